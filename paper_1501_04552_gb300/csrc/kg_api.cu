@@ -52,12 +52,14 @@ struct Ctx {
     int N = 0, NH = 0, prec = KG_DF64;
     bool cplx = false;       // complex field: full N^3 spectrum, N columns per plane
     double L = 0, dt = 0, lam = 1.0;
-    size_t nspec = 0, nphys = 0;   // complex values per spectral array, reals per physical array
+    size_t nspec = 0, nphys = 0;   // modes of the spectrum, reals per physical array
+    size_t slots = 0;              // complex values a spectral array holds (modes and padding)
     cudaStream_t own_stream = nullptr;
     const PassLaunch* pl = nullptr;
     double2* S0 = nullptr;   // FP64 state arrays; dev->phase tells which holds uh^n
     double2* S1 = nullptr;
-    void* W = nullptr;       // work array in the pass precision
+    void* W1 = nullptr;      // work arrays in the pass precision: x-lines (live between steps) and
+    void* W2 = nullptr;      // z-columns (scratch between steps, of 16 bytes a slot: FP64 scratch too)
     double2* tmp = nullptr;  // FP64 spectral scratch (set-up and read-out), allocated on demand
     double* phys = nullptr;  // physical scratch (N^3 doubles), on demand
     KgDev* dev = nullptr;
@@ -146,22 +148,18 @@ int upload_tables(Ctx* c) {
 
 int ensure_scratch(Ctx* c) {
     int rc = KG_OK;
-    if (!c->tmp) rc = dalloc(c, (void**)&c->tmp, sizeof(double2) * c->nspec, "fp64 spectral scratch");
+    if (!c->tmp) rc = dalloc(c, (void**)&c->tmp, sizeof(double2) * c->slots, "fp64 spectral scratch");
     if (!rc && !c->phys) rc = dalloc(c, (void**)&c->phys, sizeof(double) * c->nphys, "physical scratch");
     return rc;
 }
 
-// FP64 inverse of a spectral state array (phase-selected pair) into c->tmp (yz only)
+// FP64 inverse of a spectral state array (phase-selected pair) into the x-lines of c->tmp
+// (yz only), through W2
 int inverse_yz_f64(Ctx* c, const double2* src0, const double2* src1, const KgDev* sel) {
-    const int N = c->N, NH = c->NH;
+    const int N = c->N;
     cudaStream_t st = stream_of(c);
-    if (c->cplx) {
-        KG_CK(kLaunchF64.colc_from_f64(N, src0, src1, sel, c->tmp, N, (size_t)N * N, N, c->tw64, st));   // z
-        KG_CK(kLaunchF64.colc(N, +1, c->tmp, (size_t)N * N, N, N, c->tw64, st));                        // y
-        return KG_OK;
-    }
-    KG_CK(kLaunchF64.col_from_f64(N, src0, src1, sel, c->tmp, NH, (size_t)N * NH, N, c->tw64, st));   // z
-    KG_CK(kLaunchF64.col(N, +1, c->tmp, (size_t)N * NH, NH, N, c->tw64, st));                         // y
+    KG_CK((c->cplx ? kLaunchF64.zc_from_f64 : kLaunchF64.z_from_f64)(N, src0, src1, sel, c->W2, c->tw64, st));
+    KG_CK((c->cplx ? kLaunchF64.yic : kLaunchF64.yi)(N, c->W2, c->tmp, c->tw64, st));
     return KG_OK;
 }
 
@@ -286,6 +284,7 @@ int create_ctx(int N, double L, double dt, bool cplx, Ctx** out) {
     c->pl = launcher(c->prec);
     c->cplx = cplx;
     c->nspec = (size_t)N * N * (cplx ? N : c->NH);
+    c->slots = spec_slots(N, cplx);
     c->nphys = (size_t)N * N * N * (cplx ? 2 : 1);   // doubles of one physical field
     int rc = KG_OK;
 #define KG_TRY(x)              \
@@ -300,9 +299,10 @@ int create_ctx(int N, double L, double dt, bool cplx, Ctx** out) {
         cudaError_t e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking);
         if (e != cudaSuccess) KG_TRY(fail(KG_ECUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e)));
     }
-    KG_TRY(dalloc(c, (void**)&c->S0, sizeof(double2) * c->nspec, "state S0"));
-    KG_TRY(dalloc(c, (void**)&c->S1, sizeof(double2) * c->nspec, "state S1"));
-    KG_TRY(dalloc(c, &c->W, c->pl->store_bytes * c->nspec, "work array W"));
+    KG_TRY(dalloc(c, (void**)&c->S0, sizeof(double2) * c->slots, "state S0"));
+    KG_TRY(dalloc(c, (void**)&c->S1, sizeof(double2) * c->slots, "state S1"));
+    KG_TRY(dalloc(c, &c->W1, c->pl->store_bytes * c->slots, "work array W1"));
+    KG_TRY(dalloc(c, &c->W2, sizeof(double2) * c->slots, "work array W2"));
     KG_TRY(dalloc(c, (void**)&c->dev, sizeof(KgDev), "device state"));
     if (cplx) {
         c->nparts = std::max(std::max(c->pl->xc_parts(N), c->pl->updatec_parts(N)), xc_inverse_parts(N));
@@ -369,11 +369,11 @@ int init_common(int N, double L, double dt, const double* u0, const double* v0, 
                                         device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) KG_TRY(fail(KG_ECUDA, std::string("copy u0: ") + cudaGetErrorString(e)));
     }
-    // the set-up transforms run in the pass precision where it has them (double-float), with
-    // W as their work array; F^0 = R2C(lam u0^3) waits in the FP64 scratch
+    // the set-up transforms run in the pass precision where it has them (double-float), through
+    // the work arrays; F^0 = R2C(lam u0^3) waits in the FP64 scratch
     Tables tb{c->tw, c->tw64, c->coef, c->w2};
     c->scheme = g_scheme;
-    KG_TRY(init_state(N, c->prec, dt, c->lam, tb, c->phys, v0, device_ptrs, c->S0, c->S1, c->W, c->tmp, st,
+    KG_TRY(init_state(N, c->prec, dt, c->lam, tb, c->phys, v0, device_ptrs, c->S0, c->S1, c->W1, c->W2, c->tmp, st,
                       c->scheme == KG_SCHEME_COMPOSED4 ? c->kick : nullptr, true));
     KgDev d = fresh_dev();
     d.scheme = c->scheme;
@@ -412,7 +412,7 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
     // F^0 = FFT(lam |u0|^2 u0) waits in the FP64 scratch
     Tables tb{c->tw, c->tw64, c->coef, c->w2};
     rc = init_state_c(N, c->prec, dt, c->lam, tb, (double2*)c->phys, (const double2*)v0, device_ptrs, c->S0, c->S1,
-                      c->W, c->tmp, st, true);
+                      c->W1, c->W2, c->tmp, st, true);
     KgDev d = fresh_dev();
     d.complex_field = 1;
     if (!rc && cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -434,19 +434,18 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
 // (+ its finaliser), inverse z, inverse y.
 // xy = 1 or 2: the fused form (use_xy), whose first kernel runs the x pass and the forward
 // y transforms of every z-plane (after their inverse y transforms when xy = 2, i.e. on
-// every step of a kg_step call but its first); it ends with the z pass and leaves W
-// y-forward, so the caller ends the call with one inverse y pass (xy_close).  Its time
+// every step of a kg_step call but its first); it ends with the z pass and leaves W2
+// z-inverse, so the caller ends the call with one inverse y pass (xy_close).  Its time
 // goes to the x slot; the forward and inverse y slots stay empty.
 // skip_x: the x pass (and its finaliser) already ran for this step (kg_energy ran it ahead).
 int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool skip_x = false) {
-    const int N = c->N, NH = c->NH;
+    const int N = c->N;
     const double h = c->L / N;
     const double p_norm = c->lam * h * h * h / 4.0;
     const double q_norm = h * h * h * inv_n3(N);
-    // column geometry: NX columns per plane (N/2 + 1, or N for a complex field)
-    const int NX = c->cplx ? N : NH;
-    const size_t yps = (size_t)N * NX, zrs = (size_t)N * NX;
-    auto col = c->cplx ? c->pl->colc : c->pl->col;
+    auto yf = c->cplx ? c->pl->yfc : c->pl->yf;
+    auto yi = c->cplx ? c->pl->yic : c->pl->yi;
+    auto zcol = c->cplx ? c->pl->zcolc : c->pl->zcol;
     if (timed) KG_CK(cudaEventRecord(c->ev[0], st));
     if (skip_x) {
         // W already holds the x pass's output for this step; its max |u| becomes the step's
@@ -456,44 +455,44 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
                               cudaMemcpyDeviceToDevice, st));
     } else if (xy) {
         // (inverse y,) x pass, forward y of every z-plane in one cluster launch
-        KG_CK(c->pl->xy_fused(N, xy == 2, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
+        KG_CK(c->pl->xy_fused(N, xy == 2, c->W1, c->W2, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
         KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->xy_parts(N), c->dev, p_norm, st));
     } else if (c->cplx) {
-        KG_CK(c->pl->passc_x(N, MODE_STEP, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
+        KG_CK(c->pl->passc_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
         KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->xc_parts(N), c->dev, p_norm, st));
     } else {
-        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
+        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
         KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, p_norm, st));
     }
     if (timed) KG_CK(cudaEventRecord(c->ev[1], st));
-    if (!xy) KG_CK(col(N, -1, c->W, yps, NX, N, c->tw, st));                      // forward y
+    if (!xy) KG_CK(yf(N, c->W1, c->W2, c->tw, st));
     if (timed) KG_CK(cudaEventRecord(c->ev[2], st));
     const bool fused = c->pl->zstep != nullptr;
     const C4Args c4{c->kick, 3 * (N / 2) * (N / 2) + 1, {c->c4h[0], c->c4h[1], c->c4h[2]}};
     const C4Args* c4p = c->scheme == KG_SCHEME_COMPOSED4 ? &c4 : nullptr;
     if (fused) {
         // z pass: forward z FFT -> F^n, the update, inverse z FFT, in one kernel
-        KG_CK(c->pl->zstep(N, c->cplx, c->W, c->S0, c->S1, c->dev, c->part_sum, c->tw, c->coef, c->w2, 1.0 / c->dt,
+        KG_CK(c->pl->zstep(N, c->cplx, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->tw, c->coef, c->w2, 1.0 / c->dt,
                            c4p, st));
         KG_CK(launch_fin_z(c->part_sum, c->pl->zstep_parts(N, c->cplx), c->part2, c->dev, q_norm, st));
     } else {
         // the IEEE FP64 passes, bound by the FP64 pipe throughout, keep the three kernels
         // (the fused form measured slower there)
-        KG_CK(col(N, -1, c->W, NX, zrs, N, c->tw, st));                           // forward z -> F^n
+        KG_CK(zcol(N, -1, c->W2, c->tw, st));                                     // forward z -> F^n
         if (timed) KG_CK(cudaEventRecord(c->ev[3], st));
         if (c->cplx) {
-            KG_CK(c->pl->updatec(N, c->W, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, st));
+            KG_CK(c->pl->updatec(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, st));
             KG_CK(launch_fin_z(c->part_sum, c->pl->updatec_parts(N), c->part2, c->dev, q_norm, st));
         } else {
-            KG_CK(c->pl->update(N, c->W, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, c4p,
+            KG_CK(c->pl->update(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, c4p,
                                 st));
             KG_CK(launch_fin_z(c->part_sum, c->pl->update_parts(N), c->part2, c->dev, q_norm, st));
         }
         if (timed) KG_CK(cudaEventRecord(c->ev[4], st));
-        KG_CK(col(N, +1, c->W, NX, zrs, N, c->tw, st));                           // inverse z
+        KG_CK(zcol(N, +1, c->W2, c->tw, st));                                     // inverse z
     }
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    if (!xy) KG_CK(col(N, +1, c->W, yps, NX, N, c->tw, st));                      // inverse y
+    if (!xy) KG_CK(yi(N, c->W2, c->W1, c->tw, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -537,11 +536,10 @@ bool use_xy(const Ctx* c) {
            c->pl->xy_parts(c->N) > 0;
 }
 
-// the inverse y pass that ends a kg_step call of the fused form (W back to the y-inverse)
+// the inverse y pass that ends a kg_step call of the fused form (W1 back to the y-inverse)
 int xy_close(Ctx* c, cudaStream_t st, bool timed, float* ms) {
-    const int N = c->N, NX = c->NH;
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    KG_CK(c->pl->col(N, +1, c->W, (size_t)N * NX, NX, N, c->tw, st));
+    KG_CK(c->pl->yi(c->N, c->W2, c->W1, c->tw, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -596,6 +594,15 @@ int p_from_state(Ctx* c, bool older, double* out) {
     return KG_OK;
 }
 
+// a state array in the packed order [kz][ky][kx] into host memory, through the FP64 scratch
+// (enqueued: the caller synchronises)
+int state_to_host(Ctx* c, const double2* s, void* host) {
+    cudaStream_t st = stream_of(c);
+    KG_CK(launch_repack(c->N, c->cplx, true, s, c->tmp, st));
+    KG_CK(cudaMemcpyAsync(host, c->tmp, sizeof(double2) * c->nspec, cudaMemcpyDeviceToHost, st));
+    return KG_OK;
+}
+
 }  // namespace
 
 namespace kg {
@@ -628,9 +635,10 @@ int energy_composed(Ctx* c, double* E) {
     if (rc) return rc;
     KG_CK(launch_x_inverse(N, c->tmp, c->phys, c->tw64, inv_n3(N), c->part_sum, st));   // u^n, sum u^4
     KG_CK(launch_fin_sum(c->part_sum, x_inverse_parts(N), c->lam * h * h * h / 4.0, c->scal + 1, st));
-    rc = forward3d_f64(N, c->phys, c->tmp, c->tw64, 1, c->lam, st);   // F = R2C(lam u^3)
+    double2* F = (double2*)c->W2;
+    rc = forward3d_f64(N, c->phys, c->tmp, F, c->tw64, 1, c->lam, st);   // F = R2C(lam u^3)
     if (rc) return rc;
-    KG_CK(launch_energy_c4(N, c->S0, c->S1, c->tmp, c->kick, c->w2, c->part_sum, kStrideCtas, st));
+    KG_CK(launch_energy_c4(N, c->S0, c->S1, F, c->kick, c->w2, c->part_sum, kStrideCtas, st));
     KG_CK(launch_fin_sum(c->part_sum, kStrideCtas, h * h * h * inv_n3(N), c->scal, st));
     double v[2];
     KG_CK(cudaMemcpyAsync(v, c->scal, sizeof(v), cudaMemcpyDeviceToHost, st));
@@ -758,7 +766,7 @@ int kg_energy(double* E) {
         const int one = 1;
         KG_CK(cudaMemcpyAsync(reinterpret_cast<char*>(c->dev) + offsetof(KgDev, record_p), &one, sizeof(int),
                               cudaMemcpyHostToDevice, st));
-        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
+        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
         KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, c->lam * h * h * h / 4.0, st));
         c->x_ahead = true;
         KgDev d2;
@@ -768,12 +776,12 @@ int kg_energy(double* E) {
         Pn = d2.P_last;
     } else if (!d.frozen) {
         if (c->cplx) {
-            KG_CK(c->pl->passc_x(N, MODE_PEEK, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
+            KG_CK(c->pl->passc_x(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
                                  st));
             KG_CK(launch_fin_peek(c->part_sum, c->part_max, c->pl->xc_parts(N), c->dev, c->lam * h * h * h / 4.0,
                                   st));
         } else {
-            KG_CK(c->pl->pass_x(N, MODE_PEEK, c->W, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
+            KG_CK(c->pl->pass_x(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
                                 st));
             KG_CK(launch_fin_peek(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, c->lam * h * h * h / 4.0,
                                   st));
@@ -804,12 +812,12 @@ int kg_fetch_device(double* d_u) {
     if (!d_u) return fail(KG_EINVAL, "output pointer is NULL");
     if (c->cplx) return fail(KG_ESTATE, "the context holds a complex field: use kg_fetch_complex");
     if (c->pl->x_readout) {
-        // read-out in the pass precision (double-float): inverse z and y of uh^n into the FP64
-        // scratch used as a W-format array, then the inverse x into d_u
-        const int N = c->N, NH = c->NH;
+        // read-out in the pass precision (double-float): inverse z of uh^n into W2, inverse y into
+        // the FP64 scratch used as x-lines of the pass precision, then the inverse x into d_u
+        const int N = c->N;
         cudaStream_t st = stream_of(c);
-        KG_CK(c->pl->col_from_f64(N, c->S0, c->S1, c->dev, c->tmp, NH, (size_t)N * NH, N, c->tw, st));
-        KG_CK(c->pl->col(N, +1, c->tmp, (size_t)N * NH, NH, N, c->tw, st));
+        KG_CK(c->pl->z_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
+        KG_CK(c->pl->yi(N, c->W2, c->tmp, c->tw, st));
         KG_CK(c->pl->x_readout(N, c->tmp, d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -849,8 +857,8 @@ int kg_fetch_complex_device(double* d_u) {
         // read-out in the pass precision (double-float), as kg_fetch_device
         const int N = c->N;
         cudaStream_t st = stream_of(c);
-        KG_CK(c->pl->colc_from_f64(N, c->S0, c->S1, c->dev, c->tmp, N, (size_t)N * N, N, c->tw, st));
-        KG_CK(c->pl->colc(N, +1, c->tmp, (size_t)N * N, N, N, c->tw, st));
+        KG_CK(c->pl->zc_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
+        KG_CK(c->pl->yic(N, c->W2, c->tmp, c->tw, st));
         KG_CK(c->pl->xc_readout(N, c->tmp, (double2*)d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -879,10 +887,11 @@ int kg_fetch_spectral(double* a, double* b) {
     KgDev d;
     int rc = read_dev(c, &d);
     if (rc) return rc;
-    const double2* cur = d.phase ? c->S1 : c->S0;
-    const double2* old = d.phase ? c->S0 : c->S1;
-    if (a) KG_CK(cudaMemcpy(a, cur, sizeof(double2) * c->nspec, cudaMemcpyDeviceToHost));
-    if (b) KG_CK(cudaMemcpy(b, old, sizeof(double2) * c->nspec, cudaMemcpyDeviceToHost));
+    cudaStream_t st = stream_of(c);
+    if (a) rc = state_to_host(c, d.phase ? c->S1 : c->S0, a);
+    if (!rc && b) rc = state_to_host(c, d.phase ? c->S0 : c->S1, b);
+    if (rc) return rc;
+    KG_CK(cudaStreamSynchronize(st));
     return KG_OK;
 }
 
@@ -1035,12 +1044,10 @@ int kg_save_state(void* h, size_t cap, size_t* used) {
     hd.scheme = c->scheme;
     hd.payload_bytes = 2 * arr;
     unsigned char* base = (unsigned char*)h;
-    cudaStream_t st = stream_of(c);
-    const double2* cur = d.phase ? c->S1 : c->S0;
-    const double2* old = d.phase ? c->S0 : c->S1;
-    KG_CK(cudaMemcpyAsync(base + sizeof(hd), cur, arr, cudaMemcpyDeviceToHost, st));
-    KG_CK(cudaMemcpyAsync(base + sizeof(hd) + arr, old, arr, cudaMemcpyDeviceToHost, st));
-    KG_CK(cudaStreamSynchronize(st));
+    rc = state_to_host(c, d.phase ? c->S1 : c->S0, base + sizeof(hd));
+    if (!rc) rc = state_to_host(c, d.phase ? c->S0 : c->S1, base + sizeof(hd) + arr);
+    if (rc) return rc;
+    KG_CK(cudaStreamSynchronize(stream_of(c)));
     hd.checksum = kg_state_checksum(base + sizeof(hd), 2 * arr);
     std::memcpy(base, &hd, sizeof(hd));
     return KG_OK;
@@ -1083,7 +1090,7 @@ int kg_load_state(const void* h, size_t len) {
     int rc = create_ctx(hd.N, hd.L, hd.dt, cplx, &c);
     if (rc) return rc;
     c->scheme = hd.scheme;
-    const int N = c->N, NX = cplx ? N : c->NH;
+    const int N = c->N;
     cudaStream_t st = stream_of(c);
     KgDev d = fresh_dev();
     d.level = hd.level;
@@ -1096,14 +1103,14 @@ int kg_load_state(const void* h, size_t len) {
     d.Q_last_level = hd.Q_last_level;
     d.complex_field = cplx ? 1 : 0;
     d.scheme = c->scheme;
-    cudaError_t e = cudaMemcpyAsync(c->S0, base + sizeof(hd), arr, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->S1, base + sizeof(hd) + arr, arr, cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(c->tmp, base + sizeof(hd), arr, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S0, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->tmp, base + sizeof(hd) + arr, arr, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S1, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st);
-    // W = the yz inverse of uh^n in the pass precision, as the last two transforms of a step leave it
-    auto col = cplx ? c->pl->colc : c->pl->col;
-    auto col_f64 = cplx ? c->pl->colc_from_f64 : c->pl->col_from_f64;
-    if (e == cudaSuccess) e = col_f64(N, c->S0, c->S1, nullptr, c->W, NX, (size_t)N * NX, N, c->tw, st);
-    if (e == cudaSuccess) e = col(N, +1, c->W, (size_t)N * NX, NX, N, c->tw, st);
+    // W1 = the yz inverse of uh^n in the pass precision, as the last two transforms of a step leave it
+    if (e == cudaSuccess) e = (cplx ? c->pl->zc_from_f64 : c->pl->z_from_f64)(N, c->S0, c->S1, nullptr, c->W2, c->tw, st);
+    if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         destroy(c);

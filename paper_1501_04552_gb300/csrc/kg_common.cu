@@ -58,12 +58,13 @@ __global__ void __launch_bounds__(256) k_energy_c4(const double2* __restrict__ a
                                                    const double* __restrict__ w2tab, double* __restrict__ part_sum) {
     typedef ModeIndex<N, false> MI;
     __shared__ double red[96];
-    const size_t total = (size_t)MI::kModes;
+    const size_t total = (size_t)MI::kSlots;
     NSum acc;
     acc.s = 0.0;
     acc.c = 0.0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const MI mi((unsigned)i);
+        if (!mi.valid) continue;
         const double w = mi.twice ? 2.0 : 1.0;
         const double2 kc = kick0[mi.m2], ai = a[i], pi = P[i], fi = f[i];
         const double pre = pi.x + 0.5 * (kc.x * fi.x - kc.y * ai.x);
@@ -88,6 +89,16 @@ cudaError_t launch_energy_q(int N, const double2* x, const double2* y, const dou
     KG_DISPATCH_N(N, {
         if (cplx) k_energy_q<NN, true><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum);
         else k_energy_q<NN, false><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, cudaStream_t st) {
+    KG_DISPATCH_N(N, {
+        if (cplx && to_packed) k_repack<NN, true, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
+        else if (cplx) k_repack<NN, true, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
+        else if (to_packed) k_repack<NN, false, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
+        else k_repack<NN, false, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
         return cudaGetLastError();
     });
 }

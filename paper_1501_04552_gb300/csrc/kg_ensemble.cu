@@ -138,9 +138,9 @@ __global__ void k_gaussian(double* u, int N, double L, double A, double s) {
 
 // low-mode shell energies of uh^0: (h^3/N^3) sum_{shell} w_k omega_k^2 |uh_k|^2 / 2,
 // shells |m| in {0}, (0,1], (1,2], (2,4]; one CTA, one instance
-__global__ void k_shells(const double2* __restrict__ uh, int N, double L, double* __restrict__ out4) {
+template <int N>
+__global__ void k_shells(const double2* __restrict__ uh, double L, double* __restrict__ out4) {
     __shared__ double acc[4][256];
-    const int NH = N / 2 + 1;
     double loc[4] = {0, 0, 0, 0};
     const double kf = 2.0 * 3.14159265358979323846 / L;
     for (int t = threadIdx.x; t < 9 * 9 * 5; t += blockDim.x) {   // |m| <= 4 box, kx >= 0
@@ -149,7 +149,7 @@ __global__ void k_shells(const double2* __restrict__ uh, int N, double L, double
         const int sh = (m2 == 0) ? 0 : (m2 <= 1) ? 1 : (m2 <= 4) ? 2 : (m2 <= 16) ? 3 : -1;
         if (sh < 0) continue;
         const int ky = (my + N) % N, kz = (mz + N) % N;
-        const double2 v = uh[((size_t)kz * N + ky) * NH + mx];
+        const double2 v = uh[Lay<N>::zcol(ky, mx) + 8 * (size_t)kz];
         const double w = (mx == 0 || mx == N / 2) ? 1.0 : 2.0;
         loc[sh] += w * 0.5 * (1.0 + kf * kf * m2) * (v.x * v.x + v.y * v.y);
     }
@@ -217,7 +217,8 @@ struct Ens {
     unsigned long long* d_step = nullptr;
     int* d_order = nullptr;
     double* d_feat = nullptr;
-    double2* tmp = nullptr;     // FP64 spectral scratch of the largest grid
+    double2* tmp = nullptr;     // two FP64 spectral scratch arrays of the largest grid
+    double2* tmp2 = nullptr;
     double* phys = nullptr;     // physical scratch of the largest grid
     cudaStream_t stream = nullptr;
     const PassLaunch* pl = nullptr;
@@ -405,23 +406,25 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
             e->have[t] = true;
         }
     }
-    const size_t spec_max = (size_t)nmax * nmax * (nmax / 2 + 1);
+    const size_t spec_max = spec_slots(nmax, false);
     KG_ETRY(ealloc(e, (void**)&e->tmp, sizeof(double2) * spec_max, "ensemble spectral scratch"));
+    KG_ETRY(ealloc(e, (void**)&e->tmp2, sizeof(double2) * spec_max, "ensemble spectral scratch"));
     KG_ETRY(ealloc(e, (void**)&e->phys, sizeof(double) * (size_t)nmax * nmax * nmax, "ensemble physical scratch"));
     // one allocation per array class, instances at 256-byte aligned offsets
     size_t off_s = 0, off_w = 0;
     std::vector<size_t> os(count), ow(count);
     for (int i = 0; i < count; i++) {
-        const size_t ns = (size_t)Ns[i] * Ns[i] * (Ns[i] / 2 + 1);
+        const size_t ns = spec_slots(Ns[i], false);
         os[i] = off_s;
         ow[i] = off_w;
         off_s += (ns * sizeof(double2) + 255) & ~(size_t)255;
         off_w += (ns * e->pl->store_bytes + 255) & ~(size_t)255;
     }
-    char *b0 = nullptr, *b1 = nullptr, *bw = nullptr;
+    char *b0 = nullptr, *b1 = nullptr, *bw = nullptr, *bw2 = nullptr;
     KG_ETRY(ealloc(e, (void**)&b0, off_s, "ensemble S0"));
     KG_ETRY(ealloc(e, (void**)&b1, off_s, "ensemble S1"));
-    KG_ETRY(ealloc(e, (void**)&bw, off_w, "ensemble W"));
+    KG_ETRY(ealloc(e, (void**)&bw, off_w, "ensemble W1"));
+    KG_ETRY(ealloc(e, (void**)&bw2, off_w, "ensemble W2"));
     KG_ETRY(ealloc(e, (void**)&e->d_inst, sizeof(EnsInst) * count, "ensemble descriptors"));
     KG_ETRY(ealloc(e, (void**)&e->d_maxkey, sizeof(unsigned) * 2 * count, "ensemble max keys"));
     KG_ETRY(ealloc(e, (void**)&e->d_bar, sizeof(unsigned) * 2, "ensemble barrier"));
@@ -437,16 +440,16 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
         std::memset(&in, 0, sizeof(in));
         in.S0 = (double2*)(b0 + os[i]);
         in.S1 = (double2*)(b1 + os[i]);
-        in.W = (void*)(bw + ow[i]);
+        in.W1 = (void*)(bw + ow[i]);
+        in.W2 = (void*)(bw2 + ow[i]);
         in.N = N;
         in.blowup_level = -1;
         k_gaussian<<<kStrideCtas, 256, 0, e->stream>>>(e->phys, N, L, A[i], s[i]);
         if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "gaussian launch"));
-        // F^0 scratch: W itself when it holds 16-byte values, else the spectral scratch
-        double2* fbuf = e->pl->store_bytes == sizeof(double2) ? (double2*)in.W : e->tmp;
-        KG_ETRY(init_state(N, e->prec, dt, e->lam, e->tab[t], e->phys, nullptr, false, in.S0, in.S1, in.W, fbuf,
-                           e->stream));
-        k_shells<<<1, 256, 0, e->stream>>>(in.S0, N, L, e->d_feat + 4 * i);
+        // the scratch array serves as W2 (16 bytes a slot) during the set-up
+        KG_ETRY(init_state(N, e->prec, dt, e->lam, e->tab[t], e->phys, nullptr, false, in.S0, in.S1, in.W1, e->tmp,
+                           e->tmp2, e->stream));
+        (N == 64 ? k_shells<64> : k_shells<128>)<<<1, 256, 0, e->stream>>>(in.S0, L, e->d_feat + 4 * i);
         if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "shells launch"));
     }
     if (cudaMemcpyAsync(e->d_inst, e->h_inst.data(), sizeof(EnsInst) * count, cudaMemcpyHostToDevice, e->stream) != cudaSuccess ||
@@ -547,11 +550,11 @@ int kg_ens_fetch(int i, double* u) {
     KG_ECK(cudaStreamSynchronize(e->stream));
     EnsInst in;
     KG_ECK(cudaMemcpy(&in, e->d_inst + i, sizeof(EnsInst), cudaMemcpyDeviceToHost));
-    const int N = in.N, NH = N / 2 + 1;
+    const int N = in.N;
     const Tables& tb = e->tab[N == 64 ? 0 : 1];
     const double2* cur = in.phase ? in.S1 : in.S0;
-    KG_ECK(kLaunchF64.col_from_f64(N, cur, cur, nullptr, e->tmp, NH, (size_t)N * NH, N, tb.tw64, e->stream));
-    KG_ECK(kLaunchF64.col(N, +1, e->tmp, (size_t)N * NH, NH, N, tb.tw64, e->stream));
+    KG_ECK(kLaunchF64.z_from_f64(N, cur, cur, nullptr, e->tmp2, tb.tw64, e->stream));
+    KG_ECK(kLaunchF64.yi(N, e->tmp2, e->tmp, tb.tw64, e->stream));
     KG_ECK(launch_x_inverse(N, e->tmp, e->phys, tb.tw64, 1.0 / ((double)N * N * N), nullptr, e->stream));
     KG_ECK(cudaMemcpyAsync(u, e->phys, sizeof(double) * (size_t)N * N * N, cudaMemcpyDeviceToHost, e->stream));
     KG_ECK(cudaStreamSynchronize(e->stream));

@@ -23,7 +23,8 @@ constexpr int kEnsMaxInst = 1024;
 struct EnsInst {
     double2* S0;
     double2* S1;
-    void* W;
+    void* W1;            // x-lines
+    void* W2;            // z-columns (struct Lay)
     long long level;
     long long blowup_level;
     int N;
@@ -115,8 +116,8 @@ __device__ __forceinline__ bool ens_barrier(const EnsParams& p, unsigned nblocks
 }
 
 template <class P, int N, int SCHED>
-__device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, int pass, bool active_z,
-                                         int inst_phase, unsigned* maxkey_row, typename P::S* sm) {
+__device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, int pass, int inst_phase,
+                                         unsigned* maxkey_row, typename P::S* sm) {
     typedef typename P::S S;
     typedef EnsUnits<P, N, SCHED> U;
     constexpr bool RF = EnsSched<SCHED>::remfirst;
@@ -124,7 +125,8 @@ __device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, i
     const EnsInst& in = p.inst[ii];
     const EnsTab& tb = (N == 64) ? p.tab64 : p.tab128;
     const S* tw = (const S*)tb.tw;
-    S* W = (S*)in.W;
+    S* W1 = (S*)in.W1;
+    S* W2 = (S*)in.W2;
     if (pass == 0) {
         Stats<P> st;
         st.init();
@@ -135,7 +137,7 @@ __device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, i
             const int pi = threadIdx.x / XP::T, jp = threadIdx.x % XP::T;
             const size_t pair = (size_t)unit * (U::LPU / 2) + pi;
             LineSmemX<P, false> lsm{sm + pi * XP::PADN, 0u, 0u};
-            x_pair_body<P, N, MODE_STEP, LineSmemX<P, false>, RF>(W + 2 * pair * NH, jp, lsm, tw,
+            x_pair_body<P, N, MODE_STEP, LineSmemX<P, false>, RF>(W1 + 2 * pair * Lay<N>::PITCH, jp, lsm, tw,
                                                                   1.0 / ((double)N * N * N), P::from_f64(p.lam),
                                                                   false, st);
         } else {
@@ -143,7 +145,7 @@ __device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, i
             const int li = threadIdx.x / T, j = threadIdx.x % T;
             const size_t line = (size_t)unit * U::LPU + li;
             LineSmem<P> lsm{sm + li * XShape<N>::PADM};
-            x_line_body<P, N, MODE_STEP, const S*, S* __restrict__, RF>(W + line * NH, W + line * NH, j, lsm, tw,
+            x_line_body<P, N, MODE_STEP, const S*, S* __restrict__, RF>(W1 + line * Lay<N>::PITCH, W1 + line * Lay<N>::PITCH, j, lsm, tw,
                                                                         1.0 / ((double)N * N * N),
                                                                         P::from_f64(p.lam), false, st);
         }
@@ -162,17 +164,13 @@ __device__ __forceinline__ void ens_unit(const EnsParams& p, int ii, int unit, i
         const bool valid = tile_ok && kx < NH;
         ColSmem<P, C> csm{sm + sub * (N * C), c};
         if (pass == 1) {
-            col_body<P, P, P, N, -1, C, RF>(W, W, (size_t)plane * N * NH + kx, NH, valid, j, csm, tw);
+            col_body<P, P, P, N, -1, COL_YF, false, C, RF>(W1, W2, plane, kx, valid, j, csm, tw);
         } else if (pass == 3) {
-            col_body<P, P, P, N, +1, C, RF>(W, W, (size_t)plane * N * NH + kx, NH, valid, j, csm, tw);
+            col_body<P, P, P, N, +1, COL_YI, false, C, RF>(W2, W1, plane, kx, valid, j, csm, tw);
         } else {
             double2* cur = inst_phase ? in.S1 : in.S0;
             double2* old = inst_phase ? in.S0 : in.S1;
-            NSum q;
-            q.s = 0.0;
-            q.c = 0.0;
-            z_body<P, N, 0, C, RF>(W, cur, old, kx, plane, valid, j, csm, tw, tb.coef, tb.w2, p.inv_dt, active_z, false,
-                                   q);
+            z_body<P, N, C, RF>(W2, cur, old, kx, plane, valid, j, csm, tw, tb.coef);
         }
     }
 }
@@ -280,8 +278,8 @@ __global__ void __launch_bounds__(kEnsThreads, EnsMinBlocks<P>::value) k_ens_ste
             }
             const int ii = p.order_idx[lo];
             const int local = unit - s_pref[lo];
-            if (!s_n128[ii]) ens_unit<P, 64, SCHED>(p, ii, local, pass, true, s_phase0[ii], keys, sm);
-            else ens_unit<P, 128, SCHED>(p, ii, local, pass, true, s_phase0[ii], keys, sm);
+            if (!s_n128[ii]) ens_unit<P, 64, SCHED>(p, ii, local, pass, s_phase0[ii], keys, sm);
+            else ens_unit<P, 128, SCHED>(p, ii, local, pass, s_phase0[ii], keys, sm);
             __syncthreads();
         }
         if (pass == 3) break;

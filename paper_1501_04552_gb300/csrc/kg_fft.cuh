@@ -2,24 +2,23 @@
 //
 // One time step of the scheme of section 1.1.2 (Eq. (2), stepped in Fourier space
 // with the cube formed in real space, two 3D FFTs per step) is a sequence of passes
-// over the work array W (half spectrum in x, [z][y][kx] / [kz][ky][kx], kx = 0..N/2
-// fastest):
+// over two work arrays W1 and W2 (half spectrum in x, kx = 0..N/2):
 //
-//   X  : per x-line, complex-to-real inverse along x, scale 1/N^3 -> u^n on the line;
+//   X  : per x-line of W1, complex-to-real inverse along x, scale 1/N^3 -> u^n on the line;
 //        max|u|, sum u^4; F = lam u^3; real-to-complex forward along x; in place.
 //        (One line through an N/2-point complex FFT, or two lines through one N-point
 //        complex FFT.)
-//   Yf : per (z, kx) column, forward complex FFT along y, in place.
-//   Z  : per (ky, kx) column, forward complex FFT along z -> F^n_k; per mode, the FP64
+//   Yf : per (z, kx) column, forward complex FFT along y, W1 -> W2.
+//   Z  : per (ky, kx) column of W2, forward complex FFT along z -> F^n_k; per mode, the FP64
 //        update uh^{n+1} = 2 c_k uh^n - uh^{n-1} + 2 beta_k F^n_k written over uh^{n-1},
 //        optional Q^{n+1/2} partial sums; inverse complex FFT along z of uh^{n+1}, in
 //        place (one kernel; the IEEE FP64 passes run the three parts as kernels Zf, U, Zi).
-//   Yi : per (z, kx) column, inverse complex FFT along y, in place.
+//   Yi : per (z, kx) column, inverse complex FFT along y, W2 -> W1.
 //
-// The pencil transposes of a distributed 3D FFT become strided column accesses:
-// a column tile is C consecutive kx columns (C * element = 128 bytes, one full
-// line per row) by all N rows, held in registers (8 values per thread) and in
-// shared memory between radix stages.
+// The pencil transposes of a distributed 3D FFT become a change of layout that the y
+// passes carry (struct Lay): W1 holds x-lines, W2 and the FP64 state hold z-columns.
+// A column tile is C consecutive kx columns (C * element = 64 or 128 bytes per row) by all
+// N rows, held in registers (8 values per thread) and in shared memory between radix stages.
 //
 // FFT formulation: Stockham autosort, radix 8 (last stage radix 2 or 4 when log2 n
 // is not a multiple of 3).  With T = n/8 threads per line, thread j holds the
@@ -41,6 +40,30 @@ __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_
 
 // x-pass modes: one stepping pass, or a read-only pass for P^n
 enum { MODE_STEP = 0, MODE_PEEK = 1 };
+
+// Layouts of the spectral arrays, NX = N/2 + 1 columns (N for a complex field) in TL tiles of
+// eight columns:
+//   x-lines   (W1)            [z][y][kx], rows of PITCH = 8 TL values, so that every row of a
+//                             column tile starts on its own 64- or 128-byte boundary;
+//   z-columns (W2, the state) [ky][kx / 8][kz][kx % 8]: the (ky, kx) column tile of the z pass
+//                             is one contiguous run (64 KB of state at N = 512).
+// The z pass reads and writes five arrays' worth of data against two for a y pass, and with
+// rows a whole plane (2.1 MB at N = 512) apart it reached 0.7 of the copy bandwidth; the
+// scattered rows now fall to the y passes, which write or read them at no measured cost
+// (512^3: z pass 1.696 -> 1.584 ms double-float, 0.988 -> 0.808 ms FP32, before prefetching;
+// y passes 0.568 and 0.228 ms either way).
+template <int N, bool CPLX = false>
+struct Lay {
+    static constexpr int NX = CPLX ? N : N / 2 + 1;
+    static constexpr int TL = (NX + 7) / 8;
+    static constexpr int PITCH = 8 * TL;
+    static constexpr long long kSlots = (long long)N * N * PITCH;   // values an array holds, padding included
+    // z-columns: element (ky, kx, kz); consecutive kz are 8 apart
+    static __host__ __device__ __forceinline__ size_t zcol(int ky, int kx) {
+        return (size_t)(ky * TL + (kx >> 3)) * (8 * N) + (kx & 7);
+    }
+    static constexpr size_t kKyStride = (size_t)TL * 8 * N;         // consecutive ky
+};
 
 constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n >> 1); }
 

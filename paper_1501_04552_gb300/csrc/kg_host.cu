@@ -17,44 +17,46 @@ const double kPi = 3.14159265358979323846;
         if (e_ != cudaSuccess) return set_last_error(KG_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// FP64 R2C of a physical device array into out; cube: lam u^3 instead of u
-int forward3d(int N, const double* u, double2* out, const double2* tw64, int cube, double lam, cudaStream_t st) {
-    const int NH = N / 2 + 1;
-    KG_HCK(launch_x_forward(N, u, out, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.col(N, -1, out, (size_t)N * NH, NH, N, tw64, st));   // y
-    KG_HCK(kLaunchF64.col(N, -1, out, NH, (size_t)N * NH, N, tw64, st));   // z
+// FP64 R2C of a physical device array into the z-columns of out, through the x-lines in
+// `lines`; cube: lam u^3 instead of u
+int forward3d(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+              cudaStream_t st) {
+    KG_HCK(launch_x_forward(N, u, lines, tw64, cube, lam, st));
+    KG_HCK(kLaunchF64.yf(N, lines, out, tw64, st));
+    KG_HCK(kLaunchF64.zcol(N, -1, out, tw64, st));
     return KG_OK;
 }
 // FP64 forward 3D transform of a complex physical device array (full spectrum);
 // cube: of lam |u|^2 u instead of u
-int forward3d_c(int N, const double2* u, double2* out, const double2* tw64, int cube, double lam, cudaStream_t st) {
-    KG_HCK(launch_xc_forward(N, u, out, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.colc(N, -1, out, (size_t)N * N, N, N, tw64, st));   // y
-    KG_HCK(kLaunchF64.colc(N, -1, out, N, (size_t)N * N, N, tw64, st));   // z
+int forward3d_c(int N, const double2* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+                cudaStream_t st) {
+    KG_HCK(launch_xc_forward(N, u, lines, tw64, cube, lam, st));
+    KG_HCK(kLaunchF64.yfc(N, lines, out, tw64, st));
+    KG_HCK(kLaunchF64.zcolc(N, -1, out, tw64, st));
     return KG_OK;
 }
-// forward 3D transform of a physical FP64 array in the pass precision of pl, W as the
-// work array, into the FP64 spectral array out; cube: of lam u^3 instead of u
-int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W, double2* out, const void* tw, int cube,
-                   double lam, cudaStream_t st) {
-    const int NH = N / 2 + 1;
-    KG_HCK(pl->x_setup(N, u, W, tw, cube, lam, st));
-    KG_HCK(pl->col(N, -1, W, (size_t)N * NH, NH, N, tw, st));             // y
-    KG_HCK(pl->col_to_f64(N, W, out, NH, (size_t)N * NH, N, tw, st));     // z -> FP64
+// forward 3D transform of a physical FP64 array in the pass precision of pl, through the
+// work arrays, into the FP64 spectral array out; cube: of lam u^3 instead of u
+int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W1, void* W2, double2* out, const void* tw,
+                   int cube, double lam, cudaStream_t st) {
+    KG_HCK(pl->x_setup(N, u, W1, tw, cube, lam, st));
+    KG_HCK(pl->yf(N, W1, W2, tw, st));
+    KG_HCK(pl->z_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
 // the same for a complex physical field (full spectrum)
-int forward3d_c_pass(int N, const PassLaunch* pl, const double2* u, void* W, double2* out, const void* tw, int cube,
-                     double lam, cudaStream_t st) {
-    KG_HCK(pl->xc_setup(N, u, W, tw, cube, lam, st));
-    KG_HCK(pl->colc(N, -1, W, (size_t)N * N, N, N, tw, st));              // y
-    KG_HCK(pl->colc_to_f64(N, W, out, N, (size_t)N * N, N, tw, st));      // z -> FP64
+int forward3d_c_pass(int N, const PassLaunch* pl, const double2* u, void* W1, void* W2, double2* out, const void* tw,
+                     int cube, double lam, cudaStream_t st) {
+    KG_HCK(pl->xc_setup(N, u, W1, tw, cube, lam, st));
+    KG_HCK(pl->yfc(N, W1, W2, tw, st));
+    KG_HCK(pl->zc_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
 }  // namespace
 
-int forward3d_f64(int N, const double* u, double2* out, const double2* tw64, int cube, double lam, cudaStream_t st) {
-    return forward3d(N, u, out, tw64, cube, lam, st);
+int forward3d_f64(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+                  cudaStream_t st) {
+    return forward3d(N, u, lines, out, tw64, cube, lam, st);
 }
 
 const PassLaunch* launcher_for(int prec) {
@@ -142,16 +144,15 @@ int make_kick_tables(int N, double L, double dt, const AllocFn& alloc, double2**
 }
 
 int init_state(int N, int prec, double dt, double lam, const Tables& tb, double* phys, const double* v0,
-               bool v0_on_device, double2* S0, double2* S1, void* W, double2* fbuf, cudaStream_t st,
+               bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
                const double2* kick0, bool pass_precision) {
-    const int NH = N / 2 + 1;
-    const size_t nspec = (size_t)N * N * NH, n3 = (size_t)N * N * N;
+    const size_t slots = spec_slots(N, false), n3 = (size_t)N * N * N;
     const PassLaunch* pl = launcher_for(prec);
     if (!pl) return set_last_error(KG_EINVAL, "unknown precision");
     const bool pass = pass_precision && pl->x_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
-        return pass ? forward3d_pass(N, pl, phys, W, out, tb.tw, cube, lam, st)
-                    : forward3d(N, phys, out, tb.tw64, cube, lam, st);
+        return pass ? forward3d_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
+                    : forward3d(N, phys, (double2*)W2, out, tb.tw64, cube, lam, st);
     };
     int rc = fwd(fbuf, 1);              // F^0 = R2C(lam u0^3)
     if (!rc) rc = fwd(S0, 0);           // uh^0
@@ -161,25 +162,25 @@ int init_state(int N, int prec, double dt, double lam, const Tables& tb, double*
         rc = fwd(S1, 0);                // vh^0
         if (rc) return rc;
     } else {
-        KG_HCK(cudaMemsetAsync(S1, 0, sizeof(double2) * nspec, st));
+        KG_HCK(cudaMemsetAsync(S1, 0, sizeof(double2) * slots, st));
     }
     if (kick0) KG_HCK(launch_startup_c4(N, S0, S1, fbuf, kick0, st));    // S1 = P^0
     else KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, false, st));  // S1 = uh^{-1}
-    KG_HCK(pl->col_from_f64(N, S0, S1, nullptr, W, NH, (size_t)N * NH, N, tb.tw, st));   // z inverse of uh^0
-    KG_HCK(pl->col(N, +1, W, (size_t)N * NH, NH, N, tb.tw, st));                          // y inverse
+    KG_HCK(pl->z_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));   // z inverse of uh^0
+    KG_HCK(pl->yi(N, W2, W1, tb.tw, st));                        // y inverse
     return KG_OK;
 }
 
 int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, double2* phys, const double2* v0,
-                 bool v0_on_device, double2* S0, double2* S1, void* W, double2* fbuf, cudaStream_t st,
+                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
                  bool pass_precision) {
     const size_t n3 = (size_t)N * N * N;
     const PassLaunch* pl = launcher_for(prec);
     if (!pl) return set_last_error(KG_EINVAL, "unknown precision");
     const bool pass = pass_precision && pl->xc_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
-        return pass ? forward3d_c_pass(N, pl, phys, W, out, tb.tw, cube, lam, st)
-                    : forward3d_c(N, phys, out, tb.tw64, cube, lam, st);
+        return pass ? forward3d_c_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
+                    : forward3d_c(N, phys, (double2*)W2, out, tb.tw64, cube, lam, st);
     };
     int rc = fwd(fbuf, 1);              // F^0 = FFT(lam |u0|^2 u0)
     if (!rc) rc = fwd(S0, 0);           // uh^0
@@ -192,8 +193,8 @@ int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, doubl
         KG_HCK(cudaMemsetAsync(S1, 0, sizeof(double2) * n3, st));
     }
     KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, true, st));       // S1 = uh^{-1}
-    KG_HCK(pl->colc_from_f64(N, S0, S1, nullptr, W, N, (size_t)N * N, N, tb.tw, st));   // z inverse of uh^0
-    KG_HCK(pl->colc(N, +1, W, (size_t)N * N, N, N, tb.tw, st));                         // y inverse
+    KG_HCK(pl->zc_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));          // z inverse of uh^0
+    KG_HCK(pl->yic(N, W2, W1, tb.tw, st));                               // y inverse
     return KG_OK;
 }
 

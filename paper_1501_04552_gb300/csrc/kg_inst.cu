@@ -35,22 +35,27 @@ cudaError_t x_setup(int N, const double* u, void* spec, const void* tw, int cube
 cudaError_t x_readout(int N, void* spec, double* u, const void* tw, double scale, cudaStream_t st) {
     return Lp::x_readout(N, spec, u, tw, scale, st);
 }
-cudaError_t xy_fused(int N, int do_yi, void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale,
-                     double lam, cudaStream_t st) {
-    return Lp::xy_fused(N, do_yi, W, dev, ps, pm, tw, scale, lam, st);
+cudaError_t xy_fused(int N, int do_yi, const void* W1, void* W2, KgDev* dev, double* ps, double* pm, const void* tw,
+                     double scale, double lam, cudaStream_t st) {
+    return Lp::xy_fused(N, do_yi, W1, W2, dev, ps, pm, tw, scale, lam, st);
 }
 int xy_parts(int N) { return Lp::xy_parts(N); }
 #elif KG_PART == 1
-cudaError_t col(int N, int sign, void* W, size_t ps, size_t rs, int nplanes, const void* tw, cudaStream_t st) {
-    return Lp::col(N, sign, W, ps, rs, nplanes, tw, st);
+cudaError_t yf(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
+    return Lp::yf_t<false>(N, W1, W2, tw, st);
 }
-cudaError_t col_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W, size_t ps,
-                         size_t rs, int nplanes, const void* tw, cudaStream_t st) {
-    return Lp::col_from_f64(N, src0, src1, dev, W, ps, rs, nplanes, tw, st);
+cudaError_t yi(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
+    return Lp::yi_t<false>(N, W2, W1, tw, st);
 }
-cudaError_t col_to_f64(int N, const void* W, double2* out, size_t ps, size_t rs, int nplanes, const void* tw,
+cudaError_t zcol(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
+    return Lp::zcol_t<false>(N, sign, W2, tw, st);
+}
+cudaError_t z_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2, const void* tw,
                        cudaStream_t st) {
-    return Lp::col_to_f64(N, W, out, ps, rs, nplanes, tw, st);
+    return Lp::z_from_f64_t<false>(N, src0, src1, dev, W2, tw, st);
+}
+cudaError_t z_to_f64(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
+    return Lp::z_to_f64_t<false>(N, W2, out, tw, st);
 }
 #elif KG_PART == 2
 cudaError_t zstep(int N, bool cplx, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const void* tw,
@@ -76,12 +81,21 @@ cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm
     return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, st);
 }
 int xc_parts(int N) { return Lp::xc_parts(N); }
-cudaError_t colc(int N, int sign, void* W, size_t ps, size_t rs, int nplanes, const void* tw, cudaStream_t st) {
-    return Lp::colc(N, sign, W, ps, rs, nplanes, tw, st);
+cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
+    return Lp::yf_t<true>(N, W1, W2, tw, st);
 }
-cudaError_t colc_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W, size_t ps,
-                          size_t rs, int nplanes, const void* tw, cudaStream_t st) {
-    return Lp::colc_from_f64(N, src0, src1, dev, W, ps, rs, nplanes, tw, st);
+cudaError_t yic(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
+    return Lp::yi_t<true>(N, W2, W1, tw, st);
+}
+cudaError_t zcolc(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
+    return Lp::zcol_t<true>(N, sign, W2, tw, st);
+}
+cudaError_t zc_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2, const void* tw,
+                       cudaStream_t st) {
+    return Lp::z_from_f64_t<true>(N, src0, src1, dev, W2, tw, st);
+}
+cudaError_t zc_to_f64(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
+    return Lp::z_to_f64_t<true>(N, W2, out, tw, st);
 }
 cudaError_t updatec(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                     const double* w2, double inv_dt, cudaStream_t st) {
@@ -93,10 +107,6 @@ cudaError_t xc_setup(int N, const double2* u, void* spec, const void* tw, int cu
 }
 cudaError_t xc_readout(int N, void* spec, double2* u, const void* tw, double scale, cudaStream_t st) {
     return Lp::xc_readout(N, spec, u, tw, scale, st);
-}
-cudaError_t colc_to_f64(int N, const void* W, double2* out, size_t ps, size_t rs, int nplanes, const void* tw,
-                        cudaStream_t st) {
-    return Lp::colc_to_f64(N, W, out, ps, rs, nplanes, tw, st);
 }
 #elif KG_PART == 4
 cudaError_t ens_step(const EnsParams& p, int grid, int sched, cudaStream_t st) {

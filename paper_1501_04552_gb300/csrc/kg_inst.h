@@ -21,22 +21,26 @@
     KG_INST_FN(x_readout) x_readout;                                                   \
     KG_INST_FN(xy_fused) xy_fused;                                                     \
     KG_INST_FN(xy_parts) xy_parts;                                                     \
-    KG_INST_FN(col) col;                      /* share 1: column passes */             \
-    KG_INST_FN(col_from_f64) col_from_f64;                                             \
-    KG_INST_FN(col_to_f64) col_to_f64;                                                 \
+    KG_INST_FN(yf) yf;                        /* share 1: column passes */             \
+    KG_INST_FN(yi) yi;                                                                 \
+    KG_INST_FN(zcol) zcol;                                                             \
+    KG_INST_FN(z_from_f64) z_from_f64;                                                 \
+    KG_INST_FN(z_to_f64) z_to_f64;                                                     \
     KG_INST_FN(zstep) zstep;                  /* share 2: z pass and update */         \
     KG_INST_FN(zstep_parts) zstep_parts;                                               \
     KG_INST_FN(update) update;                                                         \
     KG_INST_FN(update_parts) update_parts;                                             \
     KG_INST_FN(passc_x) passc_x;              /* share 3: complex field */             \
     KG_INST_FN(xc_parts) xc_parts;                                                     \
-    KG_INST_FN(colc) colc;                                                             \
-    KG_INST_FN(colc_from_f64) colc_from_f64;                                           \
+    KG_INST_FN(yfc) yfc;                                                               \
+    KG_INST_FN(yic) yic;                                                               \
+    KG_INST_FN(zcolc) zcolc;                                                           \
+    KG_INST_FN(zc_from_f64) zc_from_f64;                                               \
     KG_INST_FN(updatec) updatec;                                                       \
     KG_INST_FN(updatec_parts) updatec_parts;                                           \
     KG_INST_FN(xc_setup) xc_setup;                                                     \
     KG_INST_FN(xc_readout) xc_readout;                                                 \
-    KG_INST_FN(colc_to_f64) colc_to_f64;                                               \
+    KG_INST_FN(zc_to_f64) zc_to_f64;                                                   \
     KG_INST_FN(ens_step) ens_step;            /* share 4: ensemble step */             \
     KG_INST_FN(ens_blocks_per_sm) ens_blocks_per_sm;                                   \
     }

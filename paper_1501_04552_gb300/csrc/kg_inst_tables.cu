@@ -6,9 +6,9 @@
 namespace kg {
 
 #define KG_TABLE_COMMON(ns, S)                                                                                 \
-    &ns::pass_x, &ns::col, &ns::col_from_f64, &ns::update, &ns::update_parts, &ns::ens_step,                 \
-        &ns::ens_blocks_per_sm, &ns::x_parts, S, &ns::passc_x, &ns::xc_parts, &ns::colc, &ns::colc_from_f64, \
-        &ns::updatec, &ns::updatec_parts
+    &ns::pass_x, &ns::yf, &ns::yi, &ns::zcol, &ns::z_from_f64, &ns::update, &ns::update_parts, &ns::ens_step, \
+        &ns::ens_blocks_per_sm, &ns::x_parts, S, &ns::passc_x, &ns::xc_parts, &ns::yfc, &ns::yic, &ns::zcolc, \
+        &ns::zc_from_f64, &ns::updatec, &ns::updatec_parts
 
 const PassLaunch kLaunchF64 = {
     KG_TABLE_COMMON(inst_f64, 16),
@@ -18,8 +18,8 @@ const PassLaunch kLaunchF64 = {
 const PassLaunch kLaunchDF = {
     KG_TABLE_COMMON(inst_df, 16),
     &inst_df::zstep, &inst_df::zstep_parts,
-    &inst_df::x_setup, &inst_df::x_readout, &inst_df::col_to_f64,
-    &inst_df::xc_setup, &inst_df::xc_readout, &inst_df::colc_to_f64,
+    &inst_df::x_setup, &inst_df::x_readout, &inst_df::z_to_f64,
+    &inst_df::xc_setup, &inst_df::xc_readout, &inst_df::zc_to_f64,
     nullptr, nullptr};   // no fused xy pass: the double-float passes are bound by the FMA pipes, not HBM
 const PassLaunch kLaunchF32 = {
     KG_TABLE_COMMON(inst_f32, 8),

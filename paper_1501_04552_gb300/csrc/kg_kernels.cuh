@@ -18,7 +18,7 @@ struct XShape {
     static constexpr int M = N / 2;
     static constexpr int T = M / 8;
     static constexpr int LPC = kXThreads / T;           // lines per CTA
-    static constexpr int PADM = M + M / 8;              // padded smem slots per line
+    static constexpr int PADM = M + M / 8 + (N == 16);  // padded smem slots per line (even: a line lands in 16-byte copies)
     static_assert(T <= 32, "one line must fit in a warp");
 };
 
@@ -130,8 +130,8 @@ struct XpShape {
     static constexpr int PPC = kXThreads / T;    // pairs per CTA
     static constexpr int PADN = N + N / 8;       // padded exchange slots per pair
     static constexpr bool CTA_SYNC = T > 32;     // a pair spans more than one warp
-    static_assert(2 * PPC == XShape<N>::LPC && PPC * PADN == XShape<N>::LPC * XShape<N>::PADM,
-                  "same lines and shared memory per CTA as the one-line form");
+    static_assert(2 * PPC == XShape<N>::LPC && PPC * PADN <= XShape<N>::LPC * XShape<N>::PADM,
+                  "same lines per CTA as the one-line form, within its shared memory");
     static_assert(!CTA_SYNC || PPC <= 15, "one named barrier per pair");
 };
 
@@ -195,8 +195,7 @@ __device__ __forceinline__ void x_pair_body(typename P::S* __restrict__ L1, int 
                                             bool want_sum, Stats<P>& st) {
     typedef typename P::R R;
     typedef cx<R> C;
-    constexpr int NH = N / 2 + 1;
-    typename P::S* __restrict__ L2 = L1 + NH;
+    typename P::S* __restrict__ L2 = L1 + Lay<N>::PITCH;
     C v[8];
     x_pair_load<P, N>(L1, L2, j, v);
 #pragma unroll 1
@@ -221,18 +220,6 @@ __device__ __forceinline__ void x_pair_body(typename P::S* __restrict__ L1, int 
         }
     }
     if (MODE == MODE_STEP) x_pair_unpack<P, N>(L1, L2, j, lsm, v);
-}
-
-// one element global -> shared without registers (8- or 16-byte values)
-template <class S>
-__device__ __forceinline__ void cp_async_elem(S* smem, const S* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    if constexpr (sizeof(S) == 16) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-    } else {
-        static_assert(sizeof(S) == 8, "8- or 16-byte elements");
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-    }
 }
 
 // The double-float and FP64 passes take x-lines in pairs (x_pair_body): fewer
@@ -281,19 +268,20 @@ struct XPipelined<PrecF64> {
     static constexpr bool value = false;
 };
 
-// Pass X.  A batch is LPC consecutive x-lines, one contiguous run of LPC (N/2+1) values
-// of W; a landed batch serves as the lines' FFT exchange space.  Each CTA writes one
-// max key and (when wanted) one Sigma u^4 partial.
+// Pass X.  A batch is LPC consecutive x-lines of W1 (rows of PITCH values, 16-byte aligned, so
+// a line lands in 16-byte copies: two FP32 values each); a landed batch serves as the lines'
+// FFT exchange space.  Each CTA writes one max key and (when wanted) one Sigma u^4 partial.
 template <class P, int N, int MODE>
 __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(typename P::S* __restrict__ W, KgDev* __restrict__ dev,
                                                       double* __restrict__ part_sum, double* __restrict__ part_max,
                                                       const typename P::S* __restrict__ tw, double scale, double lam) {
     typedef typename P::S S;
     typedef XShape<N> X;
-    constexpr int T = X::T, NH = N / 2 + 1, LPC = X::LPC, PADM = X::PADM;
+    constexpr int T = X::T, NH = N / 2 + 1, LPC = X::LPC, PADM = X::PADM, PITCH = Lay<N>::PITCH;
     constexpr int NB = N * N / LPC;     // batches
-    constexpr int CHUNK = LPC * NH;     // values of one batch
-    static_assert(PADM >= NH, "a line lands in its exchange slot");
+    constexpr int VPC = 16 / (int)sizeof(S);              // values per 16-byte copy
+    constexpr int CPL = (NH + VPC - 1) / VPC;             // copies per line (the last may bring one slot of padding)
+    static_assert(PADM >= CPL * VPC && PADM % VPC == 0 && PITCH >= CPL * VPC, "a line lands in its exchange slot");
     extern __shared__ __align__(16) unsigned char smraw[];
     S* buf = reinterpret_cast<S*>(smraw);   // (2 when pipelined) x LPC x PADM values
     __shared__ double red[96];
@@ -309,17 +297,17 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
         const int pi = threadIdx.x / XP::T, jp = threadIdx.x % XP::T;
         const size_t pair = (size_t)blockIdx.x * XP::PPC + pi;
         LineSmemX<P, XP::CTA_SYNC> lsm{buf + pi * XP::PADN, 1u + (unsigned)pi, (unsigned)XP::T};
-        x_pair_body<P, N, MODE>(W + 2 * pair * NH, jp, lsm, tw, scale, rlam, want_sum, st);
+        x_pair_body<P, N, MODE>(W + 2 * pair * PITCH, jp, lsm, tw, scale, rlam, want_sum, st);
     } else if constexpr (!XPipelined<P>::value) {
         const size_t line = (size_t)blockIdx.x * LPC + li;
         LineSmem<P> lsm{buf + li * PADM};
-        x_line_body<P, N, MODE>(W + line * NH, W + line * NH, j, lsm, tw, scale, rlam, want_sum, st);
+        x_line_body<P, N, MODE>(W + line * PITCH, W + line * PITCH, j, lsm, tw, scale, rlam, want_sum, st);
     } else {
         auto issue = [&](int batch, S* dst) {
-            const S* src = W + (size_t)batch * CHUNK;
-            for (int e = threadIdx.x; e < CHUNK; e += kXThreads) {
-                const int l = e / NH;
-                cp_async_elem(dst + l * PADM + (e - l * NH), src + e);
+            const S* src = W + (size_t)batch * LPC * PITCH;
+            for (int e = threadIdx.x; e < LPC * CPL; e += kXThreads) {
+                const int l = e / CPL, k = (e - l * CPL) * VPC;
+                cp_async16(dst + l * PADM + k, src + l * PITCH + k);
             }
         };
         int b = blockIdx.x;
@@ -332,7 +320,7 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
             cp_async_wait_1();
             __syncthreads();
             LineSmem<P> lsm{cur + li * PADM};
-            x_line_body<P, N, MODE>(cur + li * PADM, W + ((size_t)b * LPC + li) * NH, j, lsm, tw, scale, rlam, want_sum,
+            x_line_body<P, N, MODE>(cur + li * PADM, W + ((size_t)b * LPC + li) * PITCH, j, lsm, tw, scale, rlam, want_sum,
                                     st);
             __syncthreads();   // the buffer is the target of the copy issued next iteration
         }
@@ -360,51 +348,77 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
 }
 
 // ---------------------------------------------------------------------------
-// Column FFT: C consecutive kx columns of one plane, all N rows, in place or
-// from a source array in another storage format (set-up / read-out).
-// Y passes: plane = z, plane stride N*NH, row stride NH.
-// Z passes: plane = ky, plane stride NH, row stride N*NH.
+// Column FFT: C consecutive kx columns of one plane, all N rows (layouts: struct Lay).
+// COL_YF: plane z, x-lines -> z-columns; COL_YI: plane z, z-columns -> x-lines;
+// COL_Z: plane ky, z-columns, in place or between storage formats (set-up / read-out).
 // ---------------------------------------------------------------------------
+enum { COL_YF = 0, COL_YI = 1, COL_Z = 2 };
+
 template <class P>
 struct ColShape {
     static constexpr int C = 128 / (int)sizeof(typename P::S);
 };
-// Column tiles of the single-state step: 128-byte rows, except the FP32 y passes, whose
-// rows are N/2+1 values apart (the z rows are a whole plane apart): there 64-byte rows
-// gave twice the CTAs for the same occupancy and measured faster (0.227 against
-// 0.244 ms at 512^3), while every z pass and the 16-byte y passes were as fast or faster
-// with 128 bytes.
+// Column tiles of the single-state step: 128-byte rows, except the FP32 y passes (64-byte
+// rows: twice the CTAs for the same occupancy, and the width of a row of z-columns).
 template <class P, bool YPASS>
 struct ColStep {
     static constexpr int C = (YPASS && sizeof(typename P::S) == 8 ? 64 : 128) / (int)sizeof(typename P::S);
 };
 
+// where column kx of a plane starts in a source (dst == false) or destination array, and
+// the distance of its rows
+template <int N, int DIR, bool CPLX, bool DST>
+struct ColAddr {
+    typedef Lay<N, CPLX> Ly;
+    static constexpr bool kLines = DST ? DIR == COL_YI : DIR == COL_YF;   // x-lines
+    static constexpr size_t kStride = DIR == COL_Z ? 8 : kLines ? (size_t)Ly::PITCH : Ly::kKyStride;
+    static __device__ __forceinline__ size_t base(int plane, int kx) {
+        if (DIR == COL_Z) return Ly::zcol(plane, kx);
+        return kLines ? (size_t)plane * N * Ly::PITCH + kx : Ly::zcol(0, kx) + 8 * (size_t)plane;
+    }
+};
+
 // one column (T = N/8 threads, thread j) of a tile; valid == false for the columns
-// of the last tile beyond kx = N/2 (they compute on zeros and store nothing)
-template <class Pin, class P, class Pout, int N, int SIGN, int CW, bool RF = false>
-__device__ __forceinline__ void col_body(const typename Pin::S* src, typename Pout::S* dst, size_t base,
-                                         size_t row_stride, bool valid, int j, ColSmem<P, CW>& csm,
+// of the last tile beyond the plane (they compute on zeros and store nothing)
+template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, int CW, bool RF = false>
+__device__ __forceinline__ void col_body(const typename Pin::S* src, typename Pout::S* dst, int plane, int kx,
+                                         bool valid, int j, ColSmem<P, CW>& csm,
                                          const typename P::S* __restrict__ tw) {
     typedef typename P::R R;
+    typedef ColAddr<N, DIR, CPLX, false> In;
+    typedef ColAddr<N, DIR, CPLX, true> Out;
     constexpr int T = N / 8;
     cx<R> v[8];
+    {
+        const typename Pin::S* s0 = src + In::base(plane, kx);
 #pragma unroll
-    for (int s = 0; s < 8; s++) {
-        if (valid) v[s] = Convert<Pin, P>::go(Pin::load(src[base + (size_t)(j + T * s) * row_stride]));
-        else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
+        for (int s = 0; s < 8; s++) {
+            if (valid) v[s] = Convert<Pin, P>::go(Pin::load(s0[(size_t)(j + T * s) * In::kStride]));
+            else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
+        }
     }
     fft<P, N, ColSmem<P, CW>, false, RF, false, false>(v, j, tw, 1, csm, SIGN);   // outputs go to W or FP64
     if (valid) {
+        typename Pout::S* d0 = dst + Out::base(plane, kx);
 #pragma unroll
-        for (int s = 0; s < 8; s++) dst[base + (size_t)(j + T * s) * row_stride] = Pout::pack(Convert<P, Pout>::go(v[s]));
+        for (int s = 0; s < 8; s++) d0[(size_t)(j + T * s) * Out::kStride] = Pout::pack(Convert<P, Pout>::go(v[s]));
     }
 }
 
-// NC columns per plane: N/2 + 1 (half spectrum of a real field) or N (complex field)
-template <class Pin, class P, class Pout, int N, int SIGN, int NC = N / 2 + 1, int CW = ColShape<P>::C>
-__global__ void __launch_bounds__(CW * N / 8) k_col(const typename Pin::S* src, typename Pout::S* dst,
-                                                               size_t plane_stride, size_t row_stride,
-                                                               const typename P::S* __restrict__ tw) {
+// resident threads per SM a column kernel is compiled for: 1024 (64 registers) for 16-byte
+// values, 2048 (32) for FP32.  Left to itself ptxas took 74 for the double-float y passes, one
+// CTA of 512 threads per SM: 0.74 against 0.55 ms at 512^3; the FP32 ones took 0.250 ms
+// compiled for 1024 threads against 0.227.  Grids below 128^3 have too few CTAs to fill the
+// SMs anyway and keep their registers.
+template <class P, int NT, int N>
+struct ColMinBlocks {
+    static constexpr int kThreads = sizeof(typename P::S) == 8 ? 2048 : 1024;
+    static constexpr int value = N >= 128 && kThreads / NT > 1 ? kThreads / NT : 1;
+};
+
+template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, int CW>
+__global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::value) k_col(const typename Pin::S* src, typename Pout::S* dst,
+                                                    const typename P::S* __restrict__ tw) {
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
@@ -412,16 +426,14 @@ __global__ void __launch_bounds__(CW * N / 8) k_col(const typename Pin::S* src, 
     const int kx = blockIdx.x * C + c;
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
-    col_body<Pin, P, Pout, N, SIGN, C>(src, dst, (size_t)blockIdx.y * plane_stride + kx, row_stride, kx < NC, j, csm, tw);
+    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, C>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
 }
 
-// inverse column FFT from an FP64 spectral array into W (precision P); the source is
+// inverse z column FFT from an FP64 spectral array into W2 (precision P); the source is
 // src1 when dev != NULL and dev->phase == 1, src0 otherwise (the current level's array)
-template <class P, int N, int NC = N / 2 + 1, int CW = ColShape<P>::C>
-__global__ void __launch_bounds__(CW * N / 8) k_col_sel(const double2* src0, const double2* src1,
-                                                                   const KgDev* dev, typename P::S* dst,
-                                                                   size_t plane_stride, size_t row_stride,
-                                                                   const typename P::S* __restrict__ tw) {
+template <class P, int N, bool CPLX, int CW>
+__global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::value) k_col_sel(const double2* src0, const double2* src1, const KgDev* dev,
+                                                        typename P::S* dst, const typename P::S* __restrict__ tw) {
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
@@ -430,48 +442,28 @@ __global__ void __launch_bounds__(CW * N / 8) k_col_sel(const double2* src0, con
     const int kx = blockIdx.x * C + c;
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
-    col_body<PrecF64, P, P, N, +1, C>(src, dst, (size_t)blockIdx.y * plane_stride + kx, row_stride, kx < NC, j, csm, tw);
+    col_body<PrecF64, P, P, N, +1, COL_Z, CPLX, C>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
 }
 
 // ---------------------------------------------------------------------------
-// Fused z column: forward z FFT -> F^n, FP64 update, optional Q terms, inverse z FFT,
-// in one pass over W (the batched ensemble's z pass; the single-state step runs the
-// three parts as separate kernels, which measured faster at 512^3).
-// coef[m2] = (2 c_k, 2 beta_k) for integer m2 = mx^2 + my^2 + mz^2; w2[m2] = omega_k^2.
+// Fused z column of the batched ensemble: forward z FFT -> F^n, FP64 update, inverse z FFT,
+// in one pass over W2.  coef[m2] = (2 c_k, 2 beta_k) for integer m2 = mx^2 + my^2 + mz^2.
+// One (ky, kx) column (T = N/8 threads, thread j).
 // ---------------------------------------------------------------------------
-// one (ky, kx) column (T = N/8 threads, thread j); update == false leaves the state
-// untouched (a frozen instance); Q terms are added to q when want_q.
-// PF: the state rows this thread updates are prefetched into shared memory by
-// asynchronous copies issued before the forward FFT: 0 none, 1 uh^n only (st_sm holds
-// 8 nt double2, slot s nt + tid), 2 both arrays (16 nt double2, uh^n at (2s) nt + tid,
-// uh^{n-1} at (2s+1) nt + tid); nt = threads of the CTA, tid = this thread's slot.
-template <class P, int N, int PF = 0, int CW = ColShape<P>::C, bool RF = false>
+template <class P, int N, int CW = ColShape<P>::C, bool RF = false>
 __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const double2* __restrict__ cur,
                                        double2* __restrict__ old, int kx, int ky, bool valid, int j,
                                        ColSmem<P, CW>& csm, const typename P::S* __restrict__ tw,
-                                       const double2* __restrict__ coef, const double* __restrict__ w2tab,
-                                       double inv_dt, bool update, bool want_q, NSum& q, double2* st_sm = nullptr,
-                                       int tid = 0, int nt = 0) {
+                                       const double2* __restrict__ coef) {
     typedef typename P::R R;
     typedef cx<R> Cx;
-    constexpr int T = N / 8, NH = N / 2 + 1;
-    const size_t rs = (size_t)N * NH;
-    const size_t base = (size_t)ky * NH + kx;
-
-    if (PF > 0 && valid) {
-#pragma unroll
-        for (int s = 0; s < 8; s++) {
-            const size_t idx = base + (size_t)(j + T * s) * rs;
-            cp_async16(st_sm + (size_t)(PF > 1 ? 2 * s : s) * nt + tid, cur + idx);
-            if (PF > 1) cp_async16(st_sm + (size_t)(2 * s + 1) * nt + tid, old + idx);
-        }
-    }
-    if (PF > 0) cp_async_commit();
+    constexpr int T = N / 8;
+    const size_t base = Lay<N>::zcol(ky, kx);
 
     Cx v[8];
 #pragma unroll
     for (int s = 0; s < 8; s++) {
-        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * rs]);
+        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * 8]);
         else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
     }
     // forward z transform, the update, then the inverse z transform; the double-float and
@@ -481,37 +473,28 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
     for (int dir = 0; dir < 2; dir++) {
         fft<P, N, ColSmem<P, CW>, false, RF, false>(v, j, tw, 1, csm, dir == 0 ? -1 : +1);
         if (dir == 1) break;
-        if (PF > 0) cp_async_wait_all();   // each thread reads back only its own copies
         const int my = ky <= N / 2 ? ky : ky - N;
         const int mxy2 = kx * kx + my * my;
-        const double wgt = (kx == 0 || kx == N / 2) ? 1.0 : 2.0;
 #pragma unroll
         for (int s = 0; s < 8; s++) {
             const int kz = j + T * s;
             const int mz = kz <= N / 2 ? kz : kz - N;
             const int m2 = mxy2 + mz * mz;
             if (valid) {
-                const size_t idx = base + (size_t)kz * rs;
+                const size_t idx = base + (size_t)kz * 8;
                 const double2 cf = __ldg(coef + m2);
-                const double2 a = PF > 0 ? st_sm[(size_t)(PF > 1 ? 2 * s : s) * nt + tid] : cur[idx];
-                const double2 b = PF > 1 ? st_sm[(size_t)(2 * s + 1) * nt + tid] : old[idx];
+                const double2 a = cur[idx];
+                const double2 b = old[idx];
                 double nre = P::fma_into(cf.y, v[s].re, fma(cf.x, a.x, -b.x));
                 double nim = P::fma_into(cf.y, v[s].im, fma(cf.x, a.y, -b.y));
-                if (update) old[idx] = make_double2(nre, nim);
-                if (want_q) {
-                    const double dre = (nre - a.x) * inv_dt, dim = (nim - a.y) * inv_dt;
-                    const double sre = nre + a.x, sim = nim + a.y;
-                    const double term =
-                        0.5 * (dre * dre + dim * dim) + 0.125 * __ldg(w2tab + m2) * (sre * sre + sim * sim);
-                    q.add(wgt * term);
-                }
+                old[idx] = make_double2(nre, nim);
                 v[s] = cmake<R>(P::from_f64(nre), P::from_f64(nim));
             }
         }
     }
     if (valid) {
 #pragma unroll
-        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * rs] = P::pack(v[s]);
+        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * 8] = P::pack(v[s]);
     }
 }
 
@@ -560,26 +543,27 @@ __device__ __forceinline__ double2 mode_update(cx<typename P::R> f, double2* cur
 // and uh^{n+1}_k in the pass precision on exit; the state update and the Q terms are
 // those of z_body.
 // ---------------------------------------------------------------------------
-// The mode stored at index i of a spectral array: the half spectrum of a real field
-// ([kz][ky][kx], kx = 0..N/2) or the full spectrum of a complex field (kx = 0..N-1 in
-// FFT order).  m2 = mx^2 + my^2 + mz^2 indexes the coefficient tables; w is the
-// Parseval weight of the mode in the energy sums.
+// The mode in slot i of an array of z-columns (struct Lay): the half spectrum of a real
+// field (kx = 0..N/2) or the full spectrum of a complex field (kx = 0..N-1 in FFT order).
+// m2 = mx^2 + my^2 + mz^2 indexes the coefficient tables; w is the Parseval weight of the
+// mode in the energy sums; slots of padding hold no mode (valid == false).
 template <int N, bool CPLX>
 struct ModeIndex {
-    static constexpr int NX = CPLX ? N : N / 2 + 1;
-    static constexpr long long kModes = (long long)N * N * NX;
-    static_assert(kModes < (1ll << 31), "mode indexes fit 32 bits");
-    int m2;
-    bool twice;
+    typedef Lay<N, CPLX> Ly;
+    static constexpr long long kSlots = Ly::kSlots;
+    static_assert(kSlots < (1ll << 31), "slot indexes fit 32 bits");
+    int m2, kx, ky, kz;
+    bool twice, valid;
     __device__ __forceinline__ explicit ModeIndex(unsigned i) {
-        const unsigned row = i / NX;
-        const int kx = (int)(i - row * NX);
-        const int ky = (int)(row % N);
-        const int kz = (int)(row / N);
+        const unsigned row = i >> 3, tile = row / N;
+        kz = (int)(row % N);
+        ky = (int)(tile / Ly::TL);
+        kx = (int)(tile % Ly::TL) * 8 + (int)(i & 7);
         const int mx = (CPLX && kx > N / 2) ? kx - N : kx;
         const int my = ky <= N / 2 ? ky : ky - N, mz = kz <= N / 2 ? kz : kz - N;
         m2 = mx * mx + my * my + mz * mz;
         twice = !CPLX && kx != 0 && kx != N / 2;
+        valid = kx < Ly::NX;
     }
 };
 
@@ -661,8 +645,6 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
     typedef typename P::R R;
     typedef QTerm<P> Q;
     typedef ModeIndex<N, CPLX> MI;
-    constexpr unsigned kModes = (unsigned)MI::kModes;
-    static_assert(MI::kModes < (1ll << 31), "mode indexes fit 32 bits");
     __shared__ typename Q::T red[kUpdThreads / 32];
     const bool want_q = SCHEME == 0 && kg_recording(dev);
     const bool update = dev->frozen == 0;
@@ -670,8 +652,8 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
     double2* __restrict__ old = dev->phase ? S0 : S1;
     const unsigned i = blockIdx.x * kUpdThreads + threadIdx.x;
     typename Q::T q = Q::zero();
-    if (i < kModes) {
-        const MI mi((unsigned)i);
+    const MI mi(i);
+    if (i < (unsigned)MI::kSlots && mi.valid) {
         const cx<R> f = P::load(W[i]);
         const double2 a = cur[i];
         const double2 n = mode_update<P, SCHEME>(f, cur, old, i, mi.m2, coef, c4, dev->sub, update, a);
@@ -688,12 +670,24 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
 // z pass of the single-state step in one kernel: per (ky, kx) column, the forward z
 // FFT -> F^n_k, the update of k_update (uh^{n+1} over uh^{n-1}, W <- uh^{n+1} in the pass
 // precision, Q terms on recording steps), then the inverse z FFT of uh^{n+1}.  One pass
-// over W: 2 W + 3 S per launch instead of 6 W + 3 S for the three kernels.  The state
-// rows are read with plain loads after the forward transform (staging them in shared
-// memory by cp.async before it cost more occupancy than it hid latency).
-// C columns of N rows per CTA; C = 8 (128-byte double-float rows, 64-byte FP32 rows),
-// 16 at N = 16 so that a CTA is at least one warp.
+// over W2: 2 W + 3 S per launch instead of 6 W + 3 S for the three kernels.
+// C columns of N rows per CTA; C = 8 (one tile of z-columns: the tile's W2 values and each
+// of its two state arrays are one contiguous run), 16 at N = 16 so that a CTA is at least
+// one warp.  The state is read with plain loads after the forward transform; from N = 256
+// on, where the arrays do not stay in L2, one thread has asked L2 for both runs before it
+// (one bulk prefetch each): 512^3 1.584 -> 1.500 ms double-float, 0.808 -> 0.785 ms FP32;
+// 256^3 0.185 -> 0.179 and 0.118 -> 0.106 ms.
 // ---------------------------------------------------------------------------
+// [p, p + bytes) of global memory into L2 (16-byte aligned, a multiple of 16 bytes)
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
+}
+
+template <int N>
+struct ZStepPrefetch {
+    static constexpr bool value = N >= 256;   // C == 8 there: the run is one tile
+};
+
 template <int N>
 struct ZStepShape {
     static constexpr int C = N >= 32 ? 8 : 16;
@@ -705,7 +699,7 @@ struct ZStepShape {
 template <class P, int N>
 struct ZStepMinBlocks {
     static constexpr int kThreads = (sizeof(typename P::S) == 8 && N >= 512) ? 1536 : 1024;
-    static constexpr int value = kThreads / ZStepShape<N>::NT > 1 ? kThreads / ZStepShape<N>::NT : 1;
+    static constexpr int value = N >= 128 && kThreads / ZStepShape<N>::NT > 1 ? kThreads / ZStepShape<N>::NT : 1;
 };
 
 template <class P, int N, bool CPLX = false, int SCHEME = 0>
@@ -716,22 +710,26 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     typedef typename P::R R;
     typedef typename P::S S;
     typedef QTerm<P> Q;
+    typedef Lay<N, CPLX> Ly;
     constexpr int T = N / 8, C = ZStepShape<N>::C, NT = ZStepShape<N>::NT;
-    constexpr int NX = CPLX ? N : N / 2 + 1;   // columns per plane
     extern __shared__ __align__(16) unsigned char smraw[];
     S* sm = reinterpret_cast<S*>(smraw);
     __shared__ typename Q::T red[NT / 32];
     const int c = threadIdx.x % C, j = threadIdx.x / C;
     const int kx = blockIdx.x * C + c, ky = blockIdx.y;
-    const bool valid = kx < NX;   // columns of the last tile beyond the plane compute on zeros
+    const bool valid = kx < Ly::NX;   // columns of the last tile beyond the plane compute on zeros
     ColSmem<P, C> csm{sm, c};
+    const size_t base = Ly::zcol(ky, kx);
+    if (ZStepPrefetch<N>::value && threadIdx.x == 0) {
+        prefetch_l2(S0 + base, (unsigned)(N * C * sizeof(double2)));
+        prefetch_l2(S1 + base, (unsigned)(N * C * sizeof(double2)));
+    }
     tw = stage_table(tw, sm + N * C, N);
-    const size_t rs = (size_t)N * NX, base = (size_t)ky * NX + kx;
 
     cx<R> v[8];
 #pragma unroll
     for (int s = 0; s < 8; s++) {
-        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * rs]);
+        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * 8]);
         else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
     }
     typename Q::T q = Q::zero();
@@ -760,7 +758,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
             const int mz = kz <= N / 2 ? kz : kz - N;
             const int m2 = mxy2 + mz * mz;
             if (valid) {
-                const size_t idx = base + (size_t)kz * rs;
+                const size_t idx = base + (size_t)kz * 8;
                 const double2 a = cur[idx];
                 const double2 n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a);
                 if (want_q) q = Q::add(q, Q::term(n.x, n.y, a, __ldg(w2tab + m2), qr, twice));
@@ -770,7 +768,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     }
     if (valid) {
 #pragma unroll
-        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * rs] = P::pack(v[s]);
+        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * 8] = P::pack(v[s]);
     }
     if (SCHEME == 0 && kg_recording(dev)) {
         q = block_tree_sum<Q, NT>(q, red);
@@ -895,13 +893,13 @@ __global__ void __launch_bounds__(kXThreads) k_x_forward(const double* __restric
     typedef PrecF64 P;
     typedef cx<double> C;
     typedef XShape<N> X;
-    constexpr int M = X::M, T = X::T, NH = N / 2 + 1;
+    constexpr int M = X::M, T = X::T;
     extern __shared__ __align__(16) unsigned char smraw[];
     double2* sm = reinterpret_cast<double2*>(smraw);
     const int li = threadIdx.x / T, j = threadIdx.x % T;
     const size_t line = (size_t)blockIdx.x * X::LPC + li;
     const double* __restrict__ ul = u + line * N;
-    double2* __restrict__ L = out + line * NH;
+    double2* __restrict__ L = out + line * Lay<N>::PITCH;
     LineSmem<P> lsm{sm + li * X::PADM};
     C v[8];
 #pragma unroll
@@ -940,7 +938,7 @@ __global__ void __launch_bounds__(kXThreads) k_x_inverse(const double2* __restri
     typedef PrecF64 P;
     typedef cx<double> C;
     typedef XShape<N> X;
-    constexpr int M = X::M, T = X::T, NH = N / 2 + 1;
+    constexpr int M = X::M, T = X::T;
     extern __shared__ __align__(16) unsigned char smraw[];
     double2* sm = reinterpret_cast<double2*>(smraw);
     __shared__ double red[96];
@@ -948,7 +946,7 @@ __global__ void __launch_bounds__(kXThreads) k_x_inverse(const double2* __restri
     const size_t line = (size_t)blockIdx.x * X::LPC + li;
     LineSmem<P> lsm{sm + li * X::PADM};
     C v[8];
-    x_load_c2r<P, N>(in + line * NH, j, tw, v);
+    x_load_c2r<P, N>(in + line * Lay<N>::PITCH, j, tw, v);
     fft<P, M>(v, j, tw, 2, lsm, +1);
     NSum acc;
     acc.s = 0.0;
@@ -977,7 +975,7 @@ __global__ void __launch_bounds__(kXThreads) k_x_inverse(const double2* __restri
 // Set-up and read-out along x in the pass precision, two physical x-lines per N-point
 // complex transform (the pair form of the x pass), one pair per N/8 threads:
 // FWD: physical FP64 lines u_in (lam u^3 when cube) -> their half spectra, unnormalised,
-//      in the pass precision in spec (lines of N/2 + 1);
+//      in the pass precision in spec (x-lines, struct Lay);
 // else: half spectra in spec -> physical lines times scale, FP64, into u_out.
 template <class P, int N, bool FWD>
 __global__ void __launch_bounds__(kXThreads) k_x_pair_io(const double* __restrict__ u_in, typename P::S* __restrict__ spec,
@@ -987,14 +985,14 @@ __global__ void __launch_bounds__(kXThreads) k_x_pair_io(const double* __restric
     typedef typename P::R R;
     typedef cx<R> C;
     typedef XpShape<N> X;
-    constexpr int NH = N / 2 + 1, T = X::T;
+    constexpr int T = X::T;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
     const int pi = threadIdx.x / T, j = threadIdx.x % T;
     const size_t pair = (size_t)blockIdx.x * X::PPC + pi;
     LineSmemX<P, X::CTA_SYNC> lsm{sm + pi * X::PADN, 1u + (unsigned)pi, (unsigned)T};
-    typename P::S* __restrict__ L1 = spec + 2 * pair * NH;
-    typename P::S* __restrict__ L2 = L1 + NH;
+    typename P::S* __restrict__ L1 = spec + 2 * pair * Lay<N>::PITCH;
+    typename P::S* __restrict__ L2 = L1 + Lay<N>::PITCH;
     C v[8];
     if constexpr (FWD) {
         const double* __restrict__ u1 = u_in + 2 * pair * N;
@@ -1033,9 +1031,11 @@ template <int N, bool CPLX = false>
 __global__ void k_startup(const double2* __restrict__ a, double2* __restrict__ b, const double2* __restrict__ f,
                           const double2* __restrict__ coef, double dt) {
     typedef ModeIndex<N, CPLX> MI;
-    const size_t total = (size_t)MI::kModes;
+    const size_t total = (size_t)MI::kSlots;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const double2 cf = coef[MI((unsigned)i).m2];
+        const MI mi((unsigned)i);
+        if (!mi.valid) continue;
+        const double2 cf = coef[mi.m2];
         const double c = 0.5 * cf.x, beta = 0.5 * cf.y;
         const double2 a0 = a[i], v0 = b[i], f0 = f[i];
         b[i] = make_double2(c * a0.x - dt * v0.x + beta * f0.x, c * a0.y - dt * v0.y + beta * f0.y);
@@ -1050,9 +1050,11 @@ template <int N>
 __global__ void k_startup_c4(const double2* __restrict__ a, double2* __restrict__ b, const double2* __restrict__ f,
                              const double2* __restrict__ kick0) {
     typedef ModeIndex<N, false> MI;
-    const size_t total = (size_t)MI::kModes;
+    const size_t total = (size_t)MI::kSlots;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const double2 kc = kick0[MI((unsigned)i).m2];
+        const MI mi((unsigned)i);
+        if (!mi.valid) continue;
+        const double2 kc = kick0[mi.m2];
         const double2 a0 = a[i], v0 = b[i], f0 = f[i];
         b[i] = make_double2(v0.x - 0.5 * (kc.x * f0.x - kc.y * a0.x), v0.y - 0.5 * (kc.x * f0.y - kc.y * a0.y));
     }
@@ -1065,12 +1067,13 @@ __global__ void __launch_bounds__(256) k_energy_q(const double2* __restrict__ x,
                                                   double* __restrict__ part_sum) {
     typedef ModeIndex<N, CPLX> MI;
     __shared__ double red[96];
-    const size_t total = (size_t)MI::kModes;
+    const size_t total = (size_t)MI::kSlots;
     NSum acc;
     acc.s = 0.0;
     acc.c = 0.0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const MI mi((unsigned)i);
+        if (!mi.valid) continue;
         const double w = mi.twice ? 2.0 : 1.0;
         const double2 a = x[i], b = y[i];
         const double dre = (a.x - b.x) * inv_dt, dim = (a.y - b.y) * inv_dt;
@@ -1080,6 +1083,20 @@ __global__ void __launch_bounds__(256) k_energy_q(const double2* __restrict__ x,
     double mx = 0.0;
     block_reduce<256>(acc, mx, red);
     if (threadIdx.x == 0) part_sum[blockIdx.x] = acc.value();
+}
+
+// z-columns <-> the packed order [kz][ky][kx] of checkpoints and kg_fetch_spectral
+template <int N, bool CPLX, bool TO_PACKED>
+__global__ void k_repack(const double2* __restrict__ in, double2* __restrict__ out) {
+    typedef ModeIndex<N, CPLX> MI;
+    const size_t total = (size_t)MI::kSlots;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const MI mi((unsigned)i);
+        if (!mi.valid) continue;
+        const size_t p = ((size_t)mi.kz * N + mi.ky) * MI::Ly::NX + mi.kx;
+        if (TO_PACKED) out[p] = in[i];
+        else out[i] = in[p];
+    }
 }
 
 #ifdef KG_DEFINE_COMMON_KERNELS

@@ -25,15 +25,17 @@ struct C4Args {
 
 // precision ids match KG_FP64 / KG_DF64 / KG_MIXED of kg.h
 struct PassLaunch {
-    // x pass over W in the context's precision; mode 0 step, 1 peek.  Writes nparts partials.
+    // x pass over W1 in the context's precision; mode 0 step, 1 peek.  Writes nparts partials.
     cudaError_t (*pass_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
                           double scale, double lam, cudaStream_t st);
-    // column FFT in place on W (sign -1 forward, +1 inverse)
-    cudaError_t (*col)(int N, int sign, void* W, size_t plane_stride, size_t row_stride, int nplanes, const void* tw,
-                       cudaStream_t st);
-    // inverse column FFT from an FP64 spectral source (chosen by dev->phase when src1 != NULL) into W
-    cudaError_t (*col_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W,
-                                size_t plane_stride, size_t row_stride, int nplanes, const void* tw, cudaStream_t st);
+    // forward y columns W1 (x-lines) -> W2 (z-columns), inverse y columns W2 -> W1; z columns of
+    // W2 in place (sign -1 forward, +1 inverse; FP64 only)
+    cudaError_t (*yf)(int N, const void* W1, void* W2, const void* tw, cudaStream_t st);
+    cudaError_t (*yi)(int N, const void* W2, void* W1, const void* tw, cudaStream_t st);
+    cudaError_t (*zcol)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
+    // inverse z columns from an FP64 spectral source (chosen by dev->phase when dev != NULL) into W2
+    cudaError_t (*z_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
+                              const void* tw, cudaStream_t st);
     // streaming FP64 update between a forward and an inverse z column pass; writes
     // update_parts(N) Q partials when recording; c4: the composed scheme's tables (NULL:
     // Eq. (2))
@@ -51,10 +53,11 @@ struct PassLaunch {
     cudaError_t (*passc_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
                            double scale, double lam, cudaStream_t st);
     int (*xc_parts)(int N);
-    cudaError_t (*colc)(int N, int sign, void* W, size_t plane_stride, size_t row_stride, int nplanes, const void* tw,
-                        cudaStream_t st);
-    cudaError_t (*colc_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W,
-                                 size_t plane_stride, size_t row_stride, int nplanes, const void* tw, cudaStream_t st);
+    cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, cudaStream_t st);
+    cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, cudaStream_t st);
+    cudaError_t (*zcolc)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
+    cudaError_t (*zc_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
+                               const void* tw, cudaStream_t st);
     cudaError_t (*updatec)(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* part_sum,
                            const double2* coef, const double* w2tab, double inv_dt, cudaStream_t st);
     int (*updatec_parts)(int N);
@@ -68,22 +71,20 @@ struct PassLaunch {
     // set-up and read-out transforms in the pass precision (NULL: the FP64 kernels serve):
     // x_setup: physical FP64 lines (lam u^3 when cube) -> half spectra along x in W format;
     // x_readout: W-format half spectra along x -> physical FP64 lines times scale;
-    // col_to_f64: forward column FFT of a W-format array into an FP64 spectral array
+    // z_to_f64: forward z columns of W2 into an FP64 spectral array
     cudaError_t (*x_setup)(int N, const double* u, void* spec, const void* tw, int cube, double lam, cudaStream_t st);
     cudaError_t (*x_readout)(int N, void* spec, double* u, const void* tw, double scale, cudaStream_t st);
-    cudaError_t (*col_to_f64)(int N, const void* W, double2* out, size_t plane_stride, size_t row_stride,
-                              int nplanes, const void* tw, cudaStream_t st);
+    cudaError_t (*z_to_f64)(int N, const void* W2, double2* out, const void* tw, cudaStream_t st);
     // the same for a complex field (N-point lines, N columns per plane)
     cudaError_t (*xc_setup)(int N, const double2* u, void* spec, const void* tw, int cube, double lam,
                             cudaStream_t st);
     cudaError_t (*xc_readout)(int N, void* spec, double2* u, const void* tw, double scale, cudaStream_t st);
-    cudaError_t (*colc_to_f64)(int N, const void* W, double2* out, size_t plane_stride, size_t row_stride,
-                               int nplanes, const void* tw, cudaStream_t st);
+    cudaError_t (*zc_to_f64)(int N, const void* W2, double2* out, const void* tw, cudaStream_t st);
     // inverse y, x pass and forward y of every z-plane in one launch of thread-block
     // clusters (kg_xyfuse.cuh; NULL where not built): do_yi = 0 leaves out the inverse y
-    // transforms (W already holds the y-inverse); writes xy_parts(N) partials of the x
+    // transforms (W1 holds the y-inverse; otherwise W2 is read); the result goes to W2; writes xy_parts(N) partials of the x
     // pass's statistics; cudaErrorNotSupported for grids it is not built for
-    cudaError_t (*xy_fused)(int N, int do_yi, void* W, KgDev* dev, double* part_sum, double* part_max,
+    cudaError_t (*xy_fused)(int N, int do_yi, const void* W1, void* W2, KgDev* dev, double* part_sum, double* part_max,
                             const void* tw, double scale, double lam, cudaStream_t st);
     int (*xy_parts)(int N);
 };
@@ -91,6 +92,12 @@ struct PassLaunch {
 extern const PassLaunch kLaunchF64;
 extern const PassLaunch kLaunchDF;
 extern const PassLaunch kLaunchF32;
+
+// values a spectral array holds, padding included (struct Lay)
+inline size_t spec_slots(int N, bool cplx) { return (size_t)N * N * (cplx ? N : (N / 2 + 8) / 8 * 8); }
+
+// z-columns (the layout of the state) -> the packed order [kz][ky][kx], or back
+cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, cudaStream_t st);
 
 // FP64 set-up / read-out launchers
 cudaError_t launch_x_forward(int N, const double* u, double2* out, const double2* tw, int cube, double lam,
@@ -124,8 +131,10 @@ cudaError_t launch_fin_sum(const double* ps, int count, double norm, double* out
 // the synchronised velocity p formed from the stored P, F = R2C(lam u^3) and the first kick table
 cudaError_t launch_energy_c4(int N, const double2* a, const double2* P, const double2* f, const double2* kick0,
                              const double* w2tab, double* part_sum, int nparts, cudaStream_t st);
-// FP64 forward 3D transform of a physical array (cube: of lam u^3 instead of u)
-int forward3d_f64(int N, const double* u, double2* out, const double2* tw64, int cube, double lam, cudaStream_t st);
+// FP64 forward 3D transform of a physical array (cube: of lam u^3 instead of u) into z-columns;
+// lines: FP64 spectral scratch for the x-lines
+int forward3d_f64(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+                  cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // shared host helpers (kg_host.cu)
@@ -148,18 +157,18 @@ int make_kick_tables(int N, double L, double dt, const AllocFn& alloc, double2**
 
 // Set-up of one state from the physical field in phys (N^3 doubles, overwritten):
 // S0 = uh^0, S1 = uh^{-1} (startup level of Eq. (2)) or, with kick0 (the composed
-// scheme's first merged-kick table), S1 = P^0; W = yz-inverse of uh^0 in the pass
-// precision; fbuf is an FP64 spectral scratch (may alias W when W holds 16-byte values,
-// unless pass_precision).  The transforms run in FP64, or with pass_precision (and a
-// precision that has x_setup) in the pass precision with W as their work array.
+// scheme's first merged-kick table), S1 = P^0; W1 = yz-inverse of uh^0 in the pass
+// precision.  W2 and fbuf are scratch of 16 bytes per slot (W2 is the step's second work
+// array).  The transforms run in FP64, or with pass_precision (and a precision that has
+// x_setup) in the pass precision through W1 and W2.
 int init_state(int N, int prec, double dt, double lam, const Tables& tb, double* phys, const double* v0,
-               bool v0_on_device, double2* S0, double2* S1, void* W, double2* fbuf, cudaStream_t st,
+               bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
                const double2* kick0 = nullptr, bool pass_precision = false);
 
-// the same for a complex field: phys and v0 hold N^3 complex values, S0, S1, W and fbuf
+// the same for a complex field: phys and v0 hold N^3 complex values, the spectral arrays
 // the full N^3 spectrum
 int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, double2* phys, const double2* v0,
-                 bool v0_on_device, double2* S0, double2* S1, void* W, double2* fbuf, cudaStream_t st,
+                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
                  bool pass_precision = false);
 
 // record a failure for kg_last_error(); returns code

@@ -92,46 +92,57 @@ struct Launchers {
         KG_DISPATCH_N(N, return x_grid_n<NN>());
     }
 
-    template <int N, int SIGN, int NC = N / 2 + 1, int C = ColShape<P>::C>
-    static cudaError_t col_n(void* W, size_t pstride, size_t rstride, int nplanes, const void* tw, cudaStream_t st) {
+    // column passes (k_col): Pin -> Pout in the layouts of direction DIR
+    template <class Pin, class Pout, int N, int SIGN, int DIR, bool CPLX, int C>
+    static cudaError_t col_n(const void* src, void* dst, const void* tw, cudaStream_t st) {
         const size_t smem = (size_t)(N * C + N) * sizeof(S);
-        auto kern = k_col<P, P, P, N, SIGN, NC, C>;
+        auto kern = k_col<Pin, P, Pout, N, SIGN, DIR, CPLX, C>;
         cudaError_t e = set_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        dim3 grid((NC + C - 1) / C, nplanes);
-        kern<<<grid, C * N / 8, smem, st>>>((const S*)W, (S*)W, pstride, rstride, (const S*)tw);
+        dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N);
+        kern<<<grid, C * N / 8, smem, st>>>((const typename Pin::S*)src, (typename Pout::S*)dst, (const S*)tw);
         return cudaGetLastError();
     }
-    // y passes (row stride of one x-row) and z passes (row stride of a plane) take the
-    // tile widths of ColStep
-    template <int N, int SIGN, int NC>
-    static cudaError_t col_yz(void* W, size_t pstride, size_t rstride, int nplanes, const void* tw,
-                              cudaStream_t st) {
-        if (rstride <= (size_t)N)
-            return col_n<N, SIGN, NC, ColStep<P, true>::C>(W, pstride, rstride, nplanes, tw, st);
-        return col_n<N, SIGN, NC, ColStep<P, false>::C>(W, pstride, rstride, nplanes, tw, st);
+    template <bool CPLX>
+    static cudaError_t yf_t(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_YF, CPLX, ColStep<P, true>::C>(W1, W2, tw, st)));
     }
-    static cudaError_t col(int N, int sign, void* W, size_t pstride, size_t rstride, int nplanes, const void* tw,
-                           cudaStream_t st) {
-        if (sign < 0) { KG_DISPATCH_N(N, return (col_yz<NN, -1, NN / 2 + 1>(W, pstride, rstride, nplanes, tw, st))); }
-        KG_DISPATCH_N(N, return (col_yz<NN, +1, NN / 2 + 1>(W, pstride, rstride, nplanes, tw, st)));
+    template <bool CPLX>
+    static cudaError_t yi_t(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_YI, CPLX, ColStep<P, true>::C>(W2, W1, tw, st)));
     }
-
-    template <int N, int NC = N / 2 + 1>
-    static cudaError_t col_from_f64_n(const double2* src0, const double2* src1, const KgDev* dev, void* W,
-                                      size_t pstride, size_t rstride, int nplanes, const void* tw, cudaStream_t st) {
+    // z columns in place: FP64 only (the other precisions have the fused z pass)
+    template <bool CPLX>
+    static cudaError_t zcol_t(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
+        if constexpr (!std::is_same<P, PrecF64>::value) {
+            return cudaErrorNotSupported;
+        } else {
+            if (sign < 0) { KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, st))); }
+            KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, st)));
+        }
+    }
+    template <int N, bool CPLX>
+    static cudaError_t z_from_f64_n(const double2* src0, const double2* src1, const KgDev* dev, void* W2,
+                                    const void* tw, cudaStream_t st) {
         constexpr int C = ColShape<P>::C;
         const size_t smem = (size_t)(N * C + N) * sizeof(S);
-        auto kern = k_col_sel<P, N, NC, C>;
+        auto kern = k_col_sel<P, N, CPLX, C>;
         cudaError_t e = set_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        dim3 grid((NC + C - 1) / C, nplanes);
-        kern<<<grid, C * N / 8, smem, st>>>(src0, src1, dev, (S*)W, pstride, rstride, (const S*)tw);
+        dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N);
+        kern<<<grid, C * N / 8, smem, st>>>(src0, src1, dev, (S*)W2, (const S*)tw);
         return cudaGetLastError();
     }
-    static cudaError_t col_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W,
-                                    size_t pstride, size_t rstride, int nplanes, const void* tw, cudaStream_t st) {
-        KG_DISPATCH_N(N, return col_from_f64_n<NN>(src0, src1, dev, W, pstride, rstride, nplanes, tw, st));
+    template <bool CPLX>
+    static cudaError_t z_from_f64_t(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
+                                    const void* tw, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (z_from_f64_n<NN, CPLX>(src0, src1, dev, W2, tw, st)));
+    }
+    // forward z columns from W2 into an FP64 spectral array (pass-precision set-up)
+    template <bool CPLX>
+    static cudaError_t z_to_f64_t(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
+        if constexpr (!kPassIO) return cudaErrorNotSupported;
+        else { KG_DISPATCH_N(N, return (col_n<P, PrecF64, NN, -1, COL_Z, CPLX, ColShape<P>::C>(W2, out, tw, st))); }
     }
 
     // set-up and read-out transforms in the pass precision (double-float only: the FP32
@@ -157,25 +168,6 @@ struct Launchers {
         if constexpr (!kPassIO) return cudaErrorNotSupported;
         else { KG_DISPATCH_N(N, return (x_io_n<NN, false>(nullptr, spec, u, tw, 0, 0.0, scale, st))); }
     }
-    // forward column FFT from W (pass precision) into an FP64 spectral array
-    template <int N>
-    static cudaError_t col_to_f64_n(const void* W, double2* out, size_t pstride, size_t rstride, int nplanes,
-                                    const void* tw, cudaStream_t st) {
-        constexpr int C = ColShape<P>::C, NH = N / 2 + 1;
-        const size_t smem = (size_t)(N * C + N) * sizeof(S);
-        auto kern = k_col<P, P, PrecF64, N, -1, NH, C>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        dim3 grid((NH + C - 1) / C, nplanes);
-        kern<<<grid, C * N / 8, smem, st>>>((const S*)W, out, pstride, rstride, (const S*)tw);
-        return cudaGetLastError();
-    }
-    static cudaError_t col_to_f64(int N, const void* W, double2* out, size_t pstride, size_t rstride, int nplanes,
-                                  const void* tw, cudaStream_t st) {
-        if constexpr (!kPassIO) return cudaErrorNotSupported;
-        else { KG_DISPATCH_N(N, return (col_to_f64_n<NN>(W, out, pstride, rstride, nplanes, tw, st))); }
-    }
-
     // the same for a complex field (one N-point transform per line, N columns per plane)
     template <int N, bool FWD>
     static cudaError_t xc_io_n(const double2* u_in, void* spec, double2* u_out, const void* tw, int cube,
@@ -197,25 +189,9 @@ struct Launchers {
         if constexpr (!kPassIO) return cudaErrorNotSupported;
         else { KG_DISPATCH_N(N, return (xc_io_n<NN, false>(nullptr, spec, u, tw, 0, 0.0, scale, st))); }
     }
-    template <int N>
-    static cudaError_t colc_to_f64_n(const void* W, double2* out, size_t pstride, size_t rstride, int nplanes,
-                                     const void* tw, cudaStream_t st) {
-        constexpr int C = ColShape<P>::C;
-        const size_t smem = (size_t)(N * C + N) * sizeof(S);
-        auto kern = k_col<P, P, PrecF64, N, -1, N, C>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        dim3 grid((N + C - 1) / C, nplanes);
-        kern<<<grid, C * N / 8, smem, st>>>((const S*)W, out, pstride, rstride, (const S*)tw);
-        return cudaGetLastError();
+    static int update_parts(int N) {   // one partial per CTA over the padded slots
+        return (int)(((long long)N * N * ((N / 2 + 8) / 8 * 8) + kUpdThreads - 1) / kUpdThreads);
     }
-    static cudaError_t colc_to_f64(int N, const void* W, double2* out, size_t pstride, size_t rstride, int nplanes,
-                                   const void* tw, cudaStream_t st) {
-        if constexpr (!kPassIO) return cudaErrorNotSupported;
-        else { KG_DISPATCH_N(N, return (colc_to_f64_n<NN>(W, out, pstride, rstride, nplanes, tw, st))); }
-    }
-
-    static int update_parts(int N) { return (int)(((long long)N * N * (N / 2 + 1) + kUpdThreads - 1) / kUpdThreads); }
     template <int N>
     static cudaError_t update_n(void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                                 const double* w2, double inv_dt, const C4Args* c4, cudaStream_t st) {
@@ -256,15 +232,6 @@ struct Launchers {
         KG_DISPATCH_N(N, return passc_x_n<NN>(mode, W, dev, ps, pm, tw, scale, lam, st));
     }
     static int xc_parts(int N) { return N * N / (kXThreads / (N / 8)); }
-    static cudaError_t colc(int N, int sign, void* W, size_t pstride, size_t rstride, int nplanes, const void* tw,
-                            cudaStream_t st) {
-        if (sign < 0) { KG_DISPATCH_N(N, return (col_yz<NN, -1, NN>(W, pstride, rstride, nplanes, tw, st))); }
-        KG_DISPATCH_N(N, return (col_yz<NN, +1, NN>(W, pstride, rstride, nplanes, tw, st)));
-    }
-    static cudaError_t colc_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W,
-                                     size_t pstride, size_t rstride, int nplanes, const void* tw, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (col_from_f64_n<NN, NN>(src0, src1, dev, W, pstride, rstride, nplanes, tw, st)));
-    }
     static int updatec_parts(int N) { return (int)(((long long)N * N * N + kUpdThreads - 1) / kUpdThreads); }
     static cudaError_t updatec(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                                const double* w2, double inv_dt, cudaStream_t st) {
@@ -284,7 +251,7 @@ struct Launchers {
                                const double2* coef, const double* w2, double inv_dt, const C4Args& c4,
                                cudaStream_t st) {
         typedef ZStepShape<N> Z;
-        constexpr int NX = CPLX ? N : N / 2 + 1;
+        constexpr int NX = Lay<N, CPLX>::NX;
         const size_t smem = (size_t)(N * Z::C + N) * sizeof(S);
         auto kern = k_zstep<P, N, CPLX, SCHEME>;
         cudaError_t e = set_smem(kern, smem);
@@ -348,7 +315,7 @@ struct Launchers {
         return grid;
     }
     template <int N, bool DO_YI>
-    static cudaError_t xy_n(void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale, double lam,
+    static cudaError_t xy_n(const void* W1, void* W2, KgDev* dev, double* ps, double* pm, const void* tw, double scale, double lam,
                             cudaStream_t st) {
         const int grid = xy_grid_n<N>();
         if (grid < kXyCluster) return cudaErrorInvalidConfiguration;
@@ -357,17 +324,17 @@ struct Launchers {
         cudaLaunchConfig_t cfg = xy_config<N, DO_YI>(attr, grid, st);
         cudaError_t e = set_smem(kern, cfg.dynamicSmemBytes);
         if (e != cudaSuccess) return e;
-        return cudaLaunchKernelEx(&cfg, kern, (float2*)W, dev, ps, pm, (const float2*)tw, scale, lam);
+        return cudaLaunchKernelEx(&cfg, kern, (const float2*)W1, (float2*)W2, dev, ps, pm, (const float2*)tw, scale, lam);
     }
-    static cudaError_t xy_fused(int N, int do_yi, void* W, KgDev* dev, double* ps, double* pm, const void* tw,
-                                double scale, double lam, cudaStream_t st) {
+    static cudaError_t xy_fused(int N, int do_yi, const void* W1, void* W2, KgDev* dev, double* ps, double* pm,
+                                const void* tw, double scale, double lam, cudaStream_t st) {
         if constexpr (!std::is_same<P, PrecF32>::value) {
             return cudaErrorNotSupported;
         } else {
 #define KG_XY_CASE(NN)                                                                       \
     case NN:                                                                                 \
-        return do_yi ? xy_n<NN, true>(W, dev, ps, pm, tw, scale, lam, st)                    \
-                     : xy_n<NN, false>(W, dev, ps, pm, tw, scale, lam, st);
+        return do_yi ? xy_n<NN, true>(W1, W2, dev, ps, pm, tw, scale, lam, st)               \
+                     : xy_n<NN, false>(W1, W2, dev, ps, pm, tw, scale, lam, st);
             switch (N) {
                 KG_XY_CASE(64)
                 KG_XY_CASE(128)

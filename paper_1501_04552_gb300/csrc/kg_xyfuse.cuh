@@ -1,7 +1,7 @@
 // kg_xyfuse.cuh -- inverse y, x and forward y passes of one z-plane fused in a
 // thread-block cluster (FP32 work array).
 //
-// Between two z passes a step runs three in-place passes over W: the inverse y
+// Between two z passes a step runs three passes over a work array: the inverse y
 // transform that ends step n, then the x pass (C2R, cube of section 1.1.2's
 // nonlinearity, R2C) and the forward y transform that begin step n+1.  Each of them
 // reads and writes all of W once.  All three only mix values within one z-plane
@@ -110,17 +110,20 @@ struct ClusterLine {
     }
 };
 
-// DO_YI: start with the inverse y transforms (W holds the output of a z pass); without
-// it W already holds the y-inverse (the first step after set-up or a previous call).
+// DO_YI: start from W2 (z-columns, the output of a z pass) with the inverse y transforms;
+// without it W1 holds the y-inverse (the first step after set-up or a previous call).  The
+// planes go back to W2: a plane's z-column rows belong to its cluster alone, so reading and
+// writing them in place needs no order between clusters.
 template <int N, int CL, bool DO_YI>
 __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
-    k_xy_cluster(float2* __restrict__ W, KgDev* __restrict__ dev, double* __restrict__ part_sum,
+    k_xy_cluster(const float2* __restrict__ W1, float2* __restrict__ W2, KgDev* __restrict__ dev, double* __restrict__ part_sum,
                  double* __restrict__ part_max, const float2* __restrict__ tw, double scale, double lam) {
     typedef PrecF32 P;
     typedef float2 S;
     typedef cx<float> C;
     typedef XyShape<N, CL> X;
-    constexpr int NX = X::NX, CW = X::CW, LDC = X::LDC, TY = X::TY, TX = X::TX;
+    constexpr int CW = X::CW, LDC = X::LDC, TY = X::TY, TX = X::TX;
+    typedef Lay<N> Ly;
     extern __shared__ __align__(16) unsigned char smraw[];
     S* slab = reinterpret_cast<S*>(smraw);
     S* xbuf = slab + X::SLAB;
@@ -162,9 +165,10 @@ __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
 
 #pragma unroll 1
     for (int z = cid; z < N; z += nclusters) {   // the same planes for every CTA of the cluster
-        const size_t zb = (size_t)z * N * NX + c0;
         for (int row = warp; row < N; row += NWARPS)
-            for (int lc = lane; lc < ncols; lc += 32) slab[row * LDC + lc] = W[zb + (size_t)row * NX + lc];
+            for (int lc = lane; lc < ncols; lc += 32)
+                slab[row * LDC + lc] = DO_YI ? W2[Ly::zcol(row, c0 + lc) + 8 * (size_t)z]
+                                             : W1[((size_t)z * N + row) * Ly::PITCH + c0 + lc];
         __syncthreads();
         if (DO_YI) y_transforms(+1);
         cluster_barrier();   // every slab holds its columns in y
@@ -181,7 +185,8 @@ __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
         cluster_barrier();   // every remote write into this slab has landed
         y_transforms(-1);
         for (int row = warp; row < N; row += NWARPS)
-            for (int lc = lane; lc < ncols; lc += 32) W[zb + (size_t)row * NX + lc] = slab[row * LDC + lc];
+            for (int lc = lane; lc < ncols; lc += 32)
+                W2[Ly::zcol(row, c0 + lc) + 8 * (size_t)z] = slab[row * LDC + lc];
         __syncthreads();   // the slab is reloaded by the next plane
     }
 
