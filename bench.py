@@ -31,7 +31,7 @@ L_BOX = 32.0
 DT = 0.005
 ENERGY_EVERY = 10
 PRECISION = "df64"
-STEP_LAUNCHES = 7
+STEP_LAUNCHES = 4
 E2E_REPEATS = 3
 METRIC = "512^3 KG steps/s"
 L2_BYTES = 129 * 1000 * 1000          # GB300 L2
@@ -518,10 +518,9 @@ def main():
                            "l2": l2_note, "device_warmup_s": 0.5},
                 "roofline": roofline, "roofline_alu": roofline_alu, "cpu_baseline": base, "e2e": e2e,
                 "clocks": clocks,
-                # per step: x pass, its finaliser, two forward column passes, update, the
-                # second-stage Q sum, the z finaliser, two inverse column passes; per energy
-                # evaluation: the peek x pass and its finaliser
-                "gpu_launches": STEP_LAUNCHES * args.steps + 2 * len(energies),
+                # per step: x pass, forward y pass, z pass, inverse y pass (the finalisers ride in
+                # the y passes); per energy evaluation one finaliser (its x pass is the next step's)
+                "gpu_launches": STEP_LAUNCHES * args.steps + len(energies),
                 "energy_series": {"every": ENERGY_EVERY, "first": energies[0] if energies else None,
                                   "max_rel_drift": (max(abs(e - energies[0]) for e in energies) / abs(energies[0])
                                                     if energies else None)},

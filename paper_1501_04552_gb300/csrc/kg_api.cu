@@ -63,9 +63,9 @@ struct Ctx {
     double2* tmp = nullptr;  // FP64 spectral scratch (set-up and read-out), allocated on demand
     double* phys = nullptr;  // physical scratch (N^3 doubles), on demand
     KgDev* dev = nullptr;
+    KgDev* h_dev = nullptr;  // two pinned copies a finaliser can write (kg_energy)
     double* part_sum = nullptr;
     double* part_max = nullptr;
-    double* part2 = nullptr;  // second-stage partial sums of the update's Q
     int nparts = 0;
     double* scal = nullptr;  // device scalars for on-demand sums
     void* tw = nullptr;      // twiddles exp(-2 pi i j/N), j < N, in the pass precision
@@ -80,10 +80,7 @@ struct Ctx {
     bool have_E0 = false;
     double E0 = 0.0;
     cudaEvent_t ev[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    cudaGraphExec_t step_graph = nullptr;   // one captured step, replayed by kg_step
     cudaGraphExec_t xy_graph = nullptr;     // one captured step of the fused xy form (inverse y included)
-    long long launched = 0;                 // steps enqueued so far
-    bool plain_done = false;                // a step of the separate-pass form ran outside a graph
     bool x_ahead = false;                   // kg_energy ran the next step's x pass (kg_step skips it)
     long long e_level = -1;                 // level of the last kg_energy result, and the result
     double e_value = 0.0;
@@ -123,9 +120,9 @@ void destroy(Ctx* c) {
     for (void* p : c->allocs) cudaFree(p);
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
-    if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
     if (c->xy_graph) cudaGraphExecDestroy(c->xy_graph);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
+    if (c->h_dev) cudaFreeHost(c->h_dev);
     delete c;
 }
 
@@ -159,7 +156,7 @@ int inverse_yz_f64(Ctx* c, const double2* src0, const double2* src1, const KgDev
     const int N = c->N;
     cudaStream_t st = stream_of(c);
     KG_CK((c->cplx ? kLaunchF64.zc_from_f64 : kLaunchF64.z_from_f64)(N, src0, src1, sel, c->W2, c->tw64, st));
-    KG_CK((c->cplx ? kLaunchF64.yic : kLaunchF64.yi)(N, c->W2, c->tmp, c->tw64, st));
+    KG_CK((c->cplx ? kLaunchF64.yic : kLaunchF64.yi)(N, c->W2, c->tmp, c->tw64, FinArgs{}, st));
     return KG_OK;
 }
 
@@ -221,17 +218,13 @@ void release(Ctx* c, void* p, size_t bytes) {
 
 // A new run on the grid, precision and field kind of the current context keeps its
 // device buffers (several GB at 512^3, whose release and allocation cost more than the
-// set-up itself); only the tables, which depend on L and dt, and the captured step
-// graph, whose launch parameters depend on them, are rebuilt.
+// set-up itself); only the tables, which depend on L and dt, and the captured graph of the
+// fused xy form, whose launch parameters depend on them, are rebuilt.
 int reuse_ctx(Ctx* c, double L, double dt, Ctx** out) {
     cudaStream_t st = stream_of(c);
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail(KG_ECUDA, "reuse: stream sync");
-    if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
     if (c->xy_graph) cudaGraphExecDestroy(c->xy_graph);
-    c->step_graph = nullptr;
     c->xy_graph = nullptr;
-    c->launched = 0;
-    c->plain_done = false;
     c->x_ahead = false;
     c->e_level = -1;
     const int N = c->N;
@@ -313,8 +306,12 @@ int create_ctx(int N, double L, double dt, bool cplx, Ctx** out) {
     c->nparts = std::max(c->nparts, kStrideCtas);   // the on-demand Q partials
     KG_TRY(dalloc(c, (void**)&c->part_sum, sizeof(double) * c->nparts, "partials"));
     KG_TRY(dalloc(c, (void**)&c->part_max, sizeof(double) * c->nparts, "partials max"));
-    KG_TRY(dalloc(c, (void**)&c->part2, sizeof(double) * (c->nparts / 1024 + 1), "second-stage partials"));
     KG_TRY(dalloc(c, (void**)&c->scal, sizeof(double) * 8, "scalars"));
+    if (cudaMallocHost((void**)&c->h_dev, 2 * sizeof(KgDev)) != cudaSuccess) {
+        cudaGetLastError();
+        c->h_dev = nullptr;
+        KG_TRY(fail(KG_ENOMEM, "pinned run-state copies"));
+    }
     KG_TRY(upload_tables(c));
     KG_TRY(ensure_scratch(c));
     for (auto& e : c->ev) {
@@ -430,8 +427,7 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
 }
 
 // one step; with timed, CUDA events split it into six kernel groups and ms[0..5]
-// accumulate their device times: x pass (+ its finaliser), forward y, forward z, update
-// (+ its finaliser), inverse z, inverse y.
+// accumulate their device times: x pass, forward y, forward z, update, inverse z, inverse y.
 // xy = 1 or 2: the fused form (use_xy), whose first kernel runs the x pass and the forward
 // y transforms of every z-plane (after their inverse y transforms when xy = 2, i.e. on
 // every step of a kg_step call but its first); it ends with the z pass and leaves W2
@@ -447,34 +443,32 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
     auto yi = c->cplx ? c->pl->yic : c->pl->yi;
     auto zcol = c->cplx ? c->pl->zcolc : c->pl->zcol;
     if (timed) KG_CK(cudaEventRecord(c->ev[0], st));
+    // the finalisers ride in the y passes (kg_kernels.cuh), or stand alone in the fused xy form
+    FinArgs fx{FIN_X, 0, c->part_sum, c->part_max, c->dev, p_norm};
     if (skip_x) {
-        // W already holds the x pass's output for this step; its max |u| becomes the step's
-        // (k_fin_x kept it in maxabs_peek; a frozen state keeps its value, as k_fin_x would)
-        char* d = reinterpret_cast<char*>(c->dev);
-        KG_CK(cudaMemcpyAsync(d + offsetof(KgDev, maxabs_last), d + offsetof(KgDev, maxabs_peek), sizeof(double),
-                              cudaMemcpyDeviceToDevice, st));
+        fx.kind = FIN_AHEAD_DONE;   // W1 already holds the x pass's output for this step
     } else if (xy) {
         // (inverse y,) x pass, forward y of every z-plane in one cluster launch
         KG_CK(c->pl->xy_fused(N, xy == 2, c->W1, c->W2, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
-        KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->xy_parts(N), c->dev, p_norm, st));
-    } else if (c->cplx) {
-        KG_CK(c->pl->passc_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
-        KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->xc_parts(N), c->dev, p_norm, st));
+        fx.count = c->pl->xy_parts(N);
+        KG_CK(launch_fin(fx, nullptr, nullptr, st));
     } else {
-        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
-        KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, p_norm, st));
+        KG_CK((c->cplx ? c->pl->passc_x : c->pl->pass_x)(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw,
+                                                         inv_n3(N), c->lam, 0, st));
+        fx.count = c->cplx ? c->pl->xc_parts(N) : c->pl->x_parts(N);
     }
     if (timed) KG_CK(cudaEventRecord(c->ev[1], st));
-    if (!xy) KG_CK(yf(N, c->W1, c->W2, c->tw, st));
+    if (!xy) KG_CK(yf(N, c->W1, c->W2, c->tw, fx, st));
     if (timed) KG_CK(cudaEventRecord(c->ev[2], st));
     const bool fused = c->pl->zstep != nullptr;
     const C4Args c4{c->kick, 3 * (N / 2) * (N / 2) + 1, {c->c4h[0], c->c4h[1], c->c4h[2]}};
     const C4Args* c4p = c->scheme == KG_SCHEME_COMPOSED4 ? &c4 : nullptr;
+    FinArgs fz{FIN_Z, 0, c->part_sum, nullptr, c->dev, q_norm};
     if (fused) {
         // z pass: forward z FFT -> F^n, the update, inverse z FFT, in one kernel
         KG_CK(c->pl->zstep(N, c->cplx, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->tw, c->coef, c->w2, 1.0 / c->dt,
                            c4p, st));
-        KG_CK(launch_fin_z(c->part_sum, c->pl->zstep_parts(N, c->cplx), c->part2, c->dev, q_norm, st));
+        fz.count = c->pl->zstep_parts(N, c->cplx);
     } else {
         // the IEEE FP64 passes, bound by the FP64 pipe throughout, keep the three kernels
         // (the fused form measured slower there)
@@ -482,17 +476,17 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
         if (timed) KG_CK(cudaEventRecord(c->ev[3], st));
         if (c->cplx) {
             KG_CK(c->pl->updatec(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, st));
-            KG_CK(launch_fin_z(c->part_sum, c->pl->updatec_parts(N), c->part2, c->dev, q_norm, st));
+            fz.count = c->pl->updatec_parts(N);
         } else {
-            KG_CK(c->pl->update(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, c4p,
-                                st));
-            KG_CK(launch_fin_z(c->part_sum, c->pl->update_parts(N), c->part2, c->dev, q_norm, st));
+            KG_CK(c->pl->update(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, c4p, st));
+            fz.count = c->pl->update_parts(N);
         }
         if (timed) KG_CK(cudaEventRecord(c->ev[4], st));
         KG_CK(zcol(N, +1, c->W2, c->tw, st));                                     // inverse z
     }
+    if (xy) KG_CK(launch_fin(fz, nullptr, nullptr, st));
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    if (!xy) KG_CK(yi(N, c->W2, c->W1, c->tw, st));
+    if (!xy) KG_CK(yi(N, c->W2, c->W1, c->tw, fz, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -511,24 +505,6 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
     return KG_OK;
 }
 
-// capture one step (its launches) into a graph; every decision of a step is made
-// on the device from KgDev, so the same graph serves every later step
-int ensure_step_graph(Ctx* c, cudaStream_t st) {
-    if (c->step_graph) return KG_OK;
-    cudaGraph_t g = nullptr;
-    KG_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    int rc = launch_step(c, st, false, nullptr);
-    cudaError_t e = cudaStreamEndCapture(st, &g);
-    if (rc || e != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return rc ? rc : fail(KG_ECUDA, std::string("step graph capture: ") + cudaGetErrorString(e));
-    }
-    e = cudaGraphInstantiate(&c->step_graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(KG_ECUDA, std::string("step graph instantiate: ") + cudaGetErrorString(e));
-    return KG_OK;
-}
-
 // the fused xy form serves the FP32 passes of a real field under Eq. (2) from N = 64 on,
 // when kg_set_xy_fusion asked for it
 bool use_xy(const Ctx* c) {
@@ -539,7 +515,7 @@ bool use_xy(const Ctx* c) {
 // the inverse y pass that ends a kg_step call of the fused form (W1 back to the y-inverse)
 int xy_close(Ctx* c, cudaStream_t st, bool timed, float* ms) {
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    KG_CK(c->pl->yi(c->N, c->W2, c->W1, c->tw, st));
+    KG_CK(c->pl->yi(c->N, c->W2, c->W1, c->tw, FinArgs{}, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -657,11 +633,10 @@ int kg_step(int n) {
     cudaStream_t st = stream_of(c);
     long long passes = (long long)n * passes_per_step(c);
     if (c->x_ahead && passes > 0) {
-        // the first step's x pass ran in kg_energy: the rest of that step, outside the graphs
+        // the first step's x pass ran in kg_energy: the rest of that step
         c->x_ahead = false;
         const int rc = launch_step(c, st, false, nullptr, 0, true);
         if (rc) return rc;
-        c->launched++;
         passes--;
     }
     if (use_xy(c) && passes > 0) {
@@ -676,21 +651,12 @@ int kg_step(int n) {
                 if (!rc && cudaGraphLaunch(c->xy_graph, st) != cudaSuccess) rc = fail(KG_ECUDA, "cudaGraphLaunch(xy)");
             }
             if (rc) return rc;
-            c->launched++;
         }
         return xy_close(c, st, false, nullptr);
     }
     for (long long i = 0; i < passes; i++) {
-        int rc;
-        if (!c->plain_done) {
-            rc = launch_step(c, st, false, nullptr);   // first step direct: it also sets kernel attributes
-            c->plain_done = true;
-        } else {
-            rc = ensure_step_graph(c, st);
-            if (!rc && cudaGraphLaunch(c->step_graph, st) != cudaSuccess) rc = fail(KG_ECUDA, "cudaGraphLaunch(step)");
-        }
+        const int rc = launch_step(c, st, false, nullptr);
         if (rc) return rc;
-        c->launched++;
     }
     return KG_OK;
 }
@@ -706,14 +672,12 @@ int kg_step_timed(int n, float* ms) {
         c->x_ahead = false;
         const int rc = launch_step(c, st, true, ms, 0, true);
         if (rc) return rc;
-        c->launched++;
         passes--;
     }
     const bool xy = use_xy(c);
     for (long long i = 0; i < passes; i++) {
         int rc = launch_step(c, st, true, ms, xy ? (i == 0 ? 1 : 2) : 0);
         if (rc) return rc;
-        c->launched++;
     }
     if (xy && passes > 0) return xy_close(c, st, true, ms);
     return KG_OK;
@@ -727,13 +691,29 @@ int kg_energy(double* E) {
     const int N = c->N;
     const double h = c->L / N;
     cudaStream_t st = stream_of(c);
+    // P^n needs u^n.  For a real field stepped by separate passes the next step's x pass runs
+    // now with P^n recorded (it forms u^n anyway) and kg_step skips it; its finaliser also
+    // hands the host the run state before and after, so that one synchronisation serves (a
+    // frozen state changes nothing in either).  Otherwise a read-only peek pass below.
+    const double p_norm = c->lam * h * h * h / 4.0;
+    const bool ahead = !c->cplx && !use_xy(c) && !c->x_ahead;
     KgDev d;
-    int rc = read_dev(c, &d);
-    if (rc) return rc;
+    int rc;
+    if (ahead) {
+        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, 1, st));
+        c->x_ahead = true;
+        KG_CK(launch_fin(FinArgs{FIN_X_AHEAD, c->pl->x_parts(N), c->part_sum, c->part_max, c->dev, p_norm}, c->h_dev,
+                         c->h_dev + 1, st));
+        KG_CK(cudaStreamSynchronize(st));
+        d = c->h_dev[0];
+    } else {
+        rc = read_dev(c, &d);
+        if (rc) return rc;
+    }
     const long long n = d.level;
     double Q, Pm, Pn;
     if (c->e_level == n) {
-        // asked again at the same level (after an x pass run ahead W no longer holds u^n's
+        // asked again at the same level (after an x pass run ahead W1 no longer holds u^n's
         // transform to peek at): the value computed then
         *E = c->e_value;
         if (g_opt.drift_tol > 0.0 && c->have_E0 && std::fabs(*E - c->E0) > g_opt.drift_tol * std::fabs(c->E0))
@@ -759,33 +739,15 @@ int kg_energy(double* E) {
         rc = p_from_state(c, true, &Pm);
         if (rc) return rc;
     }
-    // P^n: from W (which holds the yz-inverse of uh^n) unless the state froze.  For a real
-    // field stepped by separate passes, the next step's x pass runs now with P^n recorded
-    // (it forms u^n anyway) and kg_step skips it; otherwise a read-only peek pass.
-    if (!d.frozen && !c->cplx && !use_xy(c) && !c->x_ahead) {
-        const int one = 1;
-        KG_CK(cudaMemcpyAsync(reinterpret_cast<char*>(c->dev) + offsetof(KgDev, record_p), &one, sizeof(int),
-                              cudaMemcpyHostToDevice, st));
-        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st));
-        KG_CK(launch_fin_x(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, c->lam * h * h * h / 4.0, st));
-        c->x_ahead = true;
-        KgDev d2;
-        rc = read_dev(c, &d2);
-        if (rc) return rc;
-        if (d2.P_last_level != n) return fail(KG_ECUDA, "kg_energy: the x pass run ahead recorded no P");
-        Pn = d2.P_last;
+    // P^n, unless the state froze: recorded by the x pass run ahead, or by a peek
+    if (!d.frozen && ahead) {
+        if (c->h_dev[1].P_last_level != n) return fail(KG_ECUDA, "kg_energy: the x pass run ahead recorded no P");
+        Pn = c->h_dev[1].P_last;
     } else if (!d.frozen) {
-        if (c->cplx) {
-            KG_CK(c->pl->passc_x(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
-                                 st));
-            KG_CK(launch_fin_peek(c->part_sum, c->part_max, c->pl->xc_parts(N), c->dev, c->lam * h * h * h / 4.0,
-                                  st));
-        } else {
-            KG_CK(c->pl->pass_x(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam,
-                                st));
-            KG_CK(launch_fin_peek(c->part_sum, c->part_max, c->pl->x_parts(N), c->dev, c->lam * h * h * h / 4.0,
-                                  st));
-        }
+        KG_CK((c->cplx ? c->pl->passc_x : c->pl->pass_x)(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw,
+                                                         inv_n3(N), c->lam, 0, st));
+        KG_CK(launch_fin(FinArgs{FIN_PEEK, c->cplx ? c->pl->xc_parts(N) : c->pl->x_parts(N), c->part_sum, c->part_max,
+                                 c->dev, p_norm}, nullptr, nullptr, st));
         KgDev d2;
         rc = read_dev(c, &d2);
         if (rc) return rc;
@@ -817,7 +779,7 @@ int kg_fetch_device(double* d_u) {
         const int N = c->N;
         cudaStream_t st = stream_of(c);
         KG_CK(c->pl->z_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
-        KG_CK(c->pl->yi(N, c->W2, c->tmp, c->tw, st));
+        KG_CK(c->pl->yi(N, c->W2, c->tmp, c->tw, FinArgs{}, st));
         KG_CK(c->pl->x_readout(N, c->tmp, d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -858,7 +820,7 @@ int kg_fetch_complex_device(double* d_u) {
         const int N = c->N;
         cudaStream_t st = stream_of(c);
         KG_CK(c->pl->zc_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
-        KG_CK(c->pl->yic(N, c->W2, c->tmp, c->tw, st));
+        KG_CK(c->pl->yic(N, c->W2, c->tmp, c->tw, FinArgs{}, st));
         KG_CK(c->pl->xc_readout(N, c->tmp, (double2*)d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -1110,7 +1072,7 @@ int kg_load_state(const void* h, size_t len) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st);
     // W1 = the yz inverse of uh^n in the pass precision, as the last two transforms of a step leave it
     if (e == cudaSuccess) e = (cplx ? c->pl->zc_from_f64 : c->pl->z_from_f64)(N, c->S0, c->S1, nullptr, c->W2, c->tw, st);
-    if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, st);
+    if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, FinArgs{}, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         destroy(c);

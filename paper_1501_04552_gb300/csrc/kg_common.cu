@@ -129,21 +129,8 @@ cudaError_t launch_xc_inverse(int N, const double2* in, double2* u, const double
 
 int xc_inverse_parts(int N) { return N * N / (kXThreads / (N / 8)); }
 
-cudaError_t launch_fin_x(const double* ps, const double* pm, int count, KgDev* dev, double p_norm, cudaStream_t st) {
-    k_fin_x<<<1, kFinThreads, 0, st>>>(ps, pm, count, dev, p_norm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fin_peek(const double* ps, const double* pm, int count, KgDev* dev, double p_norm,
-                            cudaStream_t st) {
-    k_fin_peek<<<1, kFinThreads, 0, st>>>(ps, pm, count, dev, p_norm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fin_z(const double* ps, int count, double* stage2, KgDev* dev, double q_norm, cudaStream_t st) {
-    const int n2 = (count + kSumThreads - 1) / kSumThreads;
-    k_sum_parts<<<n2, kSumThreads, 0, st>>>(ps, count, stage2, dev);
-    k_fin_z<<<1, kFinThreads, 0, st>>>(stage2, n2, dev, q_norm);
+cudaError_t launch_fin(const FinArgs& fin, KgDev* before, KgDev* after, cudaStream_t st) {
+    k_fin<<<1, kFinThreads, 0, st>>>(fin, before, after);
     return cudaGetLastError();
 }
 

@@ -10,39 +10,42 @@
 
 namespace kg {
 
+// threads per CTA of the stepping x pass of a complex field (as XStep)
 template <int N>
+struct XcStep {
+    static constexpr int NT = N >= 128 ? kXThreads : N >= 64 ? 128 : 32;
+};
+
+template <int N, int NT = kXThreads>
 struct XcShape {
     static constexpr int T = N / 8;             // threads per x-line
-    static constexpr int LPC = kXThreads / T;   // lines per CTA
+    static constexpr int LPC = NT / T;          // lines per CTA
     static constexpr int PADN = N + N / 8;      // padded shared-memory slots per line
     static constexpr bool CTA_SYNC = T > 32;    // a line spans more than one warp
-    static_assert(kXThreads % T == 0, "whole lines per CTA");
+    static_assert(NT % T == 0, "whole lines per CTA");
     static_assert(!CTA_SYNC || LPC <= 15, "one named barrier per line");
 };
 
-// resident CTAs per SM the complex x pass is compiled for (the largest count whose
-// register budget needs no spills, FP64 excepted)
-template <class P>
+// resident threads per SM the complex x pass is compiled for (the largest count whose
+// register budget needs no spills, FP64 excepted); as XMinBlocks below 128^3
+template <class P, int N>
 struct XcMinBlocks {
-    static constexpr int value = 4;
-};
-template <>
-struct XcMinBlocks<PrecF64> {
-    static constexpr int value = 2;
+    static constexpr int kThreads = std::is_same<P, PrecF64>::value ? 512 : 1024;
+    static constexpr int value = N >= 128 ? kThreads / XcStep<N>::NT : 1;
 };
 
 // Pass X of a complex field.  MODE_STEP: per x-line, inverse transform, scale 1/N^3 ->
 // u^n; |u|^2 keys and (when wanted) sum |u|^4; F = lam |u|^2 u; forward transform;
 // written back in place.  MODE_PEEK: inverse transform and the statistics only.
 template <class P, int N, int MODE>
-__global__ void __launch_bounds__(kXThreads, XcMinBlocks<P>::value) k_pass_xc(typename P::S* __restrict__ W, KgDev* __restrict__ dev,
-                                                         double* __restrict__ part_sum, double* __restrict__ part_max,
-                                                         const typename P::S* __restrict__ tw, double scale,
-                                                         double lam) {
+__global__ void __launch_bounds__(XcStep<N>::NT, XcMinBlocks<P, N>::value)
+    k_pass_xc(typename P::S* __restrict__ W, KgDev* __restrict__ dev, double* __restrict__ part_sum,
+              double* __restrict__ part_max, const typename P::S* __restrict__ tw, double scale, double lam, int record) {
     typedef typename P::S S;
     typedef typename P::R R;
     typedef cx<R> C;
-    typedef XcShape<N> X;
+    constexpr int NT = XcStep<N>::NT;
+    typedef XcShape<N, NT> X;
     constexpr int T = X::T;
     extern __shared__ __align__(16) unsigned char smraw[];
     S* sm = reinterpret_cast<S*>(smraw);
@@ -51,7 +54,8 @@ __global__ void __launch_bounds__(kXThreads, XcMinBlocks<P>::value) k_pass_xc(ty
     const int li = threadIdx.x / T, j = threadIdx.x % T;
     const size_t line = (size_t)blockIdx.x * X::LPC + li;
     LineSmemX<P, X::CTA_SYNC> lsm{sm + li * X::PADN, 1u + (unsigned)li, (unsigned)T};
-    const bool want_sum = (MODE == MODE_PEEK) || kg_recording(dev) || dev->record_p;
+    pdl_wait();
+    const bool want_sum = (MODE == MODE_PEEK) || record || kg_recording(dev);
     const R rlam = P::from_f64(lam);
     S* __restrict__ L = W + line * N;
     Stats<P> st;
@@ -85,15 +89,13 @@ __global__ void __launch_bounds__(kXThreads, XcMinBlocks<P>::value) k_pass_xc(ty
         for (int s = 0; s < 8; s++) L[j + T * s] = P::pack(v[s]);
     }
 
-    __shared__ unsigned long long kred[kXThreads / 32];
-    const unsigned long long key = block_max_key<kXThreads>(st.dkey(), kred);
-    if (threadIdx.x == 0) part_max[blockIdx.x] = __longlong_as_double((long long)key);
+    block_max_to<NT>(st, part_max + blockIdx.x);
     if (want_sum) {
         NSum acc;
         acc.s = st.total();
         acc.c = 0.0;
         double unused = 0.0;
-        block_reduce<kXThreads>(acc, unused, red);
+        block_reduce<NT>(acc, unused, red);
         if (threadIdx.x == 0) part_sum[blockIdx.x] = acc.value();
     }
 }

@@ -554,7 +554,7 @@ int kg_ens_fetch(int i, double* u) {
     const Tables& tb = e->tab[N == 64 ? 0 : 1];
     const double2* cur = in.phase ? in.S1 : in.S0;
     KG_ECK(kLaunchF64.z_from_f64(N, cur, cur, nullptr, e->tmp2, tb.tw64, e->stream));
-    KG_ECK(kLaunchF64.yi(N, e->tmp2, e->tmp, tb.tw64, e->stream));
+    KG_ECK(kLaunchF64.yi(N, e->tmp2, e->tmp, tb.tw64, FinArgs{}, e->stream));
     KG_ECK(launch_x_inverse(N, e->tmp, e->phys, tb.tw64, 1.0 / ((double)N * N * N), nullptr, e->stream));
     KG_ECK(cudaMemcpyAsync(u, e->phys, sizeof(double) * (size_t)N * N * N, cudaMemcpyDeviceToHost, e->stream));
     KG_ECK(cudaStreamSynchronize(e->stream));

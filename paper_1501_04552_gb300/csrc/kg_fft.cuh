@@ -29,6 +29,16 @@
 
 namespace kg {
 
+// Programmatic dependent launch: the kernels of a step are launched with it, so that one's CTAs
+// are placed, and its address arithmetic and twiddle staging run, while the last CTAs of the one
+// before finish.  Every such kernel calls pdl_wait in every thread before it touches what
+// another kernel writes (it returns when the kernels before have completed and their writes are
+// visible; at once in a plain launch), and in doing so lets the next kernel's CTAs in.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // asynchronous 16-byte global -> shared copy (L2 only), and its completion wait
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -411,6 +421,7 @@ struct Stats<PrecF64> {
     }
     // bits of max|u| as a double: unsigned order = numeric order, nan above inf
     __device__ __forceinline__ unsigned long long dkey() const { return mx; }
+    static constexpr bool kKey32 = false;
 };
 
 template <>
@@ -463,6 +474,7 @@ struct Stats<PrecDF> {
     __device__ __forceinline__ unsigned long long dkey() const {
         return (unsigned long long)__double_as_longlong(f2d_int(__uint_as_float(mx)));
     }
+    static constexpr bool kKey32 = true;   // fkey() holds all of the key
 };
 
 template <>
@@ -493,6 +505,7 @@ struct Stats<PrecF32> {
     __device__ __forceinline__ unsigned long long dkey() const {
         return (unsigned long long)__double_as_longlong(f2d_int(__uint_as_float(mx)));
     }
+    static constexpr bool kKey32 = true;   // fkey() holds all of the key
 };
 
 // ---------------------------------------------------------------------------
@@ -513,11 +526,10 @@ struct KgDev {
     double Q_last;            // Q^{l+1/2} of the last recording step
     long long Q_last_level;
     double P_peek;            // sum-based P of the last peek
-    double maxabs_peek;
+    double maxabs_peek;       // max |u| of an x pass run ahead (or of a peek)
     int status;               // nonzero: a device-side check failed
     int scheme;               // KG_SCHEME_EQ2 (0) or KG_SCHEME_COMPOSED4 (1)
     int sub;                  // composed scheme: substep 0..2 of the current step
-    int record_p;             // 1: the next x pass records P^l whatever energy_every says (cleared by k_fin_x)
 };
 
 __device__ __forceinline__ bool kg_recording(const KgDev* dev) {
@@ -551,6 +563,27 @@ __device__ __forceinline__ unsigned long long block_max_key(unsigned long long k
             for (int w = 1; w < NW; w++) k = sh[w] > k ? sh[w] : k;
     }
     return k;
+}
+
+// max |u| of the statistics st of an NT-thread CTA, as a double, into *out
+template <int NT, class ST>
+__device__ __forceinline__ void block_max_to(const ST& st, double* out) {
+    static_assert(NT % 32 == 0, "whole warps");
+    if constexpr (ST::kKey32) {
+        __shared__ unsigned sh[NT / 32];
+        unsigned k = __reduce_max_sync(0xffffffffu, st.fkey());
+        if (NT > 32) {
+            if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
+            __syncthreads();
+            if (threadIdx.x == 0)
+                for (int w = 1; w < NT / 32; w++) k = sh[w] > k ? sh[w] : k;
+        }
+        if (threadIdx.x == 0) *out = f2d_int(__uint_as_float(k));
+    } else {
+        __shared__ unsigned long long sh[NT / 32];
+        const unsigned long long k = block_max_key<NT>(st.dkey(), sh);
+        if (threadIdx.x == 0) *out = __longlong_as_double((long long)k);
+    }
 }
 
 // NT threads, a power of two; lane 0 of warp 0 ends with the block result

@@ -22,7 +22,7 @@ const double kPi = 3.14159265358979323846;
 int forward3d(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
               cudaStream_t st) {
     KG_HCK(launch_x_forward(N, u, lines, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.yf(N, lines, out, tw64, st));
+    KG_HCK(kLaunchF64.yf(N, lines, out, tw64, FinArgs{}, st));
     KG_HCK(kLaunchF64.zcol(N, -1, out, tw64, st));
     return KG_OK;
 }
@@ -31,7 +31,7 @@ int forward3d(int N, const double* u, double2* lines, double2* out, const double
 int forward3d_c(int N, const double2* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
                 cudaStream_t st) {
     KG_HCK(launch_xc_forward(N, u, lines, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.yfc(N, lines, out, tw64, st));
+    KG_HCK(kLaunchF64.yfc(N, lines, out, tw64, FinArgs{}, st));
     KG_HCK(kLaunchF64.zcolc(N, -1, out, tw64, st));
     return KG_OK;
 }
@@ -40,7 +40,7 @@ int forward3d_c(int N, const double2* u, double2* lines, double2* out, const dou
 int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W1, void* W2, double2* out, const void* tw,
                    int cube, double lam, cudaStream_t st) {
     KG_HCK(pl->x_setup(N, u, W1, tw, cube, lam, st));
-    KG_HCK(pl->yf(N, W1, W2, tw, st));
+    KG_HCK(pl->yf(N, W1, W2, tw, FinArgs{}, st));
     KG_HCK(pl->z_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
@@ -48,7 +48,7 @@ int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W1, void*
 int forward3d_c_pass(int N, const PassLaunch* pl, const double2* u, void* W1, void* W2, double2* out, const void* tw,
                      int cube, double lam, cudaStream_t st) {
     KG_HCK(pl->xc_setup(N, u, W1, tw, cube, lam, st));
-    KG_HCK(pl->yfc(N, W1, W2, tw, st));
+    KG_HCK(pl->yfc(N, W1, W2, tw, FinArgs{}, st));
     KG_HCK(pl->zc_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
@@ -167,7 +167,7 @@ int init_state(int N, int prec, double dt, double lam, const Tables& tb, double*
     if (kick0) KG_HCK(launch_startup_c4(N, S0, S1, fbuf, kick0, st));    // S1 = P^0
     else KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, false, st));  // S1 = uh^{-1}
     KG_HCK(pl->z_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));   // z inverse of uh^0
-    KG_HCK(pl->yi(N, W2, W1, tb.tw, st));                        // y inverse
+    KG_HCK(pl->yi(N, W2, W1, tb.tw, FinArgs{}, st));                        // y inverse
     return KG_OK;
 }
 
@@ -194,7 +194,7 @@ int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, doubl
     }
     KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, true, st));       // S1 = uh^{-1}
     KG_HCK(pl->zc_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));          // z inverse of uh^0
-    KG_HCK(pl->yic(N, W2, W1, tb.tw, st));                               // y inverse
+    KG_HCK(pl->yic(N, W2, W1, tb.tw, FinArgs{}, st));                               // y inverse
     return KG_OK;
 }
 

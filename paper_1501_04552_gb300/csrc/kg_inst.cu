@@ -25,8 +25,8 @@ typedef Launchers<KG_P> Lp;
 
 #if KG_PART == 0
 cudaError_t pass_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale,
-                   double lam, cudaStream_t st) {
-    return Lp::pass_x(N, mode, W, dev, ps, pm, tw, scale, lam, st);
+                   double lam, int record, cudaStream_t st) {
+    return Lp::pass_x(N, mode, W, dev, ps, pm, tw, scale, lam, record, st);
 }
 int x_parts(int N) { return Lp::x_parts(N); }
 cudaError_t x_setup(int N, const double* u, void* spec, const void* tw, int cube, double lam, cudaStream_t st) {
@@ -41,11 +41,11 @@ cudaError_t xy_fused(int N, int do_yi, const void* W1, void* W2, KgDev* dev, dou
 }
 int xy_parts(int N) { return Lp::xy_parts(N); }
 #elif KG_PART == 1
-cudaError_t yf(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
-    return Lp::yf_t<false>(N, W1, W2, tw, st);
+cudaError_t yf(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yf_t<false>(N, W1, W2, tw, fin, st);
 }
-cudaError_t yi(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
-    return Lp::yi_t<false>(N, W2, W1, tw, st);
+cudaError_t yi(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yi_t<false>(N, W2, W1, tw, fin, st);
 }
 cudaError_t zcol(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
     return Lp::zcol_t<false>(N, sign, W2, tw, st);
@@ -77,15 +77,15 @@ cudaError_t update(int N, void* W, double2* S0, double2* S1, KgDev* dev, double*
 int update_parts(int N) { return Lp::update_parts(N); }
 #elif KG_PART == 3
 cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale,
-                    double lam, cudaStream_t st) {
-    return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, st);
+                    double lam, int record, cudaStream_t st) {
+    return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, record, st);
 }
 int xc_parts(int N) { return Lp::xc_parts(N); }
-cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
-    return Lp::yf_t<true>(N, W1, W2, tw, st);
+cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yf_t<true>(N, W1, W2, tw, fin, st);
 }
-cudaError_t yic(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
-    return Lp::yi_t<true>(N, W2, W1, tw, st);
+cudaError_t yic(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yi_t<true>(N, W2, W1, tw, fin, st);
 }
 cudaError_t zcolc(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
     return Lp::zcol_t<true>(N, sign, W2, tw, st);

@@ -9,15 +9,23 @@ namespace kg {
 // ---------------------------------------------------------------------------
 // Pass X.  MODE_STEP: C2R along x, stats, F = lam u^3, R2C along x, in place.
 //          MODE_PEEK: C2R along x and stats only (W untouched).
-// One line = N/2+1 complex values; T = N/16 threads per line, 256 threads per CTA.
+// One line = N/2+1 complex values; T = N/16 threads per line.
 // ---------------------------------------------------------------------------
 constexpr int kXThreads = 256;
 
+// threads per CTA of the stepping x pass: 256, and below 128^3 few enough that the grid still
+// spreads over the SMs (a 32^3 pass is 2048 threads: with 64 CTAs of 32 in place of 8 of 256
+// the whole double-float step went from 20.4 to 18.9 us; 16^3 20.9 to 18.0, 64^3 22.6 to 21.2)
 template <int N>
+struct XStep {
+    static constexpr int NT = N >= 128 ? kXThreads : N >= 64 ? 64 : 32;
+};
+
+template <int N, int NT = kXThreads>
 struct XShape {
     static constexpr int M = N / 2;
     static constexpr int T = M / 8;
-    static constexpr int LPC = kXThreads / T;           // lines per CTA
+    static constexpr int LPC = NT / T;                  // lines per CTA
     static constexpr int PADM = M + M / 8 + (N == 16);  // padded smem slots per line (even: a line lands in 16-byte copies)
     static_assert(T <= 32, "one line must fit in a warp");
 };
@@ -124,13 +132,13 @@ __device__ __forceinline__ void x_line_body(LIN Lin, LOUT L, int j,
 //     X1[k] = (Z[k] + conj Z[N-k]) / 2,    X2[k] = -i (Z[k] - conj Z[N-k]) / 2,
 // which needs no twiddle product (the one-line form packs each line into an N/2-point
 // transform with a twiddle product per point on the way in and on the way out).
-template <int N>
+template <int N, int NT = kXThreads>
 struct XpShape {
     static constexpr int T = N / 8;              // threads per line pair
-    static constexpr int PPC = kXThreads / T;    // pairs per CTA
+    static constexpr int PPC = NT / T;           // pairs per CTA
     static constexpr int PADN = N + N / 8;       // padded exchange slots per pair
     static constexpr bool CTA_SYNC = T > 32;     // a pair spans more than one warp
-    static_assert(2 * PPC == XShape<N>::LPC && PPC * PADN <= XShape<N>::LPC * XShape<N>::PADM,
+    static_assert(2 * PPC == XShape<N, NT>::LPC && PPC * PADN <= XShape<N, NT>::LPC * XShape<N, NT>::PADM,
                   "same lines per CTA as the one-line form, within its shared memory");
     static_assert(!CTA_SYNC || PPC <= 15, "one named barrier per pair");
 };
@@ -237,16 +245,14 @@ struct XPaired<PrecF64> {
     static constexpr bool value = true;
 };
 
-// resident CTAs per SM the x pass is compiled for: the paired double-float body fits
-// four (64 registers, no spills; 1.61 -> 1.44 ms at 512^3 against two); the pipelined
-// FP32 body measured slower at three (0.48 -> 0.51 ms), and the FP64 body needs its registers
-template <class P>
+// resident threads per SM the x pass is compiled for: the paired double-float body fits
+// 1024 (64 registers, no spills; 1.61 -> 1.44 ms at 512^3 against 512); the pipelined
+// FP32 body measured slower at 768 (0.48 -> 0.51 ms), and the FP64 body needs its registers.
+// Below 128^3 the grid does not fill the SMs and every body keeps its registers.
+template <class P, int N>
 struct XMinBlocks {
-    static constexpr int value = 2;
-};
-template <>
-struct XMinBlocks<PrecDF> {
-    static constexpr int value = 4;
+    static constexpr int kThreads = std::is_same<P, PrecDF>::value ? 1024 : 512;
+    static constexpr int value = N >= 128 ? kThreads / XStep<N>::NT : 1;
 };
 
 // How pass X walks W.  Pipelined (the FP32 pass, bound by latency and the L1TEX pipe): a
@@ -270,13 +276,15 @@ struct XPipelined<PrecF64> {
 
 // Pass X.  A batch is LPC consecutive x-lines of W1 (rows of PITCH values, 16-byte aligned, so
 // a line lands in 16-byte copies: two FP32 values each); a landed batch serves as the lines'
-// FFT exchange space.  Each CTA writes one max key and (when wanted) one Sigma u^4 partial.
+// FFT exchange space.  Each CTA writes one max key and one Sigma u^4 partial when the step
+// records or `record` is set (kg_energy's pass).
 template <class P, int N, int MODE>
-__global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(typename P::S* __restrict__ W, KgDev* __restrict__ dev,
-                                                      double* __restrict__ part_sum, double* __restrict__ part_max,
-                                                      const typename P::S* __restrict__ tw, double scale, double lam) {
+__global__ void __launch_bounds__(XStep<N>::NT, XMinBlocks<P, N>::value)
+    k_pass_x(typename P::S* __restrict__ W, KgDev* __restrict__ dev, double* __restrict__ part_sum,
+             double* __restrict__ part_max, const typename P::S* __restrict__ tw, double scale, double lam, int record) {
     typedef typename P::S S;
-    typedef XShape<N> X;
+    constexpr int NT = XStep<N>::NT;
+    typedef XShape<N, NT> X;
     constexpr int T = X::T, NH = N / 2 + 1, LPC = X::LPC, PADM = X::PADM, PITCH = Lay<N>::PITCH;
     constexpr int NB = N * N / LPC;     // batches
     constexpr int VPC = 16 / (int)sizeof(S);              // values per 16-byte copy
@@ -287,13 +295,14 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
     __shared__ double red[96];
 
     const int li = threadIdx.x / T, j = threadIdx.x % T;
-    const bool want_sum = (MODE == MODE_PEEK) || kg_recording(dev) || dev->record_p;
+    pdl_wait();
+    const bool want_sum = (MODE == MODE_PEEK) || record || kg_recording(dev);
     const typename P::R rlam = P::from_f64(lam);
     Stats<P> st;
     st.init();
 
     if constexpr (!XPipelined<P>::value && XPaired<P>::value) {
-        typedef XpShape<N> XP;
+        typedef XpShape<N, NT> XP;
         const int pi = threadIdx.x / XP::T, jp = threadIdx.x % XP::T;
         const size_t pair = (size_t)blockIdx.x * XP::PPC + pi;
         LineSmemX<P, XP::CTA_SYNC> lsm{buf + pi * XP::PADN, 1u + (unsigned)pi, (unsigned)XP::T};
@@ -305,7 +314,7 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
     } else {
         auto issue = [&](int batch, S* dst) {
             const S* src = W + (size_t)batch * LPC * PITCH;
-            for (int e = threadIdx.x; e < LPC * CPL; e += kXThreads) {
+            for (int e = threadIdx.x; e < LPC * CPL; e += NT) {
                 const int l = e / CPL, k = (e - l * CPL) * VPC;
                 cp_async16(dst + l * PADM + k, src + l * PITCH + k);
             }
@@ -328,21 +337,110 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<P>::value) k_pass_x(type
     }
 
     // the max every step (integer keys), the compensated FP64 sum only when it is wanted
-    __shared__ unsigned long long kred[kXThreads / 32];
-    const unsigned long long key = block_max_key<kXThreads>(st.dkey(), kred);
-    if (threadIdx.x == 0) part_max[blockIdx.x] = __longlong_as_double((long long)key);
+    block_max_to<NT>(st, part_max + blockIdx.x);
     if (want_sum) {
         if constexpr (XPaired<P>::value && !std::is_same<P, PrecF64>::value) {
-            __shared__ df dred[kXThreads / 32];
-            const df t = block_sum_df<kXThreads>(st.total_df(), dred);
+            __shared__ df dred[NT / 32];
+            const df t = block_sum_df<NT>(st.total_df(), dred);
             if (threadIdx.x == 0) part_sum[blockIdx.x] = f2d_int(t.hi) + f2d_int(t.lo);
         } else {
             NSum acc;
             acc.s = st.total();
             acc.c = 0.0;
             double unused = 0.0;
-            block_reduce<kXThreads>(acc, unused, red);
+            block_reduce<NT>(acc, unused, red);
             if (threadIdx.x == 0) part_sum[blockIdx.x] = acc.value();
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Finalisers: reduce the partials of a pass and advance the run state.  Those of a step run in
+// one more CTA of the y pass that follows (FIN_X in the forward, FIN_Z in the inverse one, both
+// before the next reader of the state starts).  As kernels of one CTA, and without programmatic
+// dependent launch, they made a double-float step 33 us at 32^3 and 72 us at 64^3 recording
+// every level; now 18.9 and 34 us.
+// ---------------------------------------------------------------------------
+constexpr int kFinThreads = 1024;
+constexpr int kFinSmem = 128;   // doubles of shared memory a finaliser needs
+
+// all NT threads of the CTA; red: kFinSmem doubles
+template <int NT>
+__device__ __forceinline__ void fin_reduce(const double* part_sum, const double* part_max, int count, NSum& acc,
+                                           double& mx, double* red) {
+    acc.s = 0.0;
+    acc.c = 0.0;
+    unsigned long long key = 0ull;
+    for (int i = threadIdx.x; i < count; i += NT) {
+        if (part_sum) acc.add(part_sum[i]);
+        if (part_max) {
+            const unsigned long long k = (unsigned long long)__double_as_longlong(part_max[i]);
+            key = k > key ? k : key;
+        }
+    }
+    if (part_max) key = block_max_key<NT>(key, reinterpret_cast<unsigned long long*>(red + 96));
+    mx = __longlong_as_double((long long)key);
+    if (part_sum) {
+        double unused = 0.0;
+        block_reduce<NT>(acc, unused, red);
+    }
+}
+
+template <int NT>
+__device__ __noinline__ void finalise(const FinArgs f, double* red) {
+    KgDev* dev = f.dev;
+    NSum acc;
+    double mx;
+    if (f.kind == FIN_X || f.kind == FIN_X_AHEAD) {
+        // after a stepping x pass: blow-up check and P^l; norm = lam h^3 / 4.  FIN_X_AHEAD: the
+        // next step's x pass, run by kg_energy; it records P^l, and its max |u| waits in
+        // maxabs_peek until that step runs (kg_status reports the last step's)
+        const bool ahead = f.kind == FIN_X_AHEAD;
+        const bool rec = kg_recording(dev) || ahead;
+        fin_reduce<NT>(rec ? f.part_sum : nullptr, f.part_max, f.count, acc, mx, red);
+        if (dev->complex_field) mx = sqrt(mx);   // the keys were |u|^2
+        if (threadIdx.x == 0) {
+            if (ahead && dev->frozen) dev->maxabs_peek = dev->maxabs_last;
+            // the composed scheme checks the field at integer times only (its first substep)
+            if (dev->sub == 0 && !dev->frozen) {
+                if (ahead) dev->maxabs_peek = mx;
+                else dev->maxabs_last = mx;
+                if (rec) {
+                    dev->P_last = f.norm * acc.value();
+                    dev->P_last_level = dev->level;
+                }
+                if (dev->threshold > 0.0 && !(mx <= dev->threshold)) {
+                    dev->frozen = 1;
+                    dev->blowup_level = dev->level;
+                }
+            }
+        }
+    } else if (f.kind == FIN_AHEAD_DONE) {
+        // the step whose x pass ran ahead: its max |u| becomes the last step's
+        if (threadIdx.x == 0) dev->maxabs_last = dev->maxabs_peek;
+    } else if (f.kind == FIN_PEEK) {
+        fin_reduce<NT>(f.part_sum, f.part_max, f.count, acc, mx, red);
+        if (dev->complex_field) mx = sqrt(mx);
+        if (threadIdx.x == 0) {
+            dev->P_peek = f.norm * acc.value();
+            dev->maxabs_peek = mx;
+        }
+    } else {
+        // after the update: Q^{l+1/2} (norm = h^3/N^3) and the level advance
+        const bool rec = kg_recording(dev);
+        if (rec) fin_reduce<NT>(f.part_sum, nullptr, f.count, acc, mx, red);
+        if (threadIdx.x == 0 && !dev->frozen) {
+            if (rec) {
+                dev->Q_last = f.norm * acc.value();
+                dev->Q_last_level = dev->level;
+            }
+            if (dev->scheme == 0) {
+                dev->level += 1;
+                dev->phase ^= 1;
+            } else {   // composed scheme: the state arrays stay put; a step is three substeps
+                dev->sub = dev->sub == 2 ? 0 : dev->sub + 1;
+                if (dev->sub == 0) dev->level += 1;
+            }
         }
     }
 }
@@ -418,15 +516,22 @@ struct ColMinBlocks {
 
 template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, int CW>
 __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::value) k_col(const typename Pin::S* src, typename Pout::S* dst,
-                                                    const typename P::S* __restrict__ tw) {
+                                                    const typename P::S* __restrict__ tw, FinArgs fin) {
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
+    const int plane = (int)blockIdx.y - (fin.kind != FIN_NONE);   // a finaliser takes the first row of CTAs
+    if (plane < 0) {
+        pdl_wait();
+        if (blockIdx.x == 0) finalise<CW * N / 8>(fin, reinterpret_cast<double*>(smraw));
+        return;
+    }
     const int c = threadIdx.x % C, j = threadIdx.x / C;
     const int kx = blockIdx.x * C + c;
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
-    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, C>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
+    pdl_wait();
+    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, C>(src, dst, plane, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
 }
 
 // inverse z column FFT from an FP64 spectral array into W2 (precision P); the source is
@@ -437,6 +542,7 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
+    pdl_wait();
     const double2* src = (dev != nullptr && dev->phase) ? src1 : src0;
     const int c = threadIdx.x % C, j = threadIdx.x / C;
     const int kx = blockIdx.x * C + c;
@@ -568,7 +674,6 @@ struct ModeIndex {
 };
 
 constexpr int kUpdThreads = 256;
-constexpr int kSumThreads = 1024;   // second reduction stage of the update's Q partials
 
 // One term of Q^{n+1/2} without its constant factor 1/(2 dt^2):
 //     w_k ( |a1 - a0|^2 + r_k |a1 + a0|^2 ),   r_k = qr omega_k^2,  qr = dt^2 / 4,
@@ -646,6 +751,7 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
     typedef QTerm<P> Q;
     typedef ModeIndex<N, CPLX> MI;
     __shared__ typename Q::T red[kUpdThreads / 32];
+    pdl_wait();
     const bool want_q = SCHEME == 0 && kg_recording(dev);
     const bool update = dev->frozen == 0;
     double2* __restrict__ cur = dev->phase ? S1 : S0;
@@ -725,6 +831,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
         prefetch_l2(S1 + base, (unsigned)(N * C * sizeof(double2)));
     }
     tw = stage_table(tw, sm + N * C, N);
+    pdl_wait();
 
     cx<R> v[8];
 #pragma unroll
@@ -776,110 +883,17 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     }
 }
 
-// second stage of the Q sum on recording steps: CTA b sums in[b*1024 ...] pairwise into out[b]
-__global__ void __launch_bounds__(kSumThreads) k_sum_parts(const double* __restrict__ in, int count,
-                                                           double* __restrict__ out, const KgDev* __restrict__ dev);
-
-// ---------------------------------------------------------------------------
-// finalisers (one CTA of 1024 threads)
-// ---------------------------------------------------------------------------
-constexpr int kFinThreads = 1024;
-
-__device__ __forceinline__ void fin_reduce(const double* part_sum, const double* part_max, int count, NSum& acc,
-                                           double& mx) {
-    __shared__ double red[96];
-    __shared__ unsigned long long kred[kFinThreads / 32];
-    acc.s = 0.0;
-    acc.c = 0.0;
-    unsigned long long key = 0ull;
-    for (int i = threadIdx.x; i < count; i += kFinThreads) {
-        if (part_sum) acc.add(part_sum[i]);
-        if (part_max) {
-            const unsigned long long k = (unsigned long long)__double_as_longlong(part_max[i]);
-            key = k > key ? k : key;
-        }
-    }
-    if (part_max) key = block_max_key<kFinThreads>(key, kred);
-    mx = __longlong_as_double((long long)key);
-    if (part_sum) {
-        double unused = 0.0;
-        block_reduce<kFinThreads>(acc, unused, red);
-    }
-}
-
 #ifdef KG_DEFINE_COMMON_KERNELS   // defined by exactly one translation unit
-// after a stepping x pass: blow-up check and P^l; p_norm = lam h^3 / 4
-__global__ void __launch_bounds__(kFinThreads) k_fin_x(const double* part_sum, const double* part_max, int count,
-                                                       KgDev* dev, double p_norm) {
-    NSum acc;
-    double mx;
-    // record_p marks the next step's x pass run ahead by kg_energy: it records P^l, and its
-    // max |u| waits in maxabs_peek until that step runs (kg_status reports the last step's)
-    const bool ahead = dev->record_p != 0;   // read by every thread before fin_reduce's barriers
-    const bool rec = kg_recording(dev) || ahead;
-    fin_reduce(rec ? part_sum : nullptr, part_max, count, acc, mx);
-    if (dev->complex_field) mx = sqrt(mx);   // the keys were |u|^2
-    // the composed scheme checks the field at integer times only (its first substep)
-    if (threadIdx.x == 0 && dev->sub == 0) {
-        if (!dev->frozen) {
-            if (ahead) dev->maxabs_peek = mx;
-            else dev->maxabs_last = mx;
-            if (rec) {
-                dev->P_last = p_norm * acc.value();
-                dev->P_last_level = dev->level;
-            }
-            if (dev->threshold > 0.0 && !(mx <= dev->threshold)) {
-                dev->frozen = 1;
-                dev->blowup_level = dev->level;
-            }
-        }
-    }
-    if (threadIdx.x == 0) dev->record_p = 0;
+// a finaliser in a kernel of its own (one CTA): the fused xy form, kg_energy's passes.
+// before / after (host memory, may be NULL) receive the run state around it.
+__global__ void __launch_bounds__(kFinThreads) k_fin(FinArgs f, KgDev* before, KgDev* after) {
+    __shared__ double red[kFinSmem];
+    if (before && threadIdx.x == 0) *before = *f.dev;
+    __syncthreads();
+    finalise<kFinThreads>(f, red);
+    __syncthreads();
+    if (after && threadIdx.x == 0) *after = *f.dev;
 }
-
-// after a peek x pass
-__global__ void __launch_bounds__(kFinThreads) k_fin_peek(const double* part_sum, const double* part_max, int count,
-                                                          KgDev* dev, double p_norm) {
-    NSum acc;
-    double mx;
-    fin_reduce(part_sum, part_max, count, acc, mx);
-    if (dev->complex_field) mx = sqrt(mx);
-    if (threadIdx.x == 0) {
-        dev->P_peek = p_norm * acc.value();
-        dev->maxabs_peek = mx;
-    }
-}
-
-// after the update: Q^{l+1/2} (q_norm = h^3/N^3) and the level advance
-__global__ void __launch_bounds__(kSumThreads) k_sum_parts(const double* __restrict__ in, int count,
-                                                           double* __restrict__ out, const KgDev* __restrict__ dev) {
-    if (!kg_recording(dev)) return;
-    __shared__ double red[kSumThreads / 32];
-    const int i = blockIdx.x * kSumThreads + threadIdx.x;
-    double v = block_tree_sum<QTerm<PrecF64>, kSumThreads>(i < count ? in[i] : 0.0, red);
-    if (threadIdx.x == 0) out[blockIdx.x] = v;
-}
-
-__global__ void __launch_bounds__(kFinThreads) k_fin_z(const double* part_sum, int count, KgDev* dev, double q_norm) {
-    const bool rec = kg_recording(dev);
-    NSum acc;
-    double mx;
-    if (rec) fin_reduce(part_sum, nullptr, count, acc, mx);
-    if (threadIdx.x == 0 && !dev->frozen) {
-        if (rec) {
-            dev->Q_last = q_norm * acc.value();
-            dev->Q_last_level = dev->level;
-        }
-        if (dev->scheme == 0) {
-            dev->level += 1;
-            dev->phase ^= 1;
-        } else {   // composed scheme: the state arrays stay put; a step is three substeps
-            dev->sub = dev->sub == 2 ? 0 : dev->sub + 1;
-            if (dev->sub == 0) dev->level += 1;
-        }
-    }
-}
-
 #endif  // KG_DEFINE_COMMON_KERNELS
 
 // ---------------------------------------------------------------------------
@@ -1102,9 +1116,10 @@ __global__ void k_repack(const double2* __restrict__ in, double2* __restrict__ o
 #ifdef KG_DEFINE_COMMON_KERNELS
 // plain Neumaier total of partials into *out (times norm)
 __global__ void __launch_bounds__(kFinThreads) k_fin_sum(const double* part_sum, int count, double norm, double* out) {
+    __shared__ double red[kFinSmem];
     NSum acc;
     double mx;
-    fin_reduce(part_sum, nullptr, count, acc, mx);
+    fin_reduce<kFinThreads>(part_sum, nullptr, count, acc, mx, red);
     if (threadIdx.x == 0) *out = norm * acc.value();
 }
 

@@ -23,15 +23,27 @@ struct C4Args {
     double h[3];           // drift length of each substep
 };
 
+// the finaliser of a pass (kg_kernels.cuh): what it does, the pass's partials and the run state
+enum { FIN_NONE = 0, FIN_X, FIN_X_AHEAD, FIN_AHEAD_DONE, FIN_PEEK, FIN_Z };
+struct FinArgs {
+    int kind = FIN_NONE;
+    int count = 0;
+    const double* part_sum = nullptr;
+    const double* part_max = nullptr;
+    KgDev* dev = nullptr;
+    double norm = 0.0;
+};
+
 // precision ids match KG_FP64 / KG_DF64 / KG_MIXED of kg.h
 struct PassLaunch {
-    // x pass over W1 in the context's precision; mode 0 step, 1 peek.  Writes nparts partials.
+    // x pass over W1 in the context's precision; mode 0 step, 1 peek.  Writes nparts partials
+    // (of sum u^4 in a stepping pass when the step records or `record` is set).
     cudaError_t (*pass_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
-                          double scale, double lam, cudaStream_t st);
+                          double scale, double lam, int record, cudaStream_t st);
     // forward y columns W1 (x-lines) -> W2 (z-columns), inverse y columns W2 -> W1; z columns of
-    // W2 in place (sign -1 forward, +1 inverse; FP64 only)
-    cudaError_t (*yf)(int N, const void* W1, void* W2, const void* tw, cudaStream_t st);
-    cudaError_t (*yi)(int N, const void* W2, void* W1, const void* tw, cudaStream_t st);
+    // W2 in place (sign -1 forward, +1 inverse; FP64 only).  fin runs in one more CTA of the y pass.
+    cudaError_t (*yf)(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*yi)(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st);
     cudaError_t (*zcol)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
     // inverse z columns from an FP64 spectral source (chosen by dev->phase when dev != NULL) into W2
     cudaError_t (*z_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
@@ -51,10 +63,10 @@ struct PassLaunch {
     // complex field (full N^3 spectrum, N columns per plane): x pass, column FFTs,
     // column FFT from an FP64 source, update, and their partial counts
     cudaError_t (*passc_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
-                           double scale, double lam, cudaStream_t st);
+                           double scale, double lam, int record, cudaStream_t st);
     int (*xc_parts)(int N);
-    cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, cudaStream_t st);
-    cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, cudaStream_t st);
+    cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st);
     cudaError_t (*zcolc)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
     cudaError_t (*zc_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
                                const void* tw, cudaStream_t st);
@@ -120,12 +132,9 @@ cudaError_t launch_xc_forward(int N, const double2* u, double2* out, const doubl
 cudaError_t launch_xc_inverse(int N, const double2* in, double2* u, const double2* tw, double scale,
                               double* part_sum, cudaStream_t st);
 int xc_inverse_parts(int N);
-cudaError_t launch_fin_x(const double* ps, const double* pm, int count, KgDev* dev, double p_norm, cudaStream_t st);
-cudaError_t launch_fin_peek(const double* ps, const double* pm, int count, KgDev* dev, double p_norm,
-                            cudaStream_t st);
-// after the update: Q from its count partials (summed pairwise in blocks of 1024 into
-// stage2, which holds (count + 1023) / 1024 doubles), then the level/phase advance
-cudaError_t launch_fin_z(const double* ps, int count, double* stage2, KgDev* dev, double q_norm, cudaStream_t st);
+// a finaliser as a kernel of its own; before / after (host memory the device can write, or
+// NULL) receive the run state around it
+cudaError_t launch_fin(const FinArgs& fin, KgDev* before, KgDev* after, cudaStream_t st);
 cudaError_t launch_fin_sum(const double* ps, int count, double norm, double* out, cudaStream_t st);
 // composed scheme: partials of the quadratic energy sum_k w_k (|p|^2 + omega^2 |a|^2) / 2 with
 // the synchronised velocity p formed from the stored P, F = R2C(lam u^3) and the first kick table

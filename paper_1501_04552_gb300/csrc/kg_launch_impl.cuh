@@ -1,5 +1,6 @@
 // kg_launch_impl.cuh -- template launchers, instantiated once per precision.
 #pragma once
+#include <atomic>
 #include <type_traits>
 #include "kg_complex.cuh"
 #include "kg_ensemble.cuh"
@@ -18,6 +19,36 @@ constexpr int kXyCluster = 8;
 template <class K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// The attribute is set once per kernel and device (a driver call of its own on every launch
+// costs as much host time as the launch).
+template <class K>
+static cudaError_t set_smem_once(K kernel, size_t bytes, std::atomic<unsigned long long>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = set_smem(kernel, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
+// a launch that may start while the kernel before it drains (the kernel calls pdl_wait)
+template <class... KA, class... A>
+static cudaError_t launch_pdl(void (*kernel)(KA...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
 
 #define KG_DISPATCH_N(N, ...)                               \
@@ -39,24 +70,24 @@ struct Launchers {
     // one per batch; cached per grid size
     template <int N>
     static size_t x_smem() {
-        typedef XShape<N> X;
+        typedef XShape<N, XStep<N>::NT> X;
         return (size_t)(XPipelined<P>::value ? 2 : 1) * X::LPC * X::PADM * sizeof(S);
     }
     template <int N>
     static int x_grid_n() {
         static int grid = 0;
-        if (!XPipelined<P>::value) return N * N / XShape<N>::LPC;
+        if (!XPipelined<P>::value) return N * N / XShape<N, XStep<N>::NT>::LPC;
         if (grid == 0) {
-            typedef XShape<N> X;
+            typedef XShape<N, XStep<N>::NT> X;
             int dev = 0, sms = 0, occ0 = 0, occ1 = 0;
             if (cudaGetDevice(&dev) != cudaSuccess ||
                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
                 return 0;
             if (set_smem(k_pass_x<P, N, MODE_STEP>, x_smem<N>()) != cudaSuccess ||
                 set_smem(k_pass_x<P, N, MODE_PEEK>, x_smem<N>()) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ0, k_pass_x<P, N, MODE_STEP>, kXThreads,
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ0, k_pass_x<P, N, MODE_STEP>, XStep<N>::NT,
                                                               x_smem<N>()) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, k_pass_x<P, N, MODE_PEEK>, kXThreads,
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, k_pass_x<P, N, MODE_PEEK>, XStep<N>::NT,
                                                               x_smem<N>()) != cudaSuccess)
                 return 0;
             const int occ = occ0 < occ1 ? occ0 : occ1;
@@ -66,26 +97,23 @@ struct Launchers {
         }
         return grid;
     }
-    template <int N>
-    static cudaError_t pass_x_n(int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale,
-                                double lam, cudaStream_t st) {
-        const size_t smem = x_smem<N>();
+    template <int N, int MODE>
+    static cudaError_t pass_x_n(void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale, double lam,
+                                int record, cudaStream_t st) {
+        static std::atomic<unsigned long long> done{0};
         const int grid = x_grid_n<N>();
         if (grid == 0) return cudaErrorInvalidConfiguration;
-        if (mode == MODE_STEP) {
-            cudaError_t e = set_smem(k_pass_x<P, N, MODE_STEP>, smem);
-            if (e != cudaSuccess) return e;
-            k_pass_x<P, N, MODE_STEP><<<grid, kXThreads, smem, st>>>((S*)W, dev, ps, pm, (const S*)tw, scale, lam);
-        } else {
-            cudaError_t e = set_smem(k_pass_x<P, N, MODE_PEEK>, smem);
-            if (e != cudaSuccess) return e;
-            k_pass_x<P, N, MODE_PEEK><<<grid, kXThreads, smem, st>>>((S*)W, dev, ps, pm, (const S*)tw, scale, lam);
-        }
-        return cudaGetLastError();
+        cudaError_t e = set_smem_once(k_pass_x<P, N, MODE>, x_smem<N>(), done);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k_pass_x<P, N, MODE>, grid, XStep<N>::NT, x_smem<N>(), st, (S*)W, dev, ps, pm, (const S*)tw,
+                          scale, lam, record);
     }
     static cudaError_t pass_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw,
-                              double scale, double lam, cudaStream_t st) {
-        KG_DISPATCH_N(N, return pass_x_n<NN>(mode, W, dev, ps, pm, tw, scale, lam, st));
+                              double scale, double lam, int record, cudaStream_t st) {
+        if (mode == MODE_STEP) {
+            KG_DISPATCH_N(N, return (pass_x_n<NN, MODE_STEP>(W, dev, ps, pm, tw, scale, lam, record, st)));
+        }
+        KG_DISPATCH_N(N, return (pass_x_n<NN, MODE_PEEK>(W, dev, ps, pm, tw, scale, lam, record, st)));
     }
     // partials the x pass writes (its grid); 0 when the device cannot be queried
     static int x_parts(int N) {
@@ -94,22 +122,24 @@ struct Launchers {
 
     // column passes (k_col): Pin -> Pout in the layouts of direction DIR
     template <class Pin, class Pout, int N, int SIGN, int DIR, bool CPLX, int C>
-    static cudaError_t col_n(const void* src, void* dst, const void* tw, cudaStream_t st) {
-        const size_t smem = (size_t)(N * C + N) * sizeof(S);
+    static cudaError_t col_n(const void* src, void* dst, const void* tw, const FinArgs& fin, cudaStream_t st) {
+        static std::atomic<unsigned long long> done{0};
+        constexpr size_t smem = (size_t)(N * C + N) * sizeof(S);
+        static_assert(smem >= kFinSmem * sizeof(double), "a finaliser's shared memory");
         auto kern = k_col<Pin, P, Pout, N, SIGN, DIR, CPLX, C>;
-        cudaError_t e = set_smem(kern, smem);
+        cudaError_t e = set_smem_once(kern, smem, done);
         if (e != cudaSuccess) return e;
-        dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N);
-        kern<<<grid, C * N / 8, smem, st>>>((const typename Pin::S*)src, (typename Pout::S*)dst, (const S*)tw);
-        return cudaGetLastError();
+        dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N + (fin.kind != FIN_NONE));
+        return launch_pdl(kern, grid, C * N / 8, smem, st, (const typename Pin::S*)src, (typename Pout::S*)dst,
+                          (const S*)tw, fin);
     }
     template <bool CPLX>
-    static cudaError_t yf_t(int N, const void* W1, void* W2, const void* tw, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_YF, CPLX, ColStep<P, true>::C>(W1, W2, tw, st)));
+    static cudaError_t yf_t(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_YF, CPLX, ColStep<P, true>::C>(W1, W2, tw, fin, st)));
     }
     template <bool CPLX>
-    static cudaError_t yi_t(int N, const void* W2, void* W1, const void* tw, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_YI, CPLX, ColStep<P, true>::C>(W2, W1, tw, st)));
+    static cudaError_t yi_t(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_YI, CPLX, ColStep<P, true>::C>(W2, W1, tw, fin, st)));
     }
     // z columns in place: FP64 only (the other precisions have the fused z pass)
     template <bool CPLX>
@@ -117,21 +147,21 @@ struct Launchers {
         if constexpr (!std::is_same<P, PrecF64>::value) {
             return cudaErrorNotSupported;
         } else {
-            if (sign < 0) { KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, st))); }
-            KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, st)));
+            if (sign < 0) { KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, FinArgs{}, st))); }
+            KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, FinArgs{}, st)));
         }
     }
     template <int N, bool CPLX>
     static cudaError_t z_from_f64_n(const double2* src0, const double2* src1, const KgDev* dev, void* W2,
                                     const void* tw, cudaStream_t st) {
+        static std::atomic<unsigned long long> done{0};
         constexpr int C = ColShape<P>::C;
         const size_t smem = (size_t)(N * C + N) * sizeof(S);
         auto kern = k_col_sel<P, N, CPLX, C>;
-        cudaError_t e = set_smem(kern, smem);
+        cudaError_t e = set_smem_once(kern, smem, done);
         if (e != cudaSuccess) return e;
         dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N);
-        kern<<<grid, C * N / 8, smem, st>>>(src0, src1, dev, (S*)W2, (const S*)tw);
-        return cudaGetLastError();
+        return launch_pdl(kern, grid, C * N / 8, smem, st, src0, src1, dev, (S*)W2, (const S*)tw);
     }
     template <bool CPLX>
     static cudaError_t z_from_f64_t(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
@@ -142,7 +172,7 @@ struct Launchers {
     template <bool CPLX>
     static cudaError_t z_to_f64_t(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
         if constexpr (!kPassIO) return cudaErrorNotSupported;
-        else { KG_DISPATCH_N(N, return (col_n<P, PrecF64, NN, -1, COL_Z, CPLX, ColShape<P>::C>(W2, out, tw, st))); }
+        else { KG_DISPATCH_N(N, return (col_n<P, PrecF64, NN, -1, COL_Z, CPLX, ColShape<P>::C>(W2, out, tw, FinArgs{}, st))); }
     }
 
     // set-up and read-out transforms in the pass precision (double-float only: the FP32
@@ -196,50 +226,45 @@ struct Launchers {
     static cudaError_t update_n(void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                                 const double* w2, double inv_dt, const C4Args* c4, cudaStream_t st) {
         const double qr = 0.25 / (inv_dt * inv_dt), qc = 0.5 * inv_dt * inv_dt;
-        if (c4) {
-            k_update<P, N, false, 1><<<update_parts(N), kUpdThreads, 0, st>>>((S*)W, S0, S1, dev, ps, coef, w2, qr,
-                                                                              qc, *c4);
-        } else {
-            k_update<P, N><<<update_parts(N), kUpdThreads, 0, st>>>((S*)W, S0, S1, dev, ps, coef, w2, qr, qc,
-                                                                   C4Args{});
-        }
-        return cudaGetLastError();
+        if (c4)
+            return launch_pdl(k_update<P, N, false, 1>, update_parts(N), kUpdThreads, 0, st, (S*)W, S0, S1, dev, ps,
+                              coef, w2, qr, qc, *c4);
+        return launch_pdl(k_update<P, N, false, 0>, update_parts(N), kUpdThreads, 0, st, (S*)W, S0, S1, dev, ps, coef,
+                          w2, qr, qc, C4Args{});
     }
     static cudaError_t update(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                               const double* w2, double inv_dt, const C4Args* c4, cudaStream_t st) {
         KG_DISPATCH_N(N, return update_n<NN>(W, S0, S1, dev, ps, coef, w2, inv_dt, c4, st));
     }
     // ---- complex field ----
-    template <int N>
-    static cudaError_t passc_x_n(int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw,
-                                 double scale, double lam, cudaStream_t st) {
-        typedef XcShape<N> X;
+    template <int N, int MODE>
+    static cudaError_t passc_x_n(void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale, double lam,
+                                 int record, cudaStream_t st) {
+        typedef XcShape<N, XcStep<N>::NT> X;
+        static std::atomic<unsigned long long> done{0};
         const size_t smem = (size_t)X::LPC * X::PADN * sizeof(S);
-        const int grid = N * N / X::LPC;
-        if (mode == MODE_STEP) {
-            cudaError_t e = set_smem(k_pass_xc<P, N, MODE_STEP>, smem);
-            if (e != cudaSuccess) return e;
-            k_pass_xc<P, N, MODE_STEP><<<grid, kXThreads, smem, st>>>((S*)W, dev, ps, pm, (const S*)tw, scale, lam);
-        } else {
-            cudaError_t e = set_smem(k_pass_xc<P, N, MODE_PEEK>, smem);
-            if (e != cudaSuccess) return e;
-            k_pass_xc<P, N, MODE_PEEK><<<grid, kXThreads, smem, st>>>((S*)W, dev, ps, pm, (const S*)tw, scale, lam);
-        }
-        return cudaGetLastError();
+        cudaError_t e = set_smem_once(k_pass_xc<P, N, MODE>, smem, done);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k_pass_xc<P, N, MODE>, N * N / X::LPC, XcStep<N>::NT, smem, st, (S*)W, dev, ps, pm,
+                          (const S*)tw, scale, lam, record);
     }
     static cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw,
-                               double scale, double lam, cudaStream_t st) {
-        KG_DISPATCH_N(N, return passc_x_n<NN>(mode, W, dev, ps, pm, tw, scale, lam, st));
+                               double scale, double lam, int record, cudaStream_t st) {
+        if (mode == MODE_STEP) {
+            KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_STEP>(W, dev, ps, pm, tw, scale, lam, record, st)));
+        }
+        KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_PEEK>(W, dev, ps, pm, tw, scale, lam, record, st)));
     }
-    static int xc_parts(int N) { return N * N / (kXThreads / (N / 8)); }
+    static int xc_parts(int N) {
+        KG_DISPATCH_N(N, return (NN * NN / XcShape<NN, XcStep<NN>::NT>::LPC));
+    }
     static int updatec_parts(int N) { return (int)(((long long)N * N * N + kUpdThreads - 1) / kUpdThreads); }
     static cudaError_t updatec(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
                                const double* w2, double inv_dt, cudaStream_t st) {
         const double qr = 0.25 / (inv_dt * inv_dt), qc = 0.5 * inv_dt * inv_dt;
         KG_DISPATCH_N(N, {
-            k_update<P, NN, true><<<updatec_parts(NN), kUpdThreads, 0, st>>>((S*)W, S0, S1, dev, ps, coef, w2, qr,
-                                                                             qc, C4Args{});
-            return cudaGetLastError();
+            return launch_pdl(k_update<P, NN, true, 0>, updatec_parts(NN), kUpdThreads, 0, st, (S*)W, S0, S1, dev, ps,
+                              coef, w2, qr, qc, C4Args{});
         });
     }
 
@@ -251,15 +276,15 @@ struct Launchers {
                                const double2* coef, const double* w2, double inv_dt, const C4Args& c4,
                                cudaStream_t st) {
         typedef ZStepShape<N> Z;
+        static std::atomic<unsigned long long> done{0};
         constexpr int NX = Lay<N, CPLX>::NX;
         const size_t smem = (size_t)(N * Z::C + N) * sizeof(S);
         auto kern = k_zstep<P, N, CPLX, SCHEME>;
-        cudaError_t e = set_smem(kern, smem);
+        cudaError_t e = set_smem_once(kern, smem, done);
         if (e != cudaSuccess) return e;
         const double qr = 0.25 / (inv_dt * inv_dt), qc = 0.5 * inv_dt * inv_dt;
         dim3 grid((NX + Z::C - 1) / Z::C, N);
-        kern<<<grid, Z::NT, smem, st>>>((S*)W, S0, S1, dev, ps, (const S*)tw, coef, w2, qr, qc, c4);
-        return cudaGetLastError();
+        return launch_pdl(kern, grid, Z::NT, smem, st, (S*)W, S0, S1, dev, ps, (const S*)tw, coef, w2, qr, qc, c4);
     }
     static cudaError_t zstep(int N, bool cplx, void* W, double2* S0, double2* S1, KgDev* dev, double* ps,
                              const void* tw, const double2* coef, const double* w2, double inv_dt, const C4Args* c4,
