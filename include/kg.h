@@ -247,12 +247,11 @@ unsigned long long kg_state_checksum(const void* p, size_t n);
 /* ---- batched parametric ensemble (blow-up studies, section 1 of the paper) ----
  * count independent instances (1..1024) on grids Ns[i] in {64, 128}, side L, step dt,
  * u0 = A[i] exp(-|x|^2 / s[i]^2), v0 = 0, in the precision and nonlinearity of the
- * current options.  Each time step of the whole ensemble is one persistent
- * cooperative kernel launch (four passes separated by bounded grid barriers), and
- * runs of steps are replayed from a captured CUDA graph.  One ensemble per process;
- * independent of the kg_init context.  Errors: KG_EINVAL, KG_ENOTSUP, KG_ENOMEM,
- * KG_ECUDA, KG_ETIMEOUT (a grid barrier wait gave up; the ensemble state is then
- * undefined and must be re-initialised). */
+ * current options.  Up to 50 time steps of the whole ensemble are one persistent
+ * cooperative kernel launch, in which bounded waits order the passes of each
+ * instance.  One ensemble per process; independent of the kg_init context.  Errors:
+ * KG_EINVAL, KG_ENOTSUP, KG_ENOMEM, KG_ECUDA, KG_ETIMEOUT (a bounded wait gave up;
+ * the ensemble state is then undefined and must be re-initialised). */
 int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, const double* s);
 
 /* Advance every instance that has not blown up by up to max_steps steps.  With
@@ -277,8 +276,8 @@ int kg_ens_fetch(int i, double* u);
  * and remember it for later kg_ens_init calls with the same precision and grid mix (and,
  * with kg_ens_set_tune_cache, in the cache file).  A shape is a schedule -- bit 0: column
  * tiles of half the default width; bit 1: the short radix stage first in transforms whose
- * length is not a power of 8 (the 128^3 instances) -- times the unit order (0: instance
- * order, 1: larger grids first) times the resident CTAs per SM.  Every shape computes the
+ * length is not a power of 8 (the 128^3 instances) -- times the unit order (0: the grid
+ * size of the first instance first, 1: larger grids first) times the resident CTAs per SM.  Every shape computes the
  * same step; schedules with bit 1 differ from the others in the rounding of the
  * transforms only.  Advances the ensemble.  blocks_per_sm and order may be NULL. */
 int kg_ens_tune(int steps, int* blocks_per_sm, int* order);

@@ -2,9 +2,8 @@
 //
 // Many independent instances of the scheme of section 1.1.2 (Eq. (2)) on 64^3 and
 // 128^3 grids, initial data u0 = A exp(-|x|^2 / s^2), v0 = 0 (the parametric blow-up
-// studies of section 1), advanced together: each time step is one persistent
-// cooperative launch (k_ens_step), and runs of steps are replayed from a captured
-// CUDA graph.  Launch shape (CTAs per SM, unit visiting order) comes from a small
+// studies of section 1), advanced together: up to kLaunchSteps time steps of the whole
+// ensemble are one persistent cooperative launch (k_ens_run).  Launch shape (CTAs per SM, unit visiting order) comes from a small
 // autotuner that times the candidates on the actual ensemble.
 #include <cuda_runtime.h>
 
@@ -24,7 +23,17 @@ using namespace kg;
 
 namespace {
 
-constexpr int kGraphSteps = 10;
+constexpr int kLaunchSteps = 50;   // steps of one launch, and between looks at the blow-up flags
+
+// Units drawn at a time.  Drawing costs about 2 us of one thread's dependent loads and fences,
+// against 5 to 10 us of work in a unit, so runs of several pay, as long as a pass keeps about three
+// runs for every CTA (else they wait for the slowest of the pass before).  ms per step with runs of
+// 1, 2, 4, 8: 48 + 48 instances double-float 3.02, 2.83, 2.74, 2.73; 256 x 64^3 FP32 1.06, 0.89,
+// 0.81, 0.79; 48 + 48 FP32 1.78, 1.47, 1.33, 1.31.
+constexpr int kMostRun = 8;
+
+// y or z units of a pass over n64 and n128 instances (in the double-float tile width)
+constexpr int pass_units(int n64, int n128) { return 80 * n64 + 576 * n128; }
 
 // launch shape chosen by kg_ens_tune, reused by later kg_ens_init calls with the
 // same precision and the same numbers of 64^3 and 128^3 instances (in this process, and
@@ -211,10 +220,8 @@ struct Ens {
     size_t bytes = 0;
     std::vector<EnsInst> h_inst;
     EnsInst* d_inst = nullptr;
-    unsigned* d_maxkey = nullptr;
-    unsigned* d_bar = nullptr;
+    EnsPlan* d_plan = nullptr;
     int* d_status = nullptr;
-    unsigned long long* d_step = nullptr;
     int* d_order = nullptr;
     double* d_feat = nullptr;
     double2* tmp = nullptr;     // two FP64 spectral scratch arrays of the largest grid
@@ -226,7 +233,6 @@ struct Ens {
     double threshold = -1.0;
     int missing = 0;
     long long spin_limit = 1ll << 24;
-    cudaGraphExec_t gexec = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 };
 
@@ -247,7 +253,6 @@ int ealloc(Ens* e, void** p, size_t bytes, const char* what) {
 void ens_destroy(Ens* e) {
     if (!e) return;
     if (e->stream) cudaStreamSynchronize(e->stream);
-    if (e->gexec) cudaGraphExecDestroy(e->gexec);
     for (void* p : e->allocs) cudaFree(p);
     if (e->ev0) cudaEventDestroy(e->ev0);
     if (e->ev1) cudaEventDestroy(e->ev1);
@@ -268,23 +273,18 @@ EnsParams make_params(const Ens* e) {
     std::memset(&p, 0, sizeof(p));
     p.inst = e->d_inst;
     p.count = e->count;
-    p.order = e->order;
+    p.plan = e->d_plan;
     for (int t = 0; t < 2; t++) {
-        EnsTab& tb = t == 0 ? p.tab64 : p.tab128;
         if (e->have[t]) {
-            tb.tw = e->tab[t].tw;
-            tb.coef = e->tab[t].coef;
-            tb.w2 = e->tab[t].w2;
+            p.tab[t].tw = e->tab[t].tw;
+            p.tab[t].coef = e->tab[t].coef;
         }
     }
-    p.maxkey = e->d_maxkey;
-    p.bar = e->d_bar;
     p.status = e->d_status;
-    p.step_ctr = e->d_step;
     p.order_idx = e->d_order;
     p.lam = e->lam;
-    p.inv_dt = 1.0 / e->dt;
     p.thr_key = threshold_key(e->threshold);
+    p.run = kMostRun;
     p.missing = e->missing;
     p.spin_limit = e->spin_limit;
     return p;
@@ -299,31 +299,10 @@ int upload_order(Ens* e) {
     return KG_OK;
 }
 
-int rebuild_graph(Ens* e) {
-    if (e->gexec) {
-        cudaGraphExecDestroy(e->gexec);
-        e->gexec = nullptr;
-    }
-    const EnsParams p = make_params(e);
-    cudaGraph_t g = nullptr;
-    KG_ECK(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t le = cudaSuccess;
-    for (int s = 0; s < kGraphSteps && le == cudaSuccess; s++) le = e->pl->ens_step(p, e->grid, e->sched, e->stream);
-    cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
-    if (le != cudaSuccess || ce != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return efail(KG_ECUDA, std::string("ensemble graph capture: ") + cudaGetErrorString(le != cudaSuccess ? le : ce));
-    }
-    cudaError_t ie = cudaGraphInstantiate(&e->gexec, g, 0);
-    cudaGraphDestroy(g);
-    if (ie != cudaSuccess) return efail(KG_ECUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
-    return KG_OK;
-}
-
 int check_status(Ens* e) {
     int st = 0;
     KG_ECK(cudaMemcpy(&st, e->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (st != 0) return efail(KG_ETIMEOUT, "ensemble grid barrier wait timed out");
+    if (st != 0) return efail(KG_ETIMEOUT, "a bounded wait of the ensemble kernel gave up");
     return KG_OK;
 }
 
@@ -334,15 +313,15 @@ int set_shape(Ens* e, int sched, int bps, int order) {
     e->bps = std::max(1, std::min(bps, maxb));
     e->grid = e->bps * e->nsm;
     e->order = order;
-    int rc = upload_order(e);
-    if (!rc) rc = rebuild_graph(e);
-    return rc;
+    return upload_order(e);
 }
 
-// one run of n steps without the graph (used for remainders and by the tuner)
+// n steps of every live instance, in launches of at most kLaunchSteps
 int launch_steps(Ens* e, int n) {
     const EnsParams p = make_params(e);
-    for (int s = 0; s < n; s++) KG_ECK(e->pl->ens_step(p, e->grid, e->sched, e->stream));
+    for (; n > 0; n -= kLaunchSteps) {
+        KG_ECK(e->pl->ens_run(p, e->grid, e->sched, e->order, std::min(n, kLaunchSteps), e->stream));
+    }
     return KG_OK;
 }
 
@@ -426,10 +405,8 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
     KG_ETRY(ealloc(e, (void**)&bw, off_w, "ensemble W1"));
     KG_ETRY(ealloc(e, (void**)&bw2, off_w, "ensemble W2"));
     KG_ETRY(ealloc(e, (void**)&e->d_inst, sizeof(EnsInst) * count, "ensemble descriptors"));
-    KG_ETRY(ealloc(e, (void**)&e->d_maxkey, sizeof(unsigned) * 2 * count, "ensemble max keys"));
-    KG_ETRY(ealloc(e, (void**)&e->d_bar, sizeof(unsigned) * 2, "ensemble barrier"));
+    KG_ETRY(ealloc(e, (void**)&e->d_plan, sizeof(EnsPlan), "ensemble plan"));
     KG_ETRY(ealloc(e, (void**)&e->d_status, sizeof(int), "ensemble status"));
-    KG_ETRY(ealloc(e, (void**)&e->d_step, sizeof(unsigned long long), "ensemble step counter"));
     KG_ETRY(ealloc(e, (void**)&e->d_order, sizeof(int) * count, "ensemble order"));
     KG_ETRY(ealloc(e, (void**)&e->d_feat, sizeof(double) * 4 * count, "ensemble features"));
     e->h_inst.resize(count);
@@ -453,10 +430,7 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
         if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "shells launch"));
     }
     if (cudaMemcpyAsync(e->d_inst, e->h_inst.data(), sizeof(EnsInst) * count, cudaMemcpyHostToDevice, e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->d_maxkey, 0, sizeof(unsigned) * 2 * count, e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->d_bar, 0, sizeof(unsigned) * 2, e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->d_status, 0, sizeof(int), e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->d_step, 0, sizeof(unsigned long long), e->stream) != cudaSuccess)
+        cudaMemsetAsync(e->d_status, 0, sizeof(int), e->stream) != cudaSuccess)
         KG_ETRY(efail(KG_ECUDA, "ensemble state upload"));
     if (cudaStreamSynchronize(e->stream) != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "ensemble init"));
     e->threshold = -1.0;
@@ -467,7 +441,15 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
         const bool use = (g_tuned.valid && g_tuned.prec == e->prec && g_tuned.n64 == n64 && g_tuned.n128 == n128 &&
                           (t = g_tuned, true)) ||
                          cache_lookup(e->prec, n64, n128, &t);
-        KG_ETRY(set_shape(e, use ? t.sched : 0, use ? t.bps : 2, use ? t.order : 1));
+        // untuned: as many CTAs as fit, fewer where a pass has few units for each; half-width
+        // tiles for FP32 (256 x 64^3: 0.79 ms per step against 0.85; 16-byte precisions no gain).
+        // ms per step double-float with 2, 3, 4 CTAs per SM: 8 x 64^3 (640 units) 0.075, 0.074,
+        // 0.083; 128^3 (576) 0.088, 0.112, 0.109; 3 + 1 (816) 0.127, 0.127, 0.154; 12 x 64^3 (960)
+        // 0.110, 0.092, 0.094; 2 x 128^3 (1152) 0.152, 0.140, 0.133; 24 x 64^3 0.195, 0.176, 0.163
+        const int sched = e->pl->store_bytes == 8 ? 1 : 0;
+        const int maxb = e->pl->ens_blocks_per_sm(sched), units = pass_units(n64, n128);
+        const int bps = std::min(maxb, units < 5 * e->nsm ? 2 : units < 6 * e->nsm ? 3 : maxb);
+        KG_ETRY(set_shape(e, use ? t.sched : sched, use ? t.bps : bps, use ? t.order : 1));
     }
 #undef KG_ETRY
     g_ens = e;
@@ -478,25 +460,15 @@ int kg_ens_run(int max_steps, double threshold, long long* steps_done, double* m
     Ens* e = g_ens;
     if (!e) return efail(KG_ESTATE, "kg_ens_run before kg_ens_init");
     if (max_steps < 0 || !std::isfinite(threshold)) return efail(KG_EINVAL, "bad arguments");
-    if (threshold != e->threshold) {
-        e->threshold = threshold;
-        int rc = rebuild_graph(e);
-        if (rc) return rc;
-    }
+    e->threshold = threshold;
     long long done = 0;
     KG_ECK(cudaEventRecord(e->ev0, e->stream));
-    const int check_every = 5 * kGraphSteps;
     while (done < max_steps) {
-        const long long left = max_steps - done;
-        if (left >= kGraphSteps) {
-            KG_ECK(cudaGraphLaunch(e->gexec, e->stream));
-            done += kGraphSteps;
-        } else {
-            int rc = launch_steps(e, (int)left);
-            if (rc) return rc;
-            done += left;
-        }
-        if (done % check_every == 0 || done >= max_steps) {
+        const int n = (int)std::min<long long>(max_steps - done, kLaunchSteps);
+        int rl = launch_steps(e, n);
+        if (rl) return rl;
+        done += n;
+        {
             // stop early once every instance has blown up
             KG_ECK(cudaMemcpyAsync(e->h_inst.data(), e->d_inst, sizeof(EnsInst) * e->count, cudaMemcpyDeviceToHost,
                                    e->stream));

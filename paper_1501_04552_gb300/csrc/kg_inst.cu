@@ -109,8 +109,8 @@ cudaError_t xc_readout(int N, void* spec, double2* u, const void* tw, double sca
     return Lp::xc_readout(N, spec, u, tw, scale, st);
 }
 #elif KG_PART == 4
-cudaError_t ens_step(const EnsParams& p, int grid, int sched, cudaStream_t st) {
-    return Lp::ens_step(p, grid, sched, st);
+cudaError_t ens_run(const EnsParams& p, int grid, int sched, int order, int steps, cudaStream_t st) {
+    return Lp::ens_run(p, grid, sched, order, steps, st);
 }
 int ens_blocks_per_sm(int sched) { return Lp::ens_blocks_per_sm(sched); }
 #else

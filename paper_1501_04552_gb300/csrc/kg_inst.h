@@ -41,7 +41,7 @@
     KG_INST_FN(xc_setup) xc_setup;                                                     \
     KG_INST_FN(xc_readout) xc_readout;                                                 \
     KG_INST_FN(zc_to_f64) zc_to_f64;                                                   \
-    KG_INST_FN(ens_step) ens_step;            /* share 4: ensemble step */             \
+    KG_INST_FN(ens_run) ens_run;              /* share 4: ensemble step */             \
     KG_INST_FN(ens_blocks_per_sm) ens_blocks_per_sm;                                   \
     }
 

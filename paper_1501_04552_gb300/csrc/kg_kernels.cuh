@@ -478,10 +478,9 @@ struct ColAddr {
 
 // one column (T = N/8 threads, thread j) of a tile; valid == false for the columns
 // of the last tile beyond the plane (they compute on zeros and store nothing)
-template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, int CW, bool RF = false>
+template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, class SM, bool RF = false>
 __device__ __forceinline__ void col_body(const typename Pin::S* src, typename Pout::S* dst, int plane, int kx,
-                                         bool valid, int j, ColSmem<P, CW>& csm,
-                                         const typename P::S* __restrict__ tw) {
+                                         bool valid, int j, SM& csm, const typename P::S* __restrict__ tw) {
     typedef typename P::R R;
     typedef ColAddr<N, DIR, CPLX, false> In;
     typedef ColAddr<N, DIR, CPLX, true> Out;
@@ -495,7 +494,7 @@ __device__ __forceinline__ void col_body(const typename Pin::S* src, typename Po
             else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
         }
     }
-    fft<P, N, ColSmem<P, CW>, false, RF, false, false>(v, j, tw, 1, csm, SIGN);   // outputs go to W or FP64
+    fft<P, N, SM, false, RF, false, false>(v, j, tw, 1, csm, SIGN);   // outputs go to W or FP64
     if (valid) {
         typename Pout::S* d0 = dst + Out::base(plane, kx);
 #pragma unroll
@@ -531,7 +530,7 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
     pdl_wait();
-    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, C>(src, dst, plane, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
+    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, ColSmem<P, C>>(src, dst, plane, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
 }
 
 // inverse z column FFT from an FP64 spectral array into W2 (precision P); the source is
@@ -548,7 +547,7 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
     const int kx = blockIdx.x * C + c;
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
-    col_body<PrecF64, P, P, N, +1, COL_Z, CPLX, C>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
+    col_body<PrecF64, P, P, N, +1, COL_Z, CPLX, ColSmem<P, C>>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
 }
 
 // ---------------------------------------------------------------------------
@@ -556,10 +555,10 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
 // in one pass over W2.  coef[m2] = (2 c_k, 2 beta_k) for integer m2 = mx^2 + my^2 + mz^2.
 // One (ky, kx) column (T = N/8 threads, thread j).
 // ---------------------------------------------------------------------------
-template <class P, int N, int CW = ColShape<P>::C, bool RF = false>
+template <class P, int N, class SM, bool RF = false>
 __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const double2* __restrict__ cur,
                                        double2* __restrict__ old, int kx, int ky, bool valid, int j,
-                                       ColSmem<P, CW>& csm, const typename P::S* __restrict__ tw,
+                                       SM& csm, const typename P::S* __restrict__ tw,
                                        const double2* __restrict__ coef) {
     typedef typename P::R R;
     typedef cx<R> Cx;
@@ -577,7 +576,7 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
     constexpr bool kShare = sizeof(typename P::S) == 16;
 #pragma unroll(kShare ? 1 : 2)
     for (int dir = 0; dir < 2; dir++) {
-        fft<P, N, ColSmem<P, CW>, false, RF, false>(v, j, tw, 1, csm, dir == 0 ? -1 : +1);
+        fft<P, N, SM, false, RF, false>(v, j, tw, 1, csm, dir == 0 ? -1 : +1);
         if (dir == 1) break;
         const int my = ky <= N / 2 ? ky : ky - N;
         const int mxy2 = kx * kx + my * my;

@@ -384,7 +384,7 @@ struct Launchers {
         }
     }
 
-    // the ensemble step (kg_ensemble.cuh); schedules differ in tile shape and stage order,
+    // the ensemble's steps (kg_ensemble.cuh); schedules differ in tile shape and stage order,
     // not in shared memory (a unit's tiles always hold 2048 values)
     template <int SCHED>
     static size_t ens_smem_s() {
@@ -395,13 +395,13 @@ struct Launchers {
         size_t m = a > b ? a : b;
         m = m > c ? m : c;
         m = m > d ? m : d;
-        return m * sizeof(S);
+        return (m + kEnsTables) * sizeof(S);   // and both twiddle tables
     }
     template <int SCHED>
     static int ens_blocks_per_sm_s() {
-        if (set_smem(k_ens_step<P, SCHED>, ens_smem_s<SCHED>()) != cudaSuccess) return 0;
+        if (set_smem(k_ens_run<P, SCHED>, ens_smem_s<SCHED>()) != cudaSuccess) return 0;
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_step<P, SCHED>, kEnsThreads, ens_smem_s<SCHED>()) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_run<P, SCHED>, kEnsThreads, ens_smem_s<SCHED>()) !=
             cudaSuccess)
             return 0;
         return n;
@@ -416,8 +416,11 @@ struct Launchers {
         }
     }
     template <int SCHED>
-    static cudaError_t ens_step_s(const EnsParams& p, int grid, cudaStream_t st) {
-        cudaError_t e = set_smem(k_ens_step<P, SCHED>, ens_smem_s<SCHED>());
+    static cudaError_t ens_run_s(const EnsParams& p, int grid, int order, int steps, cudaStream_t st) {
+        cudaError_t e = set_smem(k_ens_run<P, SCHED>, ens_smem_s<SCHED>());
+        if (e != cudaSuccess) return e;
+        k_ens_plan<P, SCHED><<<1, kEnsMaxInst, 0, st>>>(p, order, steps, grid);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid);
@@ -429,14 +432,14 @@ struct Launchers {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_ens_step<P, SCHED>, p);
+        return cudaLaunchKernelEx(&cfg, k_ens_run<P, SCHED>, p);
     }
-    static cudaError_t ens_step(const EnsParams& p, int grid, int sched, cudaStream_t st) {
+    static cudaError_t ens_run(const EnsParams& p, int grid, int sched, int order, int steps, cudaStream_t st) {
         switch (sched) {
-            case 0: return ens_step_s<0>(p, grid, st);
-            case 1: return ens_step_s<1>(p, grid, st);
-            case 2: return ens_step_s<2>(p, grid, st);
-            case 3: return ens_step_s<3>(p, grid, st);
+            case 0: return ens_run_s<0>(p, grid, order, steps, st);
+            case 1: return ens_run_s<1>(p, grid, order, steps, st);
+            case 2: return ens_run_s<2>(p, grid, order, steps, st);
+            case 3: return ens_run_s<3>(p, grid, order, steps, st);
             default: return cudaErrorInvalidValue;
         }
     }
