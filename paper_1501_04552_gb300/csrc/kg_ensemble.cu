@@ -21,6 +21,35 @@
 
 using namespace kg;
 
+namespace kg {
+__global__ void __launch_bounds__(128) k_ens_axis(const EnsInst* inst, const double* s, double L, const double2* tw64,
+                                                  const double2* tw128, EnsAxis* out) {
+    __shared__ double g[128], g3[128];
+    const int i = blockIdx.x, t = threadIdx.x, N = inst[i].N;
+    const double2* tw = N == 64 ? tw64 : tw128;   // exp(-2 pi i j / N)
+    EnsAxis& ax = out[i];
+    if (t < N) {
+        const double x = -L / 2 + (L / N) * t;
+        const double v = exp(-x * x * (1.0 / (s[i] * s[i])));
+        g[t] = v;
+        g3[t] = v * v * v;
+        ax.g[t] = v;
+    }
+    __syncthreads();
+    if (t <= N / 2) {
+        NSum a, b;
+        a.s = a.c = b.s = b.c = 0.0;
+        for (int j = 0; j < N; j++) {
+            const double c = tw[(t * j) & (N - 1)].x;
+            a.add(g[j] * c);
+            b.add(g3[j] * c);
+        }
+        ax.G[t] = a.value();
+        ax.G3[t] = b.value();
+    }
+}
+}  // namespace kg
+
 namespace {
 
 constexpr int kLaunchSteps = 50;   // steps of one launch, and between looks at the blow-up flags
@@ -134,21 +163,10 @@ int efail(int code, const std::string& msg) { return set_last_error(code, msg); 
         if (e_ != cudaSuccess) return efail(KG_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// u = A exp(-|x|^2 / s^2) on the N^3 grid x_j = -L/2 + j L/N (an initial field, not the method)
-__global__ void k_gaussian(double* u, int N, double L, double A, double s) {
-    const size_t n3 = (size_t)N * N * N;
-    const double h = L / N, inv_s2 = 1.0 / (s * s);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % N), y = (int)((i / N) % N), z = (int)(i / ((size_t)N * N));
-        const double px = -L / 2 + h * x, py = -L / 2 + h * y, pz = -L / 2 + h * z;
-        u[i] = A * exp(-(px * px + py * py + pz * pz) * inv_s2);
-    }
-}
-
 // low-mode shell energies of uh^0: (h^3/N^3) sum_{shell} w_k omega_k^2 |uh_k|^2 / 2,
-// shells |m| in {0}, (0,1], (1,2], (2,4]; one CTA, one instance
+// shells |m| in {0}, (0,1], (1,2], (2,4]; one CTA per instance
 template <int N>
-__global__ void k_shells(const double2* __restrict__ uh, double L, double* __restrict__ out4) {
+__device__ __forceinline__ void shells(const double2* __restrict__ uh, double L, double* __restrict__ out4) {
     __shared__ double acc[4][256];
     double loc[4] = {0, 0, 0, 0};
     const double kf = 2.0 * 3.14159265358979323846 / L;
@@ -170,6 +188,12 @@ __global__ void k_shells(const double2* __restrict__ uh, double L, double* __res
         const double h = L / N;
         out4[threadIdx.x] = s * h * h * h / ((double)N * N * N);
     }
+}
+
+__global__ void __launch_bounds__(256) k_shells(const EnsInst* inst, double L, double* out) {
+    const EnsInst& in = inst[blockIdx.x];
+    if (in.N == 64) shells<64>(in.S0, L, out + 4 * blockIdx.x);
+    else shells<128>(in.S0, L, out + 4 * blockIdx.x);
 }
 
 // shell energies of many sampled Gaussians A exp(-|x|^2/s^2) on the N^3 grid: the field
@@ -388,7 +412,10 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
     const size_t spec_max = spec_slots(nmax, false);
     KG_ETRY(ealloc(e, (void**)&e->tmp, sizeof(double2) * spec_max, "ensemble spectral scratch"));
     KG_ETRY(ealloc(e, (void**)&e->tmp2, sizeof(double2) * spec_max, "ensemble spectral scratch"));
-    KG_ETRY(ealloc(e, (void**)&e->phys, sizeof(double) * (size_t)nmax * nmax * nmax, "ensemble physical scratch"));
+    static_assert(2 * kEnsMaxInst * sizeof(double) + kEnsMaxInst * sizeof(EnsAxis) <= (size_t)2 * 64 * 64 * 64 * 8,
+                  "the set-up's 1D data fits the physical scratch");
+    KG_ETRY(ealloc(e, (void**)&e->phys, sizeof(double) * std::max((size_t)nmax * nmax * nmax, (size_t)2 * 64 * 64 * 64),
+                   "ensemble physical scratch"));
     // one allocation per array class, instances at 256-byte aligned offsets
     size_t off_s = 0, off_w = 0;
     std::vector<size_t> os(count), ow(count);
@@ -411,27 +438,40 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
     KG_ETRY(ealloc(e, (void**)&e->d_feat, sizeof(double) * 4 * count, "ensemble features"));
     e->h_inst.resize(count);
     for (int i = 0; i < count; i++) {
-        const int N = Ns[i];
-        const int t = N == 64 ? 0 : 1;
         EnsInst& in = e->h_inst[i];
         std::memset(&in, 0, sizeof(in));
         in.S0 = (double2*)(b0 + os[i]);
         in.S1 = (double2*)(b1 + os[i]);
         in.W1 = (void*)(bw + ow[i]);
         in.W2 = (void*)(bw2 + ow[i]);
-        in.N = N;
+        in.N = Ns[i];
         in.blowup_level = -1;
-        k_gaussian<<<kStrideCtas, 256, 0, e->stream>>>(e->phys, N, L, A[i], s[i]);
-        if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "gaussian launch"));
-        // the scratch array serves as W2 (16 bytes a slot) during the set-up
-        KG_ETRY(init_state(N, e->prec, dt, e->lam, e->tab[t], e->phys, nullptr, false, in.S0, in.S1, in.W1, e->tmp,
-                           e->tmp2, e->stream));
-        (N == 64 ? k_shells<64> : k_shells<128>)<<<1, 256, 0, e->stream>>>(in.S0, L, e->d_feat + 4 * i);
-        if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "shells launch"));
     }
+    // A, s and the 1D transforms travel through the physical scratch
+    double* d_A = e->phys;
+    double* d_s = d_A + kEnsMaxInst;
+    EnsAxis* axis = reinterpret_cast<EnsAxis*>(d_s + kEnsMaxInst);
     if (cudaMemcpyAsync(e->d_inst, e->h_inst.data(), sizeof(EnsInst) * count, cudaMemcpyHostToDevice, e->stream) != cudaSuccess ||
+        cudaMemcpyAsync(d_A, A, sizeof(double) * count, cudaMemcpyHostToDevice, e->stream) != cudaSuccess ||
+        cudaMemcpyAsync(d_s, s, sizeof(double) * count, cudaMemcpyHostToDevice, e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_status, 0, sizeof(int), e->stream) != cudaSuccess)
         KG_ETRY(efail(KG_ECUDA, "ensemble state upload"));
+    k_ens_axis<<<count, 128, 0, e->stream>>>(e->d_inst, d_s, L, e->tab[0].tw64, e->tab[1].tw64, axis);
+    if (cudaGetLastError() != cudaSuccess ||
+        e->pl->ens_fill(e->d_inst, count, axis, d_A, e->lam, e->tab[0].coef, e->tab[1].coef, e->stream) != cudaSuccess)
+        KG_ETRY(efail(KG_ECUDA, "ensemble set-up launch"));
+    if (e->pl->store_bytes != sizeof(double2)) {
+        // FP32 work arrays: the inverse z and y transforms of uh^0, as a step leaves them
+        for (int i = 0; i < count; i++) {
+            const EnsInst& in = e->h_inst[i];
+            const Tables& tb = e->tab[in.N == 64 ? 0 : 1];
+            if (e->pl->z_from_f64(in.N, in.S0, in.S1, nullptr, in.W2, tb.tw, e->stream) != cudaSuccess ||
+                e->pl->yi(in.N, in.W2, in.W1, tb.tw, FinArgs{}, e->stream) != cudaSuccess)
+                KG_ETRY(efail(KG_ECUDA, "ensemble set-up transforms"));
+        }
+    }
+    k_shells<<<count, 256, 0, e->stream>>>(e->d_inst, L, e->d_feat);
+    if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "shells launch"));
     if (cudaStreamSynchronize(e->stream) != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "ensemble init"));
     e->threshold = -1.0;
     {

@@ -426,4 +426,62 @@ __global__ void __launch_bounds__(kEnsThreads, EnsMinBlocks<P>::value) k_ens_run
     }
 }
 
+// ---------------------------------------------------------------------------
+// Set-up of the Gaussian instances.  u0 = A exp(-|x|^2/s^2) is a product g(x) g(y) g(z) on the grid,
+// and so is u0^3; their transforms are products of 1D ones, and the yz-inverse of uh^0 that W1
+// holds is N^2 A g(z) g(y) G(kx).  So a set-up is 130 sums of N terms and one pass that writes the
+// arrays, in place of three 3D transforms in FP64: kg_ens_init of 48 + 48 double-float instances 36.1
+// -> 5.7 ms, of 256 x 64^3 FP32 ones 35.9 -> 5.4 ms (most of what is left is allocation)
+// ---------------------------------------------------------------------------
+// per instance: g_j (N values), G(m) and the transform of g^3 (m = 0..N/2 each; both real, since
+// the grid has x_{N-j} = -x_j), compensated FP64 sums
+struct EnsAxis {
+    double g[128], G[65], G3[65];
+};
+
+__global__ void __launch_bounds__(128) k_ens_axis(const EnsInst* inst, const double* s, double L, const double2* tw64,
+                                                  const double2* tw128, EnsAxis* out);
+
+// S0 = uh^0, S1 = uh^{-1} = c uh^0 + beta F^0 (v0 = 0) and, with W1 in FP64 or double-float, its
+// x-lines; the slots of padding get zeros
+template <class P, int N>
+__device__ __forceinline__ void ens_fill(const EnsInst& in, const EnsAxis& ax, double A, double lam,
+                                         const double2* __restrict__ coef) {
+    typedef ModeIndex<N, false> MI;
+    typedef typename P::S S;
+    constexpr unsigned PITCH = Lay<N>::PITCH;
+    const double A3 = lam * (A * A * A), An2 = A * ((double)N * N);
+    S* W1 = (S*)in.W1;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)MI::kSlots; i += gridDim.x * blockDim.x) {
+        const MI mi(i);
+        double a = 0.0, b = 0.0;
+        if (mi.valid) {
+            const int my = mi.ky <= N / 2 ? mi.ky : N - mi.ky, mz = mi.kz <= N / 2 ? mi.kz : N - mi.kz;
+            const double2 cf = coef[mi.m2];
+            a = A * (ax.G[mi.kx] * ax.G[my] * ax.G[mz]);
+            b = 0.5 * cf.x * a + 0.5 * cf.y * (A3 * (ax.G3[mi.kx] * ax.G3[my] * ax.G3[mz]));
+        }
+        in.S0[i] = make_double2(a, 0.0);
+        in.S1[i] = make_double2(b, 0.0);
+        if constexpr (sizeof(S) == 16) {
+            const unsigned row = i / PITCH, kx = i - row * PITCH;
+            const double w = kx <= N / 2 ? An2 * (ax.g[row / N] * ax.g[row % N] * ax.G[kx]) : 0.0;
+            W1[i] = P::pack(cmake<typename P::R>(P::from_f64(w), P::from_f64(0.0)));
+        }
+    }
+}
+
+template <class P>
+__global__ void __launch_bounds__(256) k_ens_fill(const EnsInst* inst, const EnsAxis* axis, const double* A, double lam,
+                                                  EnsTab t64, EnsTab t128) {
+    __shared__ EnsAxis ax;
+    const int i = blockIdx.y;
+    const EnsInst in = inst[i];
+    const double* src = reinterpret_cast<const double*>(axis + i);
+    for (int k = threadIdx.x; k < (int)(sizeof(EnsAxis) / 8); k += blockDim.x) reinterpret_cast<double*>(&ax)[k] = src[k];
+    __syncthreads();
+    if (in.N == 64) ens_fill<P, 64>(in, ax, A[i], lam, t64.coef);
+    else ens_fill<P, 128>(in, ax, A[i], lam, t128.coef);
+}
+
 }  // namespace kg

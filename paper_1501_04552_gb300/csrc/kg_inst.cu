@@ -113,6 +113,10 @@ cudaError_t ens_run(const EnsParams& p, int grid, int sched, int order, int step
     return Lp::ens_run(p, grid, sched, order, steps, st);
 }
 int ens_blocks_per_sm(int sched) { return Lp::ens_blocks_per_sm(sched); }
+cudaError_t ens_fill(const EnsInst* inst, int count, const EnsAxis* axis, const double* A, double lam,
+                     const double2* coef64, const double2* coef128, cudaStream_t st) {
+    return Lp::ens_fill(inst, count, axis, A, lam, coef64, coef128, st);
+}
 #else
 #error "KG_PART out of range"
 #endif

@@ -43,6 +43,7 @@
     KG_INST_FN(zc_to_f64) zc_to_f64;                                                   \
     KG_INST_FN(ens_run) ens_run;              /* share 4: ensemble step */             \
     KG_INST_FN(ens_blocks_per_sm) ens_blocks_per_sm;                                   \
+    KG_INST_FN(ens_fill) ens_fill;                                                     \
     }
 
 namespace kg {

@@ -7,7 +7,7 @@ namespace kg {
 
 #define KG_TABLE_COMMON(ns, S)                                                                                 \
     &ns::pass_x, &ns::yf, &ns::yi, &ns::zcol, &ns::z_from_f64, &ns::update, &ns::update_parts, &ns::ens_run, \
-        &ns::ens_blocks_per_sm, &ns::x_parts, S, &ns::passc_x, &ns::xc_parts, &ns::yfc, &ns::yic, &ns::zcolc, \
+        &ns::ens_blocks_per_sm, &ns::ens_fill, &ns::x_parts, S, &ns::passc_x, &ns::xc_parts, &ns::yfc, &ns::yic, &ns::zcolc, \
         &ns::zc_from_f64, &ns::updatec, &ns::updatec_parts
 
 const PassLaunch kLaunchF64 = {

@@ -15,6 +15,8 @@ constexpr int kStrideCtasDeep = 152 * 8;
 
 struct KgDev;
 struct EnsParams;
+struct EnsInst;
+struct EnsAxis;
 
 // the composed scheme's per-substep data, passed by value to the update kernels
 struct C4Args {
@@ -59,6 +61,9 @@ struct PassLaunch {
     // schedule can hold
     cudaError_t (*ens_run)(const EnsParams& p, int grid, int sched, int order, int steps, cudaStream_t st);
     int (*ens_blocks_per_sm)(int sched);
+    // fill the state (and the 16-byte work arrays) of Gaussian instances from their 1D transforms
+    cudaError_t (*ens_fill)(const EnsInst* inst, int count, const EnsAxis* axis, const double* A, double lam,
+                            const double2* coef64, const double2* coef128, cudaStream_t st);
     int (*x_parts)(int N);
     size_t store_bytes;  // bytes of one complex value of W
     // complex field (full N^3 spectrum, N columns per plane): x pass, column FFTs,

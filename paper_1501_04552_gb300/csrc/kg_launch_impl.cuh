@@ -443,6 +443,13 @@ struct Launchers {
             default: return cudaErrorInvalidValue;
         }
     }
+    static cudaError_t ens_fill(const EnsInst* inst, int count, const EnsAxis* axis, const double* A, double lam,
+                                const double2* coef64, const double2* coef128, cudaStream_t st) {
+        // 64 CTAs an instance: one slot in ten a thread at 64^3
+        k_ens_fill<P><<<dim3(64, count), 256, 0, st>>>(inst, axis, A, lam, EnsTab{nullptr, coef64},
+                                                      EnsTab{nullptr, coef128});
+        return cudaGetLastError();
+    }
 };
 
 }  // namespace kg
