@@ -56,6 +56,7 @@ struct Ctx {
     size_t slots = 0;              // complex values a spectral array holds (modes and padding)
     cudaStream_t own_stream = nullptr;
     const PassLaunch* pl = nullptr;
+    int lg = 3;              // layout of S0, S1 and W2 (struct Lay)
     double2* S0 = nullptr;   // FP64 state arrays; dev->phase tells which holds uh^n
     double2* S1 = nullptr;
     void* W1 = nullptr;      // work arrays in the pass precision: x-lines (live between steps) and
@@ -155,8 +156,8 @@ int ensure_scratch(Ctx* c) {
 int inverse_yz_f64(Ctx* c, const double2* src0, const double2* src1, const KgDev* sel) {
     const int N = c->N;
     cudaStream_t st = stream_of(c);
-    KG_CK((c->cplx ? kLaunchF64.zc_from_f64 : kLaunchF64.z_from_f64)(N, src0, src1, sel, c->W2, c->tw64, st));
-    KG_CK((c->cplx ? kLaunchF64.yic : kLaunchF64.yi)(N, c->W2, c->tmp, c->tw64, FinArgs{}, st));
+    KG_CK((c->cplx ? kLaunchF64.zc_from_f64 : kLaunchF64.z_from_f64)(N, src0, src1, sel, c->W2, c->tw64, c->lg, st));
+    KG_CK((c->cplx ? kLaunchF64.yic : kLaunchF64.yi)(N, c->W2, c->tmp, c->tw64, c->lg, FinArgs{}, st));
     return KG_OK;
 }
 
@@ -275,6 +276,7 @@ int create_ctx(int N, double L, double dt, bool cplx, Ctx** out) {
     c->lam = g_opt.nonlinearity;
     c->prec = g_opt.precision;
     c->pl = launcher(c->prec);
+    c->lg = c->pl->lg(N);
     c->cplx = cplx;
     c->nspec = (size_t)N * N * (cplx ? N : c->NH);
     c->slots = spec_slots(N, cplx);
@@ -439,6 +441,7 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
     const double h = c->L / N;
     const double p_norm = c->lam * h * h * h / 4.0;
     const double q_norm = h * h * h * inv_n3(N);
+    const int lg = c->lg;
     auto yf = c->cplx ? c->pl->yfc : c->pl->yf;
     auto yi = c->cplx ? c->pl->yic : c->pl->yi;
     auto zcol = c->cplx ? c->pl->zcolc : c->pl->zcol;
@@ -458,7 +461,7 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
         fx.count = c->cplx ? c->pl->xc_parts(N) : c->pl->x_parts(N);
     }
     if (timed) KG_CK(cudaEventRecord(c->ev[1], st));
-    if (!xy) KG_CK(yf(N, c->W1, c->W2, c->tw, fx, st));
+    if (!xy) KG_CK(yf(N, c->W1, c->W2, c->tw, lg, fx, st));
     if (timed) KG_CK(cudaEventRecord(c->ev[2], st));
     const bool fused = c->pl->zstep != nullptr;
     const C4Args c4{c->kick, 3 * (N / 2) * (N / 2) + 1, {c->c4h[0], c->c4h[1], c->c4h[2]}};
@@ -472,7 +475,7 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
     } else {
         // the IEEE FP64 passes, bound by the FP64 pipe throughout, keep the three kernels
         // (the fused form measured slower there)
-        KG_CK(zcol(N, -1, c->W2, c->tw, st));                                     // forward z -> F^n
+        KG_CK(zcol(N, -1, c->W2, c->tw, lg, st));                                     // forward z -> F^n
         if (timed) KG_CK(cudaEventRecord(c->ev[3], st));
         if (c->cplx) {
             KG_CK(c->pl->updatec(N, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->coef, c->w2, 1.0 / c->dt, st));
@@ -482,11 +485,11 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
             fz.count = c->pl->update_parts(N);
         }
         if (timed) KG_CK(cudaEventRecord(c->ev[4], st));
-        KG_CK(zcol(N, +1, c->W2, c->tw, st));                                     // inverse z
+        KG_CK(zcol(N, +1, c->W2, c->tw, lg, st));                                     // inverse z
     }
     if (xy) KG_CK(launch_fin(fz, nullptr, nullptr, st));
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    if (!xy) KG_CK(yi(N, c->W2, c->W1, c->tw, fz, st));
+    if (!xy) KG_CK(yi(N, c->W2, c->W1, c->tw, lg, fz, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -515,7 +518,7 @@ bool use_xy(const Ctx* c) {
 // the inverse y pass that ends a kg_step call of the fused form (W1 back to the y-inverse)
 int xy_close(Ctx* c, cudaStream_t st, bool timed, float* ms) {
     if (timed) KG_CK(cudaEventRecord(c->ev[5], st));
-    KG_CK(c->pl->yi(c->N, c->W2, c->W1, c->tw, FinArgs{}, st));
+    KG_CK(c->pl->yi(c->N, c->W2, c->W1, c->tw, c->lg, FinArgs{}, st));
     if (timed) {
         KG_CK(cudaEventRecord(c->ev[6], st));
         KG_CK(cudaEventSynchronize(c->ev[6]));
@@ -574,7 +577,7 @@ int p_from_state(Ctx* c, bool older, double* out) {
 // (enqueued: the caller synchronises)
 int state_to_host(Ctx* c, const double2* s, void* host) {
     cudaStream_t st = stream_of(c);
-    KG_CK(launch_repack(c->N, c->cplx, true, s, c->tmp, st));
+    KG_CK(launch_repack(c->N, c->cplx, true, s, c->tmp, c->lg, st));
     KG_CK(cudaMemcpyAsync(host, c->tmp, sizeof(double2) * c->nspec, cudaMemcpyDeviceToHost, st));
     return KG_OK;
 }
@@ -612,9 +615,9 @@ int energy_composed(Ctx* c, double* E) {
     KG_CK(launch_x_inverse(N, c->tmp, c->phys, c->tw64, inv_n3(N), c->part_sum, st));   // u^n, sum u^4
     KG_CK(launch_fin_sum(c->part_sum, x_inverse_parts(N), c->lam * h * h * h / 4.0, c->scal + 1, st));
     double2* F = (double2*)c->W2;
-    rc = forward3d_f64(N, c->phys, c->tmp, F, c->tw64, 1, c->lam, st);   // F = R2C(lam u^3)
+    rc = forward3d_f64(N, c->phys, c->tmp, F, c->tw64, 1, c->lam, c->lg, st);   // F = R2C(lam u^3)
     if (rc) return rc;
-    KG_CK(launch_energy_c4(N, c->S0, c->S1, F, c->kick, c->w2, c->part_sum, kStrideCtas, st));
+    KG_CK(launch_energy_c4(N, c->S0, c->S1, F, c->kick, c->w2, c->part_sum, kStrideCtas, c->lg, st));
     KG_CK(launch_fin_sum(c->part_sum, kStrideCtas, h * h * h * inv_n3(N), c->scal, st));
     double v[2];
     KG_CK(cudaMemcpyAsync(v, c->scal, sizeof(v), cudaMemcpyDeviceToHost, st));
@@ -727,7 +730,7 @@ int kg_energy(double* E) {
         const double2* cur = d.phase ? c->S1 : c->S0;
         const double2* old = d.phase ? c->S0 : c->S1;
         const int np = kStrideCtas;
-        KG_CK(launch_energy_q(N, cur, old, c->w2, 1.0 / c->dt, c->part_sum, np, c->cplx, st));
+        KG_CK(launch_energy_q(N, cur, old, c->w2, 1.0 / c->dt, c->part_sum, np, c->cplx, c->lg, st));
         KG_CK(launch_fin_sum(c->part_sum, np, h * h * h * inv_n3(N), c->scal, st));
         KG_CK(cudaMemcpyAsync(&Q, c->scal, sizeof(double), cudaMemcpyDeviceToHost, st));
         KG_CK(cudaStreamSynchronize(st));
@@ -778,8 +781,8 @@ int kg_fetch_device(double* d_u) {
         // the FP64 scratch used as x-lines of the pass precision, then the inverse x into d_u
         const int N = c->N;
         cudaStream_t st = stream_of(c);
-        KG_CK(c->pl->z_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
-        KG_CK(c->pl->yi(N, c->W2, c->tmp, c->tw, FinArgs{}, st));
+        KG_CK(c->pl->z_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, c->lg, st));
+        KG_CK(c->pl->yi(N, c->W2, c->tmp, c->tw, c->lg, FinArgs{}, st));
         KG_CK(c->pl->x_readout(N, c->tmp, d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -819,8 +822,8 @@ int kg_fetch_complex_device(double* d_u) {
         // read-out in the pass precision (double-float), as kg_fetch_device
         const int N = c->N;
         cudaStream_t st = stream_of(c);
-        KG_CK(c->pl->zc_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, st));
-        KG_CK(c->pl->yic(N, c->W2, c->tmp, c->tw, FinArgs{}, st));
+        KG_CK(c->pl->zc_from_f64(N, c->S0, c->S1, c->dev, c->W2, c->tw, c->lg, st));
+        KG_CK(c->pl->yic(N, c->W2, c->tmp, c->tw, c->lg, FinArgs{}, st));
         KG_CK(c->pl->xc_readout(N, c->tmp, (double2*)d_u, c->tw, inv_n3(N), st));
         return KG_OK;
     }
@@ -1066,13 +1069,13 @@ int kg_load_state(const void* h, size_t len) {
     d.complex_field = cplx ? 1 : 0;
     d.scheme = c->scheme;
     cudaError_t e = cudaMemcpyAsync(c->tmp, base + sizeof(hd), arr, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S0, st);
+    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S0, c->lg, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->tmp, base + sizeof(hd) + arr, arr, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S1, st);
+    if (e == cudaSuccess) e = launch_repack(N, cplx, false, c->tmp, c->S1, c->lg, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st);
     // W1 = the yz inverse of uh^n in the pass precision, as the last two transforms of a step leave it
-    if (e == cudaSuccess) e = (cplx ? c->pl->zc_from_f64 : c->pl->z_from_f64)(N, c->S0, c->S1, nullptr, c->W2, c->tw, st);
-    if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, FinArgs{}, st);
+    if (e == cudaSuccess) e = (cplx ? c->pl->zc_from_f64 : c->pl->z_from_f64)(N, c->S0, c->S1, nullptr, c->W2, c->tw, c->lg, st);
+    if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, c->lg, FinArgs{}, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         destroy(c);

@@ -33,18 +33,18 @@ cudaError_t launch_x_inverse(int N, const double2* in, double* u, const double2*
 int x_inverse_parts(int N) { return N * N / (kXThreads / (N / 16)); }
 
 cudaError_t launch_startup(int N, const double2* a, double2* b, const double2* f, const double2* coef, double dt,
-                           bool cplx, cudaStream_t st) {
+                           bool cplx, int lg, cudaStream_t st) {
     KG_DISPATCH_N(N, {
-        if (cplx) k_startup<NN, true><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, coef, dt);
-        else k_startup<NN, false><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, coef, dt);
+        if (cplx) k_startup<NN, true><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, coef, dt, lg);
+        else k_startup<NN, false><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, coef, dt, lg);
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_startup_c4(int N, const double2* a, double2* b, const double2* f, const double2* kick0,
-                              cudaStream_t st) {
+                              int lg, cudaStream_t st) {
     KG_DISPATCH_N(N, {
-        k_startup_c4<NN><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, kick0);
+        k_startup_c4<NN><<<kStrideCtasDeep, 256, 0, st>>>(a, b, f, kick0, lg);
         return cudaGetLastError();
     });
 }
@@ -55,15 +55,15 @@ cudaError_t launch_startup_c4(int N, const double2* a, double2* b, const double2
 template <int N>
 __global__ void __launch_bounds__(256) k_energy_c4(const double2* __restrict__ a, const double2* __restrict__ P,
                                                    const double2* __restrict__ f, const double2* __restrict__ kick0,
-                                                   const double* __restrict__ w2tab, double* __restrict__ part_sum) {
+                                                   const double* __restrict__ w2tab, double* __restrict__ part_sum, int lg) {
     typedef ModeIndex<N, false> MI;
     __shared__ double red[96];
-    const size_t total = (size_t)MI::kSlots;
+    const size_t total = MI::slots(lg);
     NSum acc;
     acc.s = 0.0;
     acc.c = 0.0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const MI mi((unsigned)i);
+        const MI mi((unsigned)i, lg);
         if (!mi.valid) continue;
         const double w = mi.twice ? 2.0 : 1.0;
         const double2 kc = kick0[mi.m2], ai = a[i], pi = P[i], fi = f[i];
@@ -77,28 +77,29 @@ __global__ void __launch_bounds__(256) k_energy_c4(const double2* __restrict__ a
 }
 
 cudaError_t launch_energy_c4(int N, const double2* a, const double2* P, const double2* f, const double2* kick0,
-                             const double* w2tab, double* part_sum, int nparts, cudaStream_t st) {
+                             const double* w2tab, double* part_sum, int nparts, int lg, cudaStream_t st) {
     KG_DISPATCH_N(N, {
-        k_energy_c4<NN><<<nparts, 256, 0, st>>>(a, P, f, kick0, w2tab, part_sum);
+        k_energy_c4<NN><<<nparts, 256, 0, st>>>(a, P, f, kick0, w2tab, part_sum, lg);
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_energy_q(int N, const double2* x, const double2* y, const double* w2tab, double inv_dt,
-                            double* part_sum, int nparts, bool cplx, cudaStream_t st) {
+                            double* part_sum, int nparts, bool cplx, int lg, cudaStream_t st) {
     KG_DISPATCH_N(N, {
-        if (cplx) k_energy_q<NN, true><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum);
-        else k_energy_q<NN, false><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum);
+        if (cplx) k_energy_q<NN, true><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum, lg);
+        else k_energy_q<NN, false><<<nparts, 256, 0, st>>>(x, y, w2tab, inv_dt, part_sum, lg);
         return cudaGetLastError();
     });
 }
 
-cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, cudaStream_t st) {
+cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, int lg,
+                          cudaStream_t st) {
     KG_DISPATCH_N(N, {
-        if (cplx && to_packed) k_repack<NN, true, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
-        else if (cplx) k_repack<NN, true, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
-        else if (to_packed) k_repack<NN, false, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
-        else k_repack<NN, false, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out);
+        if (cplx && to_packed) k_repack<NN, true, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out, lg);
+        else if (cplx) k_repack<NN, true, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out, lg);
+        else if (to_packed) k_repack<NN, false, true><<<kStrideCtasDeep, 256, 0, st>>>(in, out, lg);
+        else k_repack<NN, false, false><<<kStrideCtasDeep, 256, 0, st>>>(in, out, lg);
         return cudaGetLastError();
     });
 }

@@ -166,7 +166,7 @@ int efail(int code, const std::string& msg) { return set_last_error(code, msg); 
 // low-mode shell energies of uh^0: (h^3/N^3) sum_{shell} w_k omega_k^2 |uh_k|^2 / 2,
 // shells |m| in {0}, (0,1], (1,2], (2,4]; one CTA per instance
 template <int N>
-__device__ __forceinline__ void shells(const double2* __restrict__ uh, double L, double* __restrict__ out4) {
+__device__ __forceinline__ void shells(const double2* __restrict__ uh, int lg, double L, double* __restrict__ out4) {
     __shared__ double acc[4][256];
     double loc[4] = {0, 0, 0, 0};
     const double kf = 2.0 * 3.14159265358979323846 / L;
@@ -176,7 +176,7 @@ __device__ __forceinline__ void shells(const double2* __restrict__ uh, double L,
         const int sh = (m2 == 0) ? 0 : (m2 <= 1) ? 1 : (m2 <= 4) ? 2 : (m2 <= 16) ? 3 : -1;
         if (sh < 0) continue;
         const int ky = (my + N) % N, kz = (mz + N) % N;
-        const double2 v = uh[Lay<N>::zcol(ky, mx) + 8 * (size_t)kz];
+        const double2 v = uh[Lay<N>::zcol(ky, mx, lg) + ((size_t)kz << lg)];
         const double w = (mx == 0 || mx == N / 2) ? 1.0 : 2.0;
         loc[sh] += w * 0.5 * (1.0 + kf * kf * m2) * (v.x * v.x + v.y * v.y);
     }
@@ -190,10 +190,10 @@ __device__ __forceinline__ void shells(const double2* __restrict__ uh, double L,
     }
 }
 
-__global__ void __launch_bounds__(256) k_shells(const EnsInst* inst, double L, double* out) {
+__global__ void __launch_bounds__(256) k_shells(const EnsInst* inst, int lg, double L, double* out) {
     const EnsInst& in = inst[blockIdx.x];
-    if (in.N == 64) shells<64>(in.S0, L, out + 4 * blockIdx.x);
-    else shells<128>(in.S0, L, out + 4 * blockIdx.x);
+    if (in.N == 64) shells<64>(in.S0, lg, L, out + 4 * blockIdx.x);
+    else shells<128>(in.S0, lg, L, out + 4 * blockIdx.x);
 }
 
 // shell energies of many sampled Gaussians A exp(-|x|^2/s^2) on the N^3 grid: the field
@@ -465,12 +465,13 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
         for (int i = 0; i < count; i++) {
             const EnsInst& in = e->h_inst[i];
             const Tables& tb = e->tab[in.N == 64 ? 0 : 1];
-            if (e->pl->z_from_f64(in.N, in.S0, in.S1, nullptr, in.W2, tb.tw, e->stream) != cudaSuccess ||
-                e->pl->yi(in.N, in.W2, in.W1, tb.tw, FinArgs{}, e->stream) != cudaSuccess)
+            if (e->pl->z_from_f64(in.N, in.S0, in.S1, nullptr, in.W2, tb.tw, e->pl->lg(in.N), e->stream) != cudaSuccess ||
+                e->pl->yi(in.N, in.W2, in.W1, tb.tw, e->pl->lg(in.N), FinArgs{}, e->stream) != cudaSuccess)
                 KG_ETRY(efail(KG_ECUDA, "ensemble set-up transforms"));
         }
     }
-    k_shells<<<count, 256, 0, e->stream>>>(e->d_inst, L, e->d_feat);
+    // (the layout is the same for both grids)
+    k_shells<<<count, 256, 0, e->stream>>>(e->d_inst, e->pl->lg(64), L, e->d_feat);
     if (cudaGetLastError() != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "shells launch"));
     if (cudaStreamSynchronize(e->stream) != cudaSuccess) KG_ETRY(efail(KG_ECUDA, "ensemble init"));
     e->threshold = -1.0;
@@ -565,8 +566,8 @@ int kg_ens_fetch(int i, double* u) {
     const int N = in.N;
     const Tables& tb = e->tab[N == 64 ? 0 : 1];
     const double2* cur = in.phase ? in.S1 : in.S0;
-    KG_ECK(kLaunchF64.z_from_f64(N, cur, cur, nullptr, e->tmp2, tb.tw64, e->stream));
-    KG_ECK(kLaunchF64.yi(N, e->tmp2, e->tmp, tb.tw64, FinArgs{}, e->stream));
+    KG_ECK(kLaunchF64.z_from_f64(N, cur, cur, nullptr, e->tmp2, tb.tw64, e->pl->lg(N), e->stream));
+    KG_ECK(kLaunchF64.yi(N, e->tmp2, e->tmp, tb.tw64, e->pl->lg(N), FinArgs{}, e->stream));
     KG_ECK(launch_x_inverse(N, e->tmp, e->phys, tb.tw64, 1.0 / ((double)N * N * N), nullptr, e->stream));
     KG_ECK(cudaMemcpyAsync(u, e->phys, sizeof(double) * (size_t)N * N * N, cudaMemcpyDeviceToHost, e->stream));
     KG_ECK(cudaStreamSynchronize(e->stream));

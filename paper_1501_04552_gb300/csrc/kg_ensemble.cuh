@@ -114,8 +114,8 @@ struct TileSmem {
     typename P::S* base;
     int c;
     unsigned bar;
-    __device__ __forceinline__ void put(int row, cx<typename P::R> v) { base[row * C + c] = P::pack(v); }
-    __device__ __forceinline__ cx<typename P::R> get(int row) const { return P::load(base[row * C + c]); }
+    __device__ __forceinline__ void put(int row, cx<typename P::R> v) { base[col_slot<P, C>(row, c)] = P::pack(v); }
+    __device__ __forceinline__ cx<typename P::R> get(int row) const { return P::load(base[col_slot<P, C>(row, c)]); }
     __device__ __forceinline__ void sync() const {
         if (NT <= 32) __syncwarp();
         else asm volatile("bar.sync %0, %1;\n" ::"r"(bar), "r"(NT) : "memory");
@@ -193,7 +193,7 @@ template <class P, int N, int SCHED, int SIGN, int DIR>
 __device__ __noinline__ void ens_y(const typename P::S* src, typename P::S* dst, int unit) {
     EnsTile<P, N, SCHED> t(unit);
     col_body<P, P, P, N, SIGN, DIR, false, decltype(t.csm), EnsSched<SCHED>::remfirst>(
-        src, dst, t.plane, t.kx, t.valid, t.j, t.csm, ens_twiddles<typename P::S, N>());
+        src, dst, t.plane, t.kx, t.valid, t.j, t.csm, ens_twiddles<typename P::S, N>(), LayLg<P, N>::value);
 }
 
 template <class P, int N, int SCHED>
@@ -450,10 +450,11 @@ __device__ __forceinline__ void ens_fill(const EnsInst& in, const EnsAxis& ax, d
     typedef ModeIndex<N, false> MI;
     typedef typename P::S S;
     constexpr unsigned PITCH = Lay<N>::PITCH;
+    constexpr int LG = LayLg<P, N>::value;
     const double A3 = lam * (A * A * A), An2 = A * ((double)N * N);
     S* W1 = (S*)in.W1;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)MI::kSlots; i += gridDim.x * blockDim.x) {
-        const MI mi(i);
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < MI::slots(LG); i += gridDim.x * blockDim.x) {
+        const MI mi(i, LG);
         double a = 0.0, b = 0.0;
         if (mi.valid) {
             const int my = mi.ky <= N / 2 ? mi.ky : N - mi.ky, mz = mi.kz <= N / 2 ? mi.kz : N - mi.kz;
@@ -463,7 +464,9 @@ __device__ __forceinline__ void ens_fill(const EnsInst& in, const EnsAxis& ax, d
         }
         in.S0[i] = make_double2(a, 0.0);
         in.S1[i] = make_double2(b, 0.0);
-        if constexpr (sizeof(S) == 16) {
+    }
+    if constexpr (sizeof(S) == 16) {
+        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)Lay<N>::kSlots; i += gridDim.x * blockDim.x) {
             const unsigned row = i / PITCH, kx = i - row * PITCH;
             const double w = kx <= N / 2 ? An2 * (ax.g[row / N] * ax.g[row % N] * ax.G[kx]) : 0.0;
             W1[i] = P::pack(cmake<typename P::R>(P::from_f64(w), P::from_f64(0.0)));

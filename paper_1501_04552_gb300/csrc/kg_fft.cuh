@@ -25,6 +25,7 @@
 // values of index j + T s (s = 0..7) before every stage and after the last one, so
 // a forward transform can feed an inverse one without any exchange.
 #pragma once
+#include <type_traits>
 #include "kg_arith.cuh"
 
 namespace kg {
@@ -51,28 +52,35 @@ __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_
 // x-pass modes: one stepping pass, or a read-only pass for P^n
 enum { MODE_STEP = 0, MODE_PEEK = 1 };
 
-// Layouts of the spectral arrays, NX = N/2 + 1 columns (N for a complex field) in TL tiles of
-// eight columns:
-//   x-lines   (W1)            [z][y][kx], rows of PITCH = 8 TL values, so that every row of a
-//                             column tile starts on its own 64- or 128-byte boundary;
-//   z-columns (W2, the state) [ky][kx / 8][kz][kx % 8]: the (ky, kx) column tile of the z pass
-//                             is one contiguous run (64 KB of state at N = 512).
+// Layouts of the spectral arrays, NX = N/2 + 1 columns (N for a complex field):
+//   x-lines   (W1)            [z][y][kx], rows of PITCH values (a multiple of 8), so that every row of
+//                             a column tile starts on its own 64- or 128-byte boundary;
+//   z-columns (W2, the state) [ky][kx / TW][kz][kx % TW], tiles of TW = 2^lg columns: the column tile
+//                             a CTA of the z pass takes is one contiguous run per array.
 // The z pass reads and writes five arrays' worth of data against two for a y pass, and with
 // rows a whole plane (2.1 MB at N = 512) apart it reached 0.7 of the copy bandwidth; the
-// scattered rows now fall to the y passes, which write or read them at no measured cost
-// (512^3: z pass 1.696 -> 1.584 ms double-float, 0.988 -> 0.808 ms FP32, before prefetching;
-// y passes 0.568 and 0.228 ms either way).
+// scattered rows now fall to the y passes, which write or read them at little cost (512^3: z
+// pass 1.764 -> 1.543 ms double-float with tiles of eight columns, 1.389 with tiles of four;
+// 0.998 -> 0.785 ms FP32).  TW is a property of a context's precision and grid (LayLg): four
+// columns, 64-byte rows of 16-byte values, for double-float at 512^3 (at 256^3 the z pass gains
+// nothing, 0.185 against 0.184 ms, and the y passes lose 3 %); eight for FP32, whose y passes lose
+// more on 32-byte rows (0.213 -> 0.257 ms) than its z pass gains (0.761 -> 0.736), and for FP64,
+// which is bound by its arithmetic.  The FP64 kernels that serve every context take lg at run time.
+template <class P, int N>
+struct LayLg {
+    static constexpr int value = std::is_same<P, PrecDF>::value && N >= 512 ? 2 : 3;
+};
 template <int N, bool CPLX = false>
 struct Lay {
     static constexpr int NX = CPLX ? N : N / 2 + 1;
-    static constexpr int TL = (NX + 7) / 8;
-    static constexpr int PITCH = 8 * TL;
+    static constexpr int PITCH = (NX + 7) / 8 * 8;
     static constexpr long long kSlots = (long long)N * N * PITCH;   // values an array holds, padding included
-    // z-columns: element (ky, kx, kz); consecutive kz are 8 apart
-    static __host__ __device__ __forceinline__ size_t zcol(int ky, int kx) {
-        return (size_t)(ky * TL + (kx >> 3)) * (8 * N) + (kx & 7);
+    static __host__ __device__ __forceinline__ int tiles(int lg) { return (NX + (1 << lg) - 1) >> lg; }
+    // z-columns: element (ky, kx, kz); consecutive kz are 2^lg apart, consecutive ky ky_stride
+    static __host__ __device__ __forceinline__ size_t zcol(int ky, int kx, int lg) {
+        return ((size_t)(ky * tiles(lg) + (kx >> lg)) * N << lg) + (kx & ((1 << lg) - 1));
     }
-    static constexpr size_t kKyStride = (size_t)TL * 8 * N;         // consecutive ky
+    static __host__ __device__ __forceinline__ size_t ky_stride(int lg) { return (size_t)tiles(lg) * N << lg; }
 };
 
 constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n >> 1); }
@@ -226,12 +234,21 @@ __device__ __forceinline__ const S* stage_table(const S* __restrict__ g, S* sm, 
 // shared-memory views
 // ---------------------------------------------------------------------------
 // column tile: element (row, column c) at base[row * C + c]; the whole CTA syncs
+// Where rows are shorter than the 128 bytes of one wavefront, the rows that share 128 bytes are
+// swapped by the row's bits 3.. (a stage writes rows eight apart and reads consecutive ones), so
+// that neither side has bank conflicts (FP32 tiles of eight: z pass 0.794 -> 0.759 ms at 512^3)
+template <class P, int C>
+__device__ __forceinline__ int col_slot(int row, int c) {
+    constexpr int Q = 128 / (C * (int)sizeof(typename P::S));   // rows per 128 bytes
+    if (Q <= 1) return row * C + c;
+    return (row / Q) * (Q * C) + ((row ^ (row >> 3)) & (Q - 1)) * C + c;
+}
 template <class P, int C>
 struct ColSmem {
     typename P::S* base;
     int c;
-    __device__ __forceinline__ void put(int row, cx<typename P::R> v) { base[row * C + c] = P::pack(v); }
-    __device__ __forceinline__ cx<typename P::R> get(int row) const { return P::load(base[row * C + c]); }
+    __device__ __forceinline__ void put(int row, cx<typename P::R> v) { base[col_slot<P, C>(row, c)] = P::pack(v); }
+    __device__ __forceinline__ cx<typename P::R> get(int row) const { return P::load(base[col_slot<P, C>(row, c)]); }
     __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 

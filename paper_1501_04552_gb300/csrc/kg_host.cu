@@ -19,20 +19,20 @@ const double kPi = 3.14159265358979323846;
 
 // FP64 R2C of a physical device array into the z-columns of out, through the x-lines in
 // `lines`; cube: lam u^3 instead of u
-int forward3d(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+int forward3d(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam, int lg,
               cudaStream_t st) {
     KG_HCK(launch_x_forward(N, u, lines, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.yf(N, lines, out, tw64, FinArgs{}, st));
-    KG_HCK(kLaunchF64.zcol(N, -1, out, tw64, st));
+    KG_HCK(kLaunchF64.yf(N, lines, out, tw64, lg, FinArgs{}, st));
+    KG_HCK(kLaunchF64.zcol(N, -1, out, tw64, lg, st));
     return KG_OK;
 }
 // FP64 forward 3D transform of a complex physical device array (full spectrum);
 // cube: of lam |u|^2 u instead of u
-int forward3d_c(int N, const double2* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
+int forward3d_c(int N, const double2* u, double2* lines, double2* out, const double2* tw64, int cube, double lam, int lg,
                 cudaStream_t st) {
     KG_HCK(launch_xc_forward(N, u, lines, tw64, cube, lam, st));
-    KG_HCK(kLaunchF64.yfc(N, lines, out, tw64, FinArgs{}, st));
-    KG_HCK(kLaunchF64.zcolc(N, -1, out, tw64, st));
+    KG_HCK(kLaunchF64.yfc(N, lines, out, tw64, lg, FinArgs{}, st));
+    KG_HCK(kLaunchF64.zcolc(N, -1, out, tw64, lg, st));
     return KG_OK;
 }
 // forward 3D transform of a physical FP64 array in the pass precision of pl, through the
@@ -40,7 +40,7 @@ int forward3d_c(int N, const double2* u, double2* lines, double2* out, const dou
 int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W1, void* W2, double2* out, const void* tw,
                    int cube, double lam, cudaStream_t st) {
     KG_HCK(pl->x_setup(N, u, W1, tw, cube, lam, st));
-    KG_HCK(pl->yf(N, W1, W2, tw, FinArgs{}, st));
+    KG_HCK(pl->yf(N, W1, W2, tw, pl->lg(N), FinArgs{}, st));
     KG_HCK(pl->z_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
@@ -48,15 +48,15 @@ int forward3d_pass(int N, const PassLaunch* pl, const double* u, void* W1, void*
 int forward3d_c_pass(int N, const PassLaunch* pl, const double2* u, void* W1, void* W2, double2* out, const void* tw,
                      int cube, double lam, cudaStream_t st) {
     KG_HCK(pl->xc_setup(N, u, W1, tw, cube, lam, st));
-    KG_HCK(pl->yfc(N, W1, W2, tw, FinArgs{}, st));
+    KG_HCK(pl->yfc(N, W1, W2, tw, pl->lg(N), FinArgs{}, st));
     KG_HCK(pl->zc_to_f64(N, W2, out, tw, st));
     return KG_OK;
 }
 }  // namespace
 
 int forward3d_f64(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
-                  cudaStream_t st) {
-    return forward3d(N, u, lines, out, tw64, cube, lam, st);
+                  int lg, cudaStream_t st) {
+    return forward3d(N, u, lines, out, tw64, cube, lam, lg, st);
 }
 
 const PassLaunch* launcher_for(int prec) {
@@ -152,7 +152,7 @@ int init_state(int N, int prec, double dt, double lam, const Tables& tb, double*
     const bool pass = pass_precision && pl->x_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
         return pass ? forward3d_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
-                    : forward3d(N, phys, (double2*)W2, out, tb.tw64, cube, lam, st);
+                    : forward3d(N, phys, (double2*)W2, out, tb.tw64, cube, lam, pl->lg(N), st);
     };
     int rc = fwd(fbuf, 1);              // F^0 = R2C(lam u0^3)
     if (!rc) rc = fwd(S0, 0);           // uh^0
@@ -164,10 +164,10 @@ int init_state(int N, int prec, double dt, double lam, const Tables& tb, double*
     } else {
         KG_HCK(cudaMemsetAsync(S1, 0, sizeof(double2) * slots, st));
     }
-    if (kick0) KG_HCK(launch_startup_c4(N, S0, S1, fbuf, kick0, st));    // S1 = P^0
-    else KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, false, st));  // S1 = uh^{-1}
-    KG_HCK(pl->z_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));   // z inverse of uh^0
-    KG_HCK(pl->yi(N, W2, W1, tb.tw, FinArgs{}, st));                        // y inverse
+    if (kick0) KG_HCK(launch_startup_c4(N, S0, S1, fbuf, kick0, pl->lg(N), st));    // S1 = P^0
+    else KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, false, pl->lg(N), st));  // S1 = uh^{-1}
+    KG_HCK(pl->z_from_f64(N, S0, S1, nullptr, W2, tb.tw, pl->lg(N), st));   // z inverse of uh^0
+    KG_HCK(pl->yi(N, W2, W1, tb.tw, pl->lg(N), FinArgs{}, st));                        // y inverse
     return KG_OK;
 }
 
@@ -180,7 +180,7 @@ int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, doubl
     const bool pass = pass_precision && pl->xc_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
         return pass ? forward3d_c_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
-                    : forward3d_c(N, phys, (double2*)W2, out, tb.tw64, cube, lam, st);
+                    : forward3d_c(N, phys, (double2*)W2, out, tb.tw64, cube, lam, pl->lg(N), st);
     };
     int rc = fwd(fbuf, 1);              // F^0 = FFT(lam |u0|^2 u0)
     if (!rc) rc = fwd(S0, 0);           // uh^0
@@ -192,9 +192,9 @@ int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, doubl
     } else {
         KG_HCK(cudaMemsetAsync(S1, 0, sizeof(double2) * n3, st));
     }
-    KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, true, st));       // S1 = uh^{-1}
-    KG_HCK(pl->zc_from_f64(N, S0, S1, nullptr, W2, tb.tw, st));          // z inverse of uh^0
-    KG_HCK(pl->yic(N, W2, W1, tb.tw, FinArgs{}, st));                               // y inverse
+    KG_HCK(launch_startup(N, S0, S1, fbuf, tb.coef, dt, true, pl->lg(N), st));       // S1 = uh^{-1}
+    KG_HCK(pl->zc_from_f64(N, S0, S1, nullptr, W2, tb.tw, pl->lg(N), st));          // z inverse of uh^0
+    KG_HCK(pl->yic(N, W2, W1, tb.tw, pl->lg(N), FinArgs{}, st));                               // y inverse
     return KG_OK;
 }
 

@@ -41,18 +41,18 @@ cudaError_t xy_fused(int N, int do_yi, const void* W1, void* W2, KgDev* dev, dou
 }
 int xy_parts(int N) { return Lp::xy_parts(N); }
 #elif KG_PART == 1
-cudaError_t yf(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
-    return Lp::yf_t<false>(N, W1, W2, tw, fin, st);
+cudaError_t yf(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yf_t<false>(N, W1, W2, tw, lg, fin, st);
 }
-cudaError_t yi(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
-    return Lp::yi_t<false>(N, W2, W1, tw, fin, st);
+cudaError_t yi(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yi_t<false>(N, W2, W1, tw, lg, fin, st);
 }
-cudaError_t zcol(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
-    return Lp::zcol_t<false>(N, sign, W2, tw, st);
+cudaError_t zcol(int N, int sign, void* W2, const void* tw, int lg, cudaStream_t st) {
+    return Lp::zcol_t<false>(N, sign, W2, tw, lg, st);
 }
 cudaError_t z_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2, const void* tw,
-                       cudaStream_t st) {
-    return Lp::z_from_f64_t<false>(N, src0, src1, dev, W2, tw, st);
+                       int lg, cudaStream_t st) {
+    return Lp::z_from_f64_t<false>(N, src0, src1, dev, W2, tw, lg, st);
 }
 cudaError_t z_to_f64(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
     return Lp::z_to_f64_t<false>(N, W2, out, tw, st);
@@ -81,18 +81,18 @@ cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm
     return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, record, st);
 }
 int xc_parts(int N) { return Lp::xc_parts(N); }
-cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
-    return Lp::yf_t<true>(N, W1, W2, tw, fin, st);
+cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yf_t<true>(N, W1, W2, tw, lg, fin, st);
 }
-cudaError_t yic(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
-    return Lp::yi_t<true>(N, W2, W1, tw, fin, st);
+cudaError_t yic(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+    return Lp::yi_t<true>(N, W2, W1, tw, lg, fin, st);
 }
-cudaError_t zcolc(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
-    return Lp::zcol_t<true>(N, sign, W2, tw, st);
+cudaError_t zcolc(int N, int sign, void* W2, const void* tw, int lg, cudaStream_t st) {
+    return Lp::zcol_t<true>(N, sign, W2, tw, lg, st);
 }
 cudaError_t zc_from_f64(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2, const void* tw,
-                       cudaStream_t st) {
-    return Lp::z_from_f64_t<true>(N, src0, src1, dev, W2, tw, st);
+                       int lg, cudaStream_t st) {
+    return Lp::z_from_f64_t<true>(N, src0, src1, dev, W2, tw, lg, st);
 }
 cudaError_t zc_to_f64(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
     return Lp::z_to_f64_t<true>(N, W2, out, tw, st);

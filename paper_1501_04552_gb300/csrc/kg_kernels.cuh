@@ -456,49 +456,63 @@ template <class P>
 struct ColShape {
     static constexpr int C = 128 / (int)sizeof(typename P::S);
 };
-// Column tiles of the single-state step: 128-byte rows, except the FP32 y passes (64-byte
-// rows: twice the CTAs for the same occupancy, and the width of a row of z-columns).
-template <class P, bool YPASS>
+// Column tiles of the y passes (and the FP64 z columns): 128-byte rows, except the FP32 ones
+// (64-byte rows: twice the CTAs for the same occupancy, and the width of a row of z-columns) and
+// the double-float ones at 512^3 (four CTAs of 256 threads per SM instead of two of 512 wait less
+// at barriers: 0.509 and 0.543 ms against 0.543 and 0.584; at 256^3 0.065 and 0.068 against 0.064
+// and 0.064)
+template <class P, int N, bool YPASS>
 struct ColStep {
-    static constexpr int C = (YPASS && sizeof(typename P::S) == 8 ? 64 : 128) / (int)sizeof(typename P::S);
+    static constexpr bool kNarrow = YPASS && (sizeof(typename P::S) == 8 || (std::is_same<P, PrecDF>::value && N >= 512));
+    static constexpr int C = (kNarrow ? 64 : 128) / (int)sizeof(typename P::S);
 };
 
-// where column kx of a plane starts in a source (dst == false) or destination array, and
+// where column kx of a plane starts in a source (DST == false) or destination array, and
 // the distance of its rows
 template <int N, int DIR, bool CPLX, bool DST>
 struct ColAddr {
     typedef Lay<N, CPLX> Ly;
     static constexpr bool kLines = DST ? DIR == COL_YI : DIR == COL_YF;   // x-lines
-    static constexpr size_t kStride = DIR == COL_Z ? 8 : kLines ? (size_t)Ly::PITCH : Ly::kKyStride;
-    static __device__ __forceinline__ size_t base(int plane, int kx) {
-        if (DIR == COL_Z) return Ly::zcol(plane, kx);
-        return kLines ? (size_t)plane * N * Ly::PITCH + kx : Ly::zcol(0, kx) + 8 * (size_t)plane;
+    static __device__ __forceinline__ size_t stride(int lg) {
+        return DIR == COL_Z ? (size_t)1 << lg : kLines ? (size_t)Ly::PITCH : Ly::ky_stride(lg);
+    }
+    static __device__ __forceinline__ size_t base(int plane, int kx, int lg) {
+        if (DIR == COL_Z) return Ly::zcol(plane, kx, lg);
+        return kLines ? (size_t)plane * N * Ly::PITCH + kx : Ly::zcol(0, kx, lg) + ((size_t)plane << lg);
     }
 };
+
+// the layout a kernel of precision P works in: its own, or for FP64 the context's
+template <class P, int N>
+__device__ __forceinline__ int lay_lg(int lg) {
+    return std::is_same<P, PrecF64>::value ? lg : LayLg<P, N>::value;
+}
 
 // one column (T = N/8 threads, thread j) of a tile; valid == false for the columns
 // of the last tile beyond the plane (they compute on zeros and store nothing)
 template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, class SM, bool RF = false>
 __device__ __forceinline__ void col_body(const typename Pin::S* src, typename Pout::S* dst, int plane, int kx,
-                                         bool valid, int j, SM& csm, const typename P::S* __restrict__ tw) {
+                                         bool valid, int j, SM& csm, const typename P::S* __restrict__ tw, int lg) {
     typedef typename P::R R;
     typedef ColAddr<N, DIR, CPLX, false> In;
     typedef ColAddr<N, DIR, CPLX, true> Out;
     constexpr int T = N / 8;
     cx<R> v[8];
     {
-        const typename Pin::S* s0 = src + In::base(plane, kx);
+        const typename Pin::S* s0 = src + In::base(plane, kx, lg);
+        const size_t st = In::stride(lg);
 #pragma unroll
         for (int s = 0; s < 8; s++) {
-            if (valid) v[s] = Convert<Pin, P>::go(Pin::load(s0[(size_t)(j + T * s) * In::kStride]));
+            if (valid) v[s] = Convert<Pin, P>::go(Pin::load(s0[(size_t)(j + T * s) * st]));
             else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
         }
     }
     fft<P, N, SM, false, RF, false, false>(v, j, tw, 1, csm, SIGN);   // outputs go to W or FP64
     if (valid) {
-        typename Pout::S* d0 = dst + Out::base(plane, kx);
+        typename Pout::S* d0 = dst + Out::base(plane, kx, lg);
+        const size_t st = Out::stride(lg);
 #pragma unroll
-        for (int s = 0; s < 8; s++) d0[(size_t)(j + T * s) * Out::kStride] = Pout::pack(Convert<P, Pout>::go(v[s]));
+        for (int s = 0; s < 8; s++) d0[(size_t)(j + T * s) * st] = Pout::pack(Convert<P, Pout>::go(v[s]));
     }
 }
 
@@ -515,7 +529,7 @@ struct ColMinBlocks {
 
 template <class Pin, class P, class Pout, int N, int SIGN, int DIR, bool CPLX, int CW>
 __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::value) k_col(const typename Pin::S* src, typename Pout::S* dst,
-                                                    const typename P::S* __restrict__ tw, FinArgs fin) {
+                                                    const typename P::S* __restrict__ tw, int lg, FinArgs fin) {
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
@@ -530,14 +544,16 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
     pdl_wait();
-    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, ColSmem<P, C>>(src, dst, plane, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
+    col_body<Pin, P, Pout, N, SIGN, DIR, CPLX, ColSmem<P, C>>(src, dst, plane, kx, kx < Lay<N, CPLX>::NX, j, csm, tw,
+                                                               lay_lg<P, N>(lg));
 }
 
 // inverse z column FFT from an FP64 spectral array into W2 (precision P); the source is
 // src1 when dev != NULL and dev->phase == 1, src0 otherwise (the current level's array)
 template <class P, int N, bool CPLX, int CW>
 __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::value) k_col_sel(const double2* src0, const double2* src1, const KgDev* dev,
-                                                        typename P::S* dst, const typename P::S* __restrict__ tw) {
+                                                        typename P::S* dst, const typename P::S* __restrict__ tw,
+                                                        int lg) {
     constexpr int C = CW;
     extern __shared__ __align__(16) unsigned char smraw[];
     typename P::S* sm = reinterpret_cast<typename P::S*>(smraw);
@@ -547,7 +563,8 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
     const int kx = blockIdx.x * C + c;
     ColSmem<P, C> csm{sm, c};
     tw = stage_table(tw, sm + N * C, N);
-    col_body<PrecF64, P, P, N, +1, COL_Z, CPLX, ColSmem<P, C>>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j, csm, tw);
+    col_body<PrecF64, P, P, N, +1, COL_Z, CPLX, ColSmem<P, C>>(src, dst, (int)blockIdx.y, kx, kx < Lay<N, CPLX>::NX, j,
+                                                                  csm, tw, lay_lg<P, N>(lg));
 }
 
 // ---------------------------------------------------------------------------
@@ -562,13 +579,13 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
                                        const double2* __restrict__ coef) {
     typedef typename P::R R;
     typedef cx<R> Cx;
-    constexpr int T = N / 8;
-    const size_t base = Lay<N>::zcol(ky, kx);
+    constexpr int T = N / 8, LG = LayLg<P, N>::value, RS = 1 << LG;
+    const size_t base = Lay<N>::zcol(ky, kx, LG);
 
     Cx v[8];
 #pragma unroll
     for (int s = 0; s < 8; s++) {
-        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * 8]);
+        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * RS]);
         else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
     }
     // forward z transform, the update, then the inverse z transform; the double-float and
@@ -586,7 +603,7 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
             const int mz = kz <= N / 2 ? kz : kz - N;
             const int m2 = mxy2 + mz * mz;
             if (valid) {
-                const size_t idx = base + (size_t)kz * 8;
+                const size_t idx = base + (size_t)kz * RS;
                 const double2 cf = __ldg(coef + m2);
                 const double2 a = cur[idx];
                 const double2 b = old[idx];
@@ -599,7 +616,7 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
     }
     if (valid) {
 #pragma unroll
-        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * 8] = P::pack(v[s]);
+        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * RS] = P::pack(v[s]);
     }
 }
 
@@ -634,7 +651,8 @@ __device__ __forceinline__ double2 mode_update(cx<typename P::R> f, double2* cur
         const double2 kc = __ldg(c4.kick + (size_t)sub * c4.stride + m2);
         const double pre = P::fma_into(kc.x, f.re, fma(-kc.y, a.x, b.x));
         const double pim = P::fma_into(kc.x, f.im, fma(-kc.y, a.y, b.y));
-        const double2 n = make_double2(fma(c4.h[sub], pre, a.x), fma(c4.h[sub], pim, a.y));
+        const double h = sub == 1 ? c4.h[1] : c4.h[0];   // h = (g1, g2, g1) dt
+        const double2 n = make_double2(fma(h, pre, a.x), fma(h, pim, a.y));
         if (update) {
             old[idx] = make_double2(pre, pim);
             cur[idx] = n;
@@ -648,22 +666,22 @@ __device__ __forceinline__ double2 mode_update(cx<typename P::R> f, double2* cur
 // and uh^{n+1}_k in the pass precision on exit; the state update and the Q terms are
 // those of z_body.
 // ---------------------------------------------------------------------------
-// The mode in slot i of an array of z-columns (struct Lay): the half spectrum of a real
-// field (kx = 0..N/2) or the full spectrum of a complex field (kx = 0..N-1 in FFT order).
-// m2 = mx^2 + my^2 + mz^2 indexes the coefficient tables; w is the Parseval weight of the
+// The mode in slot i of an array of z-columns (struct Lay, tiles of 2^lg columns): the half
+// spectrum of a real field (kx = 0..N/2) or the full spectrum of a complex field (kx = 0..N-1 in FFT
+// order).  m2 = mx^2 + my^2 + mz^2 indexes the coefficient tables; w is the Parseval weight of the
 // mode in the energy sums; slots of padding hold no mode (valid == false).
 template <int N, bool CPLX>
 struct ModeIndex {
     typedef Lay<N, CPLX> Ly;
-    static constexpr long long kSlots = Ly::kSlots;
-    static_assert(kSlots < (1ll << 31), "slot indexes fit 32 bits");
+    static_assert(Ly::kSlots < (1ll << 31), "slot indexes fit 32 bits");
     int m2, kx, ky, kz;
     bool twice, valid;
-    __device__ __forceinline__ explicit ModeIndex(unsigned i) {
-        const unsigned row = i >> 3, tile = row / N;
+    static __host__ __device__ __forceinline__ unsigned slots(int lg) { return (unsigned)N * (unsigned)Ly::ky_stride(lg); }
+    __device__ __forceinline__ ModeIndex(unsigned i, int lg) {
+        const unsigned row = i >> lg, tile = row / N, tl = (unsigned)Ly::tiles(lg);
         kz = (int)(row % N);
-        ky = (int)(tile / Ly::TL);
-        kx = (int)(tile % Ly::TL) * 8 + (int)(i & 7);
+        ky = (int)(tile / tl);
+        kx = (int)((tile - ky * tl) << lg) + (int)(i & ((1u << lg) - 1u));
         const int mx = (CPLX && kx > N / 2) ? kx - N : kx;
         const int my = ky <= N / 2 ? ky : ky - N, mz = kz <= N / 2 ? kz : kz - N;
         m2 = mx * mx + my * my + mz * mz;
@@ -757,8 +775,8 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
     double2* __restrict__ old = dev->phase ? S0 : S1;
     const unsigned i = blockIdx.x * kUpdThreads + threadIdx.x;
     typename Q::T q = Q::zero();
-    const MI mi(i);
-    if (i < (unsigned)MI::kSlots && mi.valid) {
+    const MI mi(i, LayLg<P, N>::value);
+    if (i < MI::slots(LayLg<P, N>::value) && mi.valid) {
         const cx<R> f = P::load(W[i]);
         const double2 a = cur[i];
         const double2 n = mode_update<P, SCHEME>(f, cur, old, i, mi.m2, coef, c4, dev->sub, update, a);
@@ -776,27 +794,24 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
 // FFT -> F^n_k, the update of k_update (uh^{n+1} over uh^{n-1}, W <- uh^{n+1} in the pass
 // precision, Q terms on recording steps), then the inverse z FFT of uh^{n+1}.  One pass
 // over W2: 2 W + 3 S per launch instead of 6 W + 3 S for the three kernels.
-// C columns of N rows per CTA; C = 8 (one tile of z-columns: the tile's W2 values and each
-// of its two state arrays are one contiguous run), 16 at N = 16 so that a CTA is at least
-// one warp.  The state is read with plain loads after the forward transform; from N = 256
-// on, where the arrays do not stay in L2, one thread has asked L2 for both runs before it
-// (one bulk prefetch each): 512^3 1.584 -> 1.500 ms double-float, 0.808 -> 0.785 ms FP32;
-// 256^3 0.185 -> 0.179 and 0.118 -> 0.106 ms.
+// C columns of N rows per CTA (ZStepShape).  The state is read with plain loads after the forward
+// transform; on large grids, whose arrays do not stay in L2, one thread has asked L2 for the
+// tile's two contiguous state runs before it (one bulk prefetch each).  512^3: 1.561 -> 1.548 ms
+// double-float, 0.777 -> 0.746 ms FP32; 256^3: 0.185 -> 0.179 and 0.118 -> 0.106 ms.
 // ---------------------------------------------------------------------------
 // [p, p + bytes) of global memory into L2 (16-byte aligned, a multiple of 16 bytes)
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
 }
 
-template <int N>
-struct ZStepPrefetch {
-    static constexpr bool value = N >= 256;   // C == 8 there: the run is one tile
-};
-
-template <int N>
+// columns per CTA: one tile of z-columns from N = 32 on.  Four double-float columns make CTAs of 256
+// threads at 512^3, four per SM where eight made two of 512: their phases interleave more and wait
+// less (1.543 -> 1.389 ms).
+template <class P, int N>
 struct ZStepShape {
-    static constexpr int C = N >= 32 ? 8 : 16;
+    static constexpr int C = N >= 32 ? 1 << LayLg<P, N>::value : 16;
     static constexpr int NT = C * N / 8;
+    static constexpr bool kPrefetch = N >= 256;
 };
 // resident threads per SM the kernel is compiled for: 1024 (64 registers); 1536 for the
 // FP32 passes at N = 512, whose smaller body fits 40 registers and gains from the extra
@@ -804,11 +819,11 @@ struct ZStepShape {
 template <class P, int N>
 struct ZStepMinBlocks {
     static constexpr int kThreads = (sizeof(typename P::S) == 8 && N >= 512) ? 1536 : 1024;
-    static constexpr int value = N >= 128 && kThreads / ZStepShape<N>::NT > 1 ? kThreads / ZStepShape<N>::NT : 1;
+    static constexpr int value = N >= 128 && kThreads / ZStepShape<P, N>::NT > 1 ? kThreads / ZStepShape<P, N>::NT : 1;
 };
 
 template <class P, int N, bool CPLX = false, int SCHEME = 0>
-__global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value)
+__global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::value)
     k_zstep(typename P::S* __restrict__ W, double2* S0, double2* S1, KgDev* __restrict__ dev,
             double* __restrict__ part_sum, const typename P::S* __restrict__ tw, const double2* __restrict__ coef,
             const double* __restrict__ w2tab, double qr, double qc, C4Args c4) {
@@ -816,7 +831,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     typedef typename P::S S;
     typedef QTerm<P> Q;
     typedef Lay<N, CPLX> Ly;
-    constexpr int T = N / 8, C = ZStepShape<N>::C, NT = ZStepShape<N>::NT;
+    constexpr int T = N / 8, C = ZStepShape<P, N>::C, NT = ZStepShape<P, N>::NT, LG = LayLg<P, N>::value, RS = 1 << LG;
     extern __shared__ __align__(16) unsigned char smraw[];
     S* sm = reinterpret_cast<S*>(smraw);
     __shared__ typename Q::T red[NT / 32];
@@ -824,8 +839,8 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     const int kx = blockIdx.x * C + c, ky = blockIdx.y;
     const bool valid = kx < Ly::NX;   // columns of the last tile beyond the plane compute on zeros
     ColSmem<P, C> csm{sm, c};
-    const size_t base = Ly::zcol(ky, kx);
-    if (ZStepPrefetch<N>::value && threadIdx.x == 0) {
+    const size_t base = Ly::zcol(ky, kx, LG);
+    if (ZStepShape<P, N>::kPrefetch && threadIdx.x == 0) {
         prefetch_l2(S0 + base, (unsigned)(N * C * sizeof(double2)));
         prefetch_l2(S1 + base, (unsigned)(N * C * sizeof(double2)));
     }
@@ -835,7 +850,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     cx<R> v[8];
 #pragma unroll
     for (int s = 0; s < 8; s++) {
-        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * 8]);
+        if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * RS]);
         else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
     }
     typename Q::T q = Q::zero();
@@ -864,7 +879,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
             const int mz = kz <= N / 2 ? kz : kz - N;
             const int m2 = mxy2 + mz * mz;
             if (valid) {
-                const size_t idx = base + (size_t)kz * 8;
+                const size_t idx = base + (size_t)kz * RS;
                 const double2 a = cur[idx];
                 const double2 n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a);
                 if (want_q) q = Q::add(q, Q::term(n.x, n.y, a, __ldg(w2tab + m2), qr, twice));
@@ -874,7 +889,7 @@ __global__ void __launch_bounds__(ZStepShape<N>::NT, ZStepMinBlocks<P, N>::value
     }
     if (valid) {
 #pragma unroll
-        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * 8] = P::pack(v[s]);
+        for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * RS] = P::pack(v[s]);
     }
     if (SCHEME == 0 && kg_recording(dev)) {
         q = block_tree_sum<Q, NT>(q, red);
@@ -1042,11 +1057,11 @@ __global__ void __launch_bounds__(kXThreads) k_x_pair_io(const double* __restric
 // uh^{-1} = c_k uh^0 - dt vh^0 + beta_k F^0 (coef holds 2c, 2 beta); b holds vh^0 on entry
 template <int N, bool CPLX = false>
 __global__ void k_startup(const double2* __restrict__ a, double2* __restrict__ b, const double2* __restrict__ f,
-                          const double2* __restrict__ coef, double dt) {
+                          const double2* __restrict__ coef, double dt, int lg) {
     typedef ModeIndex<N, CPLX> MI;
-    const size_t total = (size_t)MI::kSlots;
+    const size_t total = MI::slots(lg);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const MI mi((unsigned)i);
+        const MI mi((unsigned)i, lg);
         if (!mi.valid) continue;
         const double2 cf = coef[mi.m2];
         const double c = 0.5 * cf.x, beta = 0.5 * cf.y;
@@ -1061,11 +1076,11 @@ __global__ void k_startup(const double2* __restrict__ a, double2* __restrict__ b
 // K_0 = h_0/(1 + omega^2 h_0^2/4)
 template <int N>
 __global__ void k_startup_c4(const double2* __restrict__ a, double2* __restrict__ b, const double2* __restrict__ f,
-                             const double2* __restrict__ kick0) {
+                             const double2* __restrict__ kick0, int lg) {
     typedef ModeIndex<N, false> MI;
-    const size_t total = (size_t)MI::kSlots;
+    const size_t total = MI::slots(lg);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const MI mi((unsigned)i);
+        const MI mi((unsigned)i, lg);
         if (!mi.valid) continue;
         const double2 kc = kick0[mi.m2];
         const double2 a0 = a[i], v0 = b[i], f0 = f[i];
@@ -1077,15 +1092,15 @@ __global__ void k_startup_c4(const double2* __restrict__ a, double2* __restrict_
 template <int N, bool CPLX = false>
 __global__ void __launch_bounds__(256) k_energy_q(const double2* __restrict__ x, const double2* __restrict__ y,
                                                   const double* __restrict__ w2tab, double inv_dt,
-                                                  double* __restrict__ part_sum) {
+                                                  double* __restrict__ part_sum, int lg) {
     typedef ModeIndex<N, CPLX> MI;
     __shared__ double red[96];
-    const size_t total = (size_t)MI::kSlots;
+    const size_t total = MI::slots(lg);
     NSum acc;
     acc.s = 0.0;
     acc.c = 0.0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const MI mi((unsigned)i);
+        const MI mi((unsigned)i, lg);
         if (!mi.valid) continue;
         const double w = mi.twice ? 2.0 : 1.0;
         const double2 a = x[i], b = y[i];
@@ -1100,11 +1115,11 @@ __global__ void __launch_bounds__(256) k_energy_q(const double2* __restrict__ x,
 
 // z-columns <-> the packed order [kz][ky][kx] of checkpoints and kg_fetch_spectral
 template <int N, bool CPLX, bool TO_PACKED>
-__global__ void k_repack(const double2* __restrict__ in, double2* __restrict__ out) {
+__global__ void k_repack(const double2* __restrict__ in, double2* __restrict__ out, int lg) {
     typedef ModeIndex<N, CPLX> MI;
-    const size_t total = (size_t)MI::kSlots;
+    const size_t total = MI::slots(lg);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const MI mi((unsigned)i);
+        const MI mi((unsigned)i, lg);
         if (!mi.valid) continue;
         const size_t p = ((size_t)mi.kz * N + mi.ky) * MI::Ly::NX + mi.kx;
         if (TO_PACKED) out[p] = in[i];

@@ -44,12 +44,14 @@ struct PassLaunch {
                           double scale, double lam, int record, cudaStream_t st);
     // forward y columns W1 (x-lines) -> W2 (z-columns), inverse y columns W2 -> W1; z columns of
     // W2 in place (sign -1 forward, +1 inverse; FP64 only).  fin runs in one more CTA of the y pass.
-    cudaError_t (*yf)(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st);
-    cudaError_t (*yi)(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st);
-    cudaError_t (*zcol)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
+    // lg: tiles of 2^lg columns in the z-columns (struct Lay): the context's, which the FP64 kernels
+    // have to be told, being used by contexts of every precision; the others know theirs.
+    cudaError_t (*yf)(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*yi)(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*zcol)(int N, int sign, void* W2, const void* tw, int lg, cudaStream_t st);
     // inverse z columns from an FP64 spectral source (chosen by dev->phase when dev != NULL) into W2
     cudaError_t (*z_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
-                              const void* tw, cudaStream_t st);
+                              const void* tw, int lg, cudaStream_t st);
     // streaming FP64 update between a forward and an inverse z column pass; writes
     // update_parts(N) Q partials when recording; c4: the composed scheme's tables (NULL:
     // Eq. (2))
@@ -66,16 +68,17 @@ struct PassLaunch {
                             const double2* coef64, const double2* coef128, cudaStream_t st);
     int (*x_parts)(int N);
     size_t store_bytes;  // bytes of one complex value of W
+    int (*lg)(int N);    // layout of the state and of W2 in an N^3 context of this precision (struct Lay)
     // complex field (full N^3 spectrum, N columns per plane): x pass, column FFTs,
     // column FFT from an FP64 source, update, and their partial counts
     cudaError_t (*passc_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
                            double scale, double lam, int record, cudaStream_t st);
     int (*xc_parts)(int N);
-    cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st);
-    cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st);
-    cudaError_t (*zcolc)(int N, int sign, void* W2, const void* tw, cudaStream_t st);
+    cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);
+    cudaError_t (*zcolc)(int N, int sign, void* W2, const void* tw, int lg, cudaStream_t st);
     cudaError_t (*zc_from_f64)(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
-                               const void* tw, cudaStream_t st);
+                               const void* tw, int lg, cudaStream_t st);
     cudaError_t (*updatec)(int N, void* W, double2* S0, double2* S1, KgDev* dev, double* part_sum,
                            const double2* coef, const double* w2tab, double inv_dt, cudaStream_t st);
     int (*updatec_parts)(int N);
@@ -115,7 +118,7 @@ extern const PassLaunch kLaunchF32;
 inline size_t spec_slots(int N, bool cplx) { return (size_t)N * N * (cplx ? N : (N / 2 + 8) / 8 * 8); }
 
 // z-columns (the layout of the state) -> the packed order [kz][ky][kx], or back
-cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, cudaStream_t st);
+cudaError_t launch_repack(int N, bool cplx, bool to_packed, const double2* in, double2* out, int lg, cudaStream_t st);
 
 // FP64 set-up / read-out launchers
 cudaError_t launch_x_forward(int N, const double* u, double2* out, const double2* tw, int cube, double lam,
@@ -125,12 +128,12 @@ cudaError_t launch_x_inverse(int N, const double2* in, double* u, const double2*
 int x_inverse_parts(int N);   // partial sums launch_x_inverse writes
 // cplx: full N^3 spectrum of a complex field instead of the half spectrum
 cudaError_t launch_startup(int N, const double2* a, double2* b, const double2* f, const double2* coef, double dt,
-                           bool cplx, cudaStream_t st);
+                           bool cplx, int lg, cudaStream_t st);
 // startup of the composed scheme (real field): b = vh^0 -> P^0 (k_startup_c4)
 cudaError_t launch_startup_c4(int N, const double2* a, double2* b, const double2* f, const double2* kick0,
-                              cudaStream_t st);
+                              int lg, cudaStream_t st);
 cudaError_t launch_energy_q(int N, const double2* x, const double2* y, const double* w2tab, double inv_dt,
-                            double* part_sum, int nparts, bool cplx, cudaStream_t st);
+                            double* part_sum, int nparts, bool cplx, int lg, cudaStream_t st);
 // complex field, FP64: forward transform along x (u -> out; cube: of lam |u|^2 u) and
 // inverse transform along x times scale (u may be NULL; part_sum: per-CTA sum |u|^4)
 cudaError_t launch_xc_forward(int N, const double2* u, double2* out, const double2* tw, int cube, double lam,
@@ -145,11 +148,11 @@ cudaError_t launch_fin_sum(const double* ps, int count, double norm, double* out
 // composed scheme: partials of the quadratic energy sum_k w_k (|p|^2 + omega^2 |a|^2) / 2 with
 // the synchronised velocity p formed from the stored P, F = R2C(lam u^3) and the first kick table
 cudaError_t launch_energy_c4(int N, const double2* a, const double2* P, const double2* f, const double2* kick0,
-                             const double* w2tab, double* part_sum, int nparts, cudaStream_t st);
+                             const double* w2tab, double* part_sum, int nparts, int lg, cudaStream_t st);
 // FP64 forward 3D transform of a physical array (cube: of lam u^3 instead of u) into z-columns;
 // lines: FP64 spectral scratch for the x-lines
 int forward3d_f64(int N, const double* u, double2* lines, double2* out, const double2* tw64, int cube, double lam,
-                  cudaStream_t st);
+                  int lg, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // shared host helpers (kg_host.cu)

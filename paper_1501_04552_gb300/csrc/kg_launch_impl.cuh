@@ -122,7 +122,7 @@ struct Launchers {
 
     // column passes (k_col): Pin -> Pout in the layouts of direction DIR
     template <class Pin, class Pout, int N, int SIGN, int DIR, bool CPLX, int C>
-    static cudaError_t col_n(const void* src, void* dst, const void* tw, const FinArgs& fin, cudaStream_t st) {
+    static cudaError_t col_n(const void* src, void* dst, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
         static std::atomic<unsigned long long> done{0};
         constexpr size_t smem = (size_t)(N * C + N) * sizeof(S);
         static_assert(smem >= kFinSmem * sizeof(double), "a finaliser's shared memory");
@@ -131,29 +131,29 @@ struct Launchers {
         if (e != cudaSuccess) return e;
         dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N + (fin.kind != FIN_NONE));
         return launch_pdl(kern, grid, C * N / 8, smem, st, (const typename Pin::S*)src, (typename Pout::S*)dst,
-                          (const S*)tw, fin);
+                          (const S*)tw, lg, fin);
     }
     template <bool CPLX>
-    static cudaError_t yf_t(int N, const void* W1, void* W2, const void* tw, const FinArgs& fin, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_YF, CPLX, ColStep<P, true>::C>(W1, W2, tw, fin, st)));
+    static cudaError_t yf_t(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_YF, CPLX, ColStep<P, NN, true>::C>(W1, W2, tw, lg, fin, st)));
     }
     template <bool CPLX>
-    static cudaError_t yi_t(int N, const void* W2, void* W1, const void* tw, const FinArgs& fin, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_YI, CPLX, ColStep<P, true>::C>(W2, W1, tw, fin, st)));
+    static cudaError_t yi_t(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_YI, CPLX, ColStep<P, NN, true>::C>(W2, W1, tw, lg, fin, st)));
     }
     // z columns in place: FP64 only (the other precisions have the fused z pass)
     template <bool CPLX>
-    static cudaError_t zcol_t(int N, int sign, void* W2, const void* tw, cudaStream_t st) {
+    static cudaError_t zcol_t(int N, int sign, void* W2, const void* tw, int lg, cudaStream_t st) {
         if constexpr (!std::is_same<P, PrecF64>::value) {
             return cudaErrorNotSupported;
         } else {
-            if (sign < 0) { KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, FinArgs{}, st))); }
-            KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_Z, CPLX, ColStep<P, false>::C>(W2, W2, tw, FinArgs{}, st)));
+            if (sign < 0) { KG_DISPATCH_N(N, return (col_n<P, P, NN, -1, COL_Z, CPLX, ColStep<P, NN, false>::C>(W2, W2, tw, lg, FinArgs{}, st))); }
+            KG_DISPATCH_N(N, return (col_n<P, P, NN, +1, COL_Z, CPLX, ColStep<P, NN, false>::C>(W2, W2, tw, lg, FinArgs{}, st)));
         }
     }
     template <int N, bool CPLX>
     static cudaError_t z_from_f64_n(const double2* src0, const double2* src1, const KgDev* dev, void* W2,
-                                    const void* tw, cudaStream_t st) {
+                                    const void* tw, int lg, cudaStream_t st) {
         static std::atomic<unsigned long long> done{0};
         constexpr int C = ColShape<P>::C;
         const size_t smem = (size_t)(N * C + N) * sizeof(S);
@@ -161,18 +161,18 @@ struct Launchers {
         cudaError_t e = set_smem_once(kern, smem, done);
         if (e != cudaSuccess) return e;
         dim3 grid((Lay<N, CPLX>::NX + C - 1) / C, N);
-        return launch_pdl(kern, grid, C * N / 8, smem, st, src0, src1, dev, (S*)W2, (const S*)tw);
+        return launch_pdl(kern, grid, C * N / 8, smem, st, src0, src1, dev, (S*)W2, (const S*)tw, lg);
     }
     template <bool CPLX>
     static cudaError_t z_from_f64_t(int N, const double2* src0, const double2* src1, const KgDev* dev, void* W2,
-                                    const void* tw, cudaStream_t st) {
-        KG_DISPATCH_N(N, return (z_from_f64_n<NN, CPLX>(src0, src1, dev, W2, tw, st)));
+                                    const void* tw, int lg, cudaStream_t st) {
+        KG_DISPATCH_N(N, return (z_from_f64_n<NN, CPLX>(src0, src1, dev, W2, tw, lg, st)));
     }
     // forward z columns from W2 into an FP64 spectral array (pass-precision set-up)
     template <bool CPLX>
     static cudaError_t z_to_f64_t(int N, const void* W2, double2* out, const void* tw, cudaStream_t st) {
         if constexpr (!kPassIO) return cudaErrorNotSupported;
-        else { KG_DISPATCH_N(N, return (col_n<P, PrecF64, NN, -1, COL_Z, CPLX, ColShape<P>::C>(W2, out, tw, FinArgs{}, st))); }
+        else { KG_DISPATCH_N(N, return (col_n<P, PrecF64, NN, -1, COL_Z, CPLX, ColShape<P>::C>(W2, out, tw, 0, FinArgs{}, st))); }
     }
 
     // set-up and read-out transforms in the pass precision (double-float only: the FP32
@@ -219,8 +219,8 @@ struct Launchers {
         if constexpr (!kPassIO) return cudaErrorNotSupported;
         else { KG_DISPATCH_N(N, return (xc_io_n<NN, false>(nullptr, spec, u, tw, 0, 0.0, scale, st))); }
     }
-    static int update_parts(int N) {   // one partial per CTA over the padded slots
-        return (int)(((long long)N * N * ((N / 2 + 8) / 8 * 8) + kUpdThreads - 1) / kUpdThreads);
+    static int update_parts(int N) {   // one partial per CTA over the slots
+        KG_DISPATCH_N(N, return (int)((ModeIndex<NN, false>::slots(LayLg<P, NN>::value) + kUpdThreads - 1) / kUpdThreads));
     }
     template <int N>
     static cudaError_t update_n(void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const double2* coef,
@@ -275,7 +275,7 @@ struct Launchers {
     static cudaError_t zstep_n(void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const void* tw,
                                const double2* coef, const double* w2, double inv_dt, const C4Args& c4,
                                cudaStream_t st) {
-        typedef ZStepShape<N> Z;
+        typedef ZStepShape<P, N> Z;
         static std::atomic<unsigned long long> done{0};
         constexpr int NX = Lay<N, CPLX>::NX;
         const size_t smem = (size_t)(N * Z::C + N) * sizeof(S);
@@ -297,9 +297,10 @@ struct Launchers {
         KG_DISPATCH_N(N, return (zstep_n<NN, false, 0>(W, S0, S1, dev, ps, tw, coef, w2, inv_dt, C4Args{}, st)));
     }
     static int zstep_parts(int N, bool cplx) {
-        const int C = N >= 32 ? ZStepShape<32>::C : ZStepShape<16>::C;
-        const int nx = cplx ? N : N / 2 + 1;
-        return (nx + C - 1) / C * N;
+        KG_DISPATCH_N(N, {
+            constexpr int C = ZStepShape<P, NN>::C;
+            return ((cplx ? NN : NN / 2 + 1) + C - 1) / C * NN;
+        });
     }
 
     // ---- fused inverse y / x / forward y pass (FP32 work array, real field) ----

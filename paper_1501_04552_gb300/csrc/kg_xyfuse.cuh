@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
     typedef XyShape<N, CL> X;
     constexpr int CW = X::CW, LDC = X::LDC, TY = X::TY, TX = X::TX;
     typedef Lay<N> Ly;
+    constexpr int LG = LayLg<P, N>::value;
     extern __shared__ __align__(16) unsigned char smraw[];
     S* slab = reinterpret_cast<S*>(smraw);
     S* xbuf = slab + X::SLAB;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
     for (int z = cid; z < N; z += nclusters) {   // the same planes for every CTA of the cluster
         for (int row = warp; row < N; row += NWARPS)
             for (int lc = lane; lc < ncols; lc += 32)
-                slab[row * LDC + lc] = DO_YI ? W2[Ly::zcol(row, c0 + lc) + 8 * (size_t)z]
+                slab[row * LDC + lc] = DO_YI ? W2[Ly::zcol(row, c0 + lc, LG) + ((size_t)z << LG)]
                                              : W1[((size_t)z * N + row) * Ly::PITCH + c0 + lc];
         __syncthreads();
         if (DO_YI) y_transforms(+1);
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(XyShape<N, CL>::NT, XyShape<N, CL>::MINB)
         y_transforms(-1);
         for (int row = warp; row < N; row += NWARPS)
             for (int lc = lane; lc < ncols; lc += 32)
-                W2[Ly::zcol(row, c0 + lc) + 8 * (size_t)z] = slab[row * LDC + lc];
+                W2[Ly::zcol(row, c0 + lc, LG) + ((size_t)z << LG)] = slab[row * LDC + lc];
         __syncthreads();   // the slab is reloaded by the next plane
     }
 
