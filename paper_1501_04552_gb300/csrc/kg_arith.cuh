@@ -293,7 +293,15 @@ struct PrecF64 {
     static __device__ __forceinline__ R from_f64(double d) { return d; }
     static __device__ __forceinline__ R from_f32(float f) { return (double)f; }
     static __device__ __forceinline__ R rsqrt2() { return 0.70710678118654752440; }
-    static __device__ __forceinline__ R scale2(R x, double p2) { return x * p2; }
+    // x p2 for a power of two p2, by the exponent field where that is exact (the FP64 pipe is what
+    // limits these passes); zeros, subnormals, infinities, NaN and results near the ends of the
+    // range take the multiplication
+    static __device__ __forceinline__ R scale2(R x, double p2) {
+        const int hi = __double2hiint(x), d = __double2hiint(p2) - 0x3FF00000;
+        const unsigned e = (unsigned)(hi & 0x7FF00000), f = e + (unsigned)d;
+        if (e - 0x00100000u < 0x7FE00000u && f - 0x00100000u < 0x7FE00000u) return __hiloint2double(hi + d, __double2loint(x));
+        return x * p2;
+    }
     // acc + s * x with x in this precision, everything else FP64
     static __device__ __forceinline__ double fma_into(double s, R x, double acc) { return fma(s, x, acc); }
     // butterfly arithmetic: sums that may leave the pair unnormalised (double-float only),

@@ -215,6 +215,82 @@ __device__ __forceinline__ void dft(cx<typename P::R>* u, int sg) {
     }
 }
 
+// IEEE FP64, where the arithmetic pipe is the limit: the same DFTs with twiddle products and the
+// sqrt(1/2) rotations fused into the sums (an FMA costs what an add does).  a + w x takes four FMAs
+// and a - w x = 2 a - (a + w x) two more, against eight operations apart; a rotated pair enters the
+// last layer through its FMAs.  A radix-8 butterfly with twiddles is 72 operations instead of 84,
+// without 52 instead of 56; a 512-point transform 24.5 per point instead of 28.
+struct F64Fma {
+    typedef cx<double> C;
+    // a + w x and a - w x
+    static __device__ __forceinline__ void tw_pair(C a, C x, C w, C& s, C& d) {
+        s.re = fma(-w.im, x.im, fma(w.re, x.re, a.re));
+        s.im = fma(w.im, x.re, fma(w.re, x.im, a.im));
+        d.re = fma(2.0, a.re, -s.re);
+        d.im = fma(2.0, a.im, -s.im);
+    }
+    static __device__ __forceinline__ void pair(C a, C x, C& s, C& d) {
+        s = a + x;
+        d = a - x;
+    }
+    // TW: u[1..] times w[1..] first
+    template <bool TW>
+    static __device__ __forceinline__ void dft2(C* u, const C* w) {
+        C s, d;
+        if (TW) tw_pair(u[0], u[1], w[1], s, d);
+        else pair(u[0], u[1], s, d);
+        u[0] = s;
+        u[1] = d;
+    }
+    template <bool TW>
+    static __device__ __forceinline__ void dft4(C* u, const C* w, int sg) {
+        C t0, t1, t2, t3;
+        if (TW) {
+            tw_pair(u[0], u[2], w[2], t0, t1);
+            tw_pair(cmul(u[1], w[1]), u[3], w[3], t2, t3);
+        } else {
+            pair(u[0], u[2], t0, t1);
+            pair(u[1], u[3], t2, t3);
+        }
+        t3 = mul_sgi<PrecF64>(t3, sg);
+        pair(t0, t2, u[0], u[2]);
+        pair(t1, t3, u[1], u[3]);
+    }
+    template <bool TW>
+    static __device__ __forceinline__ void dft8(C* u, const C* w, int sg) {
+        C a[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            if (TW) tw_pair(j ? cmul(u[j], w[j]) : u[0], u[j + 4], w[j + 4], a[j], b[j]);
+            else pair(u[j], u[j + 4], a[j], b[j]);
+        }
+        const unsigned ms = sign_mask(sg), mns = sign_mask(-sg);
+        // sqrt(2) b1 exp(sg i pi/4) and sqrt(2) b3 exp(sg 3 i pi/4)
+        const C y1 = cmake<double>(b[1].re + PrecF64::flip(b[1].im, mns), b[1].im + PrecF64::flip(b[1].re, ms));
+        const C y3 = cmake<double>(PrecF64::flip(b[3].im, mns) - b[3].re, PrecF64::flip(b[3].re, ms) - b[3].im);
+        dft4<false>(a, nullptr, sg);
+        C t0, t1, t2, t3;
+        pair(b[0], mul_sgi<PrecF64>(b[2], sg), t0, t1);
+        pair(y1, y3, t2, t3);
+        t3 = mul_sgi<PrecF64>(t3, sg);
+        const double r = PrecF64::rsqrt2();
+        u[0] = a[0];
+        u[2] = a[1];
+        u[4] = a[2];
+        u[6] = a[3];
+        u[1] = cmake<double>(fma(r, t2.re, t0.re), fma(r, t2.im, t0.im));
+        u[5] = cmake<double>(fma(-r, t2.re, t0.re), fma(-r, t2.im, t0.im));
+        u[3] = cmake<double>(fma(r, t3.re, t1.re), fma(r, t3.im, t1.im));
+        u[7] = cmake<double>(fma(-r, t3.re, t1.re), fma(-r, t3.im, t1.im));
+    }
+    template <int RADIX, bool TW>
+    static __device__ __forceinline__ void dft(C* u, const C* w, int sg) {
+        if (RADIX == 8) dft8<TW>(u, w, sg);
+        else if (RADIX == 4) dft4<TW>(u, w, sg);
+        else if (RADIX == 2) dft2<TW>(u, w);
+    }
+};
+
 // Copy a twiddle table of n entries into shared memory once per CTA (all threads call
 // it) when the values are 8-byte FP32 pairs: the FP32 column passes are limited by the
 // L1TEX pipe, where the twiddle loads outnumber the data loads.  The 16-byte passes keep
@@ -303,7 +379,14 @@ __device__ __forceinline__ void fft_stage(cx<typename P::R> (&v)[8], int j, cons
         C u[RADIX];
 #pragma unroll
         for (int r = 0; r < RADIX; r++) u[r] = v[q + r * Q];
-        if (Ns > 1) {
+        if constexpr (std::is_same<P, PrecF64>::value) {
+            C w[RADIX];
+            if (Ns > 1) {
+#pragma unroll
+                for (int r = 1; r < RADIX; r++) w[r] = twiddle<P>(tw, k * r * (n / (Ns * RADIX)) * twmul, sg);
+            }
+            F64Fma::dft<RADIX, (Ns > 1)>(u, w, sg);
+        } else if (Ns > 1) {
             if constexpr (TWPOW && RADIX == 8) {
                 // one twiddle load per butterfly, the other six powers formed on the FMA
                 // pipe with at most three products in a chain (for a pass bound by the
@@ -330,7 +413,7 @@ __device__ __forceinline__ void fft_stage(cx<typename P::R> (&v)[8], int j, cons
                     u[r] = P::ctw(u[r], twiddle<P>(tw, k * r * (n / (Ns * RADIX)) * twmul, sg));
             }
         }
-        dft<P, RADIX, LAST && NORMLAST, PROT>(u, sg);
+        if constexpr (!std::is_same<P, PrecF64>::value) dft<P, RADIX, LAST && NORMLAST, PROT>(u, sg);
         if (LAST) {
 #pragma unroll
             for (int r = 0; r < RADIX; r++) out[q + r * Q] = u[r];
