@@ -59,8 +59,9 @@ struct Ctx {
     int lg = 3;              // layout of S0, S1 and W2 (struct Lay)
     double2* S0 = nullptr;   // FP64 state arrays; dev->phase tells which holds uh^n
     double2* S1 = nullptr;
-    void* W1 = nullptr;      // work arrays in the pass precision: x-lines (live between steps) and
+    void* W1 = nullptr;      // work arrays in the pass precision: x-lines (live between steps; z-columns with plane) and
     void* W2 = nullptr;      // z-columns (scratch between steps, of 16 bytes a slot: FP64 scratch too)
+    bool plane = false;      // steps of two kernels, k_plane and the z pass (use_plane), on z-columns in W1
     double2* tmp = nullptr;  // FP64 spectral scratch (set-up and read-out), allocated on demand
     double* phys = nullptr;  // physical scratch (N^3 doubles), on demand
     KgDev* dev = nullptr;
@@ -253,6 +254,20 @@ int reuse_ctx(Ctx* c, double L, double dt, Ctx** out) {
     return KG_OK;
 }
 
+// Grids up to 64^3 of a real field in double-float, whose four kernels a step were bound by the
+// chain of launches, take two.  us a step with two | four kernels: 13.1 | 18.0 at 16^3, 14.3 | 18.9 at
+// 32^3, 19.1 | 21.2 at 64^3 (29 | 34 when every level records energies).  At 128^3 a plane needs 143 KB
+// in two CTAs, one an SM: 256 of them for 152 SMs would leave the second round nearly empty.
+// The IEEE FP64 z pass is three kernels, and the FP32 x pass is another body (one line at a time):
+// they keep the separate passes.
+bool use_plane(const Ctx* c) { return !c->cplx && c->pl->plane && c->pl->plane_parts(c->N) > 0; }
+
+// after set-up W2 holds the z-inverse that the last inverse y pass read: with plane that is the work
+// array (both have 16 bytes a slot), and the x-lines are scratch
+void take_planes(Ctx* c) {
+    if (c->plane) std::swap(c->W1, c->W2);
+}
+
 // a context for an N^3 run in the current options, with every buffer a step needs;
 // replaces the previous context (reusing its buffers when the shapes match).  On
 // failure nothing is kept.
@@ -305,6 +320,8 @@ int create_ctx(int N, double L, double dt, bool cplx, Ctx** out) {
         if (c->pl->x_parts(N) <= 0) KG_TRY(fail(KG_ECUDA, "x pass occupancy query failed"));
         c->nparts = std::max(std::max(c->pl->x_parts(N), c->pl->update_parts(N)), x_inverse_parts(N));
     }
+    c->plane = use_plane(c);
+    if (c->plane) c->nparts = std::max(c->nparts, c->pl->plane_parts(N) + c->pl->zstep_parts(N, false));
     c->nparts = std::max(c->nparts, kStrideCtas);   // the on-demand Q partials
     KG_TRY(dalloc(c, (void**)&c->part_sum, sizeof(double) * c->nparts, "partials"));
     KG_TRY(dalloc(c, (void**)&c->part_max, sizeof(double) * c->nparts, "partials max"));
@@ -374,6 +391,7 @@ int init_common(int N, double L, double dt, const double* u0, const double* v0, 
     c->scheme = g_scheme;
     KG_TRY(init_state(N, c->prec, dt, c->lam, tb, c->phys, v0, device_ptrs, c->S0, c->S1, c->W1, c->W2, c->tmp, st,
                       c->scheme == KG_SCHEME_COMPOSED4 ? c->kick : nullptr, true));
+    take_planes(c);
     KgDev d = fresh_dev();
     d.scheme = c->scheme;
     if (cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st) != cudaSuccess) KG_TRY(fail(KG_ECUDA, "dev upload"));
@@ -436,7 +454,9 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
 // z-inverse, so the caller ends the call with one inverse y pass (xy_close).  Its time
 // goes to the x slot; the forward and inverse y slots stay empty.
 // skip_x: the x pass (and its finaliser) already ran for this step (kg_energy ran it ahead).
+int launch_plane_step(Ctx* c, cudaStream_t st, bool timed, float* ms, bool skip_x);
 int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool skip_x = false) {
+    if (c->plane) return launch_plane_step(c, st, timed, ms, skip_x);
     const int N = c->N;
     const double h = c->L / N;
     const double p_norm = c->lam * h * h * h / 4.0;
@@ -470,7 +490,7 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
     if (fused) {
         // z pass: forward z FFT -> F^n, the update, inverse z FFT, in one kernel
         KG_CK(c->pl->zstep(N, c->cplx, c->W2, c->S0, c->S1, c->dev, c->part_sum, c->tw, c->coef, c->w2, 1.0 / c->dt,
-                           c4p, st));
+                           c4p, nullptr, st));
         fz.count = c->pl->zstep_parts(N, c->cplx);
     } else {
         // the IEEE FP64 passes, bound by the FP64 pipe throughout, keep the three kernels
@@ -504,6 +524,43 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
             KG_CK(cudaEventElapsedTime(&t, c->ev[sg[0]], c->ev[sg[1]]));
             ms[sg[2]] += t;
         }
+    }
+    return KG_OK;
+}
+
+// a step of a small grid: inverse y, x and forward y of every z-plane in one kernel, then the z
+// pass, whose last CTA runs both finalisers; W1 holds z-columns throughout.  With timed, clocks
+// taken inside the first kernel split its time over the x, forward y and inverse y slots.
+int launch_plane_step(Ctx* c, cudaStream_t st, bool timed, float* ms, bool skip_x) {
+    const int N = c->N;
+    const double h = c->L / N;
+    const int np = c->pl->plane_parts(N);
+    long long* clk = timed ? (long long*)(c->scal + 4) : nullptr;
+    if (timed) KG_CK(cudaEventRecord(c->ev[0], st));
+    if (!skip_x)
+        KG_CK(c->pl->plane(N, c->W1, c->dev, c->part_sum, c->tw, inv_n3(N), c->lam, FinArgs{}, nullptr, nullptr, clk, st));
+    if (timed) KG_CK(cudaEventRecord(c->ev[1], st));
+    const C4Args c4{c->kick, 3 * (N / 2) * (N / 2) + 1, {c->c4h[0], c->c4h[1], c->c4h[2]}};
+    // the z pass's partials follow those of the plane kernel, which its last CTA still reads
+    double* zpart = c->part_sum + np;
+    const FinArgs tail[2] = {
+        {skip_x ? FIN_AHEAD_DONE : FIN_X, np, c->part_sum, nullptr, c->dev, c->lam * h * h * h / 4.0},
+        {FIN_Z, c->pl->zstep_parts(N, false), zpart, nullptr, c->dev, h * h * h * inv_n3(N)}};
+    KG_CK(c->pl->zstep(N, false, c->W1, c->S0, c->S1, c->dev, zpart, c->tw, c->coef, c->w2, 1.0 / c->dt,
+                       c->scheme == KG_SCHEME_COMPOSED4 ? &c4 : nullptr, tail, st));
+    if (timed) {
+        KG_CK(cudaEventRecord(c->ev[2], st));
+        long long t[4] = {0, 1, 2, 3};
+        if (!skip_x) KG_CK(cudaMemcpyAsync(t, clk, sizeof(t), cudaMemcpyDeviceToHost, st));
+        KG_CK(cudaStreamSynchronize(st));
+        float a = 0.f, b = 0.f;
+        KG_CK(cudaEventElapsedTime(&a, c->ev[0], c->ev[1]));
+        KG_CK(cudaEventElapsedTime(&b, c->ev[1], c->ev[2]));
+        const double per = t[3] > t[0] ? a / (double)(t[3] - t[0]) : 0.0;
+        ms[5] += (float)(per * (double)(t[1] - t[0]));
+        ms[0] += (float)(per * (double)(t[2] - t[1]));
+        ms[1] += (float)(per * (double)(t[3] - t[2]));
+        ms[2] += b;
     }
     return KG_OK;
 }
@@ -703,10 +760,17 @@ int kg_energy(double* E) {
     KgDev d;
     int rc;
     if (ahead) {
-        KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, 1, st));
-        c->x_ahead = true;
-        KG_CK(launch_fin(FinArgs{FIN_X_AHEAD, c->pl->x_parts(N), c->part_sum, c->part_max, c->dev, p_norm}, c->h_dev,
-                         c->h_dev + 1, st));
+        if (c->plane) {   // the run state is advanced, and handed over, by the kernel itself
+            KG_CK(c->pl->plane(N, c->W1, c->dev, c->part_sum, c->tw, inv_n3(N), c->lam,
+                               FinArgs{FIN_X_AHEAD, c->pl->plane_parts(N), c->part_sum, nullptr, c->dev, p_norm}, c->h_dev,
+                               c->h_dev + 1, nullptr, st));
+            c->x_ahead = true;
+        } else {
+            KG_CK(c->pl->pass_x(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, 1, st));
+            c->x_ahead = true;
+            KG_CK(launch_fin(FinArgs{FIN_X_AHEAD, c->pl->x_parts(N), c->part_sum, c->part_max, c->dev, p_norm}, c->h_dev,
+                             c->h_dev + 1, st));
+        }
         KG_CK(cudaStreamSynchronize(st));
         d = c->h_dev[0];
     } else {
@@ -1076,6 +1140,7 @@ int kg_load_state(const void* h, size_t len) {
     // W1 = the yz inverse of uh^n in the pass precision, as the last two transforms of a step leave it
     if (e == cudaSuccess) e = (cplx ? c->pl->zc_from_f64 : c->pl->z_from_f64)(N, c->S0, c->S1, nullptr, c->W2, c->tw, c->lg, st);
     if (e == cudaSuccess) e = (cplx ? c->pl->yic : c->pl->yi)(N, c->W2, c->W1, c->tw, c->lg, FinArgs{}, st);
+    take_planes(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         destroy(c);

@@ -295,15 +295,17 @@ struct F64Fma {
 // it) when the values are 8-byte FP32 pairs: the FP32 column passes are limited by the
 // L1TEX pipe, where the twiddle loads outnumber the data loads.  The 16-byte passes keep
 // the table in L1: their FFT exchanges already fill the shared-memory bandwidth.
+// Kernels of small grids, which wait for every first touch of a line, copy it whatever its type.
+template <class S>
+__device__ __forceinline__ const S* stage_table_any(const S* __restrict__ g, S* sm, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = g[i];
+    __syncthreads();
+    return sm;
+}
 template <class S>
 __device__ __forceinline__ const S* stage_table(const S* __restrict__ g, S* sm, int n) {
-    if constexpr (sizeof(S) != 8) {
-        return g;
-    } else {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = g[i];
-        __syncthreads();
-        return sm;
-    }
+    if constexpr (sizeof(S) != 8) return g;
+    else return stage_table_any(g, sm, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -630,6 +632,8 @@ struct KgDev {
     int status;               // nonzero: a device-side check failed
     int scheme;               // KG_SCHEME_EQ2 (0) or KG_SCHEME_COMPOSED4 (1)
     int sub;                  // composed scheme: substep 0..2 of the current step
+    unsigned int ticket;      // CTAs of a z pass that are done (ZTail); 0 between launches
+    unsigned long long xkey;  // bits of max |u| from k_plane, taken and cleared by the finaliser
 };
 
 __device__ __forceinline__ bool kg_recording(const KgDev* dev) {

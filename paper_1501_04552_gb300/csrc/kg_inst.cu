@@ -40,6 +40,11 @@ cudaError_t xy_fused(int N, int do_yi, const void* W1, void* W2, KgDev* dev, dou
     return Lp::xy_fused(N, do_yi, W1, W2, dev, ps, pm, tw, scale, lam, st);
 }
 int xy_parts(int N) { return Lp::xy_parts(N); }
+cudaError_t plane(int N, void* W, KgDev* dev, double* ps, const void* tw, double scale, double lam, const FinArgs& ahead,
+                  KgDev* before, KgDev* after, long long* phase_clk, cudaStream_t st) {
+    return Lp::plane(N, W, dev, ps, tw, scale, lam, ahead, before, after, phase_clk, st);
+}
+int plane_parts(int N) { return Lp::plane_parts(N); }
 #elif KG_PART == 1
 cudaError_t yf(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {
     return Lp::yf_t<false>(N, W1, W2, tw, lg, fin, st);
@@ -59,14 +64,15 @@ cudaError_t z_to_f64(int N, const void* W2, double2* out, const void* tw, cudaSt
 }
 #elif KG_PART == 2
 cudaError_t zstep(int N, bool cplx, void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const void* tw,
-                  const double2* coef, const double* w2, double inv_dt, const C4Args* c4, cudaStream_t st) {
+                  const double2* coef, const double* w2, double inv_dt, const C4Args* c4,
+                  const FinArgs* tail, cudaStream_t st) {
 #if KG_PREC_ID == 0
     // the IEEE FP64 step runs forward z, update and inverse z as three kernels
     (void)N, (void)cplx, (void)W, (void)S0, (void)S1, (void)dev, (void)ps, (void)tw, (void)coef, (void)w2;
-    (void)inv_dt, (void)c4, (void)st;
+    (void)inv_dt, (void)c4, (void)tail, (void)st;
     return cudaErrorNotSupported;
 #else
-    return Lp::zstep(N, cplx, W, S0, S1, dev, ps, tw, coef, w2, inv_dt, c4, st);
+    return Lp::zstep(N, cplx, W, S0, S1, dev, ps, tw, coef, w2, inv_dt, c4, tail, st);
 #endif
 }
 int zstep_parts(int N, bool cplx) { return Lp::zstep_parts(N, cplx); }

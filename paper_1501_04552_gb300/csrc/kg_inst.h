@@ -21,6 +21,8 @@
     KG_INST_FN(x_readout) x_readout;                                                   \
     KG_INST_FN(xy_fused) xy_fused;                                                     \
     KG_INST_FN(xy_parts) xy_parts;                                                     \
+    KG_INST_FN(plane) plane;                                                           \
+    KG_INST_FN(plane_parts) plane_parts;                                               \
     KG_INST_FN(yf) yf;                        /* share 1: column passes */             \
     KG_INST_FN(yi) yi;                                                                 \
     KG_INST_FN(zcol) zcol;                                                             \

@@ -359,10 +359,54 @@ __global__ void __launch_bounds__(XStep<N>::NT, XMinBlocks<P, N>::value)
 // one more CTA of the y pass that follows (FIN_X in the forward, FIN_Z in the inverse one, both
 // before the next reader of the state starts).  As kernels of one CTA, and without programmatic
 // dependent launch, they made a double-float step 33 us at 32^3 and 72 us at 64^3 recording
-// every level; now 18.9 and 34 us.
+// every level; so 18.9 and 34 us (14.3 and 29 with k_plane, whose finalisers ride in the z pass).
 // ---------------------------------------------------------------------------
 constexpr int kFinThreads = 1024;
 constexpr int kFinSmem = 128;   // doubles of shared memory a finaliser needs
+
+// compensated sums of the first 2 from lanes of a warp -> lane 0
+__device__ __forceinline__ void warp_merge(NSum& v, int from = 16, unsigned mask = 0xffffffffu) {
+    for (int o = from; o > 0; o >>= 1) {
+        NSum b;
+        b.s = __shfl_down_sync(mask, v.s, o);
+        b.c = __shfl_down_sync(mask, v.c, o);
+        nsum_merge(v, b);
+    }
+}
+
+// the sum of count partials by one warp -> lane 0
+__device__ __forceinline__ double warp_total(const double* part, int count) {
+    NSum acc;
+    acc.s = acc.c = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x & 31; i < count; i += 32) acc.add(__ldcg(part + i));
+    warp_merge(acc);
+    return acc.value();
+}
+
+// v of the first `count` threads of an NT-thread CTA (of all of them when it has fewer) -> thread 0.
+// The SM makes two FP64 operations a clock, so the warps that hold nothing stay out (a step with its
+// energy read at 64^3: 72 -> 57 us).
+template <int NT>
+__device__ __forceinline__ void block_sum_of(NSum& v, int count, double* sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int NW = (NT + 31) / 32;   // grids of 16^3 have CTAs of half a warp
+    const int nw = count >= NT ? NW : (count + 31) / 32;
+    if (w < nw) warp_merge(v, NT >= 32 ? 16 : NT / 2, NT >= 32 ? 0xffffffffu : (1u << (NT & 31)) - 1u);
+    if (nw > 1) {
+        __syncthreads();
+        if (lane == 0 && w < nw) {
+            sh[w] = v.s;
+            sh[32 + w] = v.c;
+        }
+        __syncthreads();
+        if (w == 0) {
+            v.s = lane < nw ? sh[lane] : 0.0;
+            v.c = lane < nw ? sh[32 + lane] : 0.0;
+            warp_merge(v, nw > 16 ? 16 : nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : 1);
+        }
+    }
+}
 
 // all NT threads of the CTA; red: kFinSmem doubles
 template <int NT>
@@ -380,9 +424,42 @@ __device__ __forceinline__ void fin_reduce(const double* part_sum, const double*
     }
     if (part_max) key = block_max_key<NT>(key, reinterpret_cast<unsigned long long*>(red + 96));
     mx = __longlong_as_double((long long)key);
-    if (part_sum) {
-        double unused = 0.0;
-        block_reduce<NT>(acc, unused, red);
+    if (part_sum) block_sum_of<NT>(acc, count, red);
+}
+
+// the run state after the x pass of a step, whose largest |u| is mx and whose P^l (when rec) is P;
+// ahead: the next step's x pass, run by kg_energy; its max |u| waits in maxabs_peek until that step
+// runs (kg_status reports the last step's)
+__device__ __forceinline__ void state_after_x(KgDev* dev, bool ahead, bool rec, double mx, double P) {
+    if (ahead && dev->frozen) dev->maxabs_peek = dev->maxabs_last;
+    // the composed scheme checks the field at integer times only (its first substep)
+    if (dev->sub == 0 && !dev->frozen) {
+        if (ahead) dev->maxabs_peek = mx;
+        else dev->maxabs_last = mx;
+        if (rec) {
+            dev->P_last = P;
+            dev->P_last_level = dev->level;
+        }
+        if (dev->threshold > 0.0 && !(mx <= dev->threshold)) {
+            dev->frozen = 1;
+            dev->blowup_level = dev->level;
+        }
+    }
+}
+
+// the run state after the update: Q^{l+1/2} (when rec) and the level advance
+__device__ __forceinline__ void state_after_z(KgDev* dev, bool rec, double Q) {
+    if (dev->frozen) return;
+    if (rec) {
+        dev->Q_last = Q;
+        dev->Q_last_level = dev->level;
+    }
+    if (dev->scheme == 0) {
+        dev->level += 1;
+        dev->phase ^= 1;
+    } else {   // composed scheme: the state arrays stay put; a step is three substeps
+        dev->sub = dev->sub == 2 ? 0 : dev->sub + 1;
+        if (dev->sub == 0) dev->level += 1;
     }
 }
 
@@ -392,29 +469,12 @@ __device__ __noinline__ void finalise(const FinArgs f, double* red) {
     NSum acc;
     double mx;
     if (f.kind == FIN_X || f.kind == FIN_X_AHEAD) {
-        // after a stepping x pass: blow-up check and P^l; norm = lam h^3 / 4.  FIN_X_AHEAD: the
-        // next step's x pass, run by kg_energy; it records P^l, and its max |u| waits in
-        // maxabs_peek until that step runs (kg_status reports the last step's)
+        // after a stepping x pass: blow-up check and P^l; norm = lam h^3 / 4
         const bool ahead = f.kind == FIN_X_AHEAD;
         const bool rec = kg_recording(dev) || ahead;
         fin_reduce<NT>(rec ? f.part_sum : nullptr, f.part_max, f.count, acc, mx, red);
         if (dev->complex_field) mx = sqrt(mx);   // the keys were |u|^2
-        if (threadIdx.x == 0) {
-            if (ahead && dev->frozen) dev->maxabs_peek = dev->maxabs_last;
-            // the composed scheme checks the field at integer times only (its first substep)
-            if (dev->sub == 0 && !dev->frozen) {
-                if (ahead) dev->maxabs_peek = mx;
-                else dev->maxabs_last = mx;
-                if (rec) {
-                    dev->P_last = f.norm * acc.value();
-                    dev->P_last_level = dev->level;
-                }
-                if (dev->threshold > 0.0 && !(mx <= dev->threshold)) {
-                    dev->frozen = 1;
-                    dev->blowup_level = dev->level;
-                }
-            }
-        }
+        if (threadIdx.x == 0) state_after_x(dev, ahead, rec, mx, rec ? f.norm * acc.value() : 0.0);
     } else if (f.kind == FIN_AHEAD_DONE) {
         // the step whose x pass ran ahead: its max |u| becomes the last step's
         if (threadIdx.x == 0) dev->maxabs_last = dev->maxabs_peek;
@@ -426,22 +486,10 @@ __device__ __noinline__ void finalise(const FinArgs f, double* red) {
             dev->maxabs_peek = mx;
         }
     } else {
-        // after the update: Q^{l+1/2} (norm = h^3/N^3) and the level advance
+        // after the update; norm = h^3/N^3
         const bool rec = kg_recording(dev);
         if (rec) fin_reduce<NT>(f.part_sum, nullptr, f.count, acc, mx, red);
-        if (threadIdx.x == 0 && !dev->frozen) {
-            if (rec) {
-                dev->Q_last = f.norm * acc.value();
-                dev->Q_last_level = dev->level;
-            }
-            if (dev->scheme == 0) {
-                dev->level += 1;
-                dev->phase ^= 1;
-            } else {   // composed scheme: the state arrays stay put; a step is three substeps
-                dev->sub = dev->sub == 2 ? 0 : dev->sub + 1;
-                if (dev->sub == 0) dev->level += 1;
-            }
-        }
+        if (threadIdx.x == 0) state_after_z(dev, rec, rec ? f.norm * acc.value() : 0.0);
     }
 }
 
@@ -635,12 +683,11 @@ __device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const doub
 
 // The per-mode update of one step (or substep) at mode index idx with integer norm m2, F the
 // transform of the cube there in the pass precision; writes the state (unless frozen) and
-// returns the new uh in FP64, the value the inverse transforms start from.
+// returns the new uh in FP64, the value the inverse transforms start from.  a = cur[idx], b = old[idx].
 template <class P, int SCHEME>
 __device__ __forceinline__ double2 mode_update(cx<typename P::R> f, double2* cur, double2* old, size_t idx, int m2,
                                                const double2* __restrict__ coef, const C4Args& c4, int sub,
-                                               bool update, double2 a) {
-    const double2 b = old[idx];
+                                               bool update, double2 a, double2 b) {
     if constexpr (SCHEME == 0) {
         const double2 cf = __ldg(coef + m2);
         const double nre = P::fma_into(cf.y, f.re, fma(cf.x, a.x, -b.x));
@@ -779,7 +826,7 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
     if (i < MI::slots(LayLg<P, N>::value) && mi.valid) {
         const cx<R> f = P::load(W[i]);
         const double2 a = cur[i];
-        const double2 n = mode_update<P, SCHEME>(f, cur, old, i, mi.m2, coef, c4, dev->sub, update, a);
+        const double2 n = mode_update<P, SCHEME>(f, cur, old, i, mi.m2, coef, c4, dev->sub, update, a, old[i]);
         W[i] = P::pack(cmake<R>(P::from_f64(n.x), P::from_f64(n.y)));
         if (want_q) q = Q::term(n.x, n.y, a, __ldg(w2tab + mi.m2), qr, mi.twice);
     }
@@ -822,15 +869,34 @@ struct ZStepMinBlocks {
     static constexpr int value = N >= 128 && kThreads / ZStepShape<P, N>::NT > 1 ? kThreads / ZStepShape<P, N>::NT : 1;
 };
 
-template <class P, int N, bool CPLX = false, int SCHEME = 0>
+// What a z pass does when its last CTA is done.  After k_plane the finalisers have no y pass to
+// ride in: the CTA that draws the last ticket runs them, that of the x statistics (fx) and that of
+// the update (fz); the others have read the run state by then.  Blow-up at this level must already
+// stop the update, so every CTA compares the maximum that k_plane left in the run state.  A step
+// that records no energies has nothing to reduce: its CTAs draw once the update is done, ahead of
+// their stores, and the last one advances a copy of the run state that it has read by then.
+// (Tickets after the stores and the general finalisers on every step cost 5 us of a 12 us pass.)
+struct NoTail {};
+struct ZTail {
+    FinArgs fx, fz;
+};
+
+// bring a table entry into L1
+__device__ __forceinline__ void touch(const double2* p) {
+    double x, y;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(x), "=d"(y) : "l"(p));
+}
+
+template <class P, int N, bool CPLX = false, int SCHEME = 0, class TAIL = NoTail>
 __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::value)
     k_zstep(typename P::S* __restrict__ W, double2* S0, double2* S1, KgDev* __restrict__ dev,
             double* __restrict__ part_sum, const typename P::S* __restrict__ tw, const double2* __restrict__ coef,
-            const double* __restrict__ w2tab, double qr, double qc, C4Args c4) {
+            const double* __restrict__ w2tab, double qr, double qc, C4Args c4, TAIL tail) {
     typedef typename P::R R;
     typedef typename P::S S;
     typedef QTerm<P> Q;
     typedef Lay<N, CPLX> Ly;
+    constexpr bool kTail = std::is_same<TAIL, ZTail>::value;
     constexpr int T = N / 8, C = ZStepShape<P, N>::C, NT = ZStepShape<P, N>::NT, LG = LayLg<P, N>::value, RS = 1 << LG;
     extern __shared__ __align__(16) unsigned char smraw[];
     S* sm = reinterpret_cast<S*>(smraw);
@@ -844,7 +910,17 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
         prefetch_l2(S0 + base, (unsigned)(N * C * sizeof(double2)));
         prefetch_l2(S1 + base, (unsigned)(N * C * sizeof(double2)));
     }
-    tw = stage_table(tw, sm + N * C, N);
+    if constexpr (kTail) {
+        if (SCHEME == 0 && valid) {
+            const int my = ky <= N / 2 ? ky : ky - N;
+#pragma unroll
+            for (int s = 0; s < 8; s++) {
+                const int kz = j + T * s, mz = kz <= N / 2 ? kz : kz - N;
+                touch(coef + (kx * kx + my * my + mz * mz));
+            }
+        }
+        tw = stage_table_any(tw, sm + N * C, N);
+    } else tw = stage_table(tw, sm + N * C, N);
     pdl_wait();
 
     cx<R> v[8];
@@ -852,6 +928,24 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
     for (int s = 0; s < 8; s++) {
         if (valid) v[s] = P::load(W[base + (size_t)(j + T * s) * RS]);
         else v[s] = cmake<R>(P::from_f64(0.0), P::from_f64(0.0));
+    }
+    // a small grid waits for each load in turn and has registers to spare: everything that the
+    // update reads is on its way before the forward transform
+    double2 pre0[kTail ? 8 : 1], pre1[kTail ? 8 : 1];
+    KgDev run;
+    const unsigned ctas = gridDim.x * gridDim.y;
+    unsigned ticket = 0u;
+    bool rec = false;
+    if constexpr (kTail) {
+        run = *dev;
+#pragma unroll
+        for (int s = 0; s < 8; s++) {
+            pre0[s] = pre1[s] = make_double2(0.0, 0.0);
+            if (valid) {
+                pre0[s] = S0[base + (size_t)(j + T * s) * RS];
+                pre1[s] = S1[base + (size_t)(j + T * s) * RS];
+            }
+        }
     }
     typename Q::T q = Q::zero();
     // the 16-byte bodies are large: both transforms run through one copy of the FFT code
@@ -864,15 +958,22 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
         // the run state is read only now, so that nothing of it is live across the
         // forward transform (at 64 registers: 132 -> 8 bytes of spills, 1.98 -> 1.91 ms
         // for the double-float pass at 512^3)
-        const bool want_q = SCHEME == 0 && kg_recording(dev);
-        const bool update = dev->frozen == 0;
-        double2* __restrict__ cur = dev->phase ? S1 : S0;
-        double2* __restrict__ old = dev->phase ? S0 : S1;
+        const KgDev* rs = dev;
+        if constexpr (kTail) rs = &run;
+        rec = kg_recording(rs);
+        const bool want_q = SCHEME == 0 && rec;
+        bool update = rs->frozen == 0;
+        if constexpr (kTail) {
+            if (run.threshold > 0.0 && run.sub == 0 && !(__longlong_as_double((long long)run.xkey) <= run.threshold))
+                update = false;
+        }
+        double2* __restrict__ cur = rs->phase ? S1 : S0;
+        double2* __restrict__ old = rs->phase ? S0 : S1;
         const int mx = (CPLX && kx > N / 2) ? kx - N : kx;
         const int my = ky <= N / 2 ? ky : ky - N;
         const int mxy2 = mx * mx + my * my;
         const bool twice = !CPLX && kx != 0 && kx != N / 2;
-        const int sub = SCHEME == 0 ? 0 : dev->sub;
+        const int sub = SCHEME == 0 ? 0 : rs->sub;
 #pragma unroll
         for (int s = 0; s < 8; s++) {
             const int kz = j + T * s;
@@ -880,20 +981,77 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
             const int m2 = mxy2 + mz * mz;
             if (valid) {
                 const size_t idx = base + (size_t)kz * RS;
-                const double2 a = cur[idx];
-                const double2 n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a);
+                double2 a, n;
+                if constexpr (kTail) {
+                    a = run.phase ? pre1[s] : pre0[s];
+                    n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a,
+                                               run.phase ? pre0[s] : pre1[s]);
+                } else {
+                    a = cur[idx];
+                    n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a, old[idx]);
+                }
                 if (want_q) q = Q::add(q, Q::term(n.x, n.y, a, __ldg(w2tab + m2), qr, twice));
                 v[s] = cmake<R>(P::from_f64(n.x), P::from_f64(n.y));
             }
         }
     }
+    // the inverse transform's exchanges have passed: every thread of the CTA has read the run state
+    if (kTail && threadIdx.x == 0 && !rec) ticket = atomicAdd(&dev->ticket, 1u);
     if (valid) {
 #pragma unroll
         for (int s = 0; s < 8; s++) W[base + (size_t)(j + T * s) * RS] = P::pack(v[s]);
     }
-    if (SCHEME == 0 && kg_recording(dev)) {
+    if (SCHEME == 0 && (kTail ? rec : kg_recording(dev))) {
         q = block_tree_sum<Q, NT>(q, red);
         if (threadIdx.x == 0) part_sum[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = qc * Q::value(q);
+    }
+    if constexpr (kTail) {
+        if (rec) {
+            __shared__ int last;
+            __syncthreads();   // the CTA is done with smraw
+            if (threadIdx.x == 0) {
+                __threadfence();   // the partial is visible before the ticket
+                last = atomicAdd(&dev->ticket, 1u) == ctas - 1;
+            }
+            __syncthreads();
+            if (last) {
+                // the first warp sums P's partials, the last one Q's; one thread advances the state
+                __threadfence();
+                double* tot = reinterpret_cast<double*>(smraw);
+                const int w = threadIdx.x >> 5;
+                const bool p_now = tail.fx.kind == FIN_X;
+                if (p_now && w == 0) {
+                    const double P = warp_total(tail.fx.part_sum, tail.fx.count);
+                    if (threadIdx.x == 0) tot[0] = tail.fx.norm * P;
+                }
+                if (w == NT / 32 - 1) {
+                    const double Q = warp_total(tail.fz.part_sum, tail.fz.count);
+                    if ((threadIdx.x & 31) == 0) tot[1] = tail.fz.norm * Q;
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    if (p_now) {
+                        state_after_x(&run, false, true, __longlong_as_double((long long)run.xkey), tot[0]);
+                        run.xkey = 0ull;
+                    } else {
+                        run.maxabs_last = run.maxabs_peek;
+                    }
+                    state_after_z(&run, true, tot[1]);
+                    run.ticket = 0u;
+                    *dev = run;
+                }
+            }
+        } else if (threadIdx.x == 0 && ticket == ctas - 1) {
+            if (tail.fx.kind == FIN_AHEAD_DONE) {
+                run.maxabs_last = run.maxabs_peek;
+            } else {
+                state_after_x(&run, false, false, __longlong_as_double((long long)run.xkey), 0.0);
+                run.xkey = 0ull;
+            }
+            state_after_z(&run, false, 0.0);
+            run.ticket = 0u;
+            *dev = run;
+        }
     }
 }
 

@@ -84,10 +84,11 @@ struct PassLaunch {
     int (*updatec_parts)(int N);
     // the z pass in one kernel: forward z FFT, update (as update / updatec), inverse z
     // FFT, of a real (cplx = false) or complex field; zstep_parts(N, cplx) Q partials.
-    // NULL where the step runs forward z, update and inverse z as three kernels.
+    // NULL where the step runs forward z, update and inverse z as three kernels.  tail: the two
+    // finalisers that its last CTA runs (after plane; NULL: they ride in y passes).
     cudaError_t (*zstep)(int N, bool cplx, void* W, double2* S0, double2* S1, KgDev* dev, double* part_sum,
                          const void* tw, const double2* coef, const double* w2tab, double inv_dt, const C4Args* c4,
-                         cudaStream_t st);
+                         const FinArgs* tail, cudaStream_t st);
     int (*zstep_parts)(int N, bool cplx);
     // set-up and read-out transforms in the pass precision (NULL: the FP64 kernels serve):
     // x_setup: physical FP64 lines (lam u^3 when cube) -> half spectra along x in W format;
@@ -108,6 +109,12 @@ struct PassLaunch {
     cudaError_t (*xy_fused)(int N, int do_yi, const void* W1, void* W2, KgDev* dev, double* part_sum, double* part_max,
                             const void* tw, double scale, double lam, cudaStream_t st);
     int (*xy_parts)(int N);
+    // the same of a small grid, on z-columns in place (kg_plane.cuh; plane_parts(N) = 0, or NULL,
+    // where not built): plane_parts(N) partials of sum u^4 when the step records, max |u| in the
+    // run state; ahead (FIN_X_AHEAD, or FIN_NONE), before, after, phase_clk: see there
+    cudaError_t (*plane)(int N, void* W, KgDev* dev, double* part_sum, const void* tw, double scale, double lam,
+                         const FinArgs& ahead, KgDev* before, KgDev* after, long long* phase_clk, cudaStream_t st);
+    int (*plane_parts)(int N);
 };
 
 extern const PassLaunch kLaunchF64;

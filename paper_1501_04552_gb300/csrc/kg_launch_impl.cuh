@@ -6,6 +6,7 @@
 #include "kg_ensemble.cuh"
 #include "kg_kernels.cuh"
 #include "kg_launch.h"
+#include "kg_plane.cuh"
 #include "kg_xyfuse.cuh"
 
 namespace kg {
@@ -271,24 +272,42 @@ struct Launchers {
     // fused z pass (forward z FFT, update, inverse z FFT) of a real (cplx = false) or
     // complex field, Eq. (2) (SCHEME 0) or the composed scheme (SCHEME 1, real field);
     // zstep_parts: the Q partials it writes when recording
-    template <int N, bool CPLX, int SCHEME>
+    template <int N, bool CPLX, int SCHEME, class TAIL = NoTail>
     static cudaError_t zstep_n(void* W, double2* S0, double2* S1, KgDev* dev, double* ps, const void* tw,
                                const double2* coef, const double* w2, double inv_dt, const C4Args& c4,
-                               cudaStream_t st) {
+                               cudaStream_t st, const TAIL& tail = TAIL{}) {
         typedef ZStepShape<P, N> Z;
         static std::atomic<unsigned long long> done{0};
         constexpr int NX = Lay<N, CPLX>::NX;
         const size_t smem = (size_t)(N * Z::C + N) * sizeof(S);
-        auto kern = k_zstep<P, N, CPLX, SCHEME>;
+        auto kern = k_zstep<P, N, CPLX, SCHEME, TAIL>;
         cudaError_t e = set_smem_once(kern, smem, done);
         if (e != cudaSuccess) return e;
         const double qr = 0.25 / (inv_dt * inv_dt), qc = 0.5 * inv_dt * inv_dt;
         dim3 grid((NX + Z::C - 1) / Z::C, N);
-        return launch_pdl(kern, grid, Z::NT, smem, st, (S*)W, S0, S1, dev, ps, (const S*)tw, coef, w2, qr, qc, c4);
+        return launch_pdl(kern, grid, Z::NT, smem, st, (S*)W, S0, S1, dev, ps, (const S*)tw, coef, w2, qr, qc, c4, tail);
     }
     static cudaError_t zstep(int N, bool cplx, void* W, double2* S0, double2* S1, KgDev* dev, double* ps,
                              const void* tw, const double2* coef, const double* w2, double inv_dt, const C4Args* c4,
-                             cudaStream_t st) {
+                             const FinArgs* tail, cudaStream_t st) {
+        if (tail) {
+            if (cplx || plane_parts(N) == 0) return cudaErrorInvalidValue;
+            const ZTail t{tail[0], tail[1]};
+#define KG_TAIL_CASE(NN)                                                                                         \
+    case NN:                                                                                                     \
+        return c4 ? zstep_n<NN, false, 1, ZTail>(W, S0, S1, dev, ps, tw, coef, w2, inv_dt, *c4, st, t)            \
+                  : zstep_n<NN, false, 0, ZTail>(W, S0, S1, dev, ps, tw, coef, w2, inv_dt, C4Args{}, st, t);
+            if constexpr (kPlane) {
+                switch (N) {
+                    KG_TAIL_CASE(16)
+                    KG_TAIL_CASE(32)
+                    KG_TAIL_CASE(64)
+                    default: break;
+                }
+            }
+#undef KG_TAIL_CASE
+            return cudaErrorInvalidValue;
+        }
         if (cplx) {
             if (c4) return cudaErrorInvalidValue;   // the composed scheme is built for real fields
             KG_DISPATCH_N(N, return (zstep_n<NN, true, 0>(W, S0, S1, dev, ps, tw, coef, w2, inv_dt, C4Args{}, st)));
@@ -301,6 +320,49 @@ struct Launchers {
             constexpr int C = ZStepShape<P, NN>::C;
             return ((cplx ? NN : NN / 2 + 1) + C - 1) / C * NN;
         });
+    }
+
+    // ---- inverse y / x / forward y of a z-plane in one kernel (small grids, kg_plane.cuh) ----
+    static constexpr bool kPlane = std::is_same<P, PrecDF>::value;
+    template <int N>
+    static cudaError_t plane_n(void* W, KgDev* dev, double* ps, const void* tw, double scale, double lam, const FinArgs& ahead,
+                               KgDev* before, KgDev* after, long long* phase_clk, cudaStream_t st) {
+        typedef PlaneShape<N> X;
+        static std::atomic<unsigned long long> done{0};
+        const size_t smem = (size_t)(X::SLAB + X::LINES + N) * sizeof(S);
+        cudaError_t e = set_smem_once(k_plane<P, N>, smem, done);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(N * X::CL);
+        cfg.blockDim = dim3(X::NT);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = X::CL;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = X::CL > 1 ? 2 : 1;
+        return cudaLaunchKernelEx(&cfg, k_plane<P, N>, (S*)W, dev, ps, (const S*)tw, scale, lam, ahead, before, after, phase_clk);
+    }
+    static cudaError_t plane(int N, void* W, KgDev* dev, double* ps, const void* tw, double scale, double lam, const FinArgs& ahead,
+                             KgDev* before, KgDev* after, long long* phase_clk, cudaStream_t st) {
+        if constexpr (kPlane) {
+            switch (N) {
+                case 16: return plane_n<16>(W, dev, ps, tw, scale, lam, ahead, before, after, phase_clk, st);
+                case 32: return plane_n<32>(W, dev, ps, tw, scale, lam, ahead, before, after, phase_clk, st);
+                case 64: return plane_n<64>(W, dev, ps, tw, scale, lam, ahead, before, after, phase_clk, st);
+                default: break;
+            }
+        }
+        return cudaErrorNotSupported;
+    }
+    static int plane_parts(int N) {
+        if (!kPlane) return 0;
+        return N == 16 ? 16 * PlaneShape<16>::CL : N == 32 ? 32 * PlaneShape<32>::CL : N == 64 ? 64 * PlaneShape<64>::CL : 0;
     }
 
     // ---- fused inverse y / x / forward y pass (FP32 work array, real field) ----
