@@ -695,7 +695,7 @@ def paper_protocol(kg, stream, torch, u0, NG, local, prec):
 
 def ensemble_point(kg, prec, steps, torch, stream, early_exit=False):
     """512 instances (256 x 64^3 + 256 x 128^3, A ~ U[0.5,4], s ~ U[0.5,2], seed 4, dt = 0.005):
-    one persistent launch per step vs the plain one-instance-at-a-time loop (kg_init + kg_step),
+    persistent launches of up to 50 steps vs the plain one-instance-at-a-time loop (kg_init + kg_step),
     both for `steps` fixed steps without early exits, same precision; with early_exit also the
     blow-up run (up to 2000 steps, max|u| > 1e3 freezes an instance, only active instance-steps
     counted)"""

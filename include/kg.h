@@ -162,6 +162,8 @@ int kg_fetch_spectral(double* a, double* b);
  * of the x pass, forward y (with the x pass's finaliser), the z pass, its update part, its
  * inverse-z part and inverse y (with the z pass's finaliser).  The z pass (forward z FFT,
  * update, inverse z FFT) is one kernel, so ms[2] holds all of it and ms[3], ms[4] receive 0.
+ * On real double-float grids up to 64^3 the x and y passes are one kernel too (the finalisers
+ * run in the z pass); clocks taken inside it split its time over ms[0], ms[1] and ms[5].
  * Synchronises. */
 int kg_step_timed(int n, float* ms);
 
