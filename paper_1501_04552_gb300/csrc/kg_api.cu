@@ -255,8 +255,8 @@ int reuse_ctx(Ctx* c, double L, double dt, Ctx** out) {
 }
 
 // Grids up to 64^3 of a real field in double-float, whose four kernels a step were bound by the
-// chain of launches, take two.  us a step with two | four kernels: 13.1 | 18.0 at 16^3, 14.3 | 18.9 at
-// 32^3, 19.1 | 21.2 at 64^3 (29 | 34 when every level records energies).  At 128^3 a plane needs 143 KB
+// chain of launches, take two.  us a step with two | four kernels: 11.5 | 18.0 at 16^3, 13.0 | 18.9 at
+// 32^3, 18.0 | 21.2 at 64^3 (28.5 | 34 when every level records energies).  At 128^3 a plane needs 143 KB
 // in two CTAs, one an SM: 256 of them for 152 SMs would leave the second round nearly empty.
 // The IEEE FP64 z pass is three kernels, and the FP32 x pass is another body (one line at a time):
 // they keep the separate passes.

@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(XStep<N>::NT, XMinBlocks<P, N>::value)
 // one more CTA of the y pass that follows (FIN_X in the forward, FIN_Z in the inverse one, both
 // before the next reader of the state starts).  As kernels of one CTA, and without programmatic
 // dependent launch, they made a double-float step 33 us at 32^3 and 72 us at 64^3 recording
-// every level; so 18.9 and 34 us (14.3 and 29 with k_plane, whose finalisers ride in the z pass).
+// every level; so 18.9 and 34 us (13.0 and 28.5 with k_plane, whose finalisers ride in the z pass).
 // ---------------------------------------------------------------------------
 constexpr int kFinThreads = 1024;
 constexpr int kFinSmem = 128;   // doubles of shared memory a finaliser needs
@@ -986,12 +986,25 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
                     a = run.phase ? pre1[s] : pre0[s];
                     n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a,
                                                run.phase ? pre0[s] : pre1[s]);
+                    pre0[s] = a;   // kept for the Q terms
+                    pre1[s] = n;
                 } else {
                     a = cur[idx];
                     n = mode_update<P, SCHEME>(v[s], cur, old, idx, m2, coef, c4, sub, update, a, old[idx]);
+                    if (want_q) q = Q::add(q, Q::term(n.x, n.y, a, __ldg(w2tab + m2), qr, twice));
                 }
-                if (want_q) q = Q::add(q, Q::term(n.x, n.y, a, __ldg(w2tab + m2), qr, twice));
                 v[s] = cmake<R>(P::from_f64(n.x), P::from_f64(n.y));
+            }
+        }
+        // the Q terms' code (eight copies, 40 KB) stays out of the other steps' way, which had to fetch
+        // around it: 13.1 -> 11.5, 14.3 -> 13.0, 19.1 -> 18.0 us a step at 16, 32, 64^3
+        if constexpr (kTail) {
+            if (want_q && valid) {
+#pragma unroll
+                for (int s = 0; s < 8; s++) {
+                    const int kz = j + T * s, mz = kz <= N / 2 ? kz : kz - N;
+                    q = Q::add(q, Q::term(pre1[s].x, pre1[s].y, pre0[s], __ldg(w2tab + mxy2 + mz * mz), qr, twice));
+                }
             }
         }
     }

@@ -6,8 +6,8 @@
 // within one z-plane only, and a plane fits in the shared memory of one CTA (N <= 32) or of two
 // (N = 64: 34 KB; two so that 128 SMs share the work and not 64).  So a step is two kernels,
 // this one and the z pass, instead of four; the finalisers ride in the last CTA of the z pass.
-// Measured (us a step, before and after): 18.0 -> 13.1 at 16^3, 18.9 -> 14.3 at 32^3, 21.2 -> 19.1 at
-// 64^3; a step with its energy read 65 -> 51 at 64^3.  What is left is each kernel's start, its first
+// Measured (us a step, before and after): 18.0 -> 11.5 at 16^3, 18.9 -> 13.0 at 32^3, 21.2 -> 18.0 at
+// 64^3; a step with its energy read 65 -> 50 at 64^3.  What is left is each kernel's start, its first
 // loads and the instruction stream of eight points a thread, one warp a scheduler.
 //
 // CTA r of the CL of a plane owns the kx columns [r CW, (r+1) CW) (the last one also the Nyquist
