@@ -48,9 +48,9 @@ PAPER_TABLE1 = [("Hornet", 12288, 0.319), ("Juqueen", 262144, 0.350), ("Stampede
 # DRAM bytes (read + write) per launch of a step kernel at 512^3, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; the capture is summarised under
 # profiles/), valid only for the kernel sources it was taken on: KERNEL_SOURCES hashed
-TRAFFIC_512 = {("df64", "x"): 2099839488, ("df64", "yf"): 2096962304, ("df64", "z"): 5455137792,
-               ("df64", "yi"): 2096292352}
-TRAFFIC_SOURCES_SHA = "00869fe2215bc89a"
+TRAFFIC_512 = {("df64", "x"): 2139157504, ("df64", "yf"): 2151468032, ("df64", "z"): 5602321920,
+               ("df64", "yi"): 2132845824}
+TRAFFIC_SOURCES_SHA = "c2f7ab5660916f38"
 KERNEL_SOURCES = ["kg_arith.cuh", "kg_fft.cuh", "kg_kernels.cuh", "kg_complex.cuh", "kg_launch_impl.cuh"]
 
 
