@@ -468,28 +468,32 @@ __device__ __noinline__ void finalise(const FinArgs f, double* red) {
     KgDev* dev = f.dev;
     NSum acc;
     double mx;
+    // Thread 0 advances the run state below, the level included, and the reductions hold barriers:
+    // what the branches depend on is read by every thread before that, so that a warp which comes
+    // late still takes the branch of the others.
+    const bool recording = kg_recording(dev), cplx = dev->complex_field != 0;
+    __syncthreads();
     if (f.kind == FIN_X || f.kind == FIN_X_AHEAD) {
         // after a stepping x pass: blow-up check and P^l; norm = lam h^3 / 4
         const bool ahead = f.kind == FIN_X_AHEAD;
-        const bool rec = kg_recording(dev) || ahead;
+        const bool rec = recording || ahead;
         fin_reduce<NT>(rec ? f.part_sum : nullptr, f.part_max, f.count, acc, mx, red);
-        if (dev->complex_field) mx = sqrt(mx);   // the keys were |u|^2
+        if (cplx) mx = sqrt(mx);   // the keys were |u|^2
         if (threadIdx.x == 0) state_after_x(dev, ahead, rec, mx, rec ? f.norm * acc.value() : 0.0);
     } else if (f.kind == FIN_AHEAD_DONE) {
         // the step whose x pass ran ahead: its max |u| becomes the last step's
         if (threadIdx.x == 0) dev->maxabs_last = dev->maxabs_peek;
     } else if (f.kind == FIN_PEEK) {
         fin_reduce<NT>(f.part_sum, f.part_max, f.count, acc, mx, red);
-        if (dev->complex_field) mx = sqrt(mx);
+        if (cplx) mx = sqrt(mx);
         if (threadIdx.x == 0) {
             dev->P_peek = f.norm * acc.value();
             dev->maxabs_peek = mx;
         }
     } else {
         // after the update; norm = h^3/N^3
-        const bool rec = kg_recording(dev);
-        if (rec) fin_reduce<NT>(f.part_sum, nullptr, f.count, acc, mx, red);
-        if (threadIdx.x == 0) state_after_z(dev, rec, rec ? f.norm * acc.value() : 0.0);
+        if (recording) fin_reduce<NT>(f.part_sum, nullptr, f.count, acc, mx, red);
+        if (threadIdx.x == 0) state_after_z(dev, recording, recording ? f.norm * acc.value() : 0.0);
     }
 }
 

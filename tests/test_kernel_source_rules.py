@@ -1,0 +1,39 @@
+"""Rules of the CUDA sources whose violation is a race, which no run shows reliably: read from the
+text of the kernels, on the CPU."""
+import os
+import re
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1501_04552_gb300", "csrc")
+
+
+def source(name):
+    """a source file without its comments"""
+    text = open(os.path.join(CSRC, name), encoding="utf-8").read()
+    return re.sub(r"/\*.*?\*/", "", re.sub(r"//[^\n]*", "", text), flags=re.S)
+
+
+def body(text, head):
+    """the braces after the first match of `head`"""
+    at = text.index("{", re.search(head, text).end() - 1)
+    depth = 0
+    for i in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[at:i + 1]
+    raise AssertionError("unbalanced braces after %s" % head)
+
+
+def test_finaliser_reads_the_run_state_before_it_advances():
+    """finalise(): thread 0 advances the level, and whether a level records decides which threads
+    reach the barriers of the reductions.  So every thread reads that decision ahead of a barrier,
+    once, and no branch looks at the run state again."""
+    fin = body(source("kg_kernels.cuh"), r"void finalise\(")
+    head, rest = fin.split("__syncthreads();", 1)
+    assert head.count("kg_recording(dev)") == 1 and "complex_field" in head
+    assert not re.search(r"\bif\b|fin_reduce|state_after", head)
+    assert "kg_recording" not in rest and "complex_field" not in rest
+    # what is left of the run state in the branches belongs to thread 0
+    for line in rest.split(";"):
+        if "dev->" in line or "state_after" in line:
+            assert "threadIdx.x == 0" in line or "maxabs_peek = mx" in line, line
