@@ -144,10 +144,11 @@ struct XpShape {
 };
 
 // v[s] = X1[k] + i X2[k], k = j + T s, from the half spectra L1, L2 of two x-lines
-// (Hermitian extension; the kx = 0 and N/2 entries contribute their real parts)
+// (Hermitian extension; the kx = 0 and N/2 entries contribute their real parts).  No const
+// __restrict__ pointers: the ensemble's lines are written again within the launch.
 template <class P, int N>
-__device__ __forceinline__ void x_pair_load(const typename P::S* __restrict__ L1, const typename P::S* __restrict__ L2,
-                                            int j, cx<typename P::R> (&v)[8]) {
+__device__ __forceinline__ void x_pair_load(const typename P::S* L1, const typename P::S* L2, int j,
+                                            cx<typename P::R> (&v)[8]) {
     typedef typename P::R R;
     typedef cx<R> C;
     constexpr int T = N / 8;
@@ -623,9 +624,12 @@ __global__ void __launch_bounds__(CW * N / 8, ColMinBlocks<P, CW * N / 8, N>::va
 // Fused z column of the batched ensemble: forward z FFT -> F^n, FP64 update, inverse z FFT,
 // in one pass over W2.  coef[m2] = (2 c_k, 2 beta_k) for integer m2 = mx^2 + my^2 + mz^2.
 // One (ky, kx) column (T = N/8 threads, thread j).
+// cur and old change their roles every step of a launch, so cur is not read-only for the kernel's
+// life, and it was last written by another SM: it is no const __restrict__ pointer, whose loads may
+// take the path that nothing keeps coherent.
 // ---------------------------------------------------------------------------
 template <class P, int N, class SM, bool RF = false>
-__device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const double2* __restrict__ cur,
+__device__ __forceinline__ void z_body(typename P::S* __restrict__ W, const double2* cur,
                                        double2* __restrict__ old, int kx, int ky, bool valid, int j,
                                        SM& csm, const typename P::S* __restrict__ tw,
                                        const double2* __restrict__ coef) {

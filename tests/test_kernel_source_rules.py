@@ -37,3 +37,19 @@ def test_finaliser_reads_the_run_state_before_it_advances():
     for line in rest.split(";"):
         if "dev->" in line or "state_after" in line:
             assert "threadIdx.x == 0" in line or "maxabs_peek = mx" in line, line
+
+
+def test_ensemble_bodies_claim_nothing_read_only():
+    """The bodies of the ensemble's passes run many times in one launch on arrays that earlier
+    passes of it, on other SMs, have written.  Only the tables are read-only there: no other
+    pointer may be const __restrict__, which lets loads go past the coherent path."""
+    text = source("kg_kernels.cuh") + source("kg_ensemble.cuh")
+    called = body(source("kg_ensemble.cuh"), r"void ens_x\(") + body(source("kg_ensemble.cuh"), r"void ens_y\(") + \
+        body(source("kg_ensemble.cuh"), r"void ens_z\(")
+    bodies = {n for n in re.findall(r"\b(\w+_body)<", called)} | {"x_pair_load", "x_pair_unpack", "ens_x", "ens_y", "ens_z"}
+    assert {"x_pair_body", "x_line_body", "col_body", "z_body"} <= bodies
+    for name in sorted(bodies):
+        args = re.search(r"void %s\((.*?)\)\s*\{" % name, text, re.S).group(1)
+        for a in re.split(r",(?![^<]*>)", " ".join(args.split())):
+            if "__restrict__" in a and a.strip().startswith("const "):
+                assert re.search(r"\b(tw|coef)$", a), (name, a)
