@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -505,18 +506,30 @@ int mlp_alloc(Mlp* M, void** p, size_t b) {
     return KG_OK;
 }
 
+void release_rows(Staging& s) {
+    cudaFree(s.X);
+    cudaFree(s.Y);
+    cudaFree(s.E);
+    s.X = s.Y = s.E = nullptr;
+    s.rows = 0;
+}
+void release_orders(Staging& s) {
+    for (int k = 0; k < 2; k++) {
+        cudaFree(s.idx[k]);
+        cudaFreeHost(s.h_idx[k]);
+        s.idx[k] = s.h_idx[k] = nullptr;
+    }
+    s.idx_rows = 0;
+}
+
 void mlp_destroy(Mlp* M) {
     if (!M) return;
     cudaDeviceSynchronize();
     for (void* p : M->allocs) cudaFree(p);
-    cudaFree(M->st.X);
-    cudaFree(M->st.Y);
-    cudaFree(M->st.E);
-    for (int k = 0; k < 2; k++) {
-        cudaFree(M->st.idx[k]);
-        cudaFreeHost(M->st.h_idx[k]);
-        if (M->st.sent[k]) cudaEventDestroy(M->st.sent[k]);
-    }
+    release_rows(M->st);
+    release_orders(M->st);
+    for (cudaEvent_t e : M->st.sent)
+        if (e) cudaEventDestroy(e);
     delete M;
 }
 
@@ -559,32 +572,42 @@ int set_smem_once() {
     return KG_OK;
 }
 
-// room for n rows of inputs, labels (or outputs), and with idx for two row orders
+// Test hook: KG_TEST_FAIL_STAGING=k makes the k-th allocation of a growing staging fail
+int g_staging_allocs = 0;
+template <class T>
+bool staging_fails(cudaError_t (*alloc)(void**, size_t), T** p, size_t bytes) {
+    const char* inj = std::getenv("KG_TEST_FAIL_STAGING");
+    if (inj && ++g_staging_allocs == std::atoi(inj)) return true;
+    if (alloc((void**)p, bytes) == cudaSuccess) return false;
+    cudaGetLastError();
+    *p = nullptr;
+    return true;
+}
+
+// room for n rows of inputs, labels (or outputs), and with idx for two row orders; what cannot be
+// had in full is given back
 int reserve(Staging& s, int n, bool idx) {
+    const auto device = [](void** p, size_t b) { return cudaMalloc(p, b); };
+    const auto pinned = [](void** p, size_t b) { return cudaMallocHost(p, b); };
+    g_staging_allocs = 0;
     if (n > s.rows) {
-        cudaFree(s.X);
-        cudaFree(s.Y);
-        cudaFree(s.E);
-        s.X = s.Y = s.E = nullptr;
-        s.rows = 0;
-        if (cudaMalloc((void**)&s.X, sizeof(float) * DIN * (size_t)n) != cudaSuccess ||
-            cudaMalloc((void**)&s.Y, sizeof(float) * (size_t)n) != cudaSuccess ||
-            cudaMalloc((void**)&s.E, sizeof(float) * (size_t)n) != cudaSuccess) {
-            cudaGetLastError();
+        release_rows(s);
+        if (staging_fails<float>(device, &s.X, sizeof(float) * DIN * (size_t)n) ||
+            staging_fails<float>(device, &s.Y, sizeof(float) * (size_t)n) ||
+            staging_fails<float>(device, &s.E, sizeof(float) * (size_t)n)) {
+            release_rows(s);
             return mfail(KG_ENOMEM, "mlp data allocation");
         }
         s.rows = n;
     }
     if (idx && n > s.idx_rows) {
-        s.idx_rows = 0;
+        release_orders(s);
+        for (auto& e : s.sent)
+            if (!e) KG_MCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         for (int k = 0; k < 2; k++) {
-            cudaFree(s.idx[k]);
-            cudaFreeHost(s.h_idx[k]);
-            s.idx[k] = s.h_idx[k] = nullptr;
-            if (!s.sent[k]) KG_MCK(cudaEventCreateWithFlags(&s.sent[k], cudaEventDisableTiming));
-            if (cudaMalloc((void**)&s.idx[k], sizeof(int) * (size_t)n) != cudaSuccess ||
-                cudaMallocHost((void**)&s.h_idx[k], sizeof(int) * (size_t)n) != cudaSuccess) {
-                cudaGetLastError();
+            if (staging_fails<int>(device, &s.idx[k], sizeof(int) * (size_t)n) ||
+                staging_fails<int>(pinned, &s.h_idx[k], sizeof(int) * (size_t)n)) {
+                release_orders(s);
                 return mfail(KG_ENOMEM, "mlp row order allocation");
             }
         }
@@ -593,25 +616,18 @@ int reserve(Staging& s, int n, bool idx) {
     return KG_OK;
 }
 
-// what a call keeps for the next one is bounded: staging beyond kKeepRows goes back at its end
+// What a call keeps for the next one is bounded: staging beyond kKeepRows goes back at its end,
+// however it ends.
 constexpr int kKeepRows = 1 << 20;
-void trim(Staging& s) {
-    if (s.rows > kKeepRows) {
-        cudaFree(s.X);
-        cudaFree(s.Y);
-        cudaFree(s.E);
-        s.X = s.Y = s.E = nullptr;
-        s.rows = 0;
+struct Bounded {
+    Staging& s;
+    explicit Bounded(Staging& st) : s(st) {}
+    Bounded(const Bounded&) = delete;
+    ~Bounded() {
+        if (s.rows > kKeepRows) release_rows(s);
+        if (s.idx_rows > kKeepRows) release_orders(s);
     }
-    if (s.idx_rows > kKeepRows) {
-        for (int k = 0; k < 2; k++) {
-            cudaFree(s.idx[k]);
-            cudaFreeHost(s.h_idx[k]);
-            s.idx[k] = s.h_idx[k] = nullptr;
-        }
-        s.idx_rows = 0;
-    }
-}
+};
 
 int upload(Staging& s, const float* X, const float* y, const float* ell, int n) {
     KG_MCK(cudaMemcpyAsync(s.X, X, sizeof(float) * DIN * (size_t)n, cudaMemcpyHostToDevice, 0));
@@ -669,6 +685,7 @@ int kg_mlp_predict(const float* X, int n, float* p_blowup, float* logt) {
     if (!X || n < 1) return mfail(KG_EINVAL, "bad arguments");
     int rc = set_smem_once();
     Staging& s = g_mlp->st;
+    const Bounded bounded(s);
     if (!rc) rc = reserve(s, n, false);
     if (!rc) rc = upload(s, X, nullptr, nullptr, n);
     if (rc) return rc;
@@ -679,7 +696,6 @@ int kg_mlp_predict(const float* X, int n, float* p_blowup, float* logt) {
     if (e == cudaSuccess && p_blowup) e = cudaMemcpyAsync(p_blowup, s.Y, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, 0);
     if (e == cudaSuccess && logt) e = cudaMemcpyAsync(logt, s.E, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-    trim(s);
     if (e != cudaSuccess) return mfail(KG_ECUDA, std::string("mlp forward: ") + cudaGetErrorString(e));
     return KG_OK;
 }
@@ -689,6 +705,7 @@ int kg_mlp_grad(const float* X, const float* y, const float* logt, int n, double
     if (!X || !y || !logt || n < 1 || !(T > 0.0)) return mfail(KG_EINVAL, "bad arguments");
     int rc = set_smem_once();
     Staging& s = g_mlp->st;
+    const Bounded bounded(s);
     if (!rc) rc = reserve(s, n, false);
     if (!rc) rc = upload(s, X, y, logt, n);
     if (rc) return rc;
@@ -701,7 +718,6 @@ int kg_mlp_grad(const float* X, const float* y, const float* logt, int n, double
     float l = 0.f;
     KG_MCK(cudaMemcpy(&l, g_mlp->loss, sizeof(float), cudaMemcpyDeviceToHost));
     if (loss) *loss = (double)l / n;
-    trim(s);
     return KG_OK;
 }
 
@@ -713,6 +729,7 @@ int kg_mlp_train(const float* X, const float* y, const float* logt, int n, const
     int rc = set_smem_once();
     Mlp* M = g_mlp;
     Staging& s = M->st;
+    const Bounded bounded(s);
     if (!rc) rc = reserve(s, n, true);
     if (!rc) rc = upload(s, X, y, logt, n);
     if (rc) return rc;
@@ -754,7 +771,6 @@ int kg_mlp_train(const float* X, const float* y, const float* logt, int n, const
         lastloss /= (float)((n / batch) * batch);
     }
     KG_MCK(cudaDeviceSynchronize());
-    trim(s);
     if (final_loss) *final_loss = lastloss;
     return KG_OK;
 }
