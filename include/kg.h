@@ -81,7 +81,8 @@ int kg_init(int N, double L, double dt, const double* u0, const double* v0);
 /* As kg_init with device pointers (N^3 doubles each, v0 may be NULL). */
 int kg_init_device(int N, double L, double dt, const double* d_u0, const double* d_v0);
 
-/* Enqueue n steps of Eq. (2) on the context's stream; returns once enqueued.
+/* Enqueue n steps of Eq. (2) on the context's stream; returns once enqueued (after some thousands
+ * of steps that the GPU has not begun the driver's launch queue is full, and the call waits).
  * Errors: KG_ESTATE (no context), KG_EINVAL (n < 0), KG_ECUDA. */
 int kg_step(int n);
 
