@@ -31,7 +31,6 @@ L_BOX = 32.0
 DT = 0.005
 ENERGY_EVERY = 10
 PRECISION = "df64"
-STEP_LAUNCHES = 4
 E2E_REPEATS = 3
 METRIC = "512^3 KG steps/s"
 L2_BYTES = 129 * 1000 * 1000          # GB300 L2
@@ -97,6 +96,21 @@ def kernel_groups(k_ms):
     if k_ms[3] == 0.0 and k_ms[4] == 0.0:
         return ["x", "yf", "z", "yi"], [k_ms[0], k_ms[1], k_ms[2], k_ms[5]]
     return ["x", "yf", "zf", "update", "zi", "yi"], list(k_ms)
+
+
+def timed_launches(prec, n, schedule, xy_fusion=False):
+    """kernels launched for a real field in a timed region of the given step_schedule.  A step is the
+    x, forward y, z and inverse y pass (IEEE FP64: its z pass is three kernels), the finalisers in the y
+    passes; on double-float grids up to 64^3 one kernel for the x and y passes and the z pass, which
+    finalises; in the cluster-fused form xy pass, finaliser, z pass, finaliser, and an inverse y pass
+    closes each kg_step call.  An energy evaluation runs the next step's x pass ahead and launches its
+    finaliser, where the pass does not finalise itself; the fused form has a read-only x pass too"""
+    steps, energies = sum(k for k, _ in schedule), sum(1 for _, evaluate in schedule if evaluate)
+    if xy_fusion and prec == "mixed" and n >= 64:
+        return 4 * steps + len(schedule) + 2 * energies
+    if prec == "df64" and n <= 64:
+        return 2 * steps
+    return (6 if prec == "fp64" else 4) * steps + energies
 
 
 KERNEL_NAMES = {"x": "k_pass_x", "z": "k_zstep", "update": "k_update", "xy": "k_xy_cluster"}
@@ -518,9 +532,8 @@ def main():
                            "l2": l2_note, "device_warmup_s": 0.5},
                 "roofline": roofline, "roofline_alu": roofline_alu, "cpu_baseline": base, "e2e": e2e,
                 "clocks": clocks,
-                # per step: x pass, forward y pass, z pass, inverse y pass (the finalisers ride in
-                # the y passes); per energy evaluation one finaliser (its x pass is the next step's)
-                "gpu_launches": STEP_LAUNCHES * args.steps + len(energies),
+                "gpu_launches": timed_launches(prec, NG, step_schedule(args.warmup, args.steps, ENERGY_EVERY),
+                                               args.xy_fusion),
                 "energy_series": {"every": ENERGY_EVERY, "first": energies[0] if energies else None,
                                   "max_rel_drift": (max(abs(e - energies[0]) for e in energies) / abs(energies[0])
                                                     if energies else None)},
