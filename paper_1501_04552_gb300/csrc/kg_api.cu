@@ -457,6 +457,14 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
     return KG_OK;
 }
 
+// the x pass of a real or complex field over W1
+cudaError_t x_pass(Ctx* c, int mode, cudaStream_t st) {
+    const int N = c->N;
+    if (c->cplx)
+        return c->pl->passc_x(N, mode, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, st);
+    return c->pl->pass_x(N, mode, c->W1, c->dev, c->part_sum, c->part_max, c->tw, inv_n3(N), c->lam, 0, st);
+}
+
 // one step; with timed, CUDA events split it into six kernel groups and ms[0..5]
 // accumulate their device times: x pass, forward y, forward z, update, inverse z, inverse y.
 // xy = 1 or 2: the fused form (use_xy), whose first kernel runs the x pass and the forward
@@ -487,8 +495,7 @@ int launch_step(Ctx* c, cudaStream_t st, bool timed, float* ms, int xy = 0, bool
         fx.count = c->pl->xy_parts(N);
         KG_CK(launch_fin(fx, nullptr, nullptr, st));
     } else {
-        KG_CK((c->cplx ? c->pl->passc_x : c->pl->pass_x)(N, MODE_STEP, c->W1, c->dev, c->part_sum, c->part_max, c->tw,
-                                                         inv_n3(N), c->lam, 0, st));
+        KG_CK(x_pass(c, MODE_STEP, st));
         fx.count = c->cplx ? c->pl->xc_parts(N) : c->pl->x_parts(N);
     }
     if (timed) KG_CK(cudaEventRecord(c->ev[1], st));
@@ -850,8 +857,7 @@ int kg_energy(double* E) {
         if (c->h_dev[1].P_last_level != n) return fail(KG_ECUDA, "kg_energy: the x pass run ahead recorded no P");
         Pn = c->h_dev[1].P_last;
     } else if (!d.frozen) {
-        KG_CK((c->cplx ? c->pl->passc_x : c->pl->pass_x)(N, MODE_PEEK, c->W1, c->dev, c->part_sum, c->part_max, c->tw,
-                                                         inv_n3(N), c->lam, 0, st));
+        KG_CK(x_pass(c, MODE_PEEK, st));
         KG_CK(launch_fin(FinArgs{FIN_PEEK, c->cplx ? c->pl->xc_parts(N) : c->pl->x_parts(N), c->part_sum, c->part_max,
                                  c->dev, p_norm}, nullptr, nullptr, st));
         KgDev d2;

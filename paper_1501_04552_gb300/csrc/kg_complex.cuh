@@ -40,7 +40,7 @@ struct XcMinBlocks {
 template <class P, int N, int MODE>
 __global__ void __launch_bounds__(XcStep<N>::NT, XcMinBlocks<P, N>::value)
     k_pass_xc(typename P::S* __restrict__ W, KgDev* __restrict__ dev, double* __restrict__ part_sum,
-              double* __restrict__ part_max, const typename P::S* __restrict__ tw, double scale, double lam, int record) {
+              double* __restrict__ part_max, const typename P::S* __restrict__ tw, double scale, double lam) {
     typedef typename P::S S;
     typedef typename P::R R;
     typedef cx<R> C;
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(XcStep<N>::NT, XcMinBlocks<P, N>::value)
     const size_t line = (size_t)blockIdx.x * X::LPC + li;
     LineSmemX<P, X::CTA_SYNC> lsm{sm + li * X::PADN, 1u + (unsigned)li, (unsigned)T};
     pdl_wait();
-    const bool want_sum = (MODE == MODE_PEEK) || record || kg_recording(dev);
+    const bool want_sum = (MODE == MODE_PEEK) || kg_recording(dev);
     const R rlam = P::from_f64(lam);
     S* __restrict__ L = W + line * N;
     Stats<P> st;

@@ -83,8 +83,8 @@ cudaError_t update(int N, void* W, double2* S0, double2* S1, KgDev* dev, double*
 int update_parts(int N) { return Lp::update_parts(N); }
 #elif KG_PART == 3
 cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale,
-                    double lam, int record, cudaStream_t st) {
-    return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, record, st);
+                    double lam, cudaStream_t st) {
+    return Lp::passc_x(N, mode, W, dev, ps, pm, tw, scale, lam, st);
 }
 int xc_parts(int N) { return Lp::xc_parts(N); }
 cudaError_t yfc(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st) {

@@ -72,7 +72,7 @@ struct PassLaunch {
     // complex field (full N^3 spectrum, N columns per plane): x pass, column FFTs,
     // column FFT from an FP64 source, update, and their partial counts
     cudaError_t (*passc_x)(int N, int mode, void* W, KgDev* dev, double* part_sum, double* part_max, const void* tw,
-                           double scale, double lam, int record, cudaStream_t st);
+                           double scale, double lam, cudaStream_t st);
     int (*xc_parts)(int N);
     cudaError_t (*yfc)(int N, const void* W1, void* W2, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);
     cudaError_t (*yic)(int N, const void* W2, void* W1, const void* tw, int lg, const FinArgs& fin, cudaStream_t st);

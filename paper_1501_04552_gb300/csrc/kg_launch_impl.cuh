@@ -240,21 +240,21 @@ struct Launchers {
     // ---- complex field ----
     template <int N, int MODE>
     static cudaError_t passc_x_n(void* W, KgDev* dev, double* ps, double* pm, const void* tw, double scale, double lam,
-                                 int record, cudaStream_t st) {
+                                 cudaStream_t st) {
         typedef XcShape<N, XcStep<N>::NT> X;
         static std::atomic<unsigned long long> done{0};
         const size_t smem = (size_t)X::LPC * X::PADN * sizeof(S);
         cudaError_t e = set_smem_once(k_pass_xc<P, N, MODE>, smem, done);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_pass_xc<P, N, MODE>, N * N / X::LPC, XcStep<N>::NT, smem, st, (S*)W, dev, ps, pm,
-                          (const S*)tw, scale, lam, record);
+                          (const S*)tw, scale, lam);
     }
     static cudaError_t passc_x(int N, int mode, void* W, KgDev* dev, double* ps, double* pm, const void* tw,
-                               double scale, double lam, int record, cudaStream_t st) {
+                               double scale, double lam, cudaStream_t st) {
         if (mode == MODE_STEP) {
-            KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_STEP>(W, dev, ps, pm, tw, scale, lam, record, st)));
+            KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_STEP>(W, dev, ps, pm, tw, scale, lam, st)));
         }
-        KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_PEEK>(W, dev, ps, pm, tw, scale, lam, record, st)));
+        KG_DISPATCH_N(N, return (passc_x_n<NN, MODE_PEEK>(W, dev, ps, pm, tw, scale, lam, st)));
     }
     static int xc_parts(int N) {
         KG_DISPATCH_N(N, return (NN * NN / XcShape<NN, XcStep<NN>::NT>::LPC));
