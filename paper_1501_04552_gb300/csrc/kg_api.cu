@@ -401,7 +401,7 @@ int init_common(int N, double L, double dt, const double* u0, const double* v0, 
     Tables tb{c->tw, c->tw64, c->coef, c->w2};
     c->scheme = g_scheme;
     KG_TRY(init_state(N, c->prec, dt, c->lam, tb, c->phys, v0, device_ptrs, c->S0, c->S1, c->W1, c->W2, c->tmp, st,
-                      c->scheme == KG_SCHEME_COMPOSED4 ? c->kick : nullptr, true));
+                      c->scheme == KG_SCHEME_COMPOSED4 ? c->kick : nullptr));
     take_planes(c);
     KgDev d = fresh_dev();
     d.scheme = c->scheme;
@@ -440,7 +440,7 @@ int init_common_c(int N, double L, double dt, const double* u0, const double* v0
     // F^0 = FFT(lam |u0|^2 u0) waits in the FP64 scratch
     Tables tb{c->tw, c->tw64, c->coef, c->w2};
     rc = init_state_c(N, c->prec, dt, c->lam, tb, (double2*)c->phys, (const double2*)v0, device_ptrs, c->S0, c->S1,
-                      c->W1, c->W2, c->tmp, st, true);
+                      c->W1, c->W2, c->tmp, st);
     KgDev d = fresh_dev();
     d.complex_field = 1;
     if (!rc && cudaMemcpyAsync(c->dev, &d, sizeof(d), cudaMemcpyHostToDevice, st) != cudaSuccess)

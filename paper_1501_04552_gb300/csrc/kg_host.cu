@@ -145,11 +145,11 @@ int make_kick_tables(int N, double L, double dt, const AllocFn& alloc, double2**
 
 int init_state(int N, int prec, double dt, double lam, const Tables& tb, double* phys, const double* v0,
                bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
-               const double2* kick0, bool pass_precision) {
+               const double2* kick0) {
     const size_t slots = spec_slots(N, false), n3 = (size_t)N * N * N;
     const PassLaunch* pl = launcher_for(prec);
     if (!pl) return set_last_error(KG_EINVAL, "unknown precision");
-    const bool pass = pass_precision && pl->x_setup != nullptr;
+    const bool pass = pl->x_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
         return pass ? forward3d_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
                     : forward3d(N, phys, (double2*)W2, out, tb.tw64, cube, lam, pl->lg(N), st);
@@ -172,12 +172,11 @@ int init_state(int N, int prec, double dt, double lam, const Tables& tb, double*
 }
 
 int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, double2* phys, const double2* v0,
-                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
-                 bool pass_precision) {
+                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st) {
     const size_t n3 = (size_t)N * N * N;
     const PassLaunch* pl = launcher_for(prec);
     if (!pl) return set_last_error(KG_EINVAL, "unknown precision");
-    const bool pass = pass_precision && pl->xc_setup != nullptr;
+    const bool pass = pl->xc_setup != nullptr;
     auto fwd = [&](double2* out, int cube) {
         return pass ? forward3d_c_pass(N, pl, phys, W1, W2, out, tb.tw, cube, lam, st)
                     : forward3d_c(N, phys, (double2*)W2, out, tb.tw64, cube, lam, pl->lg(N), st);

@@ -184,17 +184,16 @@ int make_kick_tables(int N, double L, double dt, const AllocFn& alloc, double2**
 // S0 = uh^0, S1 = uh^{-1} (startup level of Eq. (2)) or, with kick0 (the composed
 // scheme's first merged-kick table), S1 = P^0; W1 = yz-inverse of uh^0 in the pass
 // precision.  W2 and fbuf are scratch of 16 bytes per slot (W2 is the step's second work
-// array).  The transforms run in FP64, or with pass_precision (and a precision that has
-// x_setup) in the pass precision through W1 and W2.
+// array).  The transforms run in the pass precision where it has x_setup, through W1 and W2, and
+// in FP64 elsewhere.
 int init_state(int N, int prec, double dt, double lam, const Tables& tb, double* phys, const double* v0,
                bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
-               const double2* kick0 = nullptr, bool pass_precision = false);
+               const double2* kick0 = nullptr);
 
 // the same for a complex field: phys and v0 hold N^3 complex values, the spectral arrays
 // the full N^3 spectrum
 int init_state_c(int N, int prec, double dt, double lam, const Tables& tb, double2* phys, const double2* v0,
-                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st,
-                 bool pass_precision = false);
+                 bool v0_on_device, double2* S0, double2* S1, void* W1, void* W2, double2* fbuf, cudaStream_t st);
 
 // record a failure for kg_last_error(); returns code
 int set_last_error(int code, const std::string& msg);
