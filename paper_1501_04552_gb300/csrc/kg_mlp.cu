@@ -39,7 +39,11 @@ constexpr int BT = 128;                          // batch rows of a tile
 constexpr int NTH = 1024;
 constexpr int RT = BT / 16;                      // row tiles: warp w has row tile w % RT, columns 32 (w / RT) ..
 static_assert(RT * (DH / 32) == NTH / 32, "the warps tile the activations");
-constexpr int kMostParts = 64;                   // CTAs (and partial gradients) of a backward launch
+// CTAs (and partial gradients) of a backward launch.  Batches up to 8192 rows have a CTA a tile.  Larger
+// ones take several tiles a CTA: training on them waits for the host, which draws the row order (16384
+// rows a batch: 101 us with 64, 128 and 152 CTAs alike); a gradient by itself would gain from the
+// other SMs (65 536 rows, kg_mlp_grad: 178 us with 64, 131 with 128 or 152).
+constexpr int kMostParts = 64;
 constexpr int NPARAM = DIN * DH + DH + DH * DH + DH + DH * DOUT + DOUT;
 // offsets of the tensors in the flat parameter vector (order W1, b1, W2, b2, W3, b3)
 constexpr int OW1 = 0, OB1 = OW1 + DIN * DH, OW2 = OB1 + DH, OB2 = OW2 + DH * DH, OW3 = OB2 + DH,
@@ -689,8 +693,11 @@ int kg_mlp_predict(const float* X, int n, float* p_blowup, float* logt) {
     if (!rc) rc = reserve(s, n, false);
     if (!rc) rc = upload(s, X, nullptr, nullptr, n);
     if (rc) return rc;
-    const int tiles = (n + BT - 1) / BT, most = 152;   // a CTA per SM, over several tiles
-    k_mlp_forward<<<tiles < most ? tiles : most, NTH, sizeof(Smem)>>>(params_of(g_mlp), s.X, n, p_blowup ? s.Y : nullptr,
+    int dev = 0, sms = 0;
+    KG_MCK(cudaGetDevice(&dev));
+    KG_MCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int tiles = (n + BT - 1) / BT;   // a CTA per SM, over several tiles
+    k_mlp_forward<<<tiles < sms ? tiles : sms, NTH, sizeof(Smem)>>>(params_of(g_mlp), s.X, n, p_blowup ? s.Y : nullptr,
                                                                       logt ? s.E : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && p_blowup) e = cudaMemcpyAsync(p_blowup, s.Y, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, 0);
