@@ -25,18 +25,20 @@ def body(text, head):
 
 
 def test_finaliser_reads_the_run_state_before_it_advances():
-    """finalise(): thread 0 advances the level, and whether a level records decides which threads
-    reach the barriers of the reductions.  So every thread reads that decision ahead of a barrier,
-    once, and no branch looks at the run state again."""
-    fin = body(source("kg_kernels.cuh"), r"void finalise\(")
-    head, rest = fin.split("__syncthreads();", 1)
-    assert head.count("kg_recording(dev)") == 1 and "complex_field" in head
-    assert not re.search(r"\bif\b|fin_reduce|state_after", head)
-    assert "kg_recording" not in rest and "complex_field" not in rest
-    # what is left of the run state in the branches belongs to thread 0
-    for line in rest.split(";"):
-        if "dev->" in line or "state_after" in line:
-            assert "threadIdx.x == 0" in line or "maxabs_peek = mx" in line, line
+    """finalise(): thread 0 advances the level after the update, and whether a level records decides
+    which threads reach the barriers of the reductions.  So every thread reads that decision once,
+    ahead of the branches, and a barrier that all threads reach stands before the advance.  The other
+    branches leave alone what the decision is made of."""
+    text = source("kg_kernels.cuh")
+    fin = body(text, r"void finalise\(")
+    assert fin.count("kg_recording(dev)") == 1
+    assert not re.search(r"\bif\b|fin_reduce|state_after", fin[:fin.index("kg_recording(dev)")])
+    last = fin[fin.rindex("else {"):]
+    assert "state_after_z" in last and fin.count("state_after_z") == 1
+    statements = [" ".join(x.split()) for x in last.strip("else {}\n ").split(";") if x.strip()]
+    assert statements[-2] == "__syncthreads()" and statements[-1].startswith("if (threadIdx.x == 0) state_after_z(")
+    writes = set(re.findall(r"dev->(\w+)\s*(?:=|\+=|\^=)[^=]", body(text, r"void state_after_x\(") + fin))
+    assert not writes & {"level", "energy_every", "complex_field"}, writes
 
 
 def test_ensemble_bodies_claim_nothing_read_only():
