@@ -49,7 +49,7 @@ const PassLaunch* launcher(int prec) { return launcher_for(prec); }
 int g_alloc_counter = 0;
 
 // kg_step: steps of a graph, and step kernels launched one by one before graphs take over
-constexpr int kGraphSteps = 16, kMostQueued = 768;
+constexpr int kGraphSteps = 32, kMostQueued = 768;
 
 struct Ctx {
     int N = 0, NH = 0, prec = KG_DF64;
@@ -738,11 +738,13 @@ int kg_step(int n) {
         }
         return xy_close(c, st, false, nullptr);
     }
-    // Launches measured as fast as graphs of 16 steps (20.4 against 19.7 us a step at 32^3) and
-    // need none built (0.1 to 0.4 ms), but about 1024 of them fill the driver's queue, and the next
-    // waits for the GPU.  So what exceeds kMostQueued since the host last waited goes out as
-    // graphs, an entry of the queue each: at 256^3 a call of 1000 steps came back after 318 of its 428 ms
-    // by launches alone.  A stream that the caller captures takes launches only.
+    // Launches measured as fast as graphs and need none built (0.1 to 0.4 ms), but about 1024 of them
+    // fill the driver's queue, and the next waits for the GPU.  So what exceeds kMostQueued since the
+    // host last waited goes out as graphs, an entry of the queue each: at 256^3 a call of 1000 steps came
+    // back after 318 of its 428 ms by launches alone.  A graph ends with a gap of some 9 us; 32 steps
+    // each (FP64 at 64^3, 1000 steps: 64.75 ms by launches, 65.27 in graphs of 16, 64.67 of 32, 64.47 of 64)
+    // leave at most 31 steps to launches at the end of a call, which the queue still holds.  A stream
+    // that the caller captures takes launches only.
     const int per = c->plane ? 2 : c->pl->zstep ? 4 : 6;
     for (long long i = 0; i < passes;) {
         bool graph = c->queued + per > kMostQueued && passes - i >= kGraphSteps;

@@ -1,5 +1,5 @@
 """kg_step returns once its steps are enqueued: the driver's queue holds about a thousand launches,
-so long calls go out as graphs of 16 steps after the first few hundred launches.  A long call must be
+so long calls go out as graphs of 32 steps after the first few hundred launches.  A long call must be
 bit for bit the same steps as single calls (energies recorded, a blow-up between, every form of a
 step), come back long before the GPU is done, and be only launches on a stream that is being captured."""
 import time
