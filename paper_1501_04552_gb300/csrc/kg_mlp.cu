@@ -39,11 +39,11 @@ constexpr int BT = 128;                          // batch rows of a tile
 constexpr int NTH = 1024;
 constexpr int RT = BT / 16;                      // row tiles: warp w has row tile w % RT, columns 32 (w / RT) ..
 static_assert(RT * (DH / 32) == NTH / 32, "the warps tile the activations");
-// CTAs (and partial gradients) of a backward launch.  Batches up to 8192 rows have a CTA a tile.  Larger
-// ones take several tiles a CTA: training on them waits for the host, which draws the row order (16384
-// rows a batch: 101 us with 64, 128 and 152 CTAs alike); a gradient by itself would gain from the
-// other SMs (65 536 rows, kg_mlp_grad: 178 us with 64, 131 with 128 or 152).
-constexpr int kMostParts = 64;
+// CTAs (and partial gradients) of a backward launch.  Batches up to 16384 rows have a CTA a tile, larger
+// ones several tiles a CTA.  Training on large batches waits for the host, which draws the row order
+// (16384 rows a batch: 98 us with 64 and 128 alike); a gradient by itself does not (kg_mlp_grad of 65 536
+// rows: 205 us with 64, 145 with 128).
+constexpr int kMostParts = 128;
 constexpr int NPARAM = DIN * DH + DH + DH * DH + DH + DH * DOUT + DOUT;
 // offsets of the tensors in the flat parameter vector (order W1, b1, W2, b2, W3, b3)
 constexpr int OW1 = 0, OB1 = OW1 + DIN * DH, OW2 = OB1 + DH, OB2 = OW2 + DH * DH, OW3 = OB2 + DH,
@@ -233,7 +233,10 @@ __global__ void __launch_bounds__(NTH) k_mlp_forward(Params P, const float* X, i
 }
 
 // partial gradients of the mean loss over rows idx[0..n) (idx may be NULL: rows 0..n), scaled by
-// inv_n, of this CTA's tiles into part[blockIdx.x], its loss sum into loss_part[blockIdx.x]
+// inv_n, of this CTA's tiles into part[blockIdx.x], its loss sum into loss_part[blockIdx.x].  A CTA
+// with several tiles adds each one's gradients to its part in global memory, with rounding: left in the
+// accumulators, whose additions truncate, they drifted with the number of tiles: 65 536 and 262 144
+// rows were 8.9e-7 and 4.1e-6 of the gradient from 64 bits, and are 2.3e-7 and 7.0e-7.
 __global__ void __launch_bounds__(NTH) k_mlp_backward(Params P, const float* X, const float* Y, const float* ELL,
                                                       const int* idx, int n, float inv_n, float logT, float* part,
                                                       float* loss_part) {
@@ -261,8 +264,8 @@ __global__ void __launch_bounds__(NTH) k_mlp_backward(Params P, const float* X, 
     for (int i = threadIdx.x; i < BT * LK; i += NTH) s.dz[i] = 0;   // columns 2..15 stay zero
     kg::pdl_wait();   // the weights of the step before
     load_weights(s, P);
-    float d1[4] = {}, d2[4][4] = {}, d3[4] = {};   // dW1, dW2, dW3 accumulators
-    float db = 0.f, lsum = 0.f, db3a = 0.f, db3b = 0.f;
+    float lsum = 0.f, db3a = 0.f, db3b = 0.f;
+    float* out = part + (size_t)blockIdx.x * NPARAM;
     unsigned a[4], b[4];
     for (int row0 = blockIdx.x * BT; row0 < n; row0 += gridDim.x * BT) {
         if (row0 != (int)blockIdx.x * BT) {
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(NTH) k_mlp_backward(Params P, const float* X, 
         }
         kg::cp_async_wait_all();
         __syncthreads();
+        float d1[4] = {}, d2[4][4] = {}, d3[4] = {}, db = 0.f;   // dW1, dW2, dW3, db1 or db2 of the tile
         float c3[4];
         forward_tile(s, c3);
         if (w < RT && t == 0) {   // dz = dL/dz per row
@@ -374,21 +378,32 @@ __global__ void __launch_bounds__(NTH) k_mlp_backward(Params P, const float* X, 
 #pragma unroll 16
             for (int r = 0; r < BT; r++) db += from_bf(col[r * LH]);
         }
-    }
-    float* out = part + (size_t)blockIdx.x * NPARAM;
+        const bool add = row0 != (int)blockIdx.x * BT;
+        auto put = [&](int at, float x, float y) {   // a thread's own pairs, the same in every tile
+            float2* p = reinterpret_cast<float2*>(out + at);
+            if (add) {
+                const float2 v = *p;
+                x += v.x;
+                y += v.y;
+            }
+            *p = make_float2(x, y);
+        };
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const int f1 = 16 * (w & 7) + g, f2 = 32 * (w >> 3) + 8 * q + 2 * t;
-        *reinterpret_cast<float2*>(out + OW2 + f1 * DH + f2) = make_float2(d2[q][0], d2[q][1]);
-        *reinterpret_cast<float2*>(out + OW2 + (f1 + 8) * DH + f2) = make_float2(d2[q][2], d2[q][3]);
+        for (int q = 0; q < 4; q++) {
+            const int at = OW2 + (16 * (w & 7) + g) * DH + 32 * (w >> 3) + 8 * q + 2 * t;
+            put(at, d2[q][0], d2[q][1]);
+            put(at + 8 * DH, d2[q][2], d2[q][3]);
+        }
+        if (w < 16 && g < DIN) put(OW1 + g * DH + 8 * w + 2 * t, d1[0], d1[1]);
+        if (w < 8 && t == 0) {
+            put(OW3 + (16 * w + g) * DOUT, d3[0], d3[1]);
+            put(OW3 + (16 * w + g + 8) * DOUT, d3[2], d3[3]);
+        }
+        if (w >= 16 && w < 24) {
+            const int i = threadIdx.x - 512, at = i < DH ? OB2 + i : OB1 + i - DH;
+            out[at] = add ? out[at] + db : db;
+        }
     }
-    if (w < 16 && g < DIN) *reinterpret_cast<float2*>(out + OW1 + g * DH + 8 * w + 2 * t) = make_float2(d1[0], d1[1]);
-    if (w < 8 && t == 0) {
-        *reinterpret_cast<float2*>(out + OW3 + (16 * w + g) * DOUT) = make_float2(d3[0], d3[1]);
-        *reinterpret_cast<float2*>(out + OW3 + (16 * w + g + 8) * DOUT) = make_float2(d3[2], d3[3]);
-    }
-    if (w >= 16 && w < 20) out[OB2 + threadIdx.x - 512] = db;
-    else if (w >= 20 && w < 24) out[OB1 + threadIdx.x - 512 - DH] = db;
     // loss and db3: warp sums, then the row warps in order
     if (w < RT) {
 #pragma unroll
