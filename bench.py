@@ -47,9 +47,9 @@ PAPER_TABLE1 = [("Hornet", 12288, 0.319), ("Juqueen", 262144, 0.350), ("Stampede
 # DRAM bytes (read + write) per launch of a step kernel at 512^3, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; the capture is summarised under
 # profiles/), valid only for the kernel sources it was taken on: KERNEL_SOURCES hashed
-TRAFFIC_512 = {("df64", "x"): 2139157504, ("df64", "yf"): 2151468032, ("df64", "z"): 5602321920,
-               ("df64", "yi"): 2132845824}
-TRAFFIC_SOURCES_SHA = "c2f7ab5660916f38"
+TRAFFIC_512 = {("df64", "x"): 2138958592, ("df64", "yf"): 2151354624, ("df64", "z"): 5602414080,
+               ("df64", "yi"): 2132867072}
+TRAFFIC_SOURCES_SHA = "3e5e7b8f99e4f13c"
 KERNEL_SOURCES = ["kg_arith.cuh", "kg_fft.cuh", "kg_kernels.cuh", "kg_complex.cuh", "kg_launch_impl.cuh"]
 
 
@@ -426,16 +426,16 @@ def main():
                 "kernels": per_kernel}
     if prec == "df64":
         roofline["limiter"] = ("arithmetic, not HBM: the double-float transforms are bound by the FP32 lanes of the "
-                               "FMA pipes (packed FP32x2 instructions; x and y passes about 0.62-0.70 of their peak, "
+                               "FMA pipes (packed FP32x2 instructions; x and y passes about 0.67-0.72 of their peak, "
                                "ncu FMA pipe 75 % busy with math-pipe-throttle stalls in the x pass), and the fused z "
-                               "pass adds the FP64 update on the FP64 pipe (frac_pipes of roofline_alu.kernels.z); "
+                               "pass runs the FP64 update on the FP64 pipe in turn with them (frac_pipes of roofline_alu.kernels.z); "
                                "their HBM fraction is low by construction")
     roofline_alu = None
     if prec == "df64" and NG == 512:
         ops = df64_fp32_ops(NG)
         # the fused z pass: two column transforms on the FP32 pipe and the update on the FP64
-        # pipe (6 DFMA per mode); frac_pipes adds the two pipes' busy fractions, the share of
-        # the kernel's time their minimum times fill when they do not overlap
+        # pipe (6 DFMA per mode); frac_pipes adds the two pipes' busy fractions: near 1 it says that
+        # the two kinds of work take turns, not that the kernel is at a bound
         kops = {n: ops["x"] if n == "x" else (2 * ops["col"] if n == "z" else ops["col"]) for n in names}
         per = {n: {"ops": kops[n], "frac": round(kops[n] / (t * 1e-3) / FP32_ISSUE_PEAK, 4)}
                for n, t in zip(names, k_avg) if n != "update"}

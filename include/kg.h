@@ -252,9 +252,11 @@ unsigned long long kg_state_checksum(const void* p, size_t n);
  * u0 = A[i] exp(-|x|^2 / s[i]^2), v0 = 0, in the precision and nonlinearity of the
  * current options.  Up to 50 time steps of the whole ensemble are one persistent
  * cooperative kernel launch, in which bounded waits order the passes of each
- * instance.  One ensemble per process; independent of the kg_init context.  Errors:
- * KG_EINVAL, KG_ENOTSUP, KG_ENOMEM, KG_ECUDA, KG_ETIMEOUT (a bounded wait gave up;
- * the ensemble state is then undefined and must be re-initialised). */
+ * instance.  An instance holds two FP64 state arrays and two work arrays: 75.5 MB at 128^3
+ * in double-float and FP64 (56.6 MB in FP32), 10.5 MB (7.9 MB) at 64^3.
+ * One ensemble per process; independent of the kg_init context.  Errors: KG_EINVAL,
+ * KG_ENOTSUP, KG_ENOMEM, KG_ECUDA, KG_ETIMEOUT (a bounded wait gave up; the ensemble
+ * state is then undefined and must be re-initialised). */
 int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, const double* s);
 
 /* Advance every instance that has not blown up by up to max_steps steps.  With
@@ -282,7 +284,10 @@ int kg_ens_fetch(int i, double* u);
  * length is not a power of 8 (the 128^3 instances) -- times the unit order (0: the grid
  * size of the first instance first, 1: larger grids first) times the resident CTAs per SM.  Every shape computes the
  * same step; schedules with bit 1 differ from the others in the rounding of the
- * transforms only.  Advances the ensemble.  blocks_per_sm and order may be NULL. */
+ * transforms only.  Advances the ensemble.  blocks_per_sm and order may be NULL.  A line of
+ * the cache file is taken whatever version of the library wrote it: a shape tuned for an
+ * earlier kernel may be slower than the untuned one, so tune again after an update (which
+ * replaces the line). */
 int kg_ens_tune(int steps, int* blocks_per_sm, int* order);
 
 /* The launch shape of the current ensemble (any pointer may be NULL). */

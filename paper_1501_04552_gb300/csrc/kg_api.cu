@@ -1043,7 +1043,7 @@ int kg_set_scheme(int scheme) {
 int kg_set_xy_fusion(int on) {
     if (on != 0 && on != 1) return fail(KG_EINVAL, "kg_set_xy_fusion: on must be 0 or 1");
     if (g_ctx && g_xy_fusion != on) {
-        // the next kg_step takes the other form; W holds the y-inverse between calls in both
+        // the next kg_step takes the other form; W1 holds the y-inverse between calls in both
         cudaStream_t st = stream_of(g_ctx);
         KG_CK(cudaStreamSynchronize(st));
     }

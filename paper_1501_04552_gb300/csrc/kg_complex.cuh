@@ -27,7 +27,7 @@ struct XcShape {
 };
 
 // resident threads per SM the complex x pass is compiled for (the largest count whose
-// register budget needs no spills, FP64 excepted); as XMinBlocks below 128^3
+// register budget needs at most 24 bytes of spills); as XMinBlocks below 128^3
 template <class P, int N>
 struct XcMinBlocks {
     static constexpr int kThreads = std::is_same<P, PrecF64>::value ? 512 : 1024;

@@ -376,7 +376,7 @@ int kg_ens_init(int count, const int* Ns, double L, double dt, const double* A, 
     e->dt = dt;
     e->lam = opt.nonlinearity;
     e->Ns.assign(Ns, Ns + count);
-    const char* miss = std::getenv("KG_TEST_ENS_MISSING_CTA");   // test hook: force a barrier timeout
+    const char* miss = std::getenv("KG_TEST_ENS_MISSING_CTA");   // test hook: force a wait to run out
     if (miss && std::atoi(miss) == 1) {
         e->missing = 1;
         e->spin_limit = 1ll << 16;

@@ -298,8 +298,10 @@ __global__ void __launch_bounds__(kEnsMaxInst) k_ens_plan(EnsParams p, int order
     }
 }
 
-// resident CTAs per SM the step kernel is compiled for (the autotuner picks up to this many);
-// FP32 compiled for five and six spilled in the z body and was 8 and 14 % slower
+// resident CTAs per SM the step kernel is compiled for (the autotuner picks up to this many).  At 64
+// registers the double-float z bodies spill 180 to 272 bytes and the FP32 ones up to 96 (128^3,
+// half-width tiles or the short stage first), and four CTAs are still the fastest of those measured: FP32
+// compiled for five and six spilled more and was 8 and 14 % slower
 template <class P>
 struct EnsMinBlocks {
     static constexpr int value = 2;

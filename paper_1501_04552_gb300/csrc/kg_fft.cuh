@@ -60,12 +60,12 @@ enum { MODE_STEP = 0, MODE_PEEK = 1 };
 // The z pass reads and writes five arrays' worth of data against two for a y pass, and with
 // rows a whole plane (2.1 MB at N = 512) apart it reached 0.7 of the copy bandwidth; the
 // scattered rows now fall to the y passes, which write or read them at little cost (512^3: z
-// pass 1.764 -> 1.543 ms double-float with tiles of eight columns, 1.389 with tiles of four;
-// 0.998 -> 0.785 ms FP32).  TW is a property of a context's precision and grid (LayLg): four
+// pass 1.764 -> 1.543 ms double-float with tiles of eight columns, 1.386 with tiles of four;
+// 0.998 -> 0.780 ms FP32).  TW is a property of a context's precision and grid (LayLg): four
 // columns, 64-byte rows of 16-byte values, for double-float at 512^3 (at 256^3 the z pass gains
 // nothing, 0.185 against 0.184 ms, and the y passes lose 3 %); eight for FP32, whose y passes lose
 // more on 32-byte rows (0.213 -> 0.257 ms) than its z pass gains (0.761 -> 0.736), and for FP64,
-// which is bound by its arithmetic.  The FP64 kernels that serve every context take lg at run time.
+// which is bound by its arithmetic (these FP32 times are of the passes alone, outside a run).  The FP64 kernels that serve every context take lg at run time.
 template <class P, int N>
 struct LayLg {
     static constexpr int value = std::is_same<P, PrecDF>::value && N >= 512 ? 2 : 3;
@@ -314,7 +314,8 @@ __device__ __forceinline__ const S* stage_table(const S* __restrict__ g, S* sm, 
 // column tile: element (row, column c) at base[row * C + c]; the whole CTA syncs
 // Where rows are shorter than the 128 bytes of one wavefront, the rows that share 128 bytes are
 // swapped by the row's bits 3.. (a stage writes rows eight apart and reads consecutive ones), so
-// that neither side has bank conflicts (FP32 tiles of eight: z pass 0.794 -> 0.759 ms at 512^3)
+// that neither side has bank conflicts (FP32 tiles of eight: z pass at 512^3 0.794 -> 0.759 ms by itself,
+// 0.789 -> 0.781 in a run)
 template <class P, int C>
 __device__ __forceinline__ int col_slot(int row, int c) {
     constexpr int Q = 128 / (C * (int)sizeof(typename P::S));   // rows per 128 bytes

@@ -247,7 +247,8 @@ struct XPaired<PrecF64> {
 };
 
 // resident threads per SM the x pass is compiled for: the paired double-float body fits
-// 1024 (64 registers, no spills; 1.61 -> 1.44 ms at 512^3 against 512); the pipelined
+// 1024 (64 registers and 8 to 20 bytes of spills; 1.61 -> 1.44 ms at 512^3 against 512 when it
+// was measured); the pipelined
 // FP32 body measured slower at 768 (0.48 -> 0.51 ms), and the FP64 body needs its registers.
 // Below 128^3 the grid does not fill the SMs and every body keeps its registers.
 template <class P, int N>
@@ -853,8 +854,9 @@ __global__ void __launch_bounds__(kUpdThreads, 6) k_update(typename P::S* __rest
 // over W2: 2 W + 3 S per launch instead of 6 W + 3 S for the three kernels.
 // C columns of N rows per CTA (ZStepShape).  The state is read with plain loads after the forward
 // transform; on large grids, whose arrays do not stay in L2, one thread has asked L2 for the
-// tile's two contiguous state runs before it (one bulk prefetch each).  512^3: 1.561 -> 1.548 ms
-// double-float, 0.777 -> 0.746 ms FP32; 256^3: 0.185 -> 0.179 and 0.118 -> 0.106 ms.
+// tile's two contiguous state runs before it (one bulk prefetch each).  The pass by itself, with
+// tiles of eight columns, 512^3: 1.561 -> 1.548 ms double-float, 0.777 -> 0.746 ms FP32; 256^3: 0.185 ->
+// 0.179 and 0.118 -> 0.106 ms.
 // ---------------------------------------------------------------------------
 // [p, p + bytes) of global memory into L2 (16-byte aligned, a multiple of 16 bytes)
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
@@ -863,16 +865,17 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
 
 // columns per CTA: one tile of z-columns from N = 32 on.  Four double-float columns make CTAs of 256
 // threads at 512^3, four per SM where eight made two of 512: their phases interleave more and wait
-// less (1.543 -> 1.389 ms).
+// less (1.543 -> 1.386 ms).
 template <class P, int N>
 struct ZStepShape {
     static constexpr int C = N >= 32 ? 1 << LayLg<P, N>::value : 16;
     static constexpr int NT = C * N / 8;
     static constexpr bool kPrefetch = N >= 256;
 };
-// resident threads per SM the kernel is compiled for: 1024 (64 registers); 1536 for the
-// FP32 passes at N = 512, whose smaller body fits 40 registers and gains from the extra
-// loads in flight (1.046 -> 1.005 ms; not measured at other sizes, which keep 1024)
+// resident threads per SM the kernel is compiled for: 1024 (64 registers; double-float 44 to 56
+// bytes of spills, complex 72 to 92, composed 108 to 248); 1536 for the FP32 passes at N = 512: 40
+// registers and 96 bytes of spills, which the extra loads in flight outweigh (0.798 -> 0.780 ms, 0.854
+// -> 0.834 with the energy every 10 steps; not measured at other sizes, which keep 1024)
 template <class P, int N>
 struct ZStepMinBlocks {
     static constexpr int kThreads = (sizeof(typename P::S) == 8 && N >= 512) ? 1536 : 1024;
@@ -967,7 +970,7 @@ __global__ void __launch_bounds__(ZStepShape<P, N>::NT, ZStepMinBlocks<P, N>::va
         if (dir == 1) break;
         // the run state is read only now, so that nothing of it is live across the
         // forward transform (at 64 registers: 132 -> 8 bytes of spills, 1.98 -> 1.91 ms
-        // for the double-float pass at 512^3)
+        // for the double-float pass at 512^3 in the layout before; 56 bytes now)
         const KgDev* rs = dev;
         if constexpr (kTail) rs = &run;
         rec = kg_recording(rs);
