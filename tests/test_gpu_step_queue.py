@@ -36,7 +36,8 @@ def result(kg, N, cplx):
 # two, four and six launches a step, three passes a step (composed); calls that end inside a graph's worth
 @pytest.mark.parametrize("N,prec,scheme,cplx,steps", [(16, "df64", "eq2", False, 450), (32, "mixed", "eq2", False, 233),
                                                       (16, "fp64", "eq2", False, 200), (16, "df64", "composed4", False, 140),
-                                                      (32, "fp64", "composed4", False, 60), (16, "df64", "eq2", True, 230)])
+                                                      (32, "fp64", "composed4", False, 60), (16, "df64", "eq2", True, 230),
+                                                      (64, "df64", "eq2", False, 450)])
 @pytest.mark.parametrize("amplitude", [0.3, 4.0])
 def test_long_calls_are_the_single_steps(kg, N, prec, scheme, cplx, steps, amplitude):
     u = I.gaussian(N, L, amplitude, 4.0)
